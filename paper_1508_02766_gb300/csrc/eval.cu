@@ -518,8 +518,11 @@ __device__ __forceinline__ void cols_body_slab(const ColsParams<T>& p, int64_t s
     }
   }
   if (MODE == COL_FWD_POWER) return;
-  // Every warp's result sits in the same buffer of its pair (same plan).
-  const int zoff = (z == a) ? 0 : P;
+  // Every line's result sits in the same buffer of its pair, told by the
+  // number of stages run (not by this thread's z: the group of a column
+  // beyond S ran none, and its threads store other columns too).
+  const int nfft = (MODE == COL_MID || MODE == COL_AUTO) ? 2 : 1;
+  const int zoff = (nfft * p.lp.nst) & 1 ? P : 0;
   __syncthreads();
   const int nout = (MODE == COL_FWD) ? P : p.Nout;
   for (int idx = threadIdx.x; idx < nout * W; idx += blockDim.x) {

@@ -71,6 +71,19 @@ def test_small_grids_every_node(K, d, M, prec, method, cols, engine):
 
 
 @pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("M", [(10, 60, 62), (10, 63, 64), (9, 64, 30)])
+def test_stockham_column_tail(K, M, prec):
+    """3-D column passes with an odd number of radix stages along axis 1 and
+    an odd number of columns (the last block holds a column beyond them)."""
+    w = W.small_case(21, 3, M, n=500, precision=prec)
+    dens, counts, _, plan = run_gpu(K, w, method="direct", engine="stockham", cols="lines")
+    assert len(plan.info.radices[1]) % 2 == 1 and plan.info.Q % 2 == 1
+    f, c_ref, _, _ = oracle_full(w)
+    assert np.array_equal(counts, c_ref)
+    assert rel_err(dens, f) <= TOL[prec]
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
 def test_support_is_whole_grid(K, prec):
     """L = M - 1 on every axis (a wide H): every lag of Eq. 5 is kept."""
     w = W.small_case(7, 2, (24, 19), n=500, precision=prec)
