@@ -31,6 +31,7 @@
 #include <cmath>
 #include <cstdint>
 
+#include "fixed_pos.h"
 #include "kde_debug.cuh"
 #include "kde_internal.h"
 #include "pdl.cuh"
@@ -76,8 +77,9 @@ __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(
 // with 0 <= q < 2^32.  A fraction that rounds to exactly 2^32 (f = 1) is
 // written as (i + 1, q = 0), which gives bit-identical weights:
 // floor((w 2^32 + 2^31) / 2^32) = w and floor((w 0 + 2^31) / 2^32) = 0.
-// The scaling by 2^32 is exact in either type; FP32 inputs stay in 32-bit
-// arithmetic throughout.  Returns false if t is outside [0, M-1] or NaN.
+// The scaling by 2^32 is exact; FP32 inputs stay in 32-bit arithmetic
+// throughout, FP64 ones take fixed_position (two FP64 instructions an axis).
+// Returns false if t is outside [0, M-1] or NaN.
 __device__ __forceinline__ bool fixed_frac(float f, int& i, unsigned& q) {
   if (f == 1.0f) {
     i += 1;
@@ -87,17 +89,6 @@ __device__ __forceinline__ bool fixed_frac(float f, int& i, unsigned& q) {
   }
   return true;
 }
-__device__ __forceinline__ bool fixed_frac(double f, int& i, unsigned& q) {
-  unsigned long long Q = __double2ull_rn(f * 4294967296.0);
-  if (Q == kOne) {
-    i += 1;
-    q = 0;
-  } else {
-    q = (unsigned)Q;
-  }
-  return true;
-}
-
 template <typename T>
 __device__ __forceinline__ bool axis_position(T x, const BinAxis<T>& a, int& i, unsigned& q) {
   T t = mul_rn(sub_rn(x, a.lo), a.s);
@@ -110,6 +101,17 @@ __device__ __forceinline__ bool axis_position(T x, const BinAxis<T>& a, int& i, 
     f = T(1);
   }
   return fixed_frac(f, i, q);
+}
+
+// FP64: the position as V = i 2^32 + q (fixed_pos.h).
+__device__ __forceinline__ bool axis_fixed(double x, const BinAxis<double>& a,
+                                           unsigned long long& V) {
+  uint64_t v = 0;
+  const bool in = kde::fixed_position(
+      (uint64_t)__double_as_longlong(mul_rn(sub_rn(x, a.lo), a.s)),
+      (uint64_t)__double_as_longlong(a.top), &v);
+  V = v;
+  return in;
 }
 
 // The 2^d corner weights of the hierarchical split (axis 0 first); corner c
@@ -138,6 +140,35 @@ __device__ __forceinline__ void corner_weights(const unsigned* q, unsigned long 
 // each warp instruction's lane pairs coalesce into one sector request where
 // one lane per sample would issue two: the scattered-sector rate of the L2
 // is what bounds this kernel.
+// The corners of lane parity par of a sample at (i, q) into counts.
+template <typename T, int D>
+__device__ __forceinline__ void add_corners(const int* i, const unsigned* q, int par,
+                                            const BinParams<T>& p,
+                                            unsigned long long* __restrict__ counts) {
+  constexpr int H = 1 << (D - 1);
+  int64_t base = par;
+#pragma unroll
+  for (int k = 0; k < D; ++k) base += (int64_t)i[k] * p.ax[k].stride;
+  // weights over the first D - 1 axes, then this lane's half of the last split
+  unsigned long long w[H];
+  if (D == 1) {
+    w[0] = kOne;
+  } else {
+    corner_weights<D - 1>(q, w);
+  }
+#pragma unroll
+  for (int c = 0; c < H; ++c) {
+    const unsigned long long hi = mulhi_round(w[c], q[D - 1]);
+    const unsigned long long wc = par ? hi : w[c] - hi;
+    if (wc == 0) continue;
+    int64_t idx = base;
+#pragma unroll
+    for (int k = 0; k < D - 1; ++k)
+      if ((c >> (D - 2 - k)) & 1) idx += p.ax[k].stride;
+    if (KDE_DCHECK(idx >= 0 && idx < p.cells, KDE_DBG_BIN_DIRECT)) atomicAdd(counts + idx, wc);
+  }
+}
+
 // Block blk of nblk blocks on samples [0, n) of X into counts.
 template <typename T, int D>
 __device__ __forceinline__ void bin_direct_body(const T* __restrict__ X, int64_t n,
@@ -145,54 +176,81 @@ __device__ __forceinline__ void bin_direct_body(const T* __restrict__ X, int64_t
                                                 unsigned long long* __restrict__ counts,
                                                 unsigned long long* __restrict__ n_out, int blk,
                                                 int nblk) {
-  constexpr int H = 1 << (D - 1);
-  constexpr int U = 8;  // samples whose coordinates are loaded before any is added
+  constexpr int U = 8;  // samples of a lane pair loaded before any is added
   const int par = threadIdx.x & 1;
   unsigned long long outside = 0;
   const int64_t step = ((int64_t)nblk * blockDim.x) >> 1;
-  for (int64_t s0 = (blk * (int64_t)blockDim.x + threadIdx.x) >> 1; s0 < n; s0 += U * step) {
-    T xs[U][D];
+  int64_t s0 = (blk * (int64_t)blockDim.x + threadIdx.x) >> 1;
+  if constexpr (sizeof(T) == 8) {
+    // FP64 samples: the position arithmetic is the expensive part (FP64
+    // pipe), so lane parity p locates the pair's samples u = p (mod 2) only
+    // and the lanes exchange the located positions.  The loop bound is the
+    // warp's first sample, so that every lane reaches each exchange.
+    // GB300 (event times): 4*10^6 FP64 samples onto 2017 x 3001 274 -> 61 us,
+    // 10^6 onto 75 x 91 x 110 113 -> 64 us, bound by the L2's scattered adds
+    // like FP32 samples.
+    const int64_t lane_s = (threadIdx.x & 31) >> 1;
+    for (; s0 - lane_s < n; s0 += U * step) {
+      T xs[U / 2][D];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int64_t s = s0 + u * step;
+      for (int v = 0; v < U / 2; ++v) {
+        const int64_t s = s0 + (2 * v + par) * step;
 #pragma unroll
-      for (int k = 0; k < D; ++k) xs[u][k] = s < n ? X[s * D + k] : T(0);
+        for (int k = 0; k < D; ++k) xs[v][k] = s < n ? X[s * D + k] : T(0);
+      }
+      kde::pdl_wait();   // as below
+#pragma unroll
+      for (int v = 0; v < U / 2; ++v) {
+        const bool mine = s0 + (2 * v + par) * step < n;
+        unsigned long long V[D];
+        bool in = mine;
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+          V[k] = 0;
+          in &= axis_fixed(xs[v][k], p.ax[k], V[k]);
+        }
+        outside += mine && !in;
+        const unsigned ok = __ballot_sync(0xffffffffu, in);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {   // sample 2 v + h, located by the lane of parity h
+          int i[D];
+          unsigned q[D];
+          const int src = (threadIdx.x & 30) | h;
+#pragma unroll
+          for (int k = 0; k < D; ++k) {
+            const unsigned long long W = __shfl_sync(0xffffffffu, V[k], src);
+            i[k] = (int)(W >> 32);
+            q[k] = (unsigned)W;
+          }
+          if ((ok >> src) & 1) add_corners<T, D>(i, q, par, p, counts);
+        }
+      }
     }
-    // launched as a dependent of the kernel that zeroes the counts: the
-    // samples' loads above overlap it; the adds below wait for it
-    kde::pdl_wait();
+  } else {
+    for (; s0 < n; s0 += U * step) {
+      T xs[U][D];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (s0 + u * step >= n) break;
-      int i[D];
-      unsigned q[D];
-      bool in = true;
+      for (int u = 0; u < U; ++u) {
+        const int64_t s = s0 + u * step;
 #pragma unroll
-      for (int k = 0; k < D; ++k) in &= axis_position<T>(xs[u][k], p.ax[k], i[k], q[k]);
-      if (!in) {
-        outside += par == 0;
-        continue;
+        for (int k = 0; k < D; ++k) xs[u][k] = s < n ? X[s * D + k] : T(0);
       }
-      int64_t base = par;
+      // launched as a dependent of the kernel that zeroes the counts: the
+      // samples' loads above overlap it; the adds below wait for it
+      kde::pdl_wait();
 #pragma unroll
-      for (int k = 0; k < D; ++k) base += (int64_t)i[k] * p.ax[k].stride;
-      // weights over the first D - 1 axes, then this lane's half of the last split
-      unsigned long long w[H];
-      if (D == 1) {
-        w[0] = kOne;
-      } else {
-        corner_weights<D - 1>(q, w);
-      }
+      for (int u = 0; u < U; ++u) {
+        if (s0 + u * step >= n) break;
+        int i[D];
+        unsigned q[D];
+        bool in = true;
 #pragma unroll
-      for (int c = 0; c < H; ++c) {
-        const unsigned long long hi = mulhi_round(w[c], q[D - 1]);
-        const unsigned long long wc = par ? hi : w[c] - hi;
-        if (wc == 0) continue;
-        int64_t idx = base;
-#pragma unroll
-        for (int k = 0; k < D - 1; ++k)
-          if ((c >> (D - 2 - k)) & 1) idx += p.ax[k].stride;
-        if (KDE_DCHECK(idx >= 0 && idx < p.cells, KDE_DBG_BIN_DIRECT)) atomicAdd(counts + idx, wc);
+        for (int k = 0; k < D; ++k) in &= axis_position<T>(xs[u][k], p.ax[k], i[k], q[k]);
+        if (!in) {
+          outside += par == 0;
+          continue;
+        }
+        add_corners<T, D>(i, q, par, p, counts);
       }
     }
   }
@@ -323,16 +381,24 @@ static_assert(pad_cells<3>() < (1 << 16) && pad_cells<2>() < (1 << 16) && pad_ce
 // fixed_frac writes a fraction of one.  kWithQ = false leaves q = 0 for
 // FP32 inputs, where i does not depend on it (f < 1 - 2^-25, so f 2^32
 // never rounds up to 2^32); FP64 fractions can round up, which moves i, so
-// they are always computed.
+// they are always computed (fixed_position).
 template <typename T, bool kWithQ = true>
 __device__ __forceinline__ bool axis_node(T x, const BinAxis<T>& a, int& i, unsigned& q) {
-  const T t = mul_rn(sub_rn(x, a.lo), a.s);
-  const bool in = t >= T(0) && t <= a.top;
-  const T fl = floor(t);
-  i = (int)fl;
-  q = 0;
-  if (kWithQ || sizeof(T) == 8) fixed_frac(sub_rn(t, fl), i, q);
-  return in;
+  if constexpr (sizeof(T) == 8) {
+    unsigned long long V = 0;
+    const bool in = axis_fixed(x, a, V);
+    i = (int)(V >> 32);
+    q = (unsigned)V;
+    return in;
+  } else {
+    const T t = mul_rn(sub_rn(x, a.lo), a.s);
+    const bool in = t >= T(0) && t <= a.top;
+    const T fl = floor(t);
+    i = (int)fl;
+    q = 0;
+    if (kWithQ) fixed_frac(sub_rn(t, fl), i, q);
+    return in;
+  }
 }
 
 // One sample located on the grid: base node i and fractions q per axis, its

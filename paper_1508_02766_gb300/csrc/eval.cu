@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "fft_engine.cuh"
+#include "fixed_pos.h"
 #include "kde_internal.h"
 #include "kde_debug.cuh"
 #include "kgen.cuh"
@@ -2651,29 +2652,27 @@ __device__ __forceinline__ bool lite_fixed(float f, int& i, unsigned& q) {
   }
   return true;
 }
-__device__ __forceinline__ bool lite_fixed(double f, int& i, unsigned& q) {
-  const unsigned long long Q = __double2ull_rn(f * 4294967296.0);
-  if (Q == (1ull << 32)) {
-    i += 1;
-    q = 0;
-  } else {
-    q = (unsigned)Q;
-  }
-  return true;
-}
-
 template <typename T>
 __device__ __forceinline__ bool lite_position(T x, const BinAxisLite<T>& a, int& i, unsigned& q) {
   const T t = rn_mul(rn_sub(x, a.lo), a.s);
-  if (!(t >= T(0) && t <= a.top)) return false;
-  const T fl = floor(t);
-  i = (int)fl;
-  T f = rn_sub(t, fl);
-  if (i == a.M - 1) {
-    i = a.M - 2;
-    f = T(1);
+  if constexpr (sizeof(T) == 8) {
+    uint64_t V = 0;
+    const bool in = fixed_position((uint64_t)__double_as_longlong(t),
+                                   (uint64_t)__double_as_longlong(a.top), &V);
+    i = (int)(V >> 32);
+    q = (unsigned)V;
+    return in;
+  } else {
+    if (!(t >= T(0) && t <= a.top)) return false;
+    const T fl = floor(t);
+    i = (int)fl;
+    T f = rn_sub(t, fl);
+    if (i == a.M - 1) {
+      i = a.M - 2;
+      f = T(1);
+    }
+    return lite_fixed(f, i, q);
   }
-  return lite_fixed(f, i, q);
 }
 
 __device__ __forceinline__ unsigned lite_mulhi(unsigned long long w, unsigned q) {
