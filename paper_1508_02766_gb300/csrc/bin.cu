@@ -187,8 +187,8 @@ __device__ __forceinline__ void bin_direct_body(const T* __restrict__ X, int64_t
     // and the lanes exchange the located positions.  The loop bound is the
     // warp's first sample, so that every lane reaches each exchange.
     // GB300 (event times): 4*10^6 FP64 samples onto 2017 x 3001 274 -> 61 us,
-    // 10^6 onto 75 x 91 x 110 113 -> 64 us, bound by the L2's scattered adds
-    // like FP32 samples.
+    // 10^6 onto 75 x 91 x 110 113 -> 64 us, then bound by the L2's scattered
+    // adds like FP32 samples.
     const int64_t lane_s = (threadIdx.x & 31) >> 1;
     for (; s0 - lane_s < n; s0 += U * step) {
       T xs[U / 2][D];

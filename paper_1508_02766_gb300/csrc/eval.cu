@@ -1409,6 +1409,9 @@ kde_status kernel_grid_impl(kde_plan_s* plan, int64_t n, void* Kspec, void* ws, 
   rp.lp = line_plan(I, dl);
   rp.tw = twiddles<T>(plan, dl);
   if (d == 1) {
+    bool taken = false;
+    const kde_status s1 = line1d_kernel_grid<T>(plan, gen, (T*)Kspec, st, &taken);
+    if (s1 != KDE_OK || taken) return s1;
     rp.nrows = 1;
     rp.out_real = (T*)Kspec;
     return launch_rows<T>(kde_rows_r2c_kgen_kernel<T>, "kde_rows_r2c_kgen_kernel", 1, rp, st, gen);
@@ -1480,6 +1483,9 @@ kde_status fft_eval_impl(kde_plan_s* plan, const int64_t* counts, const void* Ks
       return fx_fft_eval(plan, cnt, (const float*)Kspec, (float*)density, ws, st);
   }
   if (d == 1) {
+    bool taken = false;
+    const kde_status s1 = line1d_eval<T>(plan, cnt, (const T*)Kspec, (T*)density, st, &taken);
+    if (s1 != KDE_OK || taken) return s1;
     const int P = (int)I.P[0];
     auto* fn = kde_line1d_kernel<T>;
     cudaError_t e = allow_smem(fn);

@@ -55,11 +55,20 @@ kde_status dft_tc_setup(kde_plan_s* plan);
 kde_status dft_tc_rows(const kde_plan_s* plan, const long long* counts, int64_t rows, void* out,
                        cudaStream_t st);
 
+template <typename T>
+struct KGen;
+// One-dimensional plans spread over the chip (line1d.cu); *taken = false,
+// with nothing launched, where the one-block kernels are the shorter.
+template <typename T>
+kde_status line1d_eval(const kde_plan_s* plan, const long long* counts, const T* K, T* density,
+                       cudaStream_t st, bool* taken);
+template <typename T>
+kde_status line1d_kernel_grid(const kde_plan_s* plan, const KGen<T>& gen, T* Kspec,
+                              cudaStream_t st, bool* taken);
+
 // Two-phase engine (eval_fx.cu, KDE_F32 plans with engine
 // KDE_ENGINE_TWO_PHASE): the kernel grid and its spectrum, and the
 // evaluation, with the same arguments as the Stockham passes.
-template <typename T>
-struct KGen;
 kde_status fx_kernel_grid(kde_plan_s* plan, const KGen<float>& gen, void* Kspec, void* ws,
                           cudaStream_t st);
 kde_status fx_fft_eval(kde_plan_s* plan, const long long* counts, const float* Kspec,
