@@ -4,7 +4,10 @@
 // Integer addition is associative, so the counts are bit-identical whatever
 // order the additions happen in.
 //
-// Two implementations of the same arithmetic:
+// Implementations of the same arithmetic:
+//   private each block's chunk added in shared memory into a copy of the whole
+//           grid, the copies added into the counts (small grids with many
+//           samples per cell, taken by the direct method's own rule);
 //   direct  one pass, 64-bit integer atomics straight into the counts (no
 //           scratch; bound by the rate of scattered L2 sector operations,
 //           ~2^(d-1) + 1/2 per sample);
@@ -398,6 +401,97 @@ __device__ __forceinline__ bool axis_node(T x, const BinAxis<T>& a, int& i, unsi
     q = 0;
     if (kWithQ) fixed_frac(sub_rn(t, fl), i, q);
     return in;
+  }
+}
+
+// Few cells, many samples: block-private counts in shared memory.  With the
+// direct kernel every sample's adds meet in the same few cells and the L2
+// takes them one after another; here each block adds its chunk into its own
+// copy of the whole grid and then adds that copy into the counts once.  A
+// weight w <= 2^32 goes as w mod 2^16 and w >> 16 into two 32-bit sums (a
+// 64-bit shared atomic is six times slower here), exact for the at most
+// kPrivSamples = 2^15 samples between two flushes.  The blocks start their
+// flush at different cells, so that they do not queue on the same ones.
+constexpr int kPrivThreads = 512;
+constexpr int kPrivSamples = 1 << 15;
+constexpr int kPrivCells = 24576;      // 192 KB of sums
+static_assert(2ll * kPrivCells * 4 <= 227 * 1024 - 1024, "private counts fit in shared memory");
+
+// Words of one of the two sums (a multiple of 4: cleared as uint4).
+__host__ __device__ constexpr int priv_words(int64_t cells) { return (int)((cells + 3) & ~(int64_t)3); }
+
+template <typename T, int D>
+__global__ void __launch_bounds__(kPrivThreads)
+kde_bin_private_kernel(const T* __restrict__ X, int64_t n, int64_t chunk, BinParams<T> p,
+                       unsigned long long* __restrict__ counts,
+                       unsigned long long* __restrict__ n_out) {
+  extern __shared__ __align__(16) unsigned priv_sm[];
+  constexpr int U = 4;   // samples loaded before any is added
+  const int cells = (int)p.cells;
+  unsigned* lo = priv_sm;
+  unsigned* hi = priv_sm + priv_words(cells);
+  kde::pdl_trigger();
+  unsigned long long outside = 0;
+  const int64_t end = min(n, (blockIdx.x + 1) * chunk);
+  for (int64_t beg = blockIdx.x * chunk; beg < end; beg += kPrivSamples) {
+    for (int j = threadIdx.x; j < priv_words(cells) / 2; j += kPrivThreads)
+      reinterpret_cast<uint4*>(priv_sm)[j] = make_uint4(0, 0, 0, 0);   // lo and hi
+    __syncthreads();
+    const int64_t stop = min(end, beg + kPrivSamples);
+    for (int64_t s0 = beg + threadIdx.x; s0 < stop; s0 += U * kPrivThreads) {
+      T xs[U][D];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int64_t s = s0 + u * kPrivThreads;
+#pragma unroll
+        for (int k = 0; k < D; ++k) xs[u][k] = s < stop ? X[s * D + k] : T(0);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (s0 + u * kPrivThreads >= stop) break;
+        int i[D];
+        unsigned q[D];
+        bool in = true;
+#pragma unroll
+        for (int k = 0; k < D; ++k) in &= axis_node<T>(xs[u][k], p.ax[k], i[k], q[k]);
+        if (!in) {
+          ++outside;
+          continue;
+        }
+        int base = 0;
+#pragma unroll
+        for (int k = 0; k < D; ++k) base += i[k] * (int)p.ax[k].stride;
+        unsigned long long w[1 << D];
+        corner_weights<D>(q, w);
+#pragma unroll
+        for (int c = 0; c < (1 << D); ++c) {
+          int idx = base;
+#pragma unroll
+          for (int k = 0; k < D; ++k)
+            if ((c >> (D - 1 - k)) & 1) idx += (int)p.ax[k].stride;
+          // a corner beyond the last node has weight zero
+          if (w[c] == 0 || !KDE_DCHECK(idx >= 0 && idx < cells, KDE_DBG_BIN_DIRECT)) continue;
+          const unsigned l = (unsigned)w[c] & 0xFFFFu;
+          if (l) atomicAdd(lo + idx, l);
+          atomicAdd(hi + idx, (unsigned)(w[c] >> 16));
+        }
+      }
+    }
+    __syncthreads();
+    kde::pdl_wait();   // the counts have been zeroed
+    const int first = (int)((int64_t)blockIdx.x * cells / gridDim.x);
+    for (int j0 = threadIdx.x; j0 < cells; j0 += kPrivThreads) {
+      int j = j0 + first;
+      if (j >= cells) j -= cells;
+      const unsigned long long v = ((unsigned long long)hi[j] << 16) + lo[j];
+      if (v) atomicAdd(counts + j, v);
+    }
+    __syncthreads();
+  }
+  if (n_out) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) outside += __shfl_down_sync(0xffffffffu, outside, off);
+    if ((threadIdx.x & 31) == 0 && outside) atomicAdd(n_out, outside);
   }
 }
 
@@ -833,6 +927,45 @@ BinParams<T> make_params(int d, const double* lo, const double* hi, const int64_
   return p;
 }
 
+template <typename F>
+cudaError_t allow_smem(F* fn, size_t bytes) {
+  if (bytes <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+// Private counts where the grid fits and the samples are many for its cells.
+// The line per dimension is where the two kernels met for normal samples
+// (direct / private, us with the zeroing, FP32, graph of ten, GB300):
+//   d = 1: 2001 cells, 16e3 samples 3.9 / 3.3, 1e6 115 / 6.7, 5e6 567 / 12;
+//          20000 cells, 256e3 5.7 / 6.4, 1e6 16 / 8.6;
+//   d = 2: 64^2, 16e3 4.3 / 4.1, 1e6 109 / 8.9; 128^2, 64e3 4.7 / 6.8,
+//          256e3 10.8 / 6.8, 5e6 155 / 41;
+//   d = 3: 16^3, 16e3 9.2 / 5.3, 1e6 381 / 16; 28^3, 32e3 8.0 / 11,
+//          256e3 46 / 11, 5e6 861 / 69.
+// A block copies and flushes the whole grid whatever its samples, which is
+// what the line grows with; more corners per sample bring it down.
+bool use_private(int64_t n, int64_t cells, int d) {
+  const int64_t per_cell = d == 1 ? 14 : d == 2 ? 8 : 3;
+  return cells <= kPrivCells && n >= 4096 + per_cell * cells;
+}
+
+template <typename T, int D>
+kde_status launch_private(const T* X, int64_t n, const BinParams<T>& p, unsigned long long* counts,
+                          unsigned long long* n_out, cudaStream_t stream) {
+  auto* fn = kde_bin_private_kernel<T, D>;
+  const size_t smem = 2 * (size_t)priv_words(p.cells) * sizeof(unsigned);
+  cudaError_t e = allow_smem(fn, smem);
+  if (e != cudaSuccess) return kde::cuda_fail(e, "smem attr");
+  const int64_t per = std::max<int64_t>(1024, p.cells / 8);
+  const int64_t cap = (int64_t)num_sms() * (smem <= 100 * 1024 ? 2 : 1);
+  const int64_t blocks = std::min(cap, (n + per - 1) / per);
+  kde::LaunchScope ls("kde_bin_private_kernel", stream);
+  e = kde::launch_pdl(fn, dim3((unsigned)blocks), dim3(kPrivThreads), smem, stream, X, n,
+                      (n + blocks - 1) / blocks, p, counts, n_out);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  return e == cudaSuccess ? KDE_OK : kde::cuda_fail(e, "kde_bin_private_kernel launch");
+}
+
 template <typename T>
 kde_status launch_direct(const T* X, int64_t n, int d, const double* lo, const double* hi,
                          const int64_t* M, unsigned long long* counts, int64_t cells,
@@ -847,6 +980,13 @@ kde_status launch_direct(const T* X, int64_t n, int d, const double* lo, const d
   }
   if (n == 0) return KDE_OK;
   BinParams<T> p = make_params<T>(d, lo, hi, M, nullptr);
+  if (use_private(n, cells, d)) {
+    switch (d) {
+      case 1: return launch_private<T, 1>(X, n, p, counts, n_out, stream);
+      case 2: return launch_private<T, 2>(X, n, p, counts, n_out, stream);
+      default: return launch_private<T, 3>(X, n, p, counts, n_out, stream);
+    }
+  }
   int64_t want = (2 * n + 255) / 256;  // two lanes per sample
   int64_t cap = (int64_t)num_sms() * 16;
   int blocks = (int)(want < cap ? want : cap);
@@ -881,12 +1021,6 @@ kde_status launch_sets(const T* X, const int64_t* off_dev, int nsets, int64_t n_
   }
   e = cudaGetLastError();
   return e == cudaSuccess ? KDE_OK : kde::cuda_fail(e, "kde_bin_sets_kernel launch");
-}
-
-template <typename F>
-cudaError_t allow_smem(F* fn, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 // Three launches: the count kernel (after the tile counts and the item
