@@ -205,12 +205,19 @@ kde_line1d_kgen_kernel(KGen<T> gen, T* __restrict__ Kspec, int P,
   }
   __syncthreads();
   const int q = blockIdx.x * kQ + lane;
-  T s = 0;
+  T s = 0, e = 0;
   if (q < Q) {
     int m = (int)((int64_t)q * (w + 1) % P);
     const int step = (int)((int64_t)q * 8 % P);
     for (int l = w + 1; l <= L; l += 8) {
-      s = fma(kv[l], cs[2 * m <= P ? m : P - m], s);
+      const T c = cs[2 * m <= P ? m : P - m];
+      if (sizeof(T) == 4) {   // Kahan: FP32 sums of many terms lose digits the transform keeps
+        const T y = fma(kv[l], c, -e), t = s + y;
+        e = (t - s) - y;
+        s = t;
+      } else {
+        s = fma(kv[l], c, s);
+      }
       m += step;
       if (m >= P) m -= P;
     }
