@@ -916,116 +916,361 @@ __global__ void __launch_bounds__(32) kde_lscv_reduce_kernel(LscvReduce r, const
 template <typename T>
 struct AcGen {
   int L0, L1, wand;
-  int rpu;     // lag rows per work unit
-  int u0, nu;  // this matrix's work units [u0, u0 + nu)
+  int u0, nu;  // this matrix's work units [u0, u0 + nu), kAcRows lag rows each
   int set;     // whose autocorrelation: R + set * (P_0 P_1)
   T D0, D1, b_hi, b_lo, C;
 };
 
 // Up to kAcChunk candidates (2 kAcChunk matrices) per launch; their
 // parameters and work units are uploaded to the workspace.  A work unit is
-// kAcRows or more lag rows of one matrix, about kAcTerms lag terms.
+// kAcRows lag rows of one matrix (the last of a matrix fewer).
+//
+// The order of the additions is the same in every form below, so that a
+// candidate's score does not depend on how many datasets are scored with it:
+// lag l_1 belongs to class (l_1 + L_1) mod 32; a unit's class sums run over
+// its rows and, within a row, over l_1 ascending (FP32); the 32 class sums are added
+// as a warp's shuffle tree adds its lanes (FP32); a matrix's units are added
+// in order in FP64.  The FP64 part is one addition per unit: FP64 runs at 2
+// lanes a clock and SM, and a tree over 256 FP64 values for every 4096 terms
+// took longer than the terms.
 constexpr int kAcChunk = 1024;
 constexpr int kAcRows = 8;
-constexpr int kAcTerms = 4096;
 
-// Block u takes work unit units[u] = (matrix, first row), one warp per lag
-// row, and writes one FP64 partial.  blockIdx.y > 0 scores the same units
-// against autocorrelation g.set + blockIdx.y, partials at y gridDim.x.
+// K_A at lag (l0, l1) over 2 C: every lag of the half plane counts twice,
+// the lag 0 once; zero outside the support and on the other half of row 0.
+template <typename T>
+struct AcRow {
+  T t_hi, t_lo, e0;
+};
+template <typename T>
+__device__ __forceinline__ AcRow<T> ac_row(const AcGen<T>& g, int l0) {
+  const T tl = (T)l0;
+  AcRow<T> r;
+  r.t_hi = g.b_hi * tl;
+  r.t_lo = prod_lo(g.b_hi, g.b_lo, tl, r.t_hi);
+  r.e0 = g.D0 * tl * tl;
+  return r;
+}
+// 2^x by the hardware's approximation, with results below 2^-126 (1e-38 of
+// the lag 0 term) flushed to zero instead of scaled through.
+__device__ __forceinline__ float ac_ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ double ac_ex2(double x) { return exp2(x); }
+// l1: the lag as T (an integer conversion would take the exponential's unit).
+template <typename T>
+__device__ __forceinline__ T ac_term(const AcGen<T>& g, const AcRow<T>& r, T l1) {
+  const T v = ((g.wand ? fabs(l1) : l1) + r.t_hi) + r.t_lo;
+  return ac_ex2(fma(g.D1 * v, v, r.e0));
+}
+// Row 0: the lag 0 counts half, the lags below it not at all.
+template <typename T>
+__device__ __forceinline__ T ac_term0(const AcGen<T>& g, const AcRow<T>& r, T l1) {
+  const T k = ac_term(g, r, l1);
+  return l1 > T(0) ? k : l1 == T(0) ? T(0.5) * k : T(0);
+}
+// Two terms in packed arithmetic, each component rounded as ac_term's:
+// lags l.x, l.y with the parameters D1, t_hi, t_lo, e0 of each.
+__device__ __forceinline__ float2 ac_term2(float2 l, float2 D1, float2 t_hi, float2 t_lo, float2 e0) {
+  const float2 v = __fadd2_rn(__fadd2_rn(l, t_hi), t_lo);
+  const float2 e = __ffma2_rn(__fmul2_rn(D1, v), v, e0);
+  return make_float2(ac_ex2(e.x), ac_ex2(e.y));
+}
+
+// The sum over the work unit of matrix g that starts at lag row row0, by one
+// warp (lane = class); valid in lane 0.  at(r, l1): R at lag (row0 + r, l1).
+template <typename T, typename F>
+__device__ __forceinline__ double ac_unit_sum(const AcGen<T>& g, int row0, int lane, F&& at) {
+  const int r1 = min(g.L0, row0 + kAcRows - 1), first = lane - g.L1;
+  T acc = 0;
+  int l0 = row0;
+  if (l0 == 0) {
+    const AcRow<T> r = ac_row(g, 0);
+    for (int l1 = first; l1 <= g.L1; l1 += 32)
+      if (l1 >= 0) acc = fma(ac_term0(g, r, (T)l1), at(0, l1), acc);
+    ++l0;
+  }
+  for (; l0 <= r1; ++l0) {
+    const AcRow<T> r = ac_row(g, l0);
+    T f = (T)first;
+    if constexpr (sizeof(T) == 4) {
+      const float2 D1 = make_float2(g.D1, g.D1), th = make_float2(r.t_hi, r.t_hi),
+                   tl = make_float2(r.t_lo, r.t_lo), e0 = make_float2(r.e0, r.e0);
+      for (int l1 = first; l1 <= g.L1; l1 += 64, f += 64.f) {
+        float2 l = make_float2(f, f + 32.f);
+        if (g.wand) l = make_float2(fabsf(l.x), fabsf(l.y));
+        const float2 k = ac_term2(l, D1, th, tl, e0);
+        acc = fmaf(k.x, at(l0 - row0, l1), acc);
+        if (l1 + 32 <= g.L1) acc = fmaf(k.y, at(l0 - row0, l1 + 32), acc);
+      }
+    } else {
+      for (int l1 = first; l1 <= g.L1; l1 += 32, f += T(32))
+        acc = fma(ac_term(g, r, f), at(l0 - row0, l1), acc);
+    }
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+  return (double)(T(2) * g.C * acc);
+}
+
+// Lag rows row0 .. row0 + nrow - 1 of R, lags -L1 .. L1, into tile (rows of
+// 2 L1 + 1) by the whole block.
+__device__ __forceinline__ void ac_stage(float* tile, const float* __restrict__ R, int P1, int row0,
+                                         int nrow, int L1) {
+  const int W = 2 * L1 + 1;
+  for (int r = threadIdx.x >> 5; r < nrow; r += blockDim.x >> 5) {
+    const float* Rrow = R + (size_t)(row0 + r) * P1;
+#pragma unroll 4
+    for (int i = threadIdx.x & 31; i < W; i += 32)
+      tile[r * W + i] = __ldg(Rrow + (i < L1 ? i - L1 + P1 : i - L1));
+  }
+}
+
+// A block takes up to kAcBlock work units (matrix, first row) of one dataset
+// and first row, blocks[..] = (first unit, count), two to a warp:
+// partial[u nsets + y] with u the unit's place among its matrix's units, for
+// the autocorrelation g.set + y, y = blockIdx.y.  FP32: the units' lag rows are staged in shared memory once
+// (the first unit's L_1 is the largest); read from the L2 as they are used,
+// one load's latency for 32 terms was most of the kernel.
+constexpr int kAcBlock = 16;
 template <typename T>
 __global__ void __launch_bounds__(256) kde_lscv_ac_kernel(const AcGen<T>* __restrict__ gens,
                                                           const int2* __restrict__ units,
+                                                          const int2* __restrict__ blocks,
                                                           const T* __restrict__ Rall, int P1,
                                                           int64_t set_stride,
                                                           double* __restrict__ partial) {
-  const int2 u = units[blockIdx.x];
-  const AcGen<T> g = gens[u.x];
-  const T* __restrict__ R = Rall + (int64_t)(g.set + blockIdx.y) * set_stride;
-  partial += (int64_t)blockIdx.y * gridDim.x;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const int r1 = min(g.L0, u.y + g.rpu - 1);
-  T acc = 0;
-  for (int l0 = u.y + warp; l0 <= r1; l0 += nw) {
-    const T tl = (T)l0;
-    const T t_hi = g.b_hi * tl;
-    const T t_lo = prod_lo(g.b_hi, g.b_lo, tl, t_hi);
-    const T e0 = g.D0 * tl * tl;
-    const T* Rrow = R + (size_t)l0 * P1;
-    T racc = 0;
-    for (int l1 = (l0 == 0 ? 0 : -g.L1) + lane; l1 <= g.L1; l1 += 32) {
-      const T v = ((T)(g.wand ? abs(l1) : l1) + t_hi) + t_lo;
-      racc += ex2(fma(g.D1 * v, v, e0)) * __ldg(Rrow + (l1 < 0 ? l1 + P1 : l1));
-    }
-    // every lag of the half plane counts twice, the lag 0 (K = C) once
-    if (l0 == 0 && lane == 0) racc -= T(0.5) * __ldg(Rrow);
-    acc += T(2) * racc;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* tile = reinterpret_cast<T*>(smem_raw);
+  const int2 blk = blocks[blockIdx.x];
+  units += blk.x;
+  const int2 lead = units[0];
+  const AcGen<T>& gl = gens[lead.x];
+  const T* __restrict__ R = Rall + (int64_t)(gl.set + blockIdx.y) * set_stride;
+  const int lane = threadIdx.x & 31, L1 = gl.L1, W = 2 * L1 + 1, row0 = lead.y;
+  if constexpr (sizeof(T) == 4) {
+    // rows below the support of the block's longest matrix (never past R)
+    int L0 = 0;
+    for (int i = 0; i < blk.y; ++i) L0 = max(L0, gens[units[i].x].L0);
+    ac_stage(tile, R, P1, row0, min(kAcRows, L0 + 1 - row0), L1);
+    __syncthreads();
   }
-  block_sum_to((double)(g.C * acc), partial + blockIdx.x);
-}
-
-// As kde_lscv_reduce_kernel with K_{H_i}(0) and n read from memory (kn[2i],
-// kn[2i + 1]; n_all > 0 replaces every n) and scale 1; matrix 2i + h sums
-// the partials of its work units.
-template <typename T>
-__global__ void __launch_bounds__(32) kde_lscv_ac_reduce_kernel(const AcGen<T>* __restrict__ gens,
-                                                                const double* __restrict__ kn,
-                                                                double n_all,
-                                                                const double* __restrict__ partial,
-                                                                double* __restrict__ S_out,
-                                                                double* __restrict__ lscv_out) {
-  const int i = blockIdx.x;
-  double s[2];
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int u0 = gens[2 * i + h].u0, nu = gens[2 * i + h].nu;
-    double v = 0.0;
-    for (int j = threadIdx.x; j < nu; j += 32) v += partial[u0 + j];
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    s[h] = __shfl_sync(0xffffffffu, v, 0);
-  }
-  if (threadIdx.x == 0) {
-    if (S_out) {
-      S_out[2 * i] = s[0];
-      S_out[2 * i + 1] = s[1];
-    }
-    const double K0 = kn[2 * i], n = n_all > 0.0 ? n_all : kn[2 * i + 1];
-    lscv_out[i] = s[1] / (n * n) - 2.0 * (s[0] - n * K0) / (n * (n - 1.0));
+  for (int i = threadIdx.x >> 5; i < blk.y; i += 8) {
+    const AcGen<T> g = gens[units[i].x];
+    double v;
+    if constexpr (sizeof(T) == 4)
+      v = ac_unit_sum(g, row0, lane, [&](int r, int l1) { return tile[r * W + L1 + l1]; });
+    else
+      v = ac_unit_sum(g, row0, lane, [&](int r, int l1) {
+        return __ldg(R + (size_t)(row0 + r) * P1 + (l1 < 0 ? l1 + P1 : l1));
+      });
+    if (lane == 0) partial[(int64_t)(g.u0 + row0 / kAcRows) * gridDim.y + blockIdx.y] = v;
   }
 }
 
-// kde_lscv_ac_reduce_kernel for a prepared candidate set scored against
-// many autocorrelations: blockIdx.y is the dataset (its n in nset[y], its
-// partials at y nunits), outputs at y nH_all + i.
+// Many datasets scored against one candidate set.  A kernel value serves
+// every dataset, so the sums are a matrix product (matrices x lags) (lags x
+// datasets).  A warp takes the work units of kAcQuad matrices with the same
+// L_1 on one first row, lane = class as above: per lag it forms the four
+// kernel values once and sums them against kAcSets datasets, whose lags a
+// block stages in shared memory (datasets innermost, so that a lane's
+// kAcSets values are four 16-byte loads; the pitch of 20 words keeps them
+// free of bank conflicts) for its 16 warps, the next rows' copies in flight.
+// That is about 1.2 instructions a term, where one dataset at a time takes the exponential
+// again for each: 256 datasets x 2016 matrices on 256^2 grids 3181 -> 255 us
+// (event times; 1.8 G terms, 44 us at the FP32 pipes' rate; what is left is
+// the staging's copies, one block of 16 warps an SM for its registers, and
+// lanes past the supports).  Tried: the datasets innermost in memory, a
+// thread a dataset, classes one after another (897 us with four matrices a
+// thread, 323 with eight: the L2's latency at 8 to 12 warps an SM).
+constexpr int kAcQuad = 4, kAcSets = 16, kAcPitch = 20;
+constexpr int kAcTileRows = 2;   // lag rows staged at a time, two tiles in turn
+constexpr int kAcWarps = 16;
+constexpr int kAcSlab = 256;     // datasets per launch
+constexpr int kAcMinSets = 8;    // fewer are scored one by one
+
+// The matrices of one warp: the same L_1, falling L_0 (m[0]'s the largest).
+struct AcGroup {
+  int m[kAcQuad];   // matrix or -1
+  int L0, L1;
+};
+
+// Lag rows t0 .. t0 + nrow - 1 of the datasets s0 .. s0 + nset - 1 into a tile
+// (one committed group of 4-byte asynchronous copies; no copy and no value
+// for datasets beyond).
+__device__ __forceinline__ void ac_stage_sets(float* tile, const float* __restrict__ R, int P1,
+                                              int64_t set_stride, int t0, int nrow, int nset, int Lw) {
+  const int W = 2 * Lw + 1, lane = threadIdx.x & 31;
+  for (int q = threadIdx.x >> 5; q < nrow * nset; q += kAcWarps) {
+    const int r = q / nset, d = q - r * nset;
+    const float* Rrow = R + (int64_t)d * set_stride + (int64_t)(t0 + r) * P1;
+    uint32_t dst = (uint32_t)__cvta_generic_to_shared(tile + (r * W + lane) * kAcPitch + d);
+    for (int l1 = lane - Lw; l1 <= Lw; l1 += 32, dst += 32 * kAcPitch * 4)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst),
+                   "l"(__cvta_generic_to_global(Rrow + (l1 < 0 ? l1 + P1 : l1)))
+                   : "memory");
+  }
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+}
+
+__global__ void __launch_bounds__(32 * kAcWarps, 1) kde_lscv_ac_sets_kernel(
+    const AcGen<float>* __restrict__ gens, const AcGroup* __restrict__ groups,
+    const int3* __restrict__ items, const float* __restrict__ Rall, int P1, int64_t set_stride,
+    int ns, double* __restrict__ partial) {
+  extern __shared__ __align__(16) float tiles[];   // 2 x [row][l1 + Lw][kAcPitch]
+  const int3 it = items[blockIdx.x];              // first group, groups, first row
+  const int s0 = blockIdx.y * kAcSets, nset = min(kAcSets, ns - s0);
+  const int Lw = groups[it.x].L1, W = 2 * Lw + 1, row0 = it.z;   // L_1 falls along the groups
+  int Lmax = 0;
+  for (int i = 0; i < it.y; ++i) Lmax = max(Lmax, groups[it.x + i].L0);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool act = warp < it.y && groups[it.x + (warp < it.y ? warp : 0)].L0 >= row0;
+  const AcGroup gr = groups[it.x + (act ? warp : 0)];
+  AcGen<float> g[kAcQuad];
+#pragma unroll
+  for (int m = 0; m < kAcQuad; ++m) {
+    g[m] = gens[gr.m[m] >= 0 ? gr.m[m] : gr.m[0]];
+    if (gr.m[m] < 0) g[m].L0 = -1;
+  }
+  const int wand = g[0].wand;
+  float2 acc[kAcQuad][kAcSets / 2];
+#pragma unroll
+  for (int m = 0; m < kAcQuad; ++m)
+#pragma unroll
+    for (int d = 0; d < kAcSets / 2; ++d) acc[m][d] = make_float2(0.f, 0.f);
+  const float* R = Rall + (int64_t)s0 * set_stride;
+  const int end = min(Lmax + 1, row0 + kAcRows), tile_len = kAcTileRows * W * kAcPitch;
+  if (nset < kAcSets) {   // datasets beyond the last read as zeros
+    for (int i = threadIdx.x; i < 2 * tile_len; i += blockDim.x) tiles[i] = 0.f;
+    __syncthreads();
+  }
+  ac_stage_sets(tiles, R, P1, set_stride, row0, min(kAcTileRows, end - row0), nset, Lw);
+  int cur = 0;
+  for (int t0 = row0; t0 < end; t0 += kAcTileRows, cur ^= 1) {
+    const int nrow = min(kAcTileRows, end - t0);
+    const float* tile = tiles + cur * tile_len;
+    if (t0 + kAcTileRows < end)
+      ac_stage_sets(tiles + (cur ^ 1) * tile_len, R, P1, set_stride, t0 + kAcTileRows,
+                    min(kAcTileRows, end - t0 - kAcTileRows), nset, Lw);
+    else
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    __syncthreads();
+    if (act) {
+      const int r1 = min(nrow, gr.L0 + 1 - t0);
+      for (int r = 0; r < r1; ++r) {
+        const int l0 = t0 + r;
+        float2 D1[2], th[2], tl[2], e0[2];
+        float on[kAcQuad];   // 0 for a matrix whose support ends before this row
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const AcRow<float> a = ac_row(g[2 * h], l0), b = ac_row(g[2 * h + 1], l0);
+          D1[h] = make_float2(g[2 * h].D1, g[2 * h + 1].D1);
+          th[h] = make_float2(a.t_hi, b.t_hi);
+          tl[h] = make_float2(a.t_lo, b.t_lo);
+          e0[h] = make_float2(a.e0, b.e0);
+        }
+#pragma unroll
+        for (int m = 0; m < kAcQuad; ++m) on[m] = l0 <= g[m].L0 ? 1.f : 0.f;
+        float f = (float)(lane - gr.L1);
+        const float* x = tile + (r * W + lane - gr.L1 + Lw) * kAcPitch;
+        for (int l1 = lane - gr.L1; l1 - lane <= gr.L1; l1 += 32, f += 32.f, x += 32 * kAcPitch) {
+          // one factor for the lane's place: beyond the support, or row 0's
+          // other half, the terms are zero; the lag 0 counts half
+          const float w = l1 > gr.L1 ? 0.f : l0 > 0 || l1 > 0 ? 1.f : l1 == 0 ? 0.5f : 0.f;
+          const float lf = wand ? fabsf(f) : f;
+          float2 k[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            k[h] = ac_term2(make_float2(lf, lf), D1[h], th[h], tl[h], e0[h]);
+            k[h] = __fmul2_rn(k[h], make_float2(w * on[2 * h], w * on[2 * h + 1]));
+          }
+          // lanes beyond the tile's last lag read its end (times zero)
+          const float4* xv = reinterpret_cast<const float4*>(l1 > gr.L1 ? tile : x);
+          const float km[kAcQuad] = {k[0].x, k[0].y, k[1].x, k[1].y};
+#pragma unroll
+          for (int q = 0; q < kAcSets / 4; ++q) {
+            const float4 v = xv[q];
+#pragma unroll
+            for (int m = 0; m < kAcQuad; ++m) {
+              const float2 kk = make_float2(km[m], km[m]);
+              acc[m][2 * q] = __ffma2_rn(kk, make_float2(v.x, v.y), acc[m][2 * q]);
+              acc[m][2 * q + 1] = __ffma2_rn(kk, make_float2(v.z, v.w), acc[m][2 * q + 1]);
+            }
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (!act) return;
+  // the 64 sums over the lanes, halving the values a lane carries at each
+  // step: value i adds the lanes in the order of a shuffle-down tree
+  float* a = &acc[0][0].x;
+  float c[kAcQuad * kAcSets];
+#pragma unroll
+  for (int i = 0; i < kAcQuad * kAcSets; ++i) c[i] = a[i];
+  int first = 0;
+#pragma unroll
+  for (int off = 16, n = kAcQuad * kAcSets / 2; off > 0; off >>= 1, n >>= 1) {
+    const bool up = lane & off;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const float send = up ? c[i] : c[i + n], keep = up ? c[i + n] : c[i];
+      c[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+    first += up ? n : 0;
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int m = (first + i) / kAcSets, d = (first + i) % kAcSets;
+    if (d >= nset || gr.m[m] < 0) continue;
+    const AcGen<float>& gm = gens[gr.m[m]];
+    if (row0 <= gm.L0)
+      partial[(int64_t)(gm.u0 + row0 / kAcRows) * ns + s0 + d] = (double)(2.f * gm.C * c[i]);
+  }
+}
+
+// {n, 1 / n^2, 2 / (n (n - 1))}: the LSCV's factors, formed once per dataset
+// on the host (an FP64 division costs more than the rest of a score's
+// reduction).
+struct NTerms {
+  double v[3];
+};
+
+// One thread per (candidate, dataset): S(H), S(2H) as the sums of their
+// units' partials in order, and the LSCV.  The n terms are the dataset's
+// (nk_set), or nk_all, or with nk_all.v[0] = 0 the candidate's (kn: {K_H(0),
+// n terms}).  Outputs at y nH_all + i.
 template <typename T>
-__global__ void __launch_bounds__(256) kde_lscv_ac_reduce_sets_kernel(
+__global__ void __launch_bounds__(256) kde_lscv_ac_reduce_kernel(
     const AcGen<T>* __restrict__ gens, const double* __restrict__ kn,
-    const double* __restrict__ nset, const double* __restrict__ partial, int nunits, int nh,
-    int64_t nH_all, double* __restrict__ S_out, double* __restrict__ lscv_out) {
-  // one warp per candidate, eight per block
-  const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (i >= nh) return;
-  const int lane = threadIdx.x & 31;
-  const int64_t y = blockIdx.y;
-  partial += y * nunits;
+    const NTerms* __restrict__ nk_set, NTerms nk_all, const double* __restrict__ partial, int nh,
+    int ns, int64_t nH_all, double* __restrict__ S_out, double* __restrict__ lscv_out) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (int64_t)nh * ns) return;
+  const int i = (int)(t / ns), y = (int)(t - (int64_t)i * ns);
   double s[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int u0 = gens[2 * i + h].u0, nu = gens[2 * i + h].nu;
     double v = 0.0;
-    for (int j = lane; j < nu; j += 32) v += partial[u0 + j];
+#pragma unroll 8
+    for (int j = 0; j < nu; ++j) v += __ldg(partial + (int64_t)(u0 + j) * ns + y);
+    s[h] = v;
+  }
+  double nk[3];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    s[h] = __shfl_sync(0xffffffffu, v, 0);
+  for (int k = 0; k < 3; ++k)
+    nk[k] = nk_set ? nk_set[y].v[k] : nk_all.v[0] > 0.0 ? nk_all.v[k] : kn[4 * (int64_t)i + 1 + k];
+  const int64_t o = y * nH_all + i;
+  if (S_out) {
+    S_out[2 * o] = s[0];
+    S_out[2 * o + 1] = s[1];
   }
-  if (lane == 0) {
-    if (S_out) {
-      S_out[2 * (y * nH_all + i)] = s[0];
-      S_out[2 * (y * nH_all + i) + 1] = s[1];
-    }
-    const double K0 = kn[2 * i], n = nset[y];
-    lscv_out[y * nH_all + i] = s[1] / (n * n) - 2.0 * (s[0] - n * K0) / (n * (n - 1.0));
-  }
+  lscv_out[o] = s[1] * nk[1] - nk[2] * (s[0] - nk[0] * kn[4 * (int64_t)i]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1102,37 +1347,58 @@ __global__ void __launch_bounds__(128) kde_theta_gen_kernel(ThetaArgs t) {
   if (h == 0) t.K0[m >> 1] = C;
 }
 
-// One block per matrix: S(A) = sum over the support of K_A(delta o l) R(l)
-// with the lag-row arithmetic of kde_lscv_ac_kernel (one warp per lag row,
-// FP32 terms and row sums, FP64 across warps); NaN for a candidate that
-// does not fit the plan.
-__global__ void __launch_bounds__(256) kde_lscv_theta_sums_kernel(const AcGen<float>* __restrict__ gens,
-                                                                  const float* __restrict__ Rall,
-                                                                  int P1, int64_t set_stride,
-                                                                  double* __restrict__ S) {
-  const AcGen<float> g = gens[blockIdx.x];
-  if (g.L0 < 0) {
-    if (threadIdx.x == 0) S[blockIdx.x] = nan("");
-    return;
-  }
-  const float* __restrict__ R = Rall + (int64_t)g.set * set_stride;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  float acc = 0.f;
-  for (int l0 = warp; l0 <= g.L0; l0 += nw) {
-    const float tl = (float)l0;
-    const float t_hi = g.b_hi * tl;
-    const float t_lo = prod_lo(g.b_hi, g.b_lo, tl, t_hi);
-    const float e0 = g.D0 * tl * tl;
-    const float* Rrow = R + (size_t)l0 * P1;
-    float racc = 0.f;
-    for (int l1 = (l0 == 0 ? 0 : -g.L1) + lane; l1 <= g.L1; l1 += 32) {
-      const float v = ((float)(g.wand ? abs(l1) : l1) + t_hi) + t_lo;
-      racc += ex2(fmaf(g.D1 * v, v, e0)) * __ldg(Rrow + (l1 < 0 ? l1 + P1 : l1));
+// A block takes up to kThetaCands candidates of one dataset (two matrices
+// each, two to a warp): S(A) = sum over the support of K_A(delta o l) R(l),
+// kAcRows lag rows staged in shared memory at a time, the units of
+// kde_lscv_ac_kernel added in order; NaN for a matrix that does not fit the
+// plan.  256 datasets of 28 candidates with supports near the box's widest:
+// 201 -> 152 us; bound by the exponentials (336 M terms, 67 us at 16 a clock
+// and SM) and their arithmetic.
+constexpr int kThetaCands = 7;
+constexpr int kThetaThreads = 32 * kThetaCands;
+__global__ void __launch_bounds__(kThetaThreads) kde_lscv_theta_sums_kernel(
+    const AcGen<float>* __restrict__ gens, int per, const float* __restrict__ Rall, int P1,
+    int64_t set_stride, double* __restrict__ S) {
+  extern __shared__ __align__(16) float tile[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ngroups = (per + 2 * kThetaCands - 1) / (2 * kThetaCands), set = blockIdx.x / ngroups;
+  const int first = 2 * kThetaCands * (blockIdx.x - set * ngroups);
+  const int nm = min(2 * kThetaCands, per - first);
+  gens += (int64_t)set * per + first;
+  S += (int64_t)set * per + first;
+  const float* __restrict__ R = Rall + (int64_t)set * set_stride;
+  int L0 = -1, L1 = 0;
+  for (int m = 0; m < nm; ++m)
+    if (gens[m].L0 >= 0) {
+      L0 = max(L0, gens[m].L0);
+      L1 = max(L1, gens[m].L1);
     }
-    if (l0 == 0 && lane == 0) racc -= 0.5f * __ldg(Rrow);
-    acc += 2.f * racc;
+  const int W = 2 * L1 + 1;
+  AcGen<float> g[2];
+  double sum[2] = {0.0, 0.0};
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int m = warp + kThetaCands * h;
+    if (m < nm) g[h] = gens[m];
+    else g[h].L0 = -1;
   }
-  block_sum_to((double)(g.C * acc), S + blockIdx.x);
+  for (int row0 = 0; row0 <= L0; row0 += kAcRows) {
+    ac_stage(tile, R, P1, row0, min(kAcRows, L0 + 1 - row0), L1);
+    __syncthreads();
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      const AcGen<float> gh = h ? g[1] : g[0];
+      if (row0 > gh.L0) continue;
+      const double v =
+          ac_unit_sum(gh, row0, lane, [&](int r, int l1) { return tile[r * W + L1 + l1]; });
+      if (h) sum[1] += v;
+      else sum[0] += v;
+    }
+    __syncthreads();
+  }
+  if (lane == 0)
+    for (int h = 0; h < 2; ++h)
+      if (warp + kThetaCands * h < nm) S[warp + kThetaCands * h] = g[h].L0 < 0 ? nan("") : sum[h];
 }
 
 // One warp per dataset: LSCV of its J + 1 candidates (optionally stored),
@@ -1781,10 +2047,11 @@ kde_status lscv_impl(kde_plan_s* plan, int64_t n, int nH, const double* Hs, cons
 size_t ac_units_max(const kde_plan_info& I) {
   return (size_t)2 * kAcChunk * (size_t)((I.P[0] + kAcRows - 1) / kAcRows + 1);
 }
-// Uploaded per chunk: 2 nh AcGen, nh (K_H(0), n) pairs, then the work units.
+// Uploaded per chunk: 2 nh AcGen, nh x {K_H(0), n, 1/n^2, 2/(n (n-1))}, then
+// the work units and the blocks' (first unit, count).
 size_t ac_upload_bytes(const kde_plan_info& I) {
-  return ((size_t)2 * kAcChunk * sizeof(AcGen<double>) + (size_t)2 * kAcChunk * sizeof(double) +
-          ac_units_max(I) * sizeof(int2) + 255) & ~(size_t)255;
+  return ((size_t)2 * kAcChunk * sizeof(AcGen<double>) + (size_t)4 * kAcChunk * sizeof(double) +
+          2 * ac_units_max(I) * sizeof(int2) + 255) & ~(size_t)255;
 }
 
 size_t ac_workspace(const kde_plan_info& I) {
@@ -1843,18 +2110,45 @@ kde_status autocorr_impl(kde_plan_s* plan, const int64_t* counts, void* Rout, vo
   return launch_rows<T>(kde_rows_c2r_kernel<T>, "kde_rows_c2r_kernel", nsets * I.P[0], cr, st);
 }
 
+NTerms n_terms(double n) { return NTerms{{n, 1.0 / (n * n), 2.0 / (n * (n - 1.0))}}; }
+
+// The matrices by dataset (already grouped), falling L_1, then falling L_0.
+template <typename T>
+std::vector<int> ac_order(const std::vector<AcGen<T>>& gens) {
+  static_assert(KDE_MAX_P <= 4096, "supports fit in 12 bits");
+  std::vector<int64_t> key(gens.size());
+  for (size_t i = 0; i < gens.size(); ++i)
+    key[i] = (int64_t)(4095 - gens[i].L1) << 44 | (int64_t)(4095 - gens[i].L0) << 32 | (int64_t)i;
+  for (size_t i = 0, j = 0; i < key.size(); i = j) {
+    for (j = i; j < key.size() && gens[j].set == gens[i].set;) ++j;
+    std::sort(key.begin() + i, key.begin() + j);
+  }
+  std::vector<int> order(gens.size());
+  for (size_t i = 0; i < key.size(); ++i) order[i] = (int)(key[i] & 0xFFFFFFFF);
+  return order;
+}
+
+// Work units and blocks of a chunk, and its largest supports.
+struct AcShape {
+  int nunits, nblocks, L0, L1;
+};
+
 // Host side of one chunk of lag-sum candidates: candidates c = c0 ..
 // c0 + nh - 1 of set c / nH, bandwidth Hs[c], sample count ns[c / nH] (ns may
 // be NULL: n is then given at launch).  Fills `up` with the device image
-// AcGen[2 nh], (K0, n)[nh], work units; returns the unit count in *nunits.
+// AcGen[2 nh], {K0, n, 1/n^2, 2/(n (n-1))}[nh], work units (by dataset, first
+// row and falling L_1), blocks; returns their shape and, with gens_out, the
+// parameters.
 template <typename T>
 kde_status ac_build_chunk(kde_plan_s* plan, int64_t c0, int nh, int nH, const double* Hs,
-                          const int64_t* ns, std::vector<unsigned char>& up, int* nunits) {
+                          const int64_t* ns, std::vector<unsigned char>& up, AcShape* shape,
+                          std::vector<AcGen<T>>* gens_out = nullptr) {
   const kde_plan_info& I = plan->info;
   const int d = I.d;
   std::vector<AcGen<T>> gens(2 * nh, AcGen<T>{});
-  std::vector<double> kn(2 * nh, 0.0);
+  std::vector<double> kn(4 * nh, 0.0);
   std::vector<int2> units;
+  size_t nunits = 0;
   for (int i = 0; i < nh; ++i) {
     const int64_t c = c0 + i;
     const double* H = Hs + (size_t)c * d * d;
@@ -1881,51 +2175,99 @@ kde_status ac_build_chunk(kde_plan_s* plan, int64_t c0, int nh, int nH, const do
       g.b_hi = kg.Bh[0];
       g.b_lo = kg.Bl[0];
       g.C = kg.C;
-      const int W = 2 * g.L1 + 1;
-      g.rpu = std::max(kAcRows, (kAcTerms / W + kAcRows - 1) / kAcRows * kAcRows);
-      g.u0 = (int)units.size();
-      for (int r = 0; r <= g.L0; r += g.rpu) units.push_back(make_int2(2 * i + h, r));
-      g.nu = (int)units.size() - g.u0;
+      g.u0 = (int)nunits;
+      g.nu = g.L0 / kAcRows + 1;
+      nunits += g.nu;
       if (h == 0) {
-        kn[2 * i] = std::pow(6.283185307179586476925287, -0.5 * d) / std::sqrt(detA);
-        kn[2 * i + 1] = ns ? (double)ns[c / nH] : 0.0;
+        kn[4 * i] = std::pow(6.283185307179586476925287, -0.5 * d) / std::sqrt(detA);
+        const NTerms nt = ns ? n_terms((double)ns[c / nH]) : NTerms{};
+        for (int k = 0; k < 3; ++k) kn[4 * i + 1 + k] = nt.v[k];
       }
     }
   }
-  if (units.size() > ac_units_max(I)) return fail(KDE_ERR_UNSUPPORTED, "lag-sum work units overflow");
+  if (nunits > ac_units_max(I)) return fail(KDE_ERR_UNSUPPORTED, "lag-sum work units overflow");
+  // matrices by dataset and falling L_1, then each dataset's rows in turn
+  const std::vector<int> order = ac_order(gens);
+  units.reserve(nunits);
+  for (size_t i = 0, j = 0; i < order.size(); i = j) {
+    int L0 = 0;
+    for (j = i; j < order.size() && gens[order[j]].set == gens[order[i]].set; ++j)
+      L0 = std::max(L0, gens[order[j]].L0);
+    for (int r = 0; r <= L0; r += kAcRows)
+      for (size_t k = i; k < j; ++k)
+        if (r <= gens[order[k]].L0) units.push_back(make_int2(order[k], r));
+  }
+  std::vector<int2> blocks;
+  for (int u = 0; u < (int)units.size(); ++u) {
+    const bool same = !blocks.empty() && blocks.back().y < kAcBlock &&
+                      units[blocks.back().x].y == units[u].y &&
+                      gens[units[blocks.back().x].x].set == gens[units[u].x].set;
+    if (same) ++blocks.back().y;
+    else blocks.push_back(make_int2(u, 1));
+  }
+  *shape = AcShape{(int)units.size(), (int)blocks.size(), 0, 0};
+  for (const auto& g : gens) {
+    shape->L0 = std::max(shape->L0, g.L0);
+    shape->L1 = std::max(shape->L1, g.L1);
+  }
   const size_t gb = gens.size() * sizeof(AcGen<T>), kb = kn.size() * sizeof(double),
-               ub = units.size() * sizeof(int2);
-  up.resize(gb + kb + ub);
+               ub = units.size() * sizeof(int2), bb = blocks.size() * sizeof(int2);
+  up.resize(gb + kb + ub + bb);
   std::memcpy(up.data(), gens.data(), gb);
   std::memcpy(up.data() + gb, kn.data(), kb);
   std::memcpy(up.data() + gb + kb, units.data(), ub);
-  *nunits = (int)units.size();
+  std::memcpy(up.data() + gb + kb + ub, blocks.data(), bb);
+  if (gens_out) *gens_out = std::move(gens);
   return KDE_OK;
 }
 
-// Device side of one chunk whose image (ac_build_chunk) is at `img`.
+// Pointers into a chunk's device image.
 template <typename T>
-kde_status ac_launch_chunk(const kde_plan_info& I, const void* img, int nh, int nunits,
-                           const void* R, double* partial, double n_all, double* S_out,
-                           double* lscv_out, cudaStream_t st) {
-  const AcGen<T>* gens_dev = (const AcGen<T>*)img;
-  const double* kn_dev = (const double*)((const char*)img + 2 * nh * sizeof(AcGen<T>));
-  const int2* units_dev = (const int2*)((const char*)kn_dev + 2 * nh * sizeof(double));
+struct AcImage {
+  const AcGen<T>* gens;
+  const double* kn;
+  const int2 *units, *blocks;
+  AcImage(const void* img, int nh, int nunits)
+      : gens((const AcGen<T>*)img),
+        kn((const double*)((const char*)img + 2 * (size_t)nh * sizeof(AcGen<T>))),
+        units((const int2*)(kn + 4 * (size_t)nh)),
+        blocks(units + nunits) {}
+};
+
+template <typename T>
+kde_status ac_reduce(const AcImage<T>& im, int nh, int ns, const double* partial,
+                     const NTerms* nk_set, const NTerms& nk_all, int64_t nH_all, double* S_out,
+                     double* lscv_out, cudaStream_t st) {
+  LaunchScope ls("kde_lscv_ac_reduce_kernel", st);
+  const int64_t threads = (int64_t)nh * ns;
+  const int block = threads < 64 * 256 ? 64 : 256;
+  kde_lscv_ac_reduce_kernel<T><<<(unsigned)((threads + block - 1) / block), block, 0, st>>>(
+      im.gens, im.kn, nk_set, nk_all, partial, nh, ns, nH_all, S_out, lscv_out);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? KDE_OK : cuda_fail(e, "kde_lscv_ac_reduce_kernel");
+}
+
+// One chunk whose image (ac_build_chunk) is at `img` against ns
+// autocorrelations from R on, one by one (n terms as the reduction takes
+// them).  partial: nunits ns values.
+template <typename T>
+kde_status ac_launch_chunk(const kde_plan_info& I, const void* img, int nh, const AcShape& sh, const T* R,
+                           int ns, double* partial, const NTerms* nk_set, const NTerms& nk_all,
+                           int64_t nH_all, double* S_out, double* lscv_out, cudaStream_t st) {
+  const AcImage<T> im(img, nh, sh.nunits);
   cudaError_t e;
   {
+    // FP32: kAcRows staged rows of at most 2 (KDE_MAX_P / 2) - 1 lags
+    const size_t smem = sizeof(T) == 4 ? (size_t)kAcRows * (2 * sh.L1 + 1) * sizeof(T) : 0;
+    if ((e = allow_smem(kde_lscv_ac_kernel<T>)) != cudaSuccess)
+      return cuda_fail(e, "cudaFuncSetAttribute");
     LaunchScope ls("kde_lscv_ac_kernel", st);
-    kde_lscv_ac_kernel<T><<<(unsigned)nunits, 256, 0, st>>>(
-        gens_dev, units_dev, (const T*)R, (int)I.P[1], (int64_t)I.P[0] * I.P[1], partial);
+    kde_lscv_ac_kernel<T><<<dim3((unsigned)sh.nblocks, (unsigned)ns), 256, smem, st>>>(
+        im.gens, im.units, im.blocks, R, (int)I.P[1], (int64_t)I.P[0] * I.P[1], partial);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "kde_lscv_ac_kernel");
   }
-  {
-    LaunchScope ls("kde_lscv_reduce_kernel", st);
-    kde_lscv_ac_reduce_kernel<T><<<nh, 32, 0, st>>>(gens_dev, kn_dev, n_all, partial, S_out, lscv_out);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "kde_lscv_ac_reduce_kernel");
-  }
-  return KDE_OK;
+  return ac_reduce<T>(im, nh, ns, partial, nk_set, nk_all, nH_all, S_out, lscv_out, st);
 }
 
 // Candidates c = 0 .. nsets nH - 1 of set c / nH, bandwidth Hs[c], n[c / nH]:
@@ -1941,12 +2283,12 @@ kde_status lscv_ac_impl(kde_plan_s* plan, int nsets, const int64_t* ns, int nH, 
   std::vector<unsigned char> up;
   for (int64_t h0 = 0; h0 < total; h0 += kAcChunk) {
     const int nh = (int)std::min<int64_t>(kAcChunk, total - h0);
-    int nunits = 0;
-    kde_status s = ac_build_chunk<T>(plan, h0, nh, nH, Hs, ns, up, &nunits);
+    AcShape sh{};
+    kde_status s = ac_build_chunk<T>(plan, h0, nh, nH, Hs, ns, up, &sh);
     if (s != KDE_OK) return s;
     if ((s = upload_async(ws, up.data(), up.size(), st)) != KDE_OK) return s;
-    s = ac_launch_chunk<T>(I, ws, nh, nunits, R, partial, 0.0, S_out ? S_out + 2 * h0 : nullptr,
-                           lscv_out + h0, st);
+    s = ac_launch_chunk<T>(I, ws, nh, sh, (const T*)R, 1, partial, nullptr, NTerms{}, 0,
+                           S_out ? S_out + 2 * h0 : nullptr, lscv_out + h0, st);
     if (s != KDE_OK) return s;
   }
   return KDE_OK;
@@ -2349,16 +2691,21 @@ extern "C" kde_status kde_lscv_autocorr_batch(kde_plan plan, int nsets, const in
   return lscv_ac_entry(plan, nsets, n, nH, H, R, pair_sums, lscv, workspace, workspace_bytes, stream);
 }
 
-// A candidate set prepared once: its lag-sum parameters and work units live
-// on the device, so scoring it against another dataset's autocorrelation is
-// two launches per chunk of 1024 candidates with no host work.
+// A candidate set prepared once: its lag-sum parameters, work units and (FP32)
+// groups live on the device, so scoring it against other datasets'
+// autocorrelations is two launches per chunk of 1024 candidates
+// with no host work.
 struct kde_lscv_cands_s {
   kde_plan_s* plan;
   int nH;
   struct Chunk {
-    void* dev;
+    void* dev;         // image (ac_build_chunk), then groups and items
     int64_t c0;
-    int nh, nunits;
+    int nh;
+    AcShape sh;
+    AcGroup* groups;   // null: scored one by one (FP64, or a support too wide)
+    int3* items;
+    int nitems;
   };
   std::vector<Chunk> chunks;
 };
@@ -2368,17 +2715,66 @@ static void cands_free(kde_lscv_cands_s* c) {
   delete c;
 }
 
+// Supports along axis 1 up to this fit the batched sums' shared memory.
+constexpr int kAcMaxL1 = 319;
+constexpr size_t ac_tile_bytes(int L1) {
+  return (size_t)2 * kAcTileRows * (2 * L1 + 1) * kAcPitch * sizeof(float);
+}
+static_assert(ac_tile_bytes(kAcMaxL1) <= 220 * 1024, "a block's lag rows fit in shared memory");
+
+// Groups of up to kAcQuad matrices, and items of up to kAcWarps groups and a
+// first row (the widest first).
+template <typename T>
+static void cands_group(const std::vector<AcGen<T>>& gens, std::vector<AcGroup>& groups,
+                        std::vector<int3>& items) {
+  const std::vector<int> order = ac_order(gens);
+  for (size_t i = 0; i < order.size();) {
+    AcGroup g{};
+    g.L0 = gens[order[i]].L0;
+    g.L1 = gens[order[i]].L1;
+    for (int k = 0; k < kAcQuad; ++k) {
+      const bool same = i < order.size() && gens[order[i]].L1 == g.L1;
+      g.m[k] = same ? order[i++] : -1;
+    }
+    groups.push_back(g);
+  }
+  for (size_t i = 0; i < groups.size(); i += kAcWarps) {
+    const int n = (int)std::min<size_t>(kAcWarps, groups.size() - i);
+    int L0 = 0;
+    for (int k = 0; k < n; ++k) L0 = std::max(L0, groups[i + k].L0);
+    for (int r = 0; r <= L0; r += kAcRows) items.push_back(make_int3((int)i, n, r));
+  }
+}
+
 template <typename T>
 static kde_status cands_build(kde_lscv_cands_s* c, const double* H) {
   std::vector<unsigned char> up;
+  std::vector<AcGen<T>> gens;
   for (int64_t h0 = 0; h0 < c->nH; h0 += kAcChunk) {
     const int nh = (int)std::min<int64_t>(kAcChunk, c->nH - h0);
-    int nunits = 0;
-    kde_status s = ac_build_chunk<T>(c->plan, h0, nh, c->nH, H, nullptr, up, &nunits);
+    kde_lscv_cands_s::Chunk ch{};
+    kde_status s = ac_build_chunk<T>(c->plan, h0, nh, c->nH, H, nullptr, up, &ch.sh, &gens);
     if (s != KDE_OK) return s;
-    kde_lscv_cands_s::Chunk ch{nullptr, h0, nh, nunits};
+    ch.c0 = h0;
+    ch.nh = nh;
+    std::vector<AcGroup> groups;
+    std::vector<int3> items;
+    const size_t at = (up.size() + 255) & ~(size_t)255;
+    size_t at_items = at;
+    if (sizeof(T) == 4 && ch.sh.L1 <= kAcMaxL1) {
+      cands_group(gens, groups, items);
+      at_items = at + groups.size() * sizeof(AcGroup);
+      up.resize(at_items + items.size() * sizeof(int3));
+      std::memcpy(up.data() + at, groups.data(), groups.size() * sizeof(AcGroup));
+      std::memcpy(up.data() + at_items, items.data(), items.size() * sizeof(int3));
+      ch.nitems = (int)items.size();
+    }
     cudaError_t e = cudaMalloc(&ch.dev, up.size());
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(candidate set)");
+    if (ch.nitems) {
+      ch.groups = (AcGroup*)((char*)ch.dev + at);
+      ch.items = (int3*)((char*)ch.dev + at_items);
+    }
     c->chunks.push_back(ch);
     e = cudaMemcpy(ch.dev, up.data(), up.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(candidate set)");
@@ -2423,33 +2819,67 @@ extern "C" kde_status kde_lscv_autocorr_cands(kde_lscv_cands cands, int64_t n, c
   if (s != KDE_OK) return s;
   cudaStream_t st = (cudaStream_t)stream;
   double* partial = (double*)((char*)workspace + ac_upload_bytes(plan->info));
+  const NTerms nk = n_terms((double)n);
   for (const auto& ch : cands->chunks) {
     double* S = pair_sums ? pair_sums + 2 * ch.c0 : nullptr;
     s = plan->info.precision == KDE_F32
-            ? ac_launch_chunk<float>(plan->info, ch.dev, ch.nh, ch.nunits, R, partial, (double)n, S,
-                                     lscv + ch.c0, st)
-            : ac_launch_chunk<double>(plan->info, ch.dev, ch.nh, ch.nunits, R, partial, (double)n, S,
-                                      lscv + ch.c0, st);
+            ? ac_launch_chunk<float>(plan->info, ch.dev, ch.nh, ch.sh, (const float*)R, 1, partial,
+                                     nullptr, nk, 0, S, lscv + ch.c0, st)
+            : ac_launch_chunk<double>(plan->info, ch.dev, ch.nh, ch.sh, (const double*)R, 1,
+                                      partial, nullptr, nk, 0, S, lscv + ch.c0, st);
     if (s != KDE_OK) return s;
   }
   return KDE_OK;
 }
 
-// Scratch of kde_lscv_autocorr_cands_batch: the datasets' n, then one FP64
-// partial per work unit of the largest chunk and dataset.
-static size_t cands_batch_bytes(const kde_lscv_cands_s* c, int nsets) {
+// Scratch of kde_lscv_autocorr_cands_batch: the datasets' n terms, then for
+// a slab of datasets one FP64 partial per work unit of the largest chunk.
+struct CandsBatch {
+  int slab;            // datasets per launch
+  bool product;        // batched sums (else the datasets one by one)
+  size_t off_part, total;
+};
+
+static CandsBatch cands_batch_layout(const kde_lscv_cands_s* c, int nsets) {
+  auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   int units = 0;
-  for (const auto& ch : c->chunks) units = std::max(units, ch.nunits);
-  const size_t nb = ((size_t)nsets * sizeof(double) + 255) & ~(size_t)255;
-  return nb + (size_t)nsets * units * sizeof(double);
+  CandsBatch b{};
+  b.product = nsets >= kAcMinSets;
+  for (const auto& ch : c->chunks) {
+    units = std::max(units, ch.sh.nunits);
+    b.product = b.product && ch.groups;
+  }
+  b.slab = std::min(nsets, kAcSlab);
+  b.off_part = up((size_t)nsets * sizeof(NTerms));
+  b.total = b.off_part + up((size_t)b.slab * units * sizeof(double));
+  return b;
 }
 
 extern "C" kde_status kde_lscv_autocorr_cands_batch_workspace_bytes(kde_lscv_cands cands, int nsets,
                                                                     size_t* bytes) {
   if (!cands || !bytes) return fail(KDE_ERR_INVALID_ARG, "NULL argument");
   if (nsets < 0 || nsets > 65535) return fail(KDE_ERR_INVALID_ARG, "need 0 <= nsets <= 65535");
-  *bytes = cands_batch_bytes(cands, nsets);
+  *bytes = cands_batch_layout(cands, nsets).total;
   return KDE_OK;
+}
+
+// The batched sums of one chunk against ns autocorrelations from R on.
+static kde_status ac_product_chunk(const kde_plan_info& I, const kde_lscv_cands_s::Chunk& ch,
+                                   const float* R, int ns, double* partial, const NTerms* nk_set,
+                                   int64_t nH_all, double* S, double* lscv, cudaStream_t st) {
+  const AcImage<float> im(ch.dev, ch.nh, ch.sh.nunits);
+  cudaError_t e;
+  {
+    if ((e = allow_smem(kde_lscv_ac_sets_kernel)) != cudaSuccess)
+      return cuda_fail(e, "cudaFuncSetAttribute");
+    LaunchScope ls("kde_lscv_ac_sets_kernel", st);
+    kde_lscv_ac_sets_kernel<<<dim3((unsigned)ch.nitems, (unsigned)((ns + kAcSets - 1) / kAcSets)),
+                              32 * kAcWarps,
+                              ac_tile_bytes(ch.sh.L1), st>>>(
+        im.gens, ch.groups, ch.items, R, (int)I.P[1], (int64_t)I.P[0] * I.P[1], ns, partial);
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_ac_sets_kernel");
+  }
+  return ac_reduce<float>(im, ch.nh, ns, partial, nk_set, NTerms{}, nH_all, S, lscv, st);
 }
 
 extern "C" kde_status kde_lscv_autocorr_cands_batch(kde_lscv_cands cands, int nsets,
@@ -2461,12 +2891,13 @@ extern "C" kde_status kde_lscv_autocorr_cands_batch(kde_lscv_cands cands, int ns
   if (nsets < 0 || nsets > 65535) return fail(KDE_ERR_INVALID_ARG, "need 0 <= nsets <= 65535");
   if (nsets == 0) return KDE_OK;
   if (!n || !R || !lscv) return fail(KDE_ERR_INVALID_ARG, "NULL argument");
-  std::vector<double> nd((size_t)nsets);
+  std::vector<NTerms> nd((size_t)nsets);
   for (int b = 0; b < nsets; ++b) {
     if (n[b] < 2) return fail(KDE_ERR_INVALID_ARG, "LSCV needs n >= 2");
-    nd[b] = (double)n[b];
+    nd[b] = n_terms((double)n[b]);
   }
-  if (!workspace || workspace_bytes < cands_batch_bytes(cands, nsets))
+  const CandsBatch lay = cands_batch_layout(cands, nsets);
+  if (!workspace || workspace_bytes < lay.total)
     return fail(KDE_ERR_WORKSPACE, "workspace smaller than kde_lscv_autocorr_cands_batch_workspace_bytes");
   if (((uintptr_t)workspace & 255) != 0) return fail(KDE_ERR_INVALID_ARG, "workspace not 256-byte aligned");
   kde_plan_s* plan = cands->plan;
@@ -2474,41 +2905,24 @@ extern "C" kde_status kde_lscv_autocorr_cands_batch(kde_lscv_cands cands, int ns
   if (s != KDE_OK) return s;
   const kde_plan_info& I = plan->info;
   cudaStream_t st = (cudaStream_t)stream;
-  double* nset = (double*)workspace;
-  double* partial = (double*)((char*)workspace + (((size_t)nsets * sizeof(double) + 255) & ~(size_t)255));
-  if ((s = upload_async(nset, nd.data(), nd.size() * sizeof(double), st)) != KDE_OK) return s;
-  cudaError_t e = cudaSuccess;
-  const bool f32 = I.precision == KDE_F32;
-  const size_t gsz = f32 ? sizeof(AcGen<float>) : sizeof(AcGen<double>);
-  for (const auto& ch : cands->chunks) {
-    const char* img = (const char*)ch.dev;
-    const double* kn_dev = (const double*)(img + 2 * ch.nh * gsz);
-    const int2* units_dev = (const int2*)((const char*)kn_dev + 2 * ch.nh * sizeof(double));
-    const dim3 g1((unsigned)ch.nunits, (unsigned)nsets), g2((unsigned)((ch.nh + 7) / 8), (unsigned)nsets);
-    double* S = pair_sums ? pair_sums + 2 * ch.c0 : nullptr;
-    {
-      LaunchScope ls("kde_lscv_ac_kernel", st);
-      if (f32)
-        kde_lscv_ac_kernel<float><<<g1, 256, 0, st>>>((const AcGen<float>*)img, units_dev,
-                                                       (const float*)R, (int)I.P[1],
-                                                       (int64_t)I.P[0] * I.P[1], partial);
+  NTerms* nset = (NTerms*)workspace;
+  double* partial = (double*)((char*)workspace + lay.off_part);
+  if ((s = upload_async(nset, nd.data(), nd.size() * sizeof(NTerms), st)) != KDE_OK) return s;
+  const int64_t per = I.P[0] * I.P[1], nH = cands->nH;
+  for (int y = 0; y < nsets; y += lay.slab) {
+    const int ns = std::min(lay.slab, nsets - y);
+    for (const auto& ch : cands->chunks) {
+      double* S = pair_sums ? pair_sums + 2 * (y * nH + ch.c0) : nullptr;
+      double* out = lscv + y * nH + ch.c0;
+      if (lay.product)
+        s = ac_product_chunk(I, ch, (const float*)R + y * per, ns, partial, nset + y, nH, S, out, st);
+      else if (I.precision == KDE_F32)
+        s = ac_launch_chunk<float>(I, ch.dev, ch.nh, ch.sh, (const float*)R + y * per, ns, partial,
+                                   nset + y, NTerms{}, nH, S, out, st);
       else
-        kde_lscv_ac_kernel<double><<<g1, 256, 0, st>>>((const AcGen<double>*)img, units_dev,
-                                                        (const double*)R, (int)I.P[1],
-                                                        (int64_t)I.P[0] * I.P[1], partial);
-      if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_ac_kernel");
-    }
-    {
-      LaunchScope ls("kde_lscv_ac_reduce_sets_kernel", st);
-      if (f32)
-        kde_lscv_ac_reduce_sets_kernel<float><<<g2, 256, 0, st>>>(
-            (const AcGen<float>*)img, kn_dev, nset, partial, ch.nunits, ch.nh, cands->nH, S,
-            lscv + ch.c0);
-      else
-        kde_lscv_ac_reduce_sets_kernel<double><<<g2, 256, 0, st>>>(
-            (const AcGen<double>*)img, kn_dev, nset, partial, ch.nunits, ch.nh, cands->nH, S,
-            lscv + ch.c0);
-      if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_ac_reduce_sets_kernel");
+        s = ac_launch_chunk<double>(I, ch.dev, ch.nh, ch.sh, (const double*)R + y * per, ns,
+                                    partial, nset + y, NTerms{}, nH, S, out, st);
+      if (s != KDE_OK) return s;
     }
   }
   return KDE_OK;
@@ -2610,9 +3024,14 @@ extern "C" kde_status kde_lscv_theta_select(kde_plan plan, int nsets, const int6
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_theta_gen_kernel");
   }
   {
+    // a support that fits the plan has L_1 <= P_1 - M_1
+    const size_t smem = (size_t)kAcRows * (2 * (I.P[1] - I.M[1]) + 1) * sizeof(float);
+    if ((e = allow_smem(kde_lscv_theta_sums_kernel)) != cudaSuccess)
+      return cuda_fail(e, "cudaFuncSetAttribute");
     LaunchScope ls("kde_lscv_theta_sums_kernel", st);
-    kde_lscv_theta_sums_kernel<<<(unsigned)nmat, 256, 0, st>>>(t.gens, (const float*)R, (int)I.P[1],
-                                                               (int64_t)I.P[0] * I.P[1], S);
+    kde_lscv_theta_sums_kernel<<<(unsigned)((int64_t)nsets * ((J + kThetaCands) / kThetaCands)),
+                                 kThetaThreads, smem, st>>>(t.gens, 2 * (J + 1), (const float*)R,
+                                                            (int)I.P[1], (int64_t)I.P[0] * I.P[1], S);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_theta_sums_kernel");
   }
   {
