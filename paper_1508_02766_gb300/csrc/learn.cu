@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "kde_internal.h"
+#include "pdl.cuh"
 #include "tc_wait.cuh"
 
 namespace kde {
@@ -55,6 +56,12 @@ struct GemmArgs {
   bf16* Ct;            // optional BF16 transposed copy: Ct[n ldct + m]
   int ldct;
   int* status;         // set to 1 if a wait for the tensor cores gave up
+  int epi;
+  bool vec;            // C, Z, Cb rows take 16-byte accesses
+};
+// Two independent products may share a launch (blockIdx.z).
+struct GemmPair {
+  GemmArgs g[2];
 };
 
 
@@ -91,18 +98,25 @@ __device__ __forceinline__ void stage_tiles(const GemmArgs& g, uint8_t* sA, uint
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// Two shared-memory stages: the copies of K slice k+1 are in flight while
-// the tensor cores work on slice k; a stage is refilled only after the MMAs
-// that read it have completed (its mbarrier).
-template <int BN, int EPI>
-__global__ void __launch_bounds__(128) kde_gemm_tc_kernel(GemmArgs g) {
+// kStages shared-memory stages: the copies of the next kStages - 1 K slices
+// are in flight while the tensor cores work on one; a stage is refilled only
+// after the MMAs that read it have completed (its mbarrier).  The network's
+// products are a few CTAs each, so a slice's copy latency is their time: with
+// two stages the 256 x 256 x 1088 product took 17 us, 1 us a slice (figures
+// at mlp_backward).  The slices are accumulated in the same order whatever
+// the stages.
+template <int BN, int kStages>
+__global__ void __launch_bounds__(128) kde_gemm_tc_kernel(GemmPair pair) {
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr int kStageBytes = 16384 + BN * 128;  // A 128 x 64 + B BN x 64, BF16
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t mbar[kStages];
   __shared__ uint32_t tmem_slot;
   constexpr uint32_t kCols = BN < 32 ? 32 : BN;  // TMEM columns: a power of two >= 32
+  const GemmArgs g = pair.g[blockIdx.z];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int m0 = blockIdx.x * 128, n0 = blockIdx.y * BN;
+  pdl_trigger();
+  if (m0 >= g.M || n0 >= g.N) return;   // the smaller product of a pair
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&tmem_slot)),
@@ -111,14 +125,16 @@ __global__ void __launch_bounds__(128) kde_gemm_tc_kernel(GemmArgs g) {
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[0])) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[1])) : "memory");
+    for (int b = 0; b < kStages; ++b)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[b])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
+  // operands and Z come from the kernels before this one
+  pdl_wait();
   // kind::f16 instruction descriptor: D FP32 (bits 4-5 = 1), A and B BF16
   // (bits 7-9, 10-12 = 1), both K-major, N >> 3 at bit 17, M >> 4 at bit 24.
   const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
@@ -126,26 +142,17 @@ __global__ void __launch_bounds__(128) kde_gemm_tc_kernel(GemmArgs g) {
   uint32_t phase = 0u, used = 0u;  // bit b: stage b's barrier phase / MMAs pending
   bool ok = true;
   const int nk = g.K / 64;
-  stage_tiles<BN>(g, smem, smem + 16384, m0, n0, 0);
+  auto stage = [&](int kt) {       // one commit group per slice, empty past the last
+    if (kt < nk)
+      stage_tiles<BN>(g, smem + (kt % kStages) * kStageBytes,
+                      smem + (kt % kStages) * kStageBytes + 16384, m0, n0, kt * 64);
+    else
+      asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int kt = 0; kt < kStages - 1; ++kt) stage(kt);
   for (int kt = 0; kt < nk; ++kt) {
-    const int st = kt & 1, nx = st ^ 1;
-    if (kt + 1 < nk) {
-      // the other stage was read by the MMAs of slice kt - 1: wait for them
-      if ((used >> nx) & 1u) {
-        const bool done = mbar_wait(smem_u32(&mbar[nx]), (phase >> nx) & 1u);
-        if (!__syncthreads_and(done)) {
-          ok = false;
-          break;
-        }
-        phase ^= 1u << nx;
-        used &= ~(1u << nx);
-      }
-      stage_tiles<BN>(g, smem + nx * kStageBytes, smem + nx * kStageBytes + 16384, m0, n0,
-                      (kt + 1) * 64);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-    }
+    const int st = kt % kStages;
+    asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
     // the tensor cores read shared memory through the async proxy
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
@@ -169,10 +176,24 @@ __global__ void __launch_bounds__(128) kde_gemm_tc_kernel(GemmArgs g) {
           : "memory");
     }
     used |= 1u << st;
+    if (kt + kStages - 1 < nk) {
+      // the stage to refill was read by the MMAs of slice kt - 1: wait for them
+      const int nx = (kt + kStages - 1) % kStages;
+      if ((used >> nx) & 1u) {
+        const bool done = mbar_wait(smem_u32(&mbar[nx]), (phase >> nx) & 1u);
+        if (!__syncthreads_and(done)) {
+          ok = false;
+          break;
+        }
+        phase ^= 1u << nx;
+        used &= ~(1u << nx);
+      }
+    }
+    stage(kt + kStages - 1);
   }
   // every MMA has been committed; the last commit tracks them all
   if (ok) {
-    const int last = (nk - 1) & 1;
+    const int last = (nk - 1) % kStages;
     const bool done = mbar_wait(smem_u32(&mbar[last]), (phase >> last) & 1u);
     ok = __syncthreads_and(done);
   }
@@ -180,7 +201,7 @@ __global__ void __launch_bounds__(128) kde_gemm_tc_kernel(GemmArgs g) {
     if (tid == 0) atomicExch(g.status, 1);
     // one more bounded chance for the MMAs in flight before TMEM is freed
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    for (int b = 0; b < 2; ++b)
+    for (int b = 0; b < kStages; ++b)
       if ((used >> b) & 1u) mbar_wait(smem_u32(&mbar[b]), (phase >> b) & 1u);
   }
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -199,22 +220,46 @@ __global__ void __launch_bounds__(128) kde_gemm_tc_kernel(GemmArgs g) {
           : "r"(taddr)
           : "memory");
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      const int n = n0 + c0;
+      float x[16], z[16];
+      float* crow = g.C + (size_t)row * g.ldc + n;
+      if (g.epi == EPI_RELU_GRAD) {
+        const float* zrow = g.Z + (size_t)row * g.ldz + n;
+#pragma unroll
+        for (int j = 0; j < 16; j += 4) {
+          const float4 q = g.vec ? *reinterpret_cast<const float4*>(zrow + j)
+                                 : make_float4(zrow[j], zrow[j + 1], zrow[j + 2], zrow[j + 3]);
+          z[j] = q.x, z[j + 1] = q.y, z[j + 2] = q.z, z[j + 3] = q.w;
+        }
+      }
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        const int n = n0 + c0 + j;
-        float x = __uint_as_float(v[j]);
-        float a = x;
-        if (EPI == EPI_BIAS_RELU || EPI == EPI_BIAS) x += g.bias[n];
-        if (EPI == EPI_BIAS_RELU) a = fmaxf(x, 0.f);
-        if (EPI == EPI_RELU_GRAD) {
-          x = g.Z[(size_t)row * g.ldz + n] > 0.f ? x : 0.f;
-          a = x;
+        x[j] = __uint_as_float(v[j]);
+        if (g.epi == EPI_BIAS_RELU || g.epi == EPI_BIAS) x[j] += g.bias[n + j];
+        if (g.epi == EPI_RELU_GRAD) x[j] = z[j] > 0.f ? x[j] : 0.f;
+      }
+#pragma unroll
+      for (int j = 0; j < 16; j += 4) {
+        if (g.vec) {
+          *reinterpret_cast<float4*>(crow + j) = make_float4(x[j], x[j + 1], x[j + 2], x[j + 3]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) crow[j + i] = x[j + i];
         }
-        g.C[(size_t)row * g.ldc + n] = x;
-        if (EPI == EPI_BIAS_RELU || EPI == EPI_RELU_GRAD) {
-          const bf16 b = __float2bfloat16_rn(a);
-          if (g.Cb) g.Cb[(size_t)row * g.ldcb + n] = b;
-          if (g.Ct) g.Ct[(size_t)n * g.ldct + row] = b;
+      }
+      if (g.epi == EPI_BIAS_RELU || g.epi == EPI_RELU_GRAD) {
+        __align__(16) bf16 b[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          b[j] = __float2bfloat16_rn(g.epi == EPI_BIAS_RELU ? fmaxf(x[j], 0.f) : x[j]);
+        if (g.Cb) {   // rows of the network's own buffers: always 16-byte aligned
+          uint4* dst = reinterpret_cast<uint4*>(g.Cb + (size_t)row * g.ldcb + n);
+          dst[0] = reinterpret_cast<const uint4*>(b)[0];
+          dst[1] = reinterpret_cast<const uint4*>(b)[1];
+        }
+        if (g.Ct) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) g.Ct[(size_t)(n + j) * g.ldct + row] = b[j];
         }
       }
     }
@@ -226,38 +271,68 @@ __global__ void __launch_bounds__(128) kde_gemm_tc_kernel(GemmArgs g) {
                  : "memory");
 }
 
-template <int BN, int EPI>
-cudaError_t launch_gemm_bn(const GemmArgs& g, cudaStream_t st) {
-  // Two stages of A (16 KB) and B (BN x 128 bytes); 56 KB of dynamic shared
-  // memory caps the CTAs per SM at 4, so the tensor memory they hold
-  // (4 x 64 columns) stays within the SM's 512 columns.
-  const int smem = 56 * 1024;
+template <int BN, int kStages>
+cudaError_t launch_gemm_st(const GemmPair& p, dim3 grid, cudaStream_t st) {
+  // kStages stages of A (16 KB) and B (BN x 128 bytes); the narrow tiles ask
+  // for as much as the wide ones, so that at most four CTAs share an SM and
+  // their tensor memory (64 columns each) stays within its 512 columns.
+  const int smem = kStages * (16384 + 64 * 128);
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(kde_gemm_tc_kernel<BN, EPI>,
+    cudaError_t e = cudaFuncSetAttribute(kde_gemm_tc_kernel<BN, kStages>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     attr = true;
   }
   LaunchScope ls("kde_gemm_tc_kernel", st);
-  kde_gemm_tc_kernel<BN, EPI><<<dim3(g.M / 128, g.N / BN), 128, smem, st>>>(g);
-  return cudaGetLastError();
+  const cudaError_t e = launch_pdl(kde_gemm_tc_kernel<BN, kStages>, grid, dim3(128), (size_t)smem, st, p);
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
-kde_status launch_gemm(const GemmArgs& g, int epi, cudaStream_t st) {
+// Grids that leave SMs idle take eight stages (196 KB, one CTA an SM); larger
+// ones two (four CTAs an SM, one's epilogue beside the others' slices: 4096^3
+// 776 us, 792 with three stages, 889 with four).
+template <int BN>
+cudaError_t launch_gemm_bn(const GemmPair& p, int count, cudaStream_t st) {
+  int M = 0, N = 0;
+  for (int i = 0; i < count; ++i) {
+    M = std::max(M, p.g[i].M);
+    N = std::max(N, p.g[i].N);
+  }
+  const dim3 grid((unsigned)(M / 128), (unsigned)(N / BN), (unsigned)count);
+  if ((int64_t)grid.x * grid.y * grid.z <= 128) return launch_gemm_st<BN, 8>(p, grid, st);
+  return launch_gemm_st<BN, 2>(p, grid, st);
+}
+
+kde_status check_gemm(GemmArgs& g, int epi) {
   if (g.M <= 0 || g.N <= 0 || g.K <= 0 || g.M % 128 || g.N % 16 || g.K % 64 || g.lda % 8 ||
       g.ldb % 8 || ((uintptr_t)g.A & 15) || ((uintptr_t)g.B & 15) || !g.C || !g.status)
     return fail(KDE_ERR_INVALID_ARG,
                 "tensor-core GEMM: need M % 128 == 0, N % 16 == 0, K % 64 == 0, row strides "
                 "multiples of 8 elements and 16-byte aligned operands");
-  cudaError_t e;
-  const bool wide = g.N % 64 == 0;
-  switch (epi) {
-    case EPI_STORE: e = wide ? launch_gemm_bn<64, EPI_STORE>(g, st) : launch_gemm_bn<16, EPI_STORE>(g, st); break;
-    case EPI_BIAS_RELU: e = wide ? launch_gemm_bn<64, EPI_BIAS_RELU>(g, st) : launch_gemm_bn<16, EPI_BIAS_RELU>(g, st); break;
-    case EPI_BIAS: e = wide ? launch_gemm_bn<64, EPI_BIAS>(g, st) : launch_gemm_bn<16, EPI_BIAS>(g, st); break;
-    default: e = wide ? launch_gemm_bn<64, EPI_RELU_GRAD>(g, st) : launch_gemm_bn<16, EPI_RELU_GRAD>(g, st); break;
-  }
+  g.epi = epi;
+  g.vec = g.ldc % 4 == 0 && ((uintptr_t)g.C & 15) == 0 && (!g.Z || (g.ldz % 4 == 0 && ((uintptr_t)g.Z & 15) == 0));
+  return KDE_OK;
+}
+
+kde_status launch_gemm(GemmArgs g, int epi, cudaStream_t st) {
+  const kde_status s = check_gemm(g, epi);
+  if (s != KDE_OK) return s;
+  GemmPair p{};
+  p.g[0] = g;
+  const cudaError_t e = g.N % 64 == 0 ? launch_gemm_bn<64>(p, 1, st) : launch_gemm_bn<16>(p, 1, st);
+  return e == cudaSuccess ? KDE_OK : cuda_fail(e, "kde_gemm_tc_kernel");
+}
+
+// Two products of N % 64 == 0 in one launch.
+kde_status launch_gemm2(GemmArgs a, int epi_a, GemmArgs b, int epi_b, cudaStream_t st) {
+  kde_status s = check_gemm(a, epi_a);
+  if (s == KDE_OK) s = check_gemm(b, epi_b);
+  if (s != KDE_OK) return s;
+  GemmPair p{};
+  p.g[0] = a;
+  p.g[1] = b;
+  const cudaError_t e = launch_gemm_bn<64>(p, 2, st);
   return e == cudaSuccess ? KDE_OK : cuda_fail(e, "kde_gemm_tc_kernel");
 }
 
@@ -265,23 +340,38 @@ kde_status launch_gemm(const GemmArgs& g, int epi, cudaStream_t st) {
 // Element-wise and reduction kernels of the MLP.
 // ---------------------------------------------------------------------------
 // X (B x in, FP32) -> Xb (Bp x in, BF16) and its transpose Xt (in x Bp);
-// rows B .. Bp-1 are zero.
+// rows B .. Bp-1 are zero.  Tiles of 32 x 64 go through shared memory, so that
+// both copies are written in rows.  Grid (in / 64, Bp / 32).
 __global__ void __launch_bounds__(256) kde_mlp_cast_kernel(const float* __restrict__ X, int B,
                                                            int Bp, int in, bf16* __restrict__ Xb,
                                                            bf16* __restrict__ Xt) {
-  const int64_t total = (int64_t)Bp * in;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int b = (int)(i / in), k = (int)(i - (int64_t)b * in);
-    const bf16 v = __float2bfloat16_rn(b < B ? X[i] : 0.f);
-    Xb[i] = v;
-    if (Xt) Xt[(int64_t)k * Bp + b] = v;
+  __shared__ bf16 tile[32][66];
+  pdl_trigger();
+  pdl_wait();   // X, and the last reader of Xb and Xt
+  const int k0 = blockIdx.x * 64, b0 = blockIdx.y * 32, t = threadIdx.x;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int b = (t >> 6) + 4 * i, k = t & 63;
+    const bf16 v = __float2bfloat16_rn(b0 + b < B ? X[(size_t)(b0 + b) * in + k0 + k] : 0.f);
+    Xb[(size_t)(b0 + b) * in + k0 + k] = v;
+    tile[b][k] = v;
+  }
+  if (!Xt) return;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int k = (t >> 5) + 8 * i, b = t & 31;
+    Xt[(size_t)(k0 + k) * Bp + b0 + b] = tile[b][k];
   }
 }
 
 // Loss = (1/B) sum_{b < B, j < out} (Y - T)^2 and its gradient
 // dY = (2/B)(Y - T): BF16 copies dYb (Bp x 64, zero beyond out) and
-// dYt (outp x Bp), and db3 = sum_b dY (FP32, fixed order).  One block.
+// dYt (outp x Bp), and db3 = sum_b dY (FP32, b in order).  One block, tiles
+// of 256 rows: the gradient's values are formed side by side into shared
+// memory, and only their additions are one after another (read one by one
+// from global memory they took 44 us for 256 rows).
+constexpr int kMaxOut = 16;
 __global__ void __launch_bounds__(256) kde_mlp_loss_kernel(const float* __restrict__ Y, int ldy,
                                                            const float* __restrict__ T, int B,
                                                            int Bp, int out, int outp,
@@ -290,51 +380,81 @@ __global__ void __launch_bounds__(256) kde_mlp_loss_kernel(const float* __restri
                                                            float* __restrict__ db3,
                                                            float* __restrict__ loss) {
   __shared__ double part[256];
+  __shared__ float res[256][kMaxOut + 1], grd[256][kMaxOut + 1];   // Y - T, 2 (Y - T) / B
+  pdl_trigger();
+  pdl_wait();
+  const int t = threadIdx.x;
   double acc = 0.0;
-  for (int i = threadIdx.x; i < Bp * 64; i += blockDim.x) {
-    const int b = i / 64, j = i % 64;
-    float g = 0.f;
-    if (b < B && j < out) {
-      const float r = Y[(size_t)b * ldy + j] - T[(size_t)b * out + j];
-      acc += (double)r * r;
-      g = 2.f * r / (float)B;
+  float sum = 0.f;
+  for (int b0 = 0; b0 < Bp; b0 += 256) {
+    const int b = b0 + t;
+    if (b < Bp) {
+      __align__(16) bf16 row[kMaxOut];
+#pragma unroll
+      for (int j = 0; j < kMaxOut; ++j) {
+        float r = 0.f, g = 0.f;
+        if (b < B && j < out) {
+          r = Y[(size_t)b * ldy + j] - T[(size_t)b * out + j];
+          g = 2.f * r / (float)B;
+        }
+        res[t][j] = r;
+        grd[t][j] = g;
+        row[j] = __float2bfloat16_rn(g);
+        if (j < outp) dYt[(size_t)j * Bp + b] = row[j];
+      }
+      uint4* dst = reinterpret_cast<uint4*>(dYb + (size_t)b * 64);
+      dst[0] = reinterpret_cast<const uint4*>(row)[0];
+      dst[1] = reinterpret_cast<const uint4*>(row)[1];
+#pragma unroll
+      for (int q = 2; q < 8; ++q) dst[q] = make_uint4(0, 0, 0, 0);
     }
-    const bf16 gb = __float2bfloat16_rn(g);
-    dYb[i] = gb;
-    if (j < outp) dYt[(size_t)j * Bp + b] = gb;
-  }
-  part[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) part[threadIdx.x] += part[threadIdx.x + s];
+    __syncthreads();
+    const int nb = min(256, B - b0);
+    // thread (t / 64, t mod 64): output t mod 64 of every fourth row
+    if ((t & 63) < out)
+      for (int i = t >> 6; i < nb; i += 4) {
+        const float r = res[i][t & 63];
+        acc += (double)r * r;
+      }
+    if (t < out) {
+#pragma unroll 8
+      for (int i = 0; i < nb; ++i) sum += grd[i][t];
+    }
     __syncthreads();
   }
-  if (threadIdx.x == 0 && loss) *loss = (float)(part[0] / B);
-  for (int j = threadIdx.x; j < out; j += blockDim.x) {
-    float s = 0.f;
-    for (int b = 0; b < B; ++b) s += 2.f * (Y[(size_t)b * ldy + j] - T[(size_t)b * out + j]) / (float)B;
-    db3[j] = s;
+  part[t] = acc;
+  __syncthreads();
+  for (int s = 128; s > 0; s >>= 1) {
+    if (t < s) part[t] += part[t + s];
+    __syncthreads();
   }
+  if (t == 0 && loss) *loss = (float)(part[0] / B);
+  if (t < out) db3[t] = sum;
 }
 
-// db[n] = sum_{b < B} dZ[b n] (one thread per column, fixed order).
-__global__ void __launch_bounds__(256) kde_mlp_colsum_kernel(const float* __restrict__ dZ, int ld,
-                                                             int B, int N, float* __restrict__ db) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  float s = 0.f;
-  for (int b = 0; b < B; ++b) s += dZ[(size_t)b * ld + n];
-  db[n] = s;
-}
-
-// G_W3[j h] = dW3t[h j] for j < out.
-__global__ void __launch_bounds__(256) kde_mlp_w3grad_kernel(const float* __restrict__ dW3t, int hid,
-                                                             int outp, int out,
-                                                             float* __restrict__ gW3) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= out * hid) return;
-  const int j = i / hid, h = i % hid;
-  gW3[i] = dW3t[(size_t)h * outp + j];
+// The gradients that are not products, in one launch: db1 and db2 as the
+// column sums of dZ1 and dZ2 (a thread a column, b in order, 32 loads in
+// flight), and G_W3[j h] = dW3t[h j] for j < out.  Blocks of 32 threads: hid /
+// 32 for each of db1 and db2, then out hid / 32.
+__global__ void __launch_bounds__(32) kde_mlp_tail_kernel(const float* __restrict__ dZ1,
+                                                          const float* __restrict__ dZ2, int hid,
+                                                          int B, const float* __restrict__ dW3t,
+                                                          int outp, int out,
+                                                          float* __restrict__ db1,
+                                                          float* __restrict__ db2,
+                                                          float* __restrict__ gW3) {
+  pdl_trigger();
+  pdl_wait();
+  const int nb = hid / 32, i = (blockIdx.x % nb) * 32 + threadIdx.x, part = blockIdx.x / nb;
+  if (part < 2) {
+    const float* dZ = (part ? dZ2 : dZ1) + i;
+    float s = 0.f;
+#pragma unroll 32
+    for (int b = 0; b < B; ++b) s += dZ[(size_t)b * hid];
+    (part ? db2 : db1)[i] = s;
+  } else {
+    gW3[(part - 2) * hid + i] = dW3t[(size_t)i * outp + part - 2];
+  }
 }
 
 // Adam on the flat FP32 parameters.
@@ -622,8 +742,9 @@ GemmArgs gemm_args(const bf16* A, int lda, const bf16* B, int ldb, int M, int N,
 kde_status mlp_forward(kde_mlp_s* m, const float* X, int B, int Bp, bool keep_t, cudaStream_t st) {
   {
     LaunchScope ls("kde_mlp_cast_kernel", st);
-    kde_mlp_cast_kernel<<<512, 256, 0, st>>>(X, B, Bp, m->in, m->Xb, keep_t ? m->Xt : nullptr);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_pdl(kde_mlp_cast_kernel, dim3((unsigned)(m->in / 64), (unsigned)(Bp / 32)),
+                                     dim3(256), 0, st, X, B, Bp, m->in, m->Xb,
+                                     keep_t ? m->Xt : (bf16*)nullptr);
     if (e != cudaSuccess) return cuda_fail(e, "kde_mlp_cast_kernel");
   }
   GemmArgs g1 = gemm_args(m->Xb, m->in, m->W1b, m->in, Bp, m->hid, m->in, m->Z1, m->hid, m->status);
@@ -646,26 +767,18 @@ kde_status mlp_forward(kde_mlp_s* m, const float* X, int B, int Bp, bool keep_t,
   return launch_gemm(g3, EPI_BIAS, st);
 }
 
-// Loss and gradients into m->G (layout of m->P) for the first B rows.
-kde_status mlp_backward(kde_mlp_s* m, const float* T, int B, int Bp, float* loss_out,
+// Loss and gradients into G (layout of m->P) for the first B rows.  Ten
+// launches with the forward pass's four, each a programmatic dependent of the
+// one before; 256 rows of 1088-256-256-3 took 243 us with 13 (products 17 us
+// each with two stages, the loss 44, the column sums 10 each), now 87.
+kde_status mlp_backward(kde_mlp_s* m, const float* T, int B, int Bp, float* G, float* loss_out,
                         cudaStream_t st) {
   cudaError_t e;
   {
     LaunchScope ls("kde_mlp_loss_kernel", st);
-    kde_mlp_loss_kernel<<<1, 256, 0, st>>>(m->Y, m->outp, T, B, Bp, m->out, m->outp, m->dYb, m->dYt,
-                                           m->G + m->ob3, loss_out ? loss_out : m->loss);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_mlp_loss_kernel");
-  }
-  // dW3^T = A2^T dY  (M = hid, N = outp, K = Bp)
-  kde_status s = launch_gemm(gemm_args(m->A2t, Bp, m->dYt, Bp, m->hid, m->outp, Bp, m->dW3t,
-                                       m->outp, m->status),
-                             EPI_STORE, st);
-  if (s != KDE_OK) return s;
-  {
-    LaunchScope ls("kde_mlp_w3grad_kernel", st);
-    kde_mlp_w3grad_kernel<<<(m->out * m->hid + 255) / 256, 256, 0, st>>>(m->dW3t, m->hid, m->outp,
-                                                                         m->out, m->G + m->oW3);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_mlp_w3grad_kernel");
+    e = launch_pdl(kde_mlp_loss_kernel, dim3(1), dim3(256), 0, st, m->Y, m->outp, T, B, Bp, m->out,
+                   m->outp, m->dYb, m->dYt, G + m->ob3, loss_out ? loss_out : m->loss);
+    if (e != cudaSuccess) return cuda_fail(e, "kde_mlp_loss_kernel");
   }
   // dZ2 = (dY W3) * (Z2 > 0)  (M = Bp, N = hid, K = 64)
   GemmArgs g5 = gemm_args(m->dYb, 64, m->W3t, 64, Bp, m->hid, 64, m->dZ2, m->hid, m->status);
@@ -675,36 +788,36 @@ kde_status mlp_backward(kde_mlp_s* m, const float* T, int B, int Bp, float* loss
   g5.ldcb = m->hid;
   g5.Ct = m->dZ2t;
   g5.ldct = Bp;
-  if ((s = launch_gemm(g5, EPI_RELU_GRAD, st)) != KDE_OK) return s;
-  {
-    LaunchScope ls("kde_mlp_colsum_kernel", st);
-    kde_mlp_colsum_kernel<<<(m->hid + 255) / 256, 256, 0, st>>>(m->dZ2, m->hid, B, m->hid,
-                                                                m->G + m->ob2);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_mlp_colsum_kernel");
-  }
+  kde_status s = launch_gemm(g5, EPI_RELU_GRAD, st);
+  if (s != KDE_OK) return s;
+  // dZ1 = (dZ2 W2) * (Z1 > 0)  (M = Bp, N = hid, K = hid), and beside it
   // dW2 = dZ2^T A1  (M = hid, N = hid, K = Bp)
-  if ((s = launch_gemm(gemm_args(m->dZ2t, Bp, m->A1t, Bp, m->hid, m->hid, Bp, m->G + m->oW2,
-                                 m->hid, m->status),
-                       EPI_STORE, st)) != KDE_OK)
-    return s;
-  // dZ1 = (dZ2 W2) * (Z1 > 0)  (M = Bp, N = hid, K = hid)
   GemmArgs g7 = gemm_args(m->dZ2b, m->hid, m->W2t, m->hid, Bp, m->hid, m->hid, m->dZ1, m->hid,
                           m->status);
   g7.Z = m->Z1;
   g7.ldz = m->hid;
   g7.Ct = m->dZ1t;
   g7.ldct = Bp;
-  if ((s = launch_gemm(g7, EPI_RELU_GRAD, st)) != KDE_OK) return s;
-  {
-    LaunchScope ls("kde_mlp_colsum_kernel", st);
-    kde_mlp_colsum_kernel<<<(m->hid + 255) / 256, 256, 0, st>>>(m->dZ1, m->hid, B, m->hid,
-                                                                m->G + m->ob1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_mlp_colsum_kernel");
-  }
+  if ((s = launch_gemm2(g7, EPI_RELU_GRAD,
+                        gemm_args(m->dZ2t, Bp, m->A1t, Bp, m->hid, m->hid, Bp, G + m->oW2, m->hid,
+                                  m->status),
+                        EPI_STORE, st)) != KDE_OK)
+    return s;
+  // dW3^T = A2^T dY  (M = hid, N = outp, K = Bp)
+  if ((s = launch_gemm(gemm_args(m->A2t, Bp, m->dYt, Bp, m->hid, m->outp, Bp, m->dW3t, m->outp,
+                                 m->status),
+                       EPI_STORE, st)) != KDE_OK)
+    return s;
   // dW1 = dZ1^T X  (M = hid, N = in, K = Bp)
-  return launch_gemm(gemm_args(m->dZ1t, Bp, m->Xt, Bp, m->hid, m->in, Bp, m->G + m->oW1, m->in,
-                               m->status),
-                     EPI_STORE, st);
+  if ((s = launch_gemm(gemm_args(m->dZ1t, Bp, m->Xt, Bp, m->hid, m->in, Bp, G + m->oW1, m->in,
+                                 m->status),
+                       EPI_STORE, st)) != KDE_OK)
+    return s;
+  LaunchScope ls("kde_mlp_tail_kernel", st);
+  e = launch_pdl(kde_mlp_tail_kernel, dim3((unsigned)(m->hid / 32 * (2 + m->out))), dim3(32), 0, st,
+                 m->dZ1, m->dZ2, m->hid, B, m->dW3t, m->outp, m->out, G + m->ob1, G + m->ob2,
+                 G + m->oW3);
+  return e == cudaSuccess ? KDE_OK : cuda_fail(e, "kde_mlp_tail_kernel");
 }
 
 kde_status mlp_check_batch(const kde_mlp_s* m, int B, int* Bp) {
@@ -868,13 +981,7 @@ kde_status kde_mlp_loss_grad(kde_mlp m, const float* X, const float* T, int B, f
   if (!X || !T) return fail(KDE_ERR_INVALID_ARG, "NULL pointer");
   cudaStream_t st = (cudaStream_t)stream;
   if ((s = mlp_forward(m, X, B, Bp, true, st)) != KDE_OK) return s;
-  if ((s = mlp_backward(m, T, B, Bp, loss, st)) != KDE_OK) return s;
-  if (grads) {
-    cudaError_t e = cudaMemcpyAsync(grads, m->G, sizeof(float) * m->nparam,
-                                    cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(grads)");
-  }
-  return KDE_OK;
+  return mlp_backward(m, T, B, Bp, grads ? grads : m->G, loss, st);
 }
 
 kde_status kde_mlp_train_step(kde_mlp m, const float* X, const float* T, int B, float lr,
