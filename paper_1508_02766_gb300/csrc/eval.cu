@@ -2393,7 +2393,7 @@ kde_status multi_layout(const kde_plan_s* plan, MultiLayout* m) {
   m->off_gens = up(M0 * Q * 8);
   m->off_L0 = m->off_gens + up(kMultiChunk * sizeof(KGen<float>));
   m->off_t1 = m->off_L0 + up(kMultiChunk * sizeof(int));
-  m->off_K = m->off_t1 + up((size_t)kMultiChunk * (2 * m->Lmax0 + 1) * Q * 8);
+  m->off_K = m->off_t1 + up((size_t)kMultiChunk * (m->Lmax0 + 1) * Q * 8);
   m->off_S = m->off_K + up((size_t)kMultiChunk * P0 * Q * 4);
   m->total = m->off_S + up((size_t)kMultiChunk * M0 * Q * 8);
   return KDE_OK;

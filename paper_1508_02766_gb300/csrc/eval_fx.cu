@@ -287,22 +287,24 @@ kde_status fx_kernel_grid(kde_plan_s* plan, const KGen<float>& gen, void* Kspec,
   using namespace fx;
   const kde_plan_info& I = plan->info;
   const int d = I.d;
+  // rows at lags l_0 >= 0 only: the others are their conjugates (1024^2: 89
+  // -> 45 rows; 256^3, event times: rows 11.5 -> 9.7 us, axis 1 10.1 -> 8.4,
+  // axis 0 20.2 -> 18.7; a chunk of 64 bandwidths at 512^2: rows 36 -> 23)
   float2* t1 = (float2*)ws;
-  int64_t rows = 1;
-  for (int k = 0; k < d - 1; ++k) rows *= 2 * I.L[k] + 1;
+  const int64_t rows = (I.L[0] + 1) * (d == 3 ? 2 * I.L[1] + 1 : 1);
   kde_status s = rows_pass(plan, SRC_KGEN, rows, nullptr, 0, 0, &gen, t1, nullptr, nullptr, 0, st);
   if (s != KDE_OK) return s;
   if (d == 2)
     return cols_pass<COL_FWD_REAL>(plan, 0, "kde_fx_cols_kgen_real_kernel", t1, nullptr,
-                                   (float*)Kspec, nullptr, I.Q, 1, (int)(2 * I.L[0] + 1), 0,
+                                   (float*)Kspec, nullptr, I.Q, 1, (int)(I.L[0] + 1), 0,
                                    (int)I.L[0], st);
   // d == 3: axis 1 (wrapped lags) into t2, then axis 0 to the real spectrum
   float2* t2 = t1 + rows * I.Q;
   s = cols_pass<COL_FWD>(plan, 1, "kde_fx_cols_kgen_kernel", t1, t2, nullptr, nullptr, I.Q,
-                         2 * I.L[0] + 1, (int)(2 * I.L[1] + 1), (int)I.P[1], (int)I.L[1], st);
+                         I.L[0] + 1, (int)(2 * I.L[1] + 1), (int)I.P[1], (int)I.L[1], st);
   if (s != KDE_OK) return s;
   return cols_pass<COL_FWD_REAL>(plan, 0, "kde_fx_cols_kgen_real_kernel", t2, nullptr,
-                                 (float*)Kspec, nullptr, I.P[1] * I.Q, 1, (int)(2 * I.L[0] + 1), 0,
+                                 (float*)Kspec, nullptr, I.P[1] * I.Q, 1, (int)(I.L[0] + 1), 0,
                                  (int)I.L[0], st);
 }
 
@@ -371,7 +373,7 @@ kde_status fx_eval_batch2(kde_plan_s* plan, const float2* A, int nh, const KGen<
   using namespace fx;
   const kde_plan_info& I = plan->info;
   const int64_t Q = I.Q, M0 = I.M[0], M1 = I.M[1], P0 = I.P[0];
-  const int64_t rows_max = 2 * (int64_t)Lmax0 + 1;
+  const int64_t rows_max = (int64_t)Lmax0 + 1;   // lags l_0 >= 0, as in fx_kernel_grid
   Batch b;
   b.nh = nh;
   b.gens = gens;

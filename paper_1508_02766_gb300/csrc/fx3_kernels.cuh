@@ -298,15 +298,7 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kernel(ColsArgs a) {
         const int64_t s = first + 2 * c;
         const bool v0 = s < a.S, v1 = s + 1 < a.S;
 #pragma unroll
-        for (int n1 = 0; n1 < N1; ++n1) {
-          const int j = col_source(n23 + N23 * n1, P, a.Lw, a.Nin);
-          float2 p = make_float2(0.f, 0.f), q = make_float2(0.f, 0.f);
-          if (j >= 0) {
-            if (v0) p = __ldg(in + (int64_t)j * a.S + s);
-            if (v1) q = __ldg(in + (int64_t)j * a.S + s + 1);
-          }
-          x[n1] = make_float2(p.x - q.y, p.y + q.x);
-        }
+        for (int n1 = 0; n1 < N1; ++n1) x[n1] = col_pair(a, n23 + N23 * n1, P, s, v0, v1);
       } else {
         const int64_t s = first + c;
         const bool v = s < a.S;

@@ -166,7 +166,7 @@ __device__ __forceinline__ void rows_slab(RowsArgs& a, KGen<float>& g) {
   const int64_t h = blockIdx.y;
   if (a.gens) {
     g = a.gens[h];
-    a.nrows = g.d == 2 ? 2 * g.L[0] + 1 : (int64_t)(2 * g.L[0] + 1) * (2 * g.L[1] + 1);
+    a.nrows = g.d == 2 ? g.L[0] + 1 : (int64_t)(g.L[0] + 1) * (2 * g.L[1] + 1);
   }
   if (h) {
     a.out += h * a.slab_out;
@@ -253,7 +253,9 @@ __device__ __forceinline__ void rows_split_store(const RowsArgs& a, const float2
 
 // Kernel-grid rows: k at every position of the block's row pairs into the
 // staging area (zero where the wrapped lag is beyond the support).  Row r
-// enumerates the leading lags (l_0[, l_1]) with |l_k| <= L_k.
+// enumerates the leading lags (l_0[, l_1]) with 0 <= l_0 <= L_0, |l_1| <= L_1:
+// the kernel is even, so the rows at -l_0 transform to the conjugates of
+// these, which the axis-0 pass (COL_FWD_REAL) takes them from.
 __device__ __forceinline__ void rows_stage_kgen(const RowsArgs& a, const KGen<float>& g,
                                                 float2* stage) {
   const int P = a.ln.P;
@@ -269,11 +271,11 @@ __device__ __forceinline__ void rows_stage_kgen(const RowsArgs& a, const KGen<fl
         if (r >= a.nrows) break;
         int l[KDE_MAX_D] = {0, 0, 0};
         if (g.d == 2) {
-          l[0] = (int)r - g.L[0];
+          l[0] = (int)r;
           l[1] = ll;
         } else {
           const int w1 = 2 * g.L[1] + 1;
-          l[0] = (int)(r / w1) - g.L[0];
+          l[0] = (int)(r / w1);
           l[1] = (int)(r % w1) - g.L[1];
           l[2] = ll;
         }
@@ -388,13 +390,14 @@ struct ColsArgs {
   int Nin;           // input rows holding data (COL_INV: P)
   int Nout;          // output rows kept (crop); COL_FWD: P
   int Lw;            // >= 0: input row j holds lag j - Lw at position (j - Lw) mod P
+                     // (COL_FWD_REAL: row j holds lag j, lag -j its conjugate)
   Line ln;
   int B, lgB, SK;
   const float2* tw;
   // Element offsets between consecutive slabs (grid.y): outer slabs of a
   // 3-D pass, or batched bandwidths (in 0 when they share the input); with
-  // h_L0 (batched kernel spectra) the input of slab h holds 2 L0 + 1 wrapped
-  // rows with L0 = h_L0[h].
+  // h_L0 (batched kernel spectra) the input of slab h holds L0 + 1 rows (lags
+  // 0 .. L0) with L0 = h_L0[h].
   int64_t slab_in, slab_out, slab_real, slab_K;
   const int* h_L0;
   float s_pre, s_post;  // COL_AUTO scales
@@ -423,7 +426,7 @@ __device__ __forceinline__ void cols_slab(ColsArgs& a) {
   const int64_t h = blockIdx.y;
   if (a.h_L0) {
     a.Lw = a.h_L0[h];
-    a.Nin = 2 * a.Lw + 1;
+    a.Nin = a.Lw + 1;
   }
   if (h) {
     a.in += h * a.slab_in;
@@ -438,6 +441,25 @@ __device__ __forceinline__ int col_source(int pos, int P, int Lw, int Nin) {
   if (Lw < 0) return pos < Nin ? pos : -1;
   const int l = wrapped_lag(pos, P, Lw);
   return l <= Lw ? l + Lw : -1;
+}
+
+// Value at transform position pos of the two Hermitian columns s, s + 1 of a
+// COL_FWD_REAL line, as p + i q (v0, v1: the columns exist): row |l| of lag l,
+// conjugated for l < 0.
+__device__ __forceinline__ float2 col_pair(const ColsArgs& a, int pos, int P, int64_t s, bool v0,
+                                           bool v1) {
+  const int l = wrapped_lag(pos, P, a.Lw);
+  float2 p = make_float2(0.f, 0.f), q = make_float2(0.f, 0.f);
+  if (l <= a.Lw) {
+    const float2* row = a.in + (int64_t)(l < 0 ? -l : l) * a.S + s;
+    if (v0) p = __ldg(row);
+    if (v1) q = __ldg(row + 1);
+    if (l < 0) {
+      p.y = -p.y;
+      q.y = -q.y;
+    }
+  }
+  return make_float2(p.x - q.y, p.y + q.x);
 }
 
 template <int MODE>
@@ -457,15 +479,7 @@ __device__ __forceinline__ void cols_a_fwd(const ColsArgs& a, float2* sm) {
     const int64_t s = col_first<MODE>(a) + 2 * b;
     const bool v0 = s < a.S, v1 = s + 1 < a.S;
 #pragma unroll
-    for (int n1 = 0; n1 < N1; ++n1) {
-      const int j = col_source(n2 + N2 * n1, a.ln.P, a.Lw, a.Nin);
-      float2 p = make_float2(0.f, 0.f), q = make_float2(0.f, 0.f);
-      if (j >= 0) {
-        if (v0) p = __ldg(in + (int64_t)j * a.S + s);
-        if (v1) q = __ldg(in + (int64_t)j * a.S + s + 1);
-      }
-      x[n1] = make_float2(p.x - q.y, p.y + q.x);  // p + i q
-    }
+    for (int n1 = 0; n1 < N1; ++n1) x[n1] = col_pair(a, n2 + N2 * n1, a.ln.P, s, v0, v1);
   } else {
     const int64_t s = col_first<MODE>(a) + b;
     const bool v = s < a.S;
