@@ -618,9 +618,18 @@ __device__ __forceinline__ void features2_body(int by, const long long* __restri
   __shared__ unsigned long long part[8][32];
   const int t = threadIdx.x, bx = t & 31, y0 = t >> 5, w = M / 32;
   unsigned long long s = 0;
+  const bool vec = (w & 1) == 0 && ((uintptr_t)counts & 15) == 0;   // 16-byte loads
   for (int y = y0; y < w; y += 8) {
     const long long* row = counts + (size_t)(by * w + y) * M + bx * w;
-    for (int x = 0; x < w; ++x) s += (unsigned long long)row[x];
+    if (vec) {
+#pragma unroll 4
+      for (int x = 0; x < w / 2; ++x) {
+        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(row) + x);
+        s += v.x + v.y;
+      }
+    } else {
+      for (int x = 0; x < w; ++x) s += (unsigned long long)row[x];
+    }
   }
   part[y0][bx] = s;
   __syncthreads();
