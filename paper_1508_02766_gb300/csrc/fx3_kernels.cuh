@@ -232,13 +232,14 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_rows_c2r_kernel(RowsArgs a)
       const bool two = r0 + 1 < a.nrows;
       float2 x[N1];
       p3_a_inv<N1, N2, N3>(x, n23, fx_sm + b * LS, SK, 1);
-      float* o0 = a.out_real + r0 * a.Mout;
+      float *m0, *m1 = nullptr, *o0 = c2r_row(a, r0, &m0),
+                 *o1 = two ? c2r_row(a, r0 + 1, &m1) : nullptr;
 #pragma unroll
       for (int n1 = 0; n1 < N1; ++n1) {
         const int pos = n23 + N23 * n1;
         if (pos < a.Mout) {
-          o0[pos] = x[n1].x;
-          if (two) o0[a.Mout + pos] = x[n1].y;
+          c2r_store(o0, m0, pos, a.Mout, x[n1].x);
+          c2r_store(o1, m1, pos, a.Mout, x[n1].y);
         }
       }
     }

@@ -159,7 +159,30 @@ struct RowsArgs {
   // consecutive h of out, in and out_real.
   const KGen<float>* gens;
   int64_t slab_out, slab_in, slab_real;
+  // c2r of an even result (an autocorrelation): input rows p = 0 .. half - 1
+  // of every grid of P0 rows (half = P0 / 2 + 1 rounded up to even, so that
+  // every grid's rows pair alike; Mout = the whole length); row P0 - p is
+  // stored as row p reversed.  0: every row has an input row.
+  int half, P0;
 };
+
+// Where c2r row r goes: its output row (null: the mirror of an earlier row),
+// and (mirror) the row that takes it reversed, or null.
+__device__ __forceinline__ float* c2r_row(const RowsArgs& a, int64_t r, float** mirror) {
+  *mirror = nullptr;
+  if (!a.half) return a.out_real + r * a.Mout;
+  const int64_t grid = r / a.half;
+  const int p = (int)(r - grid * a.half);
+  if (2 * p > a.P0) return nullptr;
+  float* base = a.out_real + grid * (int64_t)a.P0 * a.Mout;
+  if (p > 0 && 2 * p < a.P0) *mirror = base + (int64_t)(a.P0 - p) * a.Mout;
+  return base + (int64_t)p * a.Mout;
+}
+// Value v at position pos of a row and, reversed, of its mirror.
+__device__ __forceinline__ void c2r_store(float* row, float* mirror, int pos, int M, float v) {
+  if (row) row[pos] = v;
+  if (mirror) mirror[pos ? M - pos : 0] = v;
+}
 
 // Per-bandwidth view of the arguments (h = blockIdx.y).
 __device__ __forceinline__ void rows_slab(RowsArgs& a, KGen<float>& g) {
@@ -346,13 +369,13 @@ __device__ __forceinline__ void rows_a_inv(const RowsArgs& a, const float2* sm) 
 #pragma unroll
   for (int k1 = 0; k1 < N1; ++k1) x[k1] = src[k1 * a.SK];
   idft<N1>(x);
-  float* o0 = a.out_real + r0 * a.Mout;
+  float *m0, *m1 = nullptr, *o0 = c2r_row(a, r0, &m0), *o1 = two ? c2r_row(a, r0 + 1, &m1) : nullptr;
 #pragma unroll
   for (int n1 = 0; n1 < N1; ++n1) {
     const int pos = n2 + N2 * n1;
     if (pos < a.Mout && KDE_DCHECK(r0 < a.nrows, KDE_DBG_ROWS_STORE)) {
-      o0[pos] = x[n1].x;
-      if (two) o0[a.Mout + pos] = x[n1].y;
+      c2r_store(o0, m0, pos, a.Mout, x[n1].x);
+      c2r_store(o1, m1, pos, a.Mout, x[n1].y);
     }
   }
 }
