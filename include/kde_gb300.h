@@ -93,7 +93,8 @@ enum { KDE_SLAB_OFF = 0, KDE_SLAB_ON = 1 };
  *               registers, one exchange through shared memory, an N2-point
  *               DFT per thread (P_k <= 400); longer lines, P_k = N1 N2 N3
  *               (each about 10), take three such phases.  P_k is then the
- *               smallest supported length >= M_k + L_k (at most 2048).
+ *               smallest supported length >= M_k + L_k (at most 2048; 3584
+ *               where KDE_ENGINE_AUTO chooses it, every axis above 400).
  *               KDE_ENGINE_STOCKHAM: mixed-radix passes through shared
  *               memory, P_k the smallest 7-smooth size >= M_k + L_k.
  *               KDE_ENGINE_AUTO: two-phase where it applies (KDE_F32, d >= 2,

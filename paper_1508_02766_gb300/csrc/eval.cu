@@ -31,6 +31,7 @@
 
 #include "fft_engine.cuh"
 #include "fixed_pos.h"
+#include "fx_pairs.h"
 #include "kde_internal.h"
 #include "kde_debug.cuh"
 #include "kgen.cuh"
@@ -2382,7 +2383,8 @@ struct MultiLayout {
 
 kde_status multi_layout(const kde_plan_s* plan, MultiLayout* m) {
   const kde_plan_info& I = plan->info;
-  if (I.d != 2 || I.precision != KDE_F32 || I.engine != KDE_ENGINE_TWO_PHASE)
+  if (I.d != 2 || I.precision != KDE_F32 || I.engine != KDE_ENGINE_TWO_PHASE ||
+      I.P[0] > fxp::kMaxNamedP || I.P[1] > fxp::kMaxNamedP)
     return fail(KDE_ERR_UNSUPPORTED,
                 "batched densities need a KDE_F32 2-D plan with the two-phase engine");
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };

@@ -658,6 +658,7 @@ kde_fx_cols_kernel(ColsArgs a) {
   if (l.n3) {                                                                          \
     switch (l.n1 * 4096 + l.n2 * 64 + l.n3) {                                          \
       KDE_FX_TRIPLES(KDE_FX_CASE_TRIPLE)                                               \
+      KDE_FX_LONG_TRIPLES(KDE_FX_CASE_TRIPLE)                                          \
       default:                                                                         \
         return cudaErrorInvalidConfiguration;                                          \
     }                                                                                  \

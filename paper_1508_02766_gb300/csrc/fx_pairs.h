@@ -16,6 +16,15 @@
   X(8, 12, 12) X(10, 10, 12) X(8, 10, 16) X(9, 12, 12) X(10, 12, 12) X(10, 10, 16)             \
   X(12, 12, 12) X(10, 12, 16) X(8, 16, 16)
 
+// Longer splits, taken where the planner chooses the engine and every axis has
+// more than 400 points (a caller who asks for the two-phase engine by name,
+// or for densities of many bandwidths, gets lines up to kMaxNamedP).  They take these lines from the Stockham
+// passes: on a 2017 x 3001 grid (2048 x 3072 padded, event times) counts rows
+// 53 -> 25 us, middle axis 87 -> 47, output rows 50 -> 18, kernel grid 37 ->
+// 31.
+#define KDE_FX_LONG_TRIPLES(X) \
+  X(12, 12, 16) X(10, 16, 16) X(12, 15, 16) X(12, 16, 16) X(14, 15, 16) X(14, 16, 16)
+
 namespace kde {
 namespace fxp {
 
@@ -32,9 +41,11 @@ inline constexpr Pair kPairs[] = {KDE_FX_PAIRS(KDE_FX_PAIR_ENTRY)};
 #undef KDE_FX_PAIR_ENTRY
 inline constexpr int kNumPairs = sizeof(kPairs) / sizeof(kPairs[0]);
 #define KDE_FX_TRIPLE_ENTRY(a, b, c) Triple{a, b, c},
-inline constexpr Triple kTriples[] = {KDE_FX_TRIPLES(KDE_FX_TRIPLE_ENTRY)};
+inline constexpr Triple kTriples[] = {KDE_FX_TRIPLES(KDE_FX_TRIPLE_ENTRY)
+                                      KDE_FX_LONG_TRIPLES(KDE_FX_TRIPLE_ENTRY)};
 #undef KDE_FX_TRIPLE_ENTRY
 inline constexpr int kNumTriples = sizeof(kTriples) / sizeof(kTriples[0]);
+inline constexpr int kMaxNamedP = 2048;
 inline constexpr int kGenericMax = 20;     // generic kernels: N1, N2 <= 20
 inline constexpr int kGenericMaxP = 400;
 

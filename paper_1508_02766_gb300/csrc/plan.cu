@@ -436,6 +436,8 @@ static kde_status compute_info(int d, const int64_t* M, const double* lo, const 
   int sp[KDE_MAX_D][3] = {};
   for (int k = 0; tp && k < d; ++k) {
     const int64_t P = two_phase_plan(info->P[k], sp[k]);
+    if (o.engine == KDE_ENGINE_TWO_PHASE && P > fxp::kMaxNamedP)
+      return fail(KDE_ERR_UNSUPPORTED, "padded size above the two-phase engine's largest line");
     if (P == 0) {
       if (o.engine == KDE_ENGINE_TWO_PHASE)
         return fail(KDE_ERR_UNSUPPORTED, "padded size above the two-phase engine's largest line");
@@ -443,6 +445,10 @@ static kde_status compute_info(int d, const int64_t* M, const double* lo, const 
     }
     Ptp[k] = P;
   }
+  // lines above kMaxNamedP: planes whose every axis takes three factors
+  for (int k = 0; tp && k < d; ++k)
+    for (int j = 0; j < d; ++j)
+      if (Ptp[k] > fxp::kMaxNamedP && sp[j][2] == 0) tp = false;
   info->engine = tp ? KDE_ENGINE_TWO_PHASE : KDE_ENGINE_STOCKHAM;
   for (int k = 0; k < d; ++k) {
     int64_t P = info->P[k];

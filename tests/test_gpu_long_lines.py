@@ -1,0 +1,66 @@
+"""FP32 lines between 2048 and 3584 points (the splits the planner takes by
+itself): every such split on the row and on the column axis against the
+oracle on every node, the lengths on either side of the last of them, and
+what is refused above 2048: the engine by name and densities of many
+bandwidths."""
+import os
+import re
+
+import numpy as np
+import pytest
+
+from oracle import kde_oracle as O
+from paper_1508_02766_gb300 import kde
+from paper_1508_02766_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+SRC = os.path.join(os.path.dirname(kde.__file__), "csrc", "fx_pairs.h")
+BODY = open(SRC).read().split("#define KDE_FX_LONG_TRIPLES")[1].split("\n\n")[0]
+SPLITS = [tuple(int(v) for v in m.split(",")) for m in re.findall(r"X\(([\d,\s]+)\)", BODY)]
+
+
+def _density(w, **opts):
+    X = torch.from_numpy(np.ascontiguousarray(w.X)).cuda()
+    plan = kde.Plan(w.M, w.lo, w.hi, w.H, precision="f32", tau=w.tau, **opts)
+    c = kde.kde_bin(X, w.lo, w.hi, w.M)
+    return kde.kde_fft_eval(plan, c, kde.kde_kernel_grid(plan, w.n)).cpu().numpy(), plan
+
+
+@pytest.mark.parametrize("axis", [0, 1])
+@pytest.mark.parametrize("split", SPLITS + [(3585, 1, 1)])
+def test_every_long_split(split, axis):
+    P = int(np.prod(split))
+    M, P_min = [12, 13], [401, 401]
+    M[axis], P_min[axis] = P - 100, P
+    w = W.small_case(P, 2, tuple(M), n=3000, precision="f32", scale=1e-4)
+    dens, plan = _density(w, P_min=P_min)
+    if P > 3584:
+        assert plan.info.engine == "stockham"
+    else:
+        assert plan.info.engine == "two_phase" and plan.info.split[axis] == split
+    f, _, _, _ = O.binned_estimate(w.X, w.H, w.lo, w.hi, w.M, tau=w.tau)
+    assert np.max(np.abs(dens - f)) <= 1e-5 * np.max(np.abs(f))
+
+
+def test_short_other_axis_keeps_the_stockham_engine():
+    args = ((40, 40), [0, 0], [1, 1], np.eye(2) * 1e-6)
+    assert kde.kde_plan_info_compute(*args, P_min=(2049, 401)).engine == "two_phase"
+    assert kde.kde_plan_info_compute(*args, P_min=(2049, 400)).engine == "stockham"
+
+
+def test_refusals_above_2048():
+    args = ((40, 40), [0, 0], [1, 1], np.eye(2) * 1e-6)
+    for P, ok in ((2048, True), (2049, False), (3000, False)):
+        if ok:
+            assert kde.kde_plan_info_compute(*args, engine="two_phase", P_min=(P, 0)).engine == "two_phase"
+        else:
+            with pytest.raises(kde.KDEError, match="UNSUPPORTED"):
+                kde.kde_plan_info_compute(*args, engine="two_phase", P_min=(P, 0))
+        plan = kde.Plan(*args, P_min=(P, 401))
+        if ok:
+            assert kde.kde_fft_eval_multi_workspace_bytes(plan) > 0
+        else:
+            with pytest.raises(kde.KDEError, match="UNSUPPORTED"):
+                kde.kde_fft_eval_multi_workspace_bytes(plan)
