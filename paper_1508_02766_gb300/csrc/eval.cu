@@ -2375,10 +2375,13 @@ namespace kde {
 namespace {
 
 constexpr int kMultiChunk = 64;
+// Bandwidths whose parameters go up in one copy: a copy between every two
+// chunks cost 8 us of idle device each.
+constexpr int kMultiUpload = 1024;
 
 struct MultiLayout {
   int Lmax0;
-  size_t off_A, off_gens, off_L0, off_t1, off_K, off_S, total;
+  size_t off_A, off_C, off_gens, off_t1, off_S, total;
 };
 
 kde_status multi_layout(const kde_plan_s* plan, MultiLayout* m) {
@@ -2392,11 +2395,10 @@ kde_status multi_layout(const kde_plan_s* plan, MultiLayout* m) {
   m->Lmax0 = (int)(I.P[0] - I.M[0]);
   const size_t Q = (size_t)I.Q, M0 = (size_t)I.M[0], P0 = (size_t)I.P[0];
   m->off_A = 0;
-  m->off_gens = up(M0 * Q * 8);
-  m->off_L0 = m->off_gens + up(kMultiChunk * sizeof(KGen<float>));
-  m->off_t1 = m->off_L0 + up(kMultiChunk * sizeof(int));
-  m->off_K = m->off_t1 + up((size_t)kMultiChunk * (m->Lmax0 + 1) * Q * 8);
-  m->off_S = m->off_K + up((size_t)kMultiChunk * P0 * Q * 4);
+  m->off_C = up(M0 * Q * 8);
+  m->off_gens = m->off_C + up(P0 * Q * 8);
+  m->off_t1 = m->off_gens + up(kMultiUpload * (sizeof(KGen<float>) + sizeof(int)));
+  m->off_S = m->off_t1 + up((size_t)kMultiChunk * (m->Lmax0 + 1) * Q * 8);
   m->total = m->off_S + up((size_t)kMultiChunk * M0 * Q * 8);
   return KDE_OK;
 }
@@ -2445,20 +2447,28 @@ extern "C" kde_status kde_fft_eval_multi(kde_plan plan, int64_t n, int nH, const
   }
   cudaStream_t st = (cudaStream_t)stream;
   char* ws = (char*)workspace;
-  float2* A = (float2*)(ws + m.off_A);
-  if ((s = fx_count_spectra(plan, reinterpret_cast<const long long*>(counts), A, st)) != KDE_OK)
+  float2* C = (float2*)(ws + m.off_C);
+  if ((s = fx_count_spectrum2(plan, reinterpret_cast<const long long*>(counts),
+                              (float2*)(ws + m.off_A), C, st)) != KDE_OK)
     return s;
   const size_t cells = (size_t)I.M[0] * I.M[1];
-  for (int h0 = 0; h0 < nH; h0 += kMultiChunk) {
-    const int nh = std::min(kMultiChunk, nH - h0);
-    // the chunk's parameters: stream-ordered after the previous chunk's kernels
-    if ((s = upload_async(ws + m.off_gens, gens.data() + h0, nh * sizeof(KGen<float>), st)) != KDE_OK ||
-        (s = upload_async(ws + m.off_L0, L0.data() + h0, nh * sizeof(int), st)) != KDE_OK)
-      return s;
-    s = fx_eval_batch2(plan, A, nh, (const KGen<float>*)(ws + m.off_gens), (const int*)(ws + m.off_L0),
-                       m.Lmax0, (float2*)(ws + m.off_t1), (float*)(ws + m.off_K),
-                       (float2*)(ws + m.off_S), (float*)density + (size_t)h0 * cells, st);
-    if (s != KDE_OK) return s;
+  std::vector<unsigned char> up;
+  for (int u0 = 0; u0 < nH; u0 += kMultiUpload) {
+    const int nu = std::min(kMultiUpload, nH - u0);
+    // parameters, then supports: stream-ordered after the kernels of the last ones
+    const size_t gb = (size_t)nu * sizeof(KGen<float>), lb = (size_t)nu * sizeof(int);
+    up.resize(gb + lb);
+    std::memcpy(up.data(), gens.data() + u0, gb);
+    std::memcpy(up.data() + gb, L0.data() + u0, lb);
+    if ((s = upload_async(ws + m.off_gens, up.data(), up.size(), st)) != KDE_OK) return s;
+    const auto* gens_dev = (const KGen<float>*)(ws + m.off_gens);
+    const int* L0_dev = (const int*)(ws + m.off_gens + gb);
+    for (int h0 = 0; h0 < nu; h0 += kMultiChunk) {
+      s = fx_eval_batch2(plan, C, std::min(kMultiChunk, nu - h0), gens_dev + h0, L0_dev + h0, m.Lmax0,
+                         (float2*)(ws + m.off_t1), (float2*)(ws + m.off_S),
+                         (float*)density + (size_t)(u0 + h0) * cells, st);
+      if (s != KDE_OK) return s;
+    }
   }
   return KDE_OK;
 }

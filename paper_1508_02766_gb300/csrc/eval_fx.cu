@@ -172,7 +172,7 @@ kde_status rows_pass(const kde_plan_s* plan, int kind, int64_t nrows, const long
                  threads, smem, st};
   if (kind == 2) {
     LaunchScope ls("kde_fx_rows_c2r_kernel", st);
-    return done(launch_rows_c2r(l, a), "kde_fx_rows_c2r_kernel");
+    return done(half ? launch_rows_c2r_even(l, a) : launch_rows_c2r(l, a), "kde_fx_rows_c2r_kernel");
   }
   if (kind == SRC_COUNTS) {
     LaunchScope ls("kde_fx_rows_r2c_counts_kernel", st);
@@ -188,7 +188,7 @@ kde_status cols_pass(const kde_plan_s* plan, int k, const char* name, const floa
                      float2* out, float* out_real, const float* K, int64_t S, int64_t O, int Nin,
                      int Nout, int Lw, cudaStream_t st, const Batch* bt = nullptr,
                      float s_pre = 0.f, float s_post = 0.f, unsigned long long* clear = nullptr,
-                     int64_t clear_n = 0) {
+                     int64_t clear_n = 0, const float2* C = nullptr) {
   const kde_plan_info& I = plan->info;
   ColsArgs a{};
   a.s_pre = s_pre;
@@ -210,13 +210,14 @@ kde_status cols_pass(const kde_plan_s* plan, int k, const char* name, const floa
   a.out = out;
   a.out_real = out_real;
   a.K = K;
+  a.C = C;
   a.S = S;
   a.Nin = Nin;
   a.Nout = Nout;
   a.Lw = Lw;
   a.ln = line_of(I, k);
   a.tw = twiddles(plan, k);
-  const int64_t lines = (MODE == COL_FWD_REAL ? (S + 1) / 2 : S);
+  const int64_t lines = (MODE == COL_FWD_REAL || MODE == COL_KMID ? (S + 1) / 2 : S);
   // lines per block over all slabs: at least 4 adjacent columns (a 32-byte
   // sector per row; fewer make every load a partial sector), at most 16
   int B = std::max(4, pick_lines(lines * O, a.ln, true));
@@ -230,7 +231,8 @@ kde_status cols_pass(const kde_plan_s* plan, int k, const char* name, const floa
   if (B < 16)
     while (a.SK % 16 != B % 16) ++a.SK;   // conflict-free reads across k1
   const int threads = (B * threads_per_line(a.ln) + 31) / 32 * 32;
-  const size_t smem = (size_t)a.ln.N1 * a.SK * sizeof(float2);
+  const size_t smem = ((size_t)a.ln.N1 * a.SK + (MODE == COL_KMID && !a.ln.N3 ? (size_t)B * a.ln.P : 0)) *
+                      sizeof(float2);
   if (smem > kSmemMax) return fail(KDE_ERR_UNSUPPORTED, "two-phase column block too large");
   const Launch l{a.ln.N1, a.ln.N2, a.ln.N3, dim3((unsigned)((lines + B - 1) / B), (unsigned)O), threads, smem, st};
   LaunchScope ls(name, st);
@@ -240,6 +242,7 @@ kde_status cols_pass(const kde_plan_s* plan, int k, const char* name, const floa
     case COL_FWD_REAL: e = launch_cols_real(l, a); break;
     case COL_MID: e = launch_cols_mid(l, a); break;
     case COL_AUTO: e = launch_cols_auto(l, a); break;
+    case COL_KMID: e = launch_cols_kmid(l, a); break;
     default: e = launch_cols_inv(l, a); break;
   }
   return done(e, name);
@@ -363,18 +366,22 @@ kde_status fx_fft_eval(kde_plan_s* plan, const long long* counts, const float* K
 
 namespace kde {
 
-// Densities for nh bandwidths of a 2-D plan that share the counts' half
-// spectra A (Eq. 10 with C = F(c) reused; only K changes with H): per
-// bandwidth the kernel-grid rows, its real spectrum, the middle axis
-// (forward, times K, inverse) and the output rows, each pass one launch over
-// all nh bandwidths.  gens and L0 (device) hold each bandwidth's kernel-grid
-// parameters and support along axis 0; Lmax0 bounds the supports.
-kde_status fx_eval_batch2(kde_plan_s* plan, const float2* A, int nh, const KGen<float>* gens,
-                          const int* L0, int Lmax0, float2* t1, float* Kb, float2* Sb,
-                          float* density, cudaStream_t st) {
+// Densities for nh bandwidths of a 2-D plan that share the counts' spectrum C
+// ([P_0][Q], Eq. 10 with C = F(c) reused; only K changes with H): per
+// bandwidth the kernel-grid rows, the axis-0 pass that transforms a pair of
+// their columns to K, multiplies the counts' columns and inverts them
+// (COL_KMID), and the output rows, each pass one launch over all nh
+// bandwidths.  gens and L0 (device) hold each bandwidth's kernel-grid
+// parameters and support along axis 0; Lmax0 bounds the supports.  Against a
+// kernel-spectrum pass and a middle pass that transformed the counts' columns
+// again for every bandwidth, 1024 densities at 512^2 take 2608 us, 3014
+// before (of a chunk of 64: 39 + 86 us -> 96).
+kde_status fx_eval_batch2(kde_plan_s* plan, const float2* C, int nh, const KGen<float>* gens,
+                          const int* L0, int Lmax0, float2* t1, float2* Sb, float* density,
+                          cudaStream_t st) {
   using namespace fx;
   const kde_plan_info& I = plan->info;
-  const int64_t Q = I.Q, M0 = I.M[0], M1 = I.M[1], P0 = I.P[0];
+  const int64_t Q = I.Q, M0 = I.M[0], M1 = I.M[1];
   const int64_t rows_max = (int64_t)Lmax0 + 1;   // lags l_0 >= 0, as in fx_kernel_grid
   Batch b;
   b.nh = nh;
@@ -389,17 +396,9 @@ kde_status fx_eval_batch2(kde_plan_s* plan, const float2* A, int nh, const KGen<
   b.nh = nh;
   b.L0 = L0;
   b.slab_in = rows_max * Q;
-  b.slab_real = P0 * Q;
-  s = cols_pass<COL_FWD_REAL>(plan, 0, "kde_fx_cols_kgen_real_kernel", t1, nullptr, Kb, nullptr,
-                              Q, 1, (int)rows_max, 0, Lmax0, st, &b);
-  if (s != KDE_OK) return s;
-  b = Batch();
-  b.nh = nh;
-  b.slab_in = 0;          // every bandwidth reads the same count spectra
   b.slab_out = M0 * Q;
-  b.slab_K = P0 * Q;
-  s = cols_pass<COL_MID>(plan, 0, "kde_fx_cols_mid_kernel", A, Sb, nullptr, Kb, Q, 1, (int)M0,
-                         (int)M0, -1, st, &b);
+  s = cols_pass<COL_KMID>(plan, 0, "kde_fx_cols_kmid_kernel", t1, Sb, nullptr, nullptr, Q, 1,
+                          (int)rows_max, (int)M0, Lmax0, st, &b, 0.f, 0.f, nullptr, 0, C);
   if (s != KDE_OK) return s;
   b = Batch();
   b.nh = nh;
@@ -429,6 +428,18 @@ kde_status fx_autocorr(kde_plan_s* plan, const long long* counts, float* R, floa
   if (s != KDE_OK) return s;
   return rows_pass(plan, 2, nsets * half, nullptr, 0, 0, nullptr, nullptr, B, R, (int)I.P[1], st,
                    Batch(), half);
+}
+
+// The counts' spectrum of a 2-D plan: half spectra into A, then axis 0 into C
+// ([P_0][Q]).
+kde_status fx_count_spectrum2(kde_plan_s* plan, const long long* counts, float2* A, float2* C,
+                              cudaStream_t st) {
+  using namespace fx;
+  const kde_plan_info& I = plan->info;
+  const kde_status s = fx_count_spectra(plan, counts, A, st);
+  if (s != KDE_OK) return s;
+  return cols_pass<COL_FWD>(plan, 0, "kde_fx_cols_fwd_kernel", A, C, nullptr, nullptr, I.Q, 1,
+                            (int)I.M[0], (int)I.P[0], -1, st);
 }
 
 // The counts' half spectra (first pass of the evaluation) into A.

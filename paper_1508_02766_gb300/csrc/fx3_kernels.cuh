@@ -188,7 +188,7 @@ kde_fx3_rows_fwd_kernel(RowsArgs a, const long long* __restrict__ counts, KGen<f
   }
 }
 
-template <int N1, int N2, int N3>
+template <int N1, int N2, int N3, bool EVEN>
 __global__ void __launch_bounds__(kThreads3) kde_fx3_rows_c2r_kernel(RowsArgs a) {
   pdl_trigger();
   pdl_wait();
@@ -232,14 +232,14 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_rows_c2r_kernel(RowsArgs a)
       const bool two = r0 + 1 < a.nrows;
       float2 x[N1];
       p3_a_inv<N1, N2, N3>(x, n23, fx_sm + b * LS, SK, 1);
-      float *m0, *m1 = nullptr, *o0 = c2r_row(a, r0, &m0),
-                 *o1 = two ? c2r_row(a, r0 + 1, &m1) : nullptr;
+      float *m0, *m1 = nullptr, *o0 = c2r_row<EVEN>(a, r0, &m0),
+                 *o1 = two ? c2r_row<EVEN>(a, r0 + 1, &m1) : nullptr;
 #pragma unroll
       for (int n1 = 0; n1 < N1; ++n1) {
         const int pos = n23 + N23 * n1;
         if (pos < a.Mout) {
-          c2r_store(o0, m0, pos, a.Mout, x[n1].x);
-          c2r_store(o1, m1, pos, a.Mout, x[n1].y);
+          c2r_store<EVEN>(o0, m0, pos, a.Mout, x[n1].x);
+          if (two) c2r_store<EVEN>(o1, m1, pos, a.Mout, x[n1].y);
         }
       }
     }
@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kernel(ColsArgs a) {
   const int W = a.B, SK = a.SK;
   const int t = threadIdx.x;
   const int c = t & (W - 1), r = t >> a.lgB;
-  const int64_t first = (int64_t)blockIdx.x * W * (MODE == COL_FWD_REAL ? 2 : 1);
+  const int64_t first = (int64_t)blockIdx.x * W;
   float2* line = fx_sm + c;
   // COL_MID: the kernel spectrum values of this thread's phase C, loaded
   // now so that their latency hides behind phases A and B
@@ -296,8 +296,8 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kernel(ColsArgs a) {
       const float2* in = a.in;
       float2 x[N1];
       if constexpr (MODE == COL_FWD_REAL) {
-        const int64_t s = first + 2 * c;
-        const bool v0 = s < a.S, v1 = s + 1 < a.S;
+        const int64_t s = first + c;
+        const bool v0 = s < pair_step(a.S), v1 = v0 && s + pair_step(a.S) < a.S;
 #pragma unroll
         for (int n1 = 0; n1 < N1; ++n1) x[n1] = col_pair(a, n23 + N23 * n1, P, s, v0, v1);
       } else {
@@ -340,15 +340,15 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kernel(ColsArgs a) {
           }
         }
       } else if constexpr (MODE == COL_FWD_REAL) {
-        const int64_t s = first + 2 * c;
-        if (s < a.S) {
-          const bool v1 = s + 1 < a.S;
+        const int64_t s = first + c, half = pair_step(a.S);
+        if (s < half) {
+          const bool v1 = s + half < a.S;
           float* out = a.out_real + s;
 #pragma unroll
           for (int k3 = 0; k3 < N3; ++k3) {
             const int64_t k = k1 + N1 * (k2 + N2 * k3);
             out[k * a.S] = z[k3].x;
-            if (v1) out[k * a.S + 1] = z[k3].y;
+            if (v1) out[k * a.S + half] = z[k3].y;
           }
         }
       } else {  // COL_MID: times K, inverse phase C back to the slots
@@ -389,6 +389,72 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kernel(ColsArgs a) {
     }
   }
   if (a.clear) clear_words(a.clear, a.clear_n);
+}
+
+// COL_KMID, three factors: the line's kernel spectra stay in the registers of
+// phase C between the two inverses; the first column's counts are loaded at
+// the start, the second's while the first is transformed.
+template <int N1, int N2, int N3>
+__global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kmid_kernel(ColsArgs a) {
+  pdl_trigger();
+  pdl_wait();
+  constexpr int N23 = N2 * N3, P = N1 * N23;
+  extern __shared__ float2 fx_sm[];
+  cols_slab(a);
+  const int W = a.B, SK = a.SK;
+  const int t = threadIdx.x;
+  const int c = t & (W - 1), r = t >> a.lgB;
+  const int64_t s = (int64_t)blockIdx.x * W + c, half = pair_step(a.S);
+  const bool v0 = s < half, v1 = v0 && s + half < a.S;
+  float2* line = fx_sm + c;
+  const int k1 = r % N1, k2 = r / N1;
+  const int64_t step = (int64_t)(N1 * N2) * a.S;
+  const float2* pc = a.C + s + (int64_t)(k1 + N1 * k2) * a.S;
+  const bool vc = r < N1 * N2;
+  float2 cv[N3], z[N3];
+#pragma unroll
+  for (int k3 = 0; k3 < N3; ++k3) cv[k3] = vc && v0 ? __ldg(pc + k3 * step) : make_float2(0.f, 0.f);
+  if (r < N23) {
+    float2 x[N1];
+#pragma unroll
+    for (int n1 = 0; n1 < N1; ++n1) x[n1] = col_pair(a, r + N23 * n1, P, s, v0, v1);
+    p3_a_fwd<N1, N2, N3>(x, r, a.tw, line, SK, W);
+  }
+  __syncthreads();
+  if (r < N1 * N3) p3_b_fwd<N1, N2, N3>(r / N3, r % N3, a.tw, line, SK, W);
+  __syncthreads();
+  if (vc) p3_c_fwd<N1, N2, N3>(z, k1, k2, line, SK, W);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    if (vc) {
+#pragma unroll
+      for (int k3 = 0; k3 < N3; ++k3) {
+        const float k = h ? z[k3].y : z[k3].x;
+        cv[k3].x *= k;
+        cv[k3].y *= k;
+      }
+      p3_c_inv<N1, N2, N3>(cv, k1, k2, a.tw, line, SK, W);
+      if (h == 0) {
+#pragma unroll
+        for (int k3 = 0; k3 < N3; ++k3) cv[k3] = v1 ? __ldg(pc + half + k3 * step) : make_float2(0.f, 0.f);
+      }
+    }
+    __syncthreads();
+    if (r < N1 * N3) p3_b_inv<N1, N2, N3>(r / N3, r % N3, a.tw, line, SK, W);
+    __syncthreads();
+    if (r < N23 && (h ? v1 : v0)) {
+      float2 x[N1];
+      p3_a_inv<N1, N2, N3>(x, r, line, SK, W);
+      float2* out = a.out + s + (h ? half : 0) + (int64_t)r * a.S;
+      const int64_t ostep = (int64_t)N23 * a.S;
+#pragma unroll
+      for (int n1 = 0; n1 < N1; ++n1) {
+        if (r + N23 * n1 < a.Nout) *out = x[n1];
+        out += ostep;
+      }
+    }
+    if (h == 0) __syncthreads();   // the second inverse rewrites the line
+  }
 }
 
 }  // namespace fx

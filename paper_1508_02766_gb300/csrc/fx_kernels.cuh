@@ -167,10 +167,12 @@ struct RowsArgs {
 };
 
 // Where c2r row r goes: its output row (null: the mirror of an earlier row),
-// and (mirror) the row that takes it reversed, or null.
+// and (mirror) the row that takes it reversed, or null.  EVEN: half > 0 (its
+// own kernels: the branches cost the others' stores 10%).
+template <bool EVEN>
 __device__ __forceinline__ float* c2r_row(const RowsArgs& a, int64_t r, float** mirror) {
   *mirror = nullptr;
-  if (!a.half) return a.out_real + r * a.Mout;
+  if constexpr (!EVEN) return a.out_real + r * a.Mout;
   const int64_t grid = r / a.half;
   const int p = (int)(r - grid * a.half);
   if (2 * p > a.P0) return nullptr;
@@ -179,9 +181,10 @@ __device__ __forceinline__ float* c2r_row(const RowsArgs& a, int64_t r, float** 
   return base + (int64_t)p * a.Mout;
 }
 // Value v at position pos of a row and, reversed, of its mirror.
+template <bool EVEN>
 __device__ __forceinline__ void c2r_store(float* row, float* mirror, int pos, int M, float v) {
-  if (row) row[pos] = v;
-  if (mirror) mirror[pos ? M - pos : 0] = v;
+  if (!EVEN || row) row[pos] = v;
+  if (EVEN && mirror) mirror[pos ? M - pos : 0] = v;
 }
 
 // Per-bandwidth view of the arguments (h = blockIdx.y).
@@ -355,7 +358,7 @@ __device__ __forceinline__ void rows_b_inv(const RowsArgs& a, float2* sm) {
 }
 
 // Inverse row pass, phase A: inverse N1-point DFT, rows cropped to Mout.
-template <int N1, int N2T = 0>
+template <int N1, int N2T, bool EVEN>
 __device__ __forceinline__ void rows_a_inv(const RowsArgs& a, const float2* sm) {
   const int N2 = factor<N2T>(a.ln.N2);
   const int t = threadIdx.x;
@@ -369,18 +372,19 @@ __device__ __forceinline__ void rows_a_inv(const RowsArgs& a, const float2* sm) 
 #pragma unroll
   for (int k1 = 0; k1 < N1; ++k1) x[k1] = src[k1 * a.SK];
   idft<N1>(x);
-  float *m0, *m1 = nullptr, *o0 = c2r_row(a, r0, &m0), *o1 = two ? c2r_row(a, r0 + 1, &m1) : nullptr;
+  float *m0, *m1 = nullptr, *o0 = c2r_row<EVEN>(a, r0, &m0),
+             *o1 = two ? c2r_row<EVEN>(a, r0 + 1, &m1) : nullptr;
 #pragma unroll
   for (int n1 = 0; n1 < N1; ++n1) {
     const int pos = n2 + N2 * n1;
     if (pos < a.Mout && KDE_DCHECK(r0 < a.nrows, KDE_DBG_ROWS_STORE)) {
-      c2r_store(o0, m0, pos, a.Mout, x[n1].x);
-      c2r_store(o1, m1, pos, a.Mout, x[n1].y);
+      c2r_store<EVEN>(o0, m0, pos, a.Mout, x[n1].x);
+      if (two) c2r_store<EVEN>(o1, m1, pos, a.Mout, x[n1].y);
     }
   }
 }
 
-template <int CLS, int N1T, int N2T>
+template <int CLS, int N1T, int N2T, bool EVEN>
 __global__ void __launch_bounds__(block_limit<N1T, N2T>())
 kde_fx_rows_c2r_kernel(RowsArgs a) {
   pdl_trigger();
@@ -390,7 +394,7 @@ kde_fx_rows_c2r_kernel(RowsArgs a) {
   rows_slab(a, g_unused);
   size_call<N2T, CLS>(a.ln.N2, [&](auto N) { rows_b_inv<decltype(N)::value, N1T>(a, fx_sm); });
   __syncthreads();
-  size_call<N1T, CLS>(a.ln.N1, [&](auto N) { rows_a_inv<decltype(N)::value, N2T>(a, fx_sm); });
+  size_call<N1T, CLS>(a.ln.N1, [&](auto N) { rows_a_inv<decltype(N)::value, N2T, EVEN>(a, fx_sm); });
 }
 
 // ---------------------------------------------------------------------------
@@ -402,13 +406,18 @@ kde_fx_rows_c2r_kernel(RowsArgs a) {
 // ---------------------------------------------------------------------------
 // COL_AUTO: COL_MID with z <- |s_pre z|^2 s_post in place of the product
 // with K (the counts' power spectrum, for their autocorrelation).
-enum { COL_FWD = 0, COL_FWD_REAL = 1, COL_MID = 2, COL_INV = 3, COL_AUTO = 4 };
+// COL_KMID: COL_FWD_REAL and, in place of its store, the product with the
+// transformed count columns C and the inverse with crop, for both columns of
+// the line (densities of many bandwidths: the counts' columns are transformed
+// once, the kernel spectrum never leaves the block).
+enum { COL_FWD = 0, COL_FWD_REAL = 1, COL_MID = 2, COL_INV = 3, COL_AUTO = 4, COL_KMID = 5 };
 
 struct ColsArgs {
   const float2* in;
   float2* out;
   float* out_real;   // COL_FWD_REAL: [P][S]
   const float* K;    // COL_MID: real spectrum [P][S]
+  const float2* C;   // COL_KMID: transformed count columns [P][S]
   int64_t S;         // columns
   int Nin;           // input rows holding data (COL_INV: P)
   int Nout;          // output rows kept (crop); COL_FWD: P
@@ -466,9 +475,14 @@ __device__ __forceinline__ int col_source(int pos, int P, int Lw, int Nin) {
   return l <= Lw ? l + Lw : -1;
 }
 
-// Value at transform position pos of the two Hermitian columns s, s + 1 of a
-// COL_FWD_REAL line, as p + i q (v0, v1: the columns exist): row |l| of lag l,
-// conjugated for l < 0.
+// A COL_FWD_REAL line holds columns s and s + pair_step(S), s below the step:
+// neighbouring lines then read and write neighbouring columns (columns 2 s
+// and 2 s + 1 used half of each sector at a time: the many-bandwidth pass 101
+// -> 96 us a chunk, the 256^3 kernel grid level).
+__device__ __forceinline__ int64_t pair_step(int64_t S) { return (S + 1) / 2; }
+
+// Value at transform position pos of the line's two Hermitian columns, as
+// p + i q (v0, v1: the columns exist): row |l| of lag l, conjugated for l < 0.
 __device__ __forceinline__ float2 col_pair(const ColsArgs& a, int pos, int P, int64_t s, bool v0,
                                            bool v1) {
   const int l = wrapped_lag(pos, P, a.Lw);
@@ -476,7 +490,7 @@ __device__ __forceinline__ float2 col_pair(const ColsArgs& a, int pos, int P, in
   if (l <= a.Lw) {
     const float2* row = a.in + (int64_t)(l < 0 ? -l : l) * a.S + s;
     if (v0) p = __ldg(row);
-    if (v1) q = __ldg(row + 1);
+    if (v1) q = __ldg(row + pair_step(a.S));
     if (l < 0) {
       p.y = -p.y;
       q.y = -q.y;
@@ -485,10 +499,7 @@ __device__ __forceinline__ float2 col_pair(const ColsArgs& a, int pos, int P, in
   return make_float2(p.x - q.y, p.y + q.x);
 }
 
-template <int MODE>
-__device__ __forceinline__ int64_t col_first(const ColsArgs& a) {
-  return (int64_t)blockIdx.x * a.B * (MODE == COL_FWD_REAL ? 2 : 1);
-}
+__device__ __forceinline__ int64_t col_first(const ColsArgs& a) { return (int64_t)blockIdx.x * a.B; }
 
 template <int N1, int MODE, int N2T = 0>
 __device__ __forceinline__ void cols_a_fwd(const ColsArgs& a, float2* sm) {
@@ -499,12 +510,12 @@ __device__ __forceinline__ void cols_a_fwd(const ColsArgs& a, float2* sm) {
   const float2* in = a.in;
   float2 x[N1];
   if constexpr (MODE == COL_FWD_REAL) {
-    const int64_t s = col_first<MODE>(a) + 2 * b;
-    const bool v0 = s < a.S, v1 = s + 1 < a.S;
+    const int64_t s = col_first(a) + b;
+    const bool v0 = s < pair_step(a.S), v1 = v0 && s + pair_step(a.S) < a.S;
 #pragma unroll
     for (int n1 = 0; n1 < N1; ++n1) x[n1] = col_pair(a, n2 + N2 * n1, a.ln.P, s, v0, v1);
   } else {
-    const int64_t s = col_first<MODE>(a) + b;
+    const int64_t s = col_first(a) + b;
     const bool v = s < a.S;
     if (a.Lw < 0) {
       // plain rows: position pos reads row pos < Nin; the row pointer steps
@@ -542,7 +553,7 @@ __device__ __forceinline__ void cols_b_fwd(const ColsArgs& a, float2* sm) {
   for (int n2 = 0; n2 < N2; ++n2) y[n2] = src[n2 * a.B];
   dft<N2>(y);
   if constexpr (MODE == COL_FWD) {
-    const int64_t s = col_first<MODE>(a) + b;
+    const int64_t s = col_first(a) + b;
     if (s >= a.S) return;
     float2* out = a.out + s + (int64_t)k1 * a.S;
     const int64_t step = (int64_t)N1 * a.S;
@@ -552,15 +563,15 @@ __device__ __forceinline__ void cols_b_fwd(const ColsArgs& a, float2* sm) {
       out += step;
     }
   } else if constexpr (MODE == COL_FWD_REAL) {
-    const int64_t s = col_first<MODE>(a) + 2 * b;
-    if (s >= a.S) return;
-    const bool v1 = s + 1 < a.S;
+    const int64_t s = col_first(a) + b, half = pair_step(a.S);
+    if (s >= half) return;
+    const bool v1 = s + half < a.S;
     float* out = a.out_real + s;
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) {
       const int64_t k = k1 + N1 * k2;
       out[k * a.S] = y[k2].x;
-      if (v1) out[k * a.S + 1] = y[k2].y;
+      if (v1) out[k * a.S + half] = y[k2].y;
     }
   } else if constexpr (MODE == COL_AUTO) {  // power spectrum, inverse, back to the slots
 #pragma unroll
@@ -570,7 +581,7 @@ __device__ __forceinline__ void cols_b_fwd(const ColsArgs& a, float2* sm) {
     }
     b_inv_store<N2>(y, k1, a.tw, src, a.B);
   } else {  // COL_MID: times K, inverse, back to the same slots
-    const int64_t s = col_first<MODE>(a) + b;
+    const int64_t s = col_first(a) + b;
     const bool v = s < a.S;
     const float* pk = a.K + s + (int64_t)k1 * a.S;
     const int64_t step = (int64_t)N1 * a.S;
@@ -592,7 +603,7 @@ __device__ __forceinline__ void cols_b_inv(const ColsArgs& a, float2* sm) {
   const int t = threadIdx.x;
   if (t >= a.B * N1) return;
   const int b = t & (a.B - 1), k1 = t >> a.lgB;
-  const int64_t s = col_first<COL_INV>(a) + b;
+  const int64_t s = col_first(a) + b;
   const bool v = s < a.S;
   const float2* in = a.in + s + (int64_t)k1 * a.S;
   const int64_t step = (int64_t)N1 * a.S;
@@ -612,7 +623,7 @@ __device__ __forceinline__ void cols_a_inv(const ColsArgs& a, const float2* sm) 
   const int t = threadIdx.x;
   if (t >= a.B * N2) return;
   const int b = t & (a.B - 1), n2 = t >> a.lgB;
-  const int64_t s = col_first<MODE>(a) + b;
+  const int64_t s = col_first(a) + b;
   if (s >= a.S) return;
   const float2* src = sm + b + n2 * a.B;
   float2 x[N1];
@@ -650,6 +661,87 @@ kde_fx_cols_kernel(ColsArgs a) {
     }
   }
   if (a.clear) clear_words(a.clear, a.clear_n);
+}
+
+// Inverse phase A into column s (nothing stored for s >= S).
+template <int N1, int N2T>
+__device__ __forceinline__ void cols_a_inv_at(const ColsArgs& a, const float2* sm, bool second) {
+  const int N2 = factor<N2T>(a.ln.N2);
+  const int t = threadIdx.x;
+  if (t >= a.B * N2) return;
+  const int b = t & (a.B - 1), n2 = t >> a.lgB;
+  const int64_t half = pair_step(a.S), s0 = col_first(a) + b, s = s0 + (second ? half : 0);
+  if (s0 >= half || s >= a.S) return;
+  const float2* src = sm + b + n2 * a.B;
+  float2 x[N1];
+#pragma unroll
+  for (int k1 = 0; k1 < N1; ++k1) x[k1] = src[k1 * a.SK];
+  idft<N1>(x);
+  float2* out = a.out + s + (int64_t)n2 * a.S;
+  const int64_t step = (int64_t)N2 * a.S;
+#pragma unroll
+  for (int n1 = 0; n1 < N1; ++n1) {
+    if (n2 + N2 * n1 < a.Nout) *out = x[n1];
+    out += step;
+  }
+}
+
+// COL_KMID, two factors: the line's kernel spectra (its two columns as the
+// real and imaginary part) stay in shared memory between the two inverses,
+// entry (column pair b, k) at kb[b + B k].
+template <int CLS, int N1T, int N2T>
+__global__ void __launch_bounds__(block_limit<N1T, N2T>())
+kde_fx_cols_kmid_kernel(ColsArgs a) {
+  pdl_trigger();
+  pdl_wait();
+  extern __shared__ float2 fx_sm[];
+  cols_slab(a);
+  const int n1r = factor<N1T>(a.ln.N1);
+  float2* kb = fx_sm + n1r * a.SK;
+  const int t = threadIdx.x, b = t & (a.B - 1), k1 = t >> a.lgB;
+  size_call<N1T, CLS>(a.ln.N1, [&](auto N) {
+    cols_a_fwd<decltype(N)::value, COL_FWD_REAL, N2T>(a, fx_sm);
+  });
+  __syncthreads();
+  size_call<N2T, CLS>(a.ln.N2, [&](auto N) {
+    constexpr int N2 = decltype(N)::value;
+    if (t >= a.B * n1r) return;
+    const float2* src = fx_sm + b + k1 * a.SK;
+    float2 y[N2];
+#pragma unroll
+    for (int n2 = 0; n2 < N2; ++n2) y[n2] = src[n2 * a.B];
+    dft<N2>(y);
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) kb[b + a.B * (k1 + n1r * k2)] = y[k2];
+  });
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    size_call<N2T, CLS>(a.ln.N2, [&](auto N) {
+      constexpr int N2 = decltype(N)::value;
+      if (t >= a.B * n1r) return;
+      const int64_t half = pair_step(a.S), s0 = col_first(a) + b, s = s0 + (h ? half : 0);
+      const bool v = s0 < half && s < a.S;
+      const float2* pc = a.C + s + (int64_t)k1 * a.S;
+      const int64_t step = (int64_t)n1r * a.S;
+      float2 y[N2];
+#pragma unroll
+      for (int k2 = 0; k2 < N2; ++k2) {
+        y[k2] = v ? __ldg(pc) : make_float2(0.f, 0.f);
+        pc += step;
+      }
+#pragma unroll
+      for (int k2 = 0; k2 < N2; ++k2) {
+        const float2 kk = kb[b + a.B * (k1 + n1r * k2)];   // this thread's own entries
+        const float k = h ? kk.y : kk.x;
+        y[k2].x *= k;
+        y[k2].y *= k;
+      }
+      b_inv_store<N2>(y, k1, a.tw, fx_sm + b + k1 * a.SK, a.B);
+    });
+    __syncthreads();
+    size_call<N1T, CLS>(a.ln.N1, [&](auto N) { cols_a_inv_at<decltype(N)::value, N2T>(a, fx_sm, h); });
+    __syncthreads();
+  }
 }
 
 // Launch of the kernel for the split (N1, N2): the one compiled for it if it
@@ -713,11 +805,13 @@ struct Launch {
 cudaError_t launch_rows_counts(const Launch& l, const RowsArgs& a, const long long* counts);
 cudaError_t launch_rows_kgen(const Launch& l, const RowsArgs& a, const KGen<float>& g);
 cudaError_t launch_rows_c2r(const Launch& l, const RowsArgs& a);
+cudaError_t launch_rows_c2r_even(const Launch& l, const RowsArgs& a);
 cudaError_t launch_cols_fwd(const Launch& l, const ColsArgs& a);
 cudaError_t launch_cols_real(const Launch& l, const ColsArgs& a);
 cudaError_t launch_cols_mid(const Launch& l, const ColsArgs& a);
 cudaError_t launch_cols_auto(const Launch& l, const ColsArgs& a);
 cudaError_t launch_cols_inv(const Launch& l, const ColsArgs& a);
+cudaError_t launch_cols_kmid(const Launch& l, const ColsArgs& a);
 
 }  // namespace fx
 }  // namespace kde

@@ -77,9 +77,11 @@ kde_status fx_fft_eval(kde_plan_s* plan, const long long* counts, const float* K
 kde_status fx_count_spectra(kde_plan_s* plan, const long long* counts, float2* A, cudaStream_t st);
 kde_status fx_autocorr(kde_plan_s* plan, const long long* counts, float* R, float2* A, float2* B,
                        int64_t nsets, cudaStream_t st);
-kde_status fx_eval_batch2(kde_plan_s* plan, const float2* A, int nh, const KGen<float>* gens,
-                          const int* L0, int Lmax0, float2* t1, float* Kb, float2* Sb,
-                          float* density, cudaStream_t st);
+kde_status fx_count_spectrum2(kde_plan_s* plan, const long long* counts, float2* A, float2* C,
+                              cudaStream_t st);
+kde_status fx_eval_batch2(kde_plan_s* plan, const float2* C, int nh, const KGen<float>* gens,
+                          const int* L0, int Lmax0, float2* t1, float2* Sb, float* density,
+                          cudaStream_t st);
 
 // Prepared batches of 2-D datasets (kde_prepare2_batch): binning of nsets
 // datasets onto one grid (bin.cu; samples rows [off[s], off[s+1]) of X,
@@ -101,11 +103,13 @@ int debug_read_eval();
 int debug_read_fx_rows_counts();
 int debug_read_fx_rows_kgen();
 int debug_read_fx_rows_c2r();
+int debug_read_fx_rows_c2r_even();
 int debug_read_fx_cols_fwd();
 int debug_read_fx_cols_real();
 int debug_read_fx_cols_mid();
 int debug_read_fx_cols_auto();
 int debug_read_fx_cols_inv();
+int debug_read_fx_cols_kmid();
 int debug_read_fx_slab_fwd();
 int debug_read_fx_slab_inv();
 

@@ -607,8 +607,10 @@ kde_status kde_debug_status(int* enabled, int* code) {
   if (e != cudaSuccess) return cuda_fail(e, "kde_debug_status");
   int (*readers[])() = {kde::debug_read_bin, kde::debug_read_eval, kde::debug_read_fx_rows_counts,
                         kde::debug_read_fx_rows_kgen, kde::debug_read_fx_rows_c2r,
+                        kde::debug_read_fx_rows_c2r_even,
                         kde::debug_read_fx_cols_fwd, kde::debug_read_fx_cols_real,
                         kde::debug_read_fx_cols_mid, kde::debug_read_fx_cols_inv,
+                        kde::debug_read_fx_cols_kmid,
                         kde::debug_read_fx_cols_auto, kde::debug_read_fx_slab_fwd,
                         kde::debug_read_fx_slab_inv};
   for (auto rd : readers) {
