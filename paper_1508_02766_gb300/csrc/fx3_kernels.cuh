@@ -118,7 +118,7 @@ template <int N1, int N2, int N3, int SRC>
 __global__ void __launch_bounds__(kThreads3)
 kde_fx3_rows_fwd_kernel(RowsArgs a, const long long* __restrict__ counts, KGen<float> g) {
   pdl_trigger();
-  pdl_wait();
+  rows_wait_early<SRC>(a);
   constexpr int N23 = N2 * N3, P = N1 * N23;
   extern __shared__ float2 fx_sm[];
   rows_slab(a, g);
@@ -171,6 +171,7 @@ kde_fx3_rows_fwd_kernel(RowsArgs a, const long long* __restrict__ counts, KGen<f
     for (int k3 = 0; k3 < N3; ++k3) base[k3] = z[k3];
   }
   __syncthreads();
+  rows_wait_late<SRC>(a);
   // X = F(x), Y = F(y) from Z = F(x + i y) on [0, Q)
   for (int b = 0; b < a.B; ++b) {
     const int64_t r0 = 2 * ((int64_t)blockIdx.x * a.B + b);

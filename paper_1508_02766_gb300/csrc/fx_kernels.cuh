@@ -312,11 +312,25 @@ __device__ __forceinline__ void rows_stage_kgen(const RowsArgs& a, const KGen<fl
   }
 }
 
+// Where the forward row pass waits for the kernels before it: the counts are
+// theirs, but a kernel grid whose parameters are kernel arguments is formed
+// and transformed beside them (usually the binning's last wave) and only its
+// store waits (a 1024^2 estimate of 10^6 samples 62.8 -> 58.2 us, 2017 x 3001
+// of 4*10^6 177 -> 169).
+template <int SRC>
+__device__ __forceinline__ void rows_wait_early(const RowsArgs& a) {
+  if (SRC == SRC_COUNTS || a.gens) pdl_wait();
+}
+template <int SRC>
+__device__ __forceinline__ void rows_wait_late(const RowsArgs& a) {
+  if (SRC == SRC_KGEN && !a.gens) pdl_wait();
+}
+
 template <int CLS, int N1T, int N2T, int SRC>
 __global__ void __launch_bounds__(block_limit<N1T, N2T>())
 kde_fx_rows_fwd_kernel(RowsArgs a, const long long* __restrict__ counts, KGen<float> g) {
   pdl_trigger();
-  pdl_wait();
+  rows_wait_early<SRC>(a);
   extern __shared__ float2 fx_sm[];
   rows_slab(a, g);
   if constexpr (SRC == SRC_KGEN) {
@@ -328,6 +342,7 @@ kde_fx_rows_fwd_kernel(RowsArgs a, const long long* __restrict__ counts, KGen<fl
   __syncthreads();
   size_call<N2T, CLS>(a.ln.N2, [&](auto N) { rows_b_fwd<decltype(N)::value, N1T>(a, fx_sm); });
   __syncthreads();
+  rows_wait_late<SRC>(a);
   rows_split_store<N1T, N2T>(a, fx_sm);
 }
 
