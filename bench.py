@@ -96,13 +96,17 @@ def algorithmic_bytes(info, n, x_itemsize):
     # second read of the samples and its records are overhead
     b.update({"kde_bin_count_kernel": n * d * x_itemsize, "kde_bin_scatter_kernel": 0,
               "kde_bin_accum_kernel": 8 * cells})
+    b["kde_bin_private_kernel"] = b["kde_bin_kernel"]
     if d == 1:
-        b["kde_rows_r2c_kgen_kernel"] = Q * r
-        b["kde_line1d_kernel"] = 8 * cells + Q * r + cells * r
+        b["kde_rows_r2c_kgen_kernel"] = b["kde_line1d_kgen_kernel"] = Q * r
+        b["kde_line1d_kernel"] = b["kde_line1d_cluster_kernel"] = 8 * cells + Q * r + cells * r
     elif d == 2:
         w0 = 2 * L[0] + 1
         b["kde_rows_r2c_kgen_kernel"] = w0 * Q * cs
         b["kde_cols_kgen_real_kernel"] = w0 * Q * cs + P[0] * Q * r
+        # the direct sums keep the rows at lags l_0 >= 0 only
+        b["kde_rows_kgen_sums_kernel"] = (L[0] + 1) * Q * cs
+        b["kde_cols_kgen_sums_kernel"] = (L[0] + 1) * Q * cs + P[0] * Q * r
         b["kde_rows_r2c_counts_kernel"] = 8 * cells + M[0] * Q * cs
         b["kde_cols_mid_kernel"] = 2 * M[0] * Q * cs + P[0] * Q * r
         b["kde_rows_c2r_kernel"] = M[0] * Q * cs + cells * r
@@ -1492,7 +1496,7 @@ def learned_main(args):
     Lv = np.minimum(Mg - 1.0, np.ceil(sc.tau * np.sqrt(lam)[:, None] / dlt[None, :]))
     # every matrix scored in the profiled pass (its first nprof datasets)
     ac_total = float(np.sum(8.0 * (Lv[:, 0] + 1.0) * (2.0 * Lv[:, 1] + 1.0)))
-    flops = {"kde_lscv_ac_kernel": ac_total, "kde_lscv_theta_sums_kernel": ac_total,
+    flops = {"kde_lscv_ac_kernel": ac_total, "kde_lscv_ac_sets_kernel": ac_total, "kde_lscv_theta_sums_kernel": ac_total,
              "kde_gemm_tc_kernel": nprof * 2.0 * 128 * (din * hid + hid * hid + hid * 16)}
     dom = max(prof, key=lambda k: prof[k][0])
     sm_max = clocks.get("sm_max_mhz") or 2070.0
@@ -1503,8 +1507,9 @@ def learned_main(args):
               "kde_bin_sets_kernel": Bsel * (8.0 * n + 8.0 * cells),
               "kde_features2_sets_kernel": Bsel * (8.0 * cells + 4.0 * kde.FEAT_DIM),
               "kde_rows_r2c_counts_kernel": Bsel * (8.0 * cells + Lm.GRID_M * Q * 8.0),
-              "kde_cols_auto_kernel": Bsel * (Lm.GRID_M * Q * 8.0 + P0 * Q * 8.0),
-              "kde_rows_c2r_kernel": Bsel * (P0 * Q * 8.0 + P0 * P1 * 4.0)}
+              # R is even: half of its rows are transformed, all are stored
+              "kde_cols_auto_kernel": Bsel * (Lm.GRID_M * Q * 8.0 + (P0 // 2 + 1) * Q * 8.0),
+              "kde_rows_c2r_kernel": Bsel * ((P0 // 2 + 1) * Q * 8.0 + P0 * P1 * 4.0)}
     # the same passes on the two-phase engine
     for k in ("kde_rows_r2c_counts_kernel", "kde_cols_auto_kernel", "kde_rows_c2r_kernel"):
         nbytes[k.replace("kde_", "kde_fx_", 1)] = nbytes[k]

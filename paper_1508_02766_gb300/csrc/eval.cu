@@ -35,6 +35,7 @@
 #include "kde_internal.h"
 #include "kde_debug.cuh"
 #include "kgen.cuh"
+#include "pdl.cuh"
 
 namespace kde {
 namespace {
@@ -1653,6 +1654,77 @@ kde_status kgen_for(const kde_plan_info& I, const double* A, double detA, const 
   return KDE_OK;
 }
 
+// FP64 2-D kernel grids with small supports: both passes as direct sums over
+// the lags, spread over the chip.  An FP64 line transform is one warp's (or a
+// few) dependent stages whatever the support; the sums are (L_0 + 1) Q L_1 and
+// P_0 Q L_0 terms.  Transforms against sums, both passes (us, graph of ten,
+// GB300): 32^2, L = 3 17.4 / 2.7; 128^2, L = 15 23.8 / 4.5; 256^2, L = 30 26.4
+// / 11.9; 400^2, L = 24 (2.2 M terms) 34 / 22; 256^2, L = 64 (3.1 M) 27 / 27.
+//
+// Rows: block l_0 forms T(l_0, q) = sum_{l_1} k e^{-2 pi i q l_1 / P_1} for the
+// lags l_0 >= 0, a thread a frequency: with s, d = k(l_0, l_1) +- k(l_0, -l_1),
+// Re T = k(l_0, 0) + sum s cos, Im T = -sum d sin.  Nothing here reads what the
+// kernels before it write, so only the store waits for them.
+__global__ void __launch_bounds__(128) kde_rows_kgen_sums_kernel(KGen<double> gen, int P, int Q,
+                                                                 const double2* __restrict__ tw,
+                                                                 double2* __restrict__ out) {
+  extern __shared__ __align__(16) double2 ks[];   // (s, d) of lag l_1 >= 1; ks[0].x = k(l_0, 0)
+  pdl_trigger();
+  const int l0 = blockIdx.x, L1 = gen.L[1];
+  for (int l1 = threadIdx.x; l1 <= L1; l1 += blockDim.x) {
+    const int p[KDE_MAX_D] = {l0, l1, 0}, m[KDE_MAX_D] = {l0, -l1, 0};
+    const double kp = kernel_value(gen, p), km = kernel_value(gen, m);
+    ks[l1] = l1 ? make_double2(kp + km, kp - km) : make_double2(kp, 0.0);
+  }
+  __syncthreads();
+  const int q = blockIdx.y * blockDim.x + threadIdx.x;
+  double re = ks[0].x, im = 0.0;
+  if (q < Q) {
+    int m = 0;
+#pragma unroll 4
+    for (int l1 = 1; l1 <= L1; ++l1) {
+      m += q;
+      if (m >= P) m -= P;
+      const double2 w = __ldg(tw + m), k = ks[l1];
+      re = fma(k.x, w.x, re);
+      im = fma(k.y, w.y, im);
+    }
+  }
+  pdl_wait();
+  if (q < Q) out[(int64_t)l0 * Q + q] = make_double2(re, im);
+}
+
+// Columns: block q forms K(w, q) = T(0, q) + 2 Re sum_{l_0 >= 1} T(l_0, q)
+// e^{-2 pi i w l_0 / P_0}, a thread a frequency (T(-l_0) is T(l_0)'s
+// conjugate); stored at w sw + q sq.
+__global__ void __launch_bounds__(128) kde_cols_kgen_sums_kernel(const double2* __restrict__ in, int L0,
+                                                                 int P, int Q,
+                                                                 const double2* __restrict__ tw,
+                                                                 double* __restrict__ K, int64_t sw,
+                                                                 int64_t sq) {
+  extern __shared__ __align__(16) double2 t_sm[];
+  pdl_trigger();
+  pdl_wait();
+  const int q = blockIdx.x;
+  for (int l = threadIdx.x; l <= L0; l += blockDim.x) t_sm[l] = in[(int64_t)l * Q + q];
+  __syncthreads();
+  const int w = blockIdx.y * blockDim.x + threadIdx.x;
+  if (w >= P) return;
+  double s = 0.0;
+  int m = 0;
+#pragma unroll 4
+  for (int l = 1; l <= L0; ++l) {
+    m += w;
+    if (m >= P) m -= P;
+    const double2 e = __ldg(tw + m), t = t_sm[l];
+    s = fma(t.x, e.x, fma(-t.y, e.y, s));
+  }
+  K[w * sw + q * sq] = t_sm[0].x + 2.0 * s;
+}
+
+// Terms up to which each pass is the shorter as sums.
+constexpr int64_t kKgenSums = 3 << 20;
+
 template <typename T>
 kde_status kernel_grid_impl(kde_plan_s* plan, int64_t n, void* Kspec, void* ws, cudaStream_t st) {
   using V = typename Cplx<T>::type;
@@ -1684,6 +1756,29 @@ kde_status kernel_grid_impl(kde_plan_s* plan, int64_t n, void* Kspec, void* ws, 
     return launch_rows<T>(kde_rows_r2c_kgen_kernel<T>, "kde_rows_r2c_kgen_kernel", 1, rp, st, gen);
   }
   V* t1 = (V*)ws;
+  if constexpr (std::is_same<T, double>::value) {
+    if (d == 2 && (I.L[0] + 1) * I.Q * I.L[1] <= kKgenSums && I.P[0] * I.Q * I.L[0] <= kKgenSums) {
+      const int Q = (int)I.Q, P0 = (int)I.P[0], L0 = (int)I.L[0];
+      cudaError_t e;
+      {
+        LaunchScope ls("kde_rows_kgen_sums_kernel", st);
+        e = launch_pdl(kde_rows_kgen_sums_kernel, dim3((unsigned)(L0 + 1), (unsigned)((Q + 127) / 128)),
+                       dim3(128), (size_t)(I.L[1] + 1) * sizeof(double2), st, gen, (int)I.P[1], Q,
+                       twiddles<T>(plan, 1), t1);
+        if (e == cudaSuccess) e = cudaGetLastError();
+        if (e != cudaSuccess) return cuda_fail(e, "kde_rows_kgen_sums_kernel");
+      }
+      // the layout the middle pass reads (launch_cols)
+      const bool simd = simd_cols<T>(plan->cols_variant, I.Q, P0);
+      LaunchScope ls("kde_cols_kgen_sums_kernel", st);
+      e = launch_pdl(kde_cols_kgen_sums_kernel, dim3((unsigned)Q, (unsigned)((P0 + 127) / 128)),
+                     dim3(128), (size_t)(L0 + 1) * sizeof(double2), st, (const double2*)t1, L0, P0, Q,
+                     twiddles<T>(plan, 0), (double*)Kspec, simd ? (int64_t)Q : (int64_t)1,
+                     simd ? (int64_t)1 : (int64_t)P0);
+      if (e == cudaSuccess) e = cudaGetLastError();
+      return e == cudaSuccess ? KDE_OK : cuda_fail(e, "kde_cols_kgen_sums_kernel");
+    }
+  }
   int64_t rows = 1;
   for (int k = 0; k < d - 1; ++k) rows *= 2 * I.L[k] + 1;
   rp.nrows = rows;
