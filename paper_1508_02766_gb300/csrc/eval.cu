@@ -1298,8 +1298,9 @@ struct ThetaArgs {
 
 // One thread per matrix: the same FP64 steps as the host path (H from
 // theta, support by Eq. 15, Cholesky factor, completed-square constants),
-// rounded to the lag sums' FP32 parameters.
-__global__ void __launch_bounds__(128) kde_theta_gen_kernel(ThetaArgs t) {
+// rounded to the lag sums' FP32 parameters.  Blocks of one warp: FP64 bound,
+// so the warps are spread over every SM.
+__global__ void __launch_bounds__(32) kde_theta_gen_kernel(ThetaArgs t) {
   const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t per = 2 * (int64_t)(t.J + 1);
   if (m >= (int64_t)t.nsets * per) return;
@@ -3127,7 +3128,7 @@ extern "C" kde_status kde_lscv_theta_select(kde_plan plan, int nsets, const int6
   const int64_t nmat = (int64_t)nsets * 2 * (J + 1);
   {
     LaunchScope ls("kde_theta_gen_kernel", st);
-    kde_theta_gen_kernel<<<(unsigned)((nmat + 127) / 128), 128, 0, st>>>(t);
+    kde_theta_gen_kernel<<<(unsigned)((nmat + 31) / 32), 32, 0, st>>>(t);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_theta_gen_kernel");
   }
   {
@@ -3652,7 +3653,7 @@ struct kde_batch_plan_s {
   // the kernel-grid passes need no samples: they run on this stream beside
   // the binning (fork and join events on the caller's stream)
   cudaStream_t side;
-  cudaEvent_t fork, join;
+  cudaEvent_t fork, zeroed, join;
 };
 
 namespace kde {
@@ -3860,6 +3861,7 @@ kde_status batch_eval_impl(kde_batch_plan_s* bp, const void* X, void* density, v
   if (e == cudaSuccess) e = cudaStreamWaitEvent(bp->side, bp->fork, 0);
   if (e != cudaSuccess) return cuda_fail(e, "fork (batch kernel grid)");
   e = cudaMemsetAsync(a.counts, 0, bp->counts_elems * 8, st);
+  if (e == cudaSuccess) e = cudaEventRecord(bp->zeroed, st);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(batch counts)");
   const int sms = num_sms();
   const int c = bp->count;
@@ -3870,16 +3872,6 @@ kde_status batch_eval_impl(kde_batch_plan_s* bp, const void* X, void* density, v
       kde_batch_bin_kernel<T><<<std::min(total, sms * 8), 256, 0, st>>>(a);
       if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_batch_bin_kernel");
     }
-  }
-  for (int cls = 0; cls < 2; ++cls) {
-    const int total = bp->wstart[(size_t)(BP_PBIN + cls) * (c + 1) + c];
-    if (total == 0) continue;
-    auto* fn = kde_batch_bin_private_kernel<T>;
-    if ((e = allow_smem(fn)) != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
-    const size_t smem = 2 * (size_t)((bp->priv_cells[cls] + 3) & ~3) * sizeof(unsigned);
-    LaunchScope ls("kde_batch_bin_private_kernel", st);
-    fn<<<total, kBatchPrivThreads, smem, st>>>(a, BP_PBIN + cls);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_batch_bin_private_kernel");
   }
   auto run = [&](auto fn, int pass, int tpl, const char* name, cudaStream_t ss) -> kde_status {
     const int total = bp->wstart[(size_t)pass * (c + 1) + c];
@@ -3896,6 +3888,19 @@ kde_status batch_eval_impl(kde_batch_plan_s* bp, const void* X, void* density, v
   kde_status s;
   if ((s = run(kde_batch_pass_kernel<T, BP_KROWS>, BP_KROWS, bp->tpl_rows, "kde_batch_krows_kernel", bp->side)) != KDE_OK) return s;
   if ((s = run(kde_batch_pass_kernel<T, BP_KCOLS>, BP_KCOLS, bp->tpl_cols, "kde_batch_kcols_kernel", bp->side)) != KDE_OK) return s;
+  // the private counts' problems beside the others' binning, once zeroed
+  if ((e = cudaStreamWaitEvent(bp->side, bp->zeroed, 0)) != cudaSuccess)
+    return cuda_fail(e, "cudaStreamWaitEvent(batch counts)");
+  for (int cls = 0; cls < 2; ++cls) {
+    const int total = bp->wstart[(size_t)(BP_PBIN + cls) * (c + 1) + c];
+    if (total == 0) continue;
+    auto* fn = kde_batch_bin_private_kernel<T>;
+    if ((e = allow_smem(fn)) != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
+    const size_t smem = 2 * (size_t)((bp->priv_cells[cls] + 3) & ~3) * sizeof(unsigned);
+    LaunchScope ls("kde_batch_bin_private_kernel", bp->side);
+    fn<<<total, kBatchPrivThreads, smem, bp->side>>>(a, BP_PBIN + cls);
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_batch_bin_private_kernel");
+  }
   e = cudaEventRecord(bp->join, bp->side);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(st, bp->join, 0);
   if (e != cudaSuccess) return cuda_fail(e, "join (batch kernel grid)");
@@ -4001,7 +4006,7 @@ extern "C" kde_status kde_batch_plan_create(int count, const kde_batch_item* ite
   bp->items_dev = nullptr;
   bp->wstart_dev = nullptr;
   bp->side = nullptr;
-  bp->fork = bp->join = nullptr;
+  bp->fork = bp->zeroed = bp->join = nullptr;
   kde_opts o{};
   o.tau = 3.7;
   if (opts) o = *opts;
@@ -4015,6 +4020,7 @@ extern "C" kde_status kde_batch_plan_create(int count, const kde_batch_item* ite
     if (bp->queue_dev) cudaFree(bp->queue_dev);
     if (bp->side) cudaStreamDestroy(bp->side);
     if (bp->fork) cudaEventDestroy(bp->fork);
+    if (bp->zeroed) cudaEventDestroy(bp->zeroed);
     if (bp->join) cudaEventDestroy(bp->join);
     delete bp;
     return s;
@@ -4046,6 +4052,7 @@ extern "C" kde_status kde_batch_plan_create(int count, const kde_batch_item* ite
   cudaDeviceGetStreamPriorityRange(&lo_prio, &hi_prio);
   e = cudaStreamCreateWithPriority(&bp->side, cudaStreamNonBlocking, hi_prio);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&bp->fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&bp->zeroed, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&bp->join, cudaEventDisableTiming);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "side stream (batch kernel grid)"));
   *out = bp;
@@ -4121,6 +4128,7 @@ extern "C" kde_status kde_batch_plan_destroy(kde_batch_plan bp) {
   cudaError_t e = cudaSuccess;
   if (bp->side) cudaStreamDestroy(bp->side);
   if (bp->fork) cudaEventDestroy(bp->fork);
+  if (bp->zeroed) cudaEventDestroy(bp->zeroed);
   if (bp->join) cudaEventDestroy(bp->join);
   if (bp->items_dev) e = cudaFree(bp->items_dev);
   if (bp->wstart_dev) cudaFree(bp->wstart_dev);
