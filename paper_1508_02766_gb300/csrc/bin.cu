@@ -954,7 +954,8 @@ kde_status launch_private(const T* X, int64_t n, const BinParams<T>& p, unsigned
                           unsigned long long* n_out, cudaStream_t stream) {
   auto* fn = kde_bin_private_kernel<T, D>;
   const size_t smem = 2 * (size_t)priv_words(p.cells) * sizeof(unsigned);
-  cudaError_t e = allow_smem(fn, smem);
+  // the largest grid's, so that calls from several threads set the same limit
+  cudaError_t e = allow_smem(fn, 2 * (size_t)priv_words(kPrivCells) * sizeof(unsigned));
   if (e != cudaSuccess) return kde::cuda_fail(e, "smem attr");
   const int64_t per = std::max<int64_t>(1024, p.cells / 8);
   const int64_t cap = (int64_t)num_sms() * (smem <= 100 * 1024 ? 2 : 1);
