@@ -77,12 +77,17 @@ kde_status upload_async(void* dst, const void* src, size_t bytes, cudaStream_t s
   if (!sl.ev && (e = cudaEventCreateWithFlags(&sl.ev, cudaEventDisableTiming)) != cudaSuccess)
     return cuda_fail(e, "cudaEventCreate(upload)");
   if (sl.cap < bytes) {
+    const size_t cap = std::max<size_t>(bytes, 64 << 10);
+    // a call of many bandwidths takes one slot, so a captured one can be the
+    // first to reach its slot: the allocation is allowed while capturing
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
     if (sl.host) cudaFreeHost(sl.host);
     sl.host = nullptr;
     sl.cap = 0;
-    const size_t cap = std::max<size_t>(bytes, 64 << 10);
-    if ((e = cudaHostAlloc(&sl.host, cap, cudaHostAllocPortable)) != cudaSuccess)
-      return cuda_fail(e, "cudaHostAlloc(upload)");
+    e = cudaHostAlloc(&sl.host, cap, cudaHostAllocPortable);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaHostAlloc(upload)");
     sl.cap = cap;
   }
   std::memcpy(sl.host, src, bytes);
