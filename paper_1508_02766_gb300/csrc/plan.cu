@@ -454,6 +454,14 @@ static kde_status compute_info(int d, const int64_t* M, const double* lo, const 
   for (int k = 0; tp && k < d; ++k)
     for (int j = 0; j < d; ++j)
       if (Ptp[k] > fxp::kMaxNamedP && sp[j][2] == 0) tp = false;
+  // nor a plan that only the 7-smooth length keeps within kde_fft_eval_noalloc's
+  // scratch (2-D; a 3-D plane this long is far above it)
+  if (tp && d == 2 && (Ptp[0] > fxp::kMaxNamedP || Ptp[1] > fxp::kMaxNamedP)) {
+    int64_t P = info->P[1];
+    while (!is_7smooth(P)) ++P;
+    const int64_t row = std::max(M[0], 2 * info->L[0] + 1) * 8;  // bytes per column of scratch
+    tp = row * (P / 2 + 1) > KDE_NOALLOC_SCRATCH_BYTES || row * (Ptp[1] / 2 + 1) <= KDE_NOALLOC_SCRATCH_BYTES;
+  }
   info->engine = tp ? KDE_ENGINE_TWO_PHASE : KDE_ENGINE_STOCKHAM;
   for (int k = 0; k < d; ++k) {
     int64_t P = info->P[k];

@@ -59,3 +59,14 @@ def test_requirements_above_the_limit_are_refused(d, precision):
 def test_last_axis_at_the_limit_sets_the_half_spectrum():
     info = _plan((20, 30), "f32", P_min=[0, MAX_P])
     assert info.P[1] == MAX_P and info.Q == MAX_P // 2 + 1
+
+
+@pytest.mark.parametrize("M", [(3480, 595), (2050, 1000), (500, 2050), (900, 2290)])
+def test_long_lines_keep_plans_within_the_fixed_scratch(M):
+    """A line above 2048 points leaves no plan above the fixed scratch that the
+    7-smooth lengths keep within it; where both fit, the two-phase engine stays."""
+    limit = 8 << 20
+    for m1 in range(M[1], M[1] + 40):
+        auto = _plan((M[0], m1), "f32")
+        smooth = _plan((M[0], m1), "f32", engine="stockham")
+        assert (auto.workspace_bytes <= limit) == (smooth.workspace_bytes <= limit), (M[0], m1)
