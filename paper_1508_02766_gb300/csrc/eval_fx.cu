@@ -144,8 +144,6 @@ kde_status rows_pass(const kde_plan_s* plan, int kind, int64_t nrows, const long
   const kde_plan_info& I = plan->info;
   const int dl = I.d - 1;
   RowsArgs a{};
-  a.half = half;
-  a.P0 = (int)I.P[0];
   a.nrows = nrows;
   a.Min = Min;
   a.in_stride = in_stride;
@@ -172,7 +170,8 @@ kde_status rows_pass(const kde_plan_s* plan, int kind, int64_t nrows, const long
                  threads, smem, st};
   if (kind == 2) {
     LaunchScope ls("kde_fx_rows_c2r_kernel", st);
-    return done(half ? launch_rows_c2r_even(l, a) : launch_rows_c2r(l, a), "kde_fx_rows_c2r_kernel");
+    return done(half ? launch_rows_c2r_even(l, RowsEvenArgs{a, half, (int)I.P[0]}) : launch_rows_c2r(l, a),
+                "kde_fx_rows_c2r_kernel");
   }
   if (kind == SRC_COUNTS) {
     LaunchScope ls("kde_fx_rows_r2c_counts_kernel", st);
@@ -210,7 +209,6 @@ kde_status cols_pass(const kde_plan_s* plan, int k, const char* name, const floa
   a.out = out;
   a.out_real = out_real;
   a.K = K;
-  a.C = C;
   a.S = S;
   a.Nin = Nin;
   a.Nout = Nout;
@@ -242,7 +240,7 @@ kde_status cols_pass(const kde_plan_s* plan, int k, const char* name, const floa
     case COL_FWD_REAL: e = launch_cols_real(l, a); break;
     case COL_MID: e = launch_cols_mid(l, a); break;
     case COL_AUTO: e = launch_cols_auto(l, a); break;
-    case COL_KMID: e = launch_cols_kmid(l, a); break;
+    case COL_KMID: e = launch_cols_kmid(l, KmidArgs{a, C}); break;
     default: e = launch_cols_inv(l, a); break;
   }
   return done(e, name);

@@ -121,7 +121,7 @@ kde_fx3_rows_fwd_kernel(RowsArgs a, const long long* __restrict__ counts, KGen<f
   rows_wait_early<SRC>(a);
   constexpr int N23 = N2 * N3, P = N1 * N23;
   extern __shared__ float2 fx_sm[];
-  rows_slab(a, g);
+  if constexpr (SRC == SRC_KGEN) rows_slab(a, g);   // counts come as one slab
   const int SK = a.SK, LS = N1 * SK;
   const int t = threadIdx.x;
   if constexpr (SRC == SRC_KGEN) {
@@ -190,7 +190,7 @@ kde_fx3_rows_fwd_kernel(RowsArgs a, const long long* __restrict__ counts, KGen<f
 }
 
 template <int N1, int N2, int N3, bool EVEN>
-__global__ void __launch_bounds__(kThreads3) kde_fx3_rows_c2r_kernel(RowsArgs a) {
+__global__ void __launch_bounds__(kThreads3) kde_fx3_rows_c2r_kernel(C2rArgs<EVEN> a) {
   pdl_trigger();
   pdl_wait();
   constexpr int N23 = N2 * N3, P = N1 * N23;
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kernel(ColsArgs a) {
 // phase C between the two inverses; the first column's counts are loaded at
 // the start, the second's while the first is transformed.
 template <int N1, int N2, int N3>
-__global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kmid_kernel(ColsArgs a) {
+__global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kmid_kernel(KmidArgs a) {
   pdl_trigger();
   pdl_wait();
   constexpr int N23 = N2 * N3, P = N1 * N23;

@@ -5,7 +5,7 @@
 namespace kde {
 namespace fx {
 
-cudaError_t launch_cols_kmid(const Launch& l, const ColsArgs& a) {
+cudaError_t launch_cols_kmid(const Launch& l, const KmidArgs& a) {
 #define KDE_FX_KERNEL(n1, n2) kde_fx_cols_kmid_kernel<0, n1, n2>
 #define KDE_FX_CASE_PAIR(n1, n2) \
   case n1 * 64 + n2:             \

@@ -5,7 +5,7 @@
 namespace kde {
 namespace fx {
 
-cudaError_t launch_rows_c2r_even(const Launch& l, const RowsArgs& a) {
+cudaError_t launch_rows_c2r_even(const Launch& l, const RowsEvenArgs& a) {
 #define KDE_FX_KERNEL(n1, n2) kde_fx_rows_c2r_kernel<0, n1, n2, true>
 #define KDE_FX_CASE_PAIR(n1, n2) \
   case n1 * 64 + n2:             \
