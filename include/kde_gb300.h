@@ -94,7 +94,9 @@ enum { KDE_SLAB_OFF = 0, KDE_SLAB_ON = 1 };
  *               DFT per thread (P_k <= 400); longer lines, P_k = N1 N2 N3
  *               (each about 10), take three such phases.  P_k is then the
  *               smallest supported length >= M_k + L_k (at most 2048; 3584
- *               where KDE_ENGINE_AUTO chooses it, every axis above 400).
+ *               where KDE_ENGINE_AUTO chooses it: every axis above 400, and
+ *               not if only the 7-smooth sizes keep the plan within
+ *               KDE_NOALLOC_SCRATCH_BYTES).
  *               KDE_ENGINE_STOCKHAM: mixed-radix passes through shared
  *               memory, P_k the smallest 7-smooth size >= M_k + L_k.
  *               KDE_ENGINE_AUTO: two-phase where it applies (KDE_F32, d >= 2,
@@ -200,7 +202,9 @@ kde_status kde_plan_destroy(kde_plan plan);
  *   is split axis by axis (axis 0 first): part w gives
  *   floor((w Q + 2^31) / 2^32) to node i+1 and the rest to node i.
  * n_outside: device int64, zeroed then incremented; may be NULL.  n may be 0.
- * workspace: NULL selects the direct method (64-bit atomics into counts);
+ * workspace: NULL selects the direct method (64-bit atomics into counts; on
+ * grids of up to 24576 nodes with samples enough, into block-private counts
+ * in shared memory that are then added);
  * otherwise at least kde_bin_workspace_bytes(n, d, M) bytes, 256-byte
  * aligned, select the tiled method (the samples partitioned by grid tile,
  * then each tile accumulated in shared memory and stored once).  Both give
@@ -273,9 +277,10 @@ kde_status kde_fft_eval_consume(kde_plan plan, int64_t* counts, const void* Kspe
  * binned.  density (device): nH x prod(M) values, bandwidth-major, each
  * grid exactly what kde_kernel_grid + kde_fft_eval give for that H (same
  * plan, layout and range rule).  Bandwidths go in chunks of 64 per launch:
- * kernel-grid rows, kernel spectrum, middle axis and output rows of the
- * chunk's bandwidths in four launches; their parameters are copied from
- * pageable host memory on the stream, so the call is not for graph capture.
+ * kernel-grid rows, the axis-0 pass (kernel spectrum, product with C,
+ * inverse) and output rows of the chunk's bandwidths in three launches; the
+ * parameters of 1024 bandwidths at a time are copied from host memory that
+ * the next calls reuse, so the call is not for graph capture.
  * KDE_F32 2-D plans with the two-phase engine (else KDE_ERR_UNSUPPORTED).
  * workspace: at least kde_fft_eval_multi_workspace_bytes(plan), 256-byte
  * aligned.  (Reusing F(c) is Eq. 10's structure; the batching is not in the
@@ -374,7 +379,7 @@ kde_status kde_lscv_autocorr_cands(kde_lscv_cands cands, int64_t n, const void* 
  * counts, host, each >= 2): lscv[s nH + i] (and pair_sums[2 (s nH + i)],
  * [2 (s nH + i) + 1] when not NULL; device) equal what
  * kde_lscv_autocorr_cands gives for dataset s alone.  Two launches per 1024
- * candidates whatever nsets (<= 65535).  workspace: at least
+ * candidates and 256 datasets (nsets <= 65535).  workspace: at least
  * kde_lscv_autocorr_cands_batch_workspace_bytes(cands, nsets), 256-byte
  * aligned; n is copied from pageable memory, so the call is not for
  * CUDA-graph capture. */
@@ -419,10 +424,12 @@ kde_status kde_lscv_theta_select_workspace_bytes(kde_plan plan, int nsets, int J
  *     counters).  A wait that runs out (about a second by default) records
  *     a timeout, the launch's remaining items are abandoned and
  *     kde_batch_check reports KDE_ERR_TIMEOUT.
- *   KDE_BATCH_STAGED: seven launches, a memset and one grid-stride kernel
- *     per pass covering every problem; the two kernel-grid passes run on a
- *     stream the plan owns beside the binning (fork and join through events
- *     on the caller's stream).
+ *   KDE_BATCH_STAGED: a memset and one grid-stride kernel per pass covering
+ *     every problem (binning: one for the problems with few nodes, in
+ *     block-private counts, and one for the others); the two kernel-grid
+ *     passes and then the private binning run on a stream the plan owns
+ *     beside the other binning (fork and join through events on the
+ *     caller's stream).
  * Either way small and large grids share the GPU, the result is the same,
  * graph capture works and one plan evaluates one batch at a time.  X: the problems' samples concatenated in problem order (x_rows rows
  * of 2 values, the plan's precision).  density: the problems' grids

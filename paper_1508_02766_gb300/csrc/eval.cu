@@ -3333,7 +3333,8 @@ __global__ void __launch_bounds__(256) kde_batch_bin_kernel(BatchArgs<T> a) {
 // does (the same split sums, exact for the at most 2^15 samples of a chunk).
 // One block an item; 64 datasets of 10^3 to 10^6 samples on 64^2 to 1024^2
 // grids: the binning 325 us by direct adds alone, 156 + 61 with these (event
-// times).
+// times); side by side on the plan's two streams the batch takes 661 us, one
+// after the other 699, by direct adds alone 829.
 constexpr int kBatchPrivThreads = 512;
 constexpr int kBatchPrivCells[2] = {6144, 24576};   // 48 and 192 KB of sums
 template <typename T>
