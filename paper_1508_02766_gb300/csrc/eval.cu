@@ -3132,8 +3132,10 @@ extern "C" kde_status kde_lscv_theta_select(kde_plan plan, int nsets, const int6
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_theta_gen_kernel");
   }
   {
-    // a support that fits the plan has L_1 <= P_1 - M_1
-    const size_t smem = (size_t)kAcRows * (2 * (I.P[1] - I.M[1]) + 1) * sizeof(float);
+    // a candidate's support that fits has L_1 <= P_1 - M_1, and never more than
+    // M_1 - 1 (the padding alone can be far wider than any support)
+    const int64_t L1 = std::min(I.P[1] - I.M[1], I.M[1] - 1);
+    const size_t smem = (size_t)kAcRows * (2 * L1 + 1) * sizeof(float);
     if ((e = allow_smem(kde_lscv_theta_sums_kernel)) != cudaSuccess)
       return cuda_fail(e, "cudaFuncSetAttribute");
     LaunchScope ls("kde_lscv_theta_sums_kernel", st);
