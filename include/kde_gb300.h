@@ -279,8 +279,8 @@ kde_status kde_fft_eval_consume(kde_plan plan, int64_t* counts, const void* Kspe
  * plan, layout and range rule).  Bandwidths go in chunks of 64 per launch:
  * kernel-grid rows, the axis-0 pass (kernel spectrum, product with C,
  * inverse) and output rows of the chunk's bandwidths in three launches; the
- * parameters of 1024 bandwidths at a time are copied from host memory that
- * the next calls reuse, so the call is not for graph capture.
+ * parameters go up 1024 bandwidths at a time (captured into a graph, the
+ * call's bandwidths stay in the graph).
  * KDE_F32 2-D plans with the two-phase engine (else KDE_ERR_UNSUPPORTED).
  * workspace: at least kde_fft_eval_multi_workspace_bytes(plan), 256-byte
  * aligned.  (Reusing F(c) is Eq. 10's structure; the batching is not in the
@@ -335,10 +335,9 @@ kde_status kde_lscv_workspace_bytes(kde_plan plan, size_t* bytes);
  * Both take a workspace of at least kde_lscv_autocorr_workspace_bytes,
  * 256-byte aligned.  kde_lscv_autocorr copies the candidates' kernel
  * parameters (host-prepared, FP64 factorisations) into the workspace with
- * host-to-device copies on the stream, up to 1024 candidates per launch;
- * the copies read pageable host memory that the call frees on return, so
- * these calls are not for CUDA-graph capture (kde_lscv_autocorr_cands,
- * below, launches kernels only and can be captured). */
+ * host-to-device copies on the stream, up to 1024 candidates per launch
+ * (captured into a graph, they stay in the graph; kde_lscv_autocorr_cands,
+ * below, copies nothing). */
 kde_status kde_lscv_autocorr_workspace_bytes(kde_plan plan, size_t* bytes);
 kde_status kde_autocorrelation(kde_plan plan, const int64_t* counts, void* R, void* workspace,
                                size_t workspace_bytes, kde_stream_t stream);
@@ -381,8 +380,7 @@ kde_status kde_lscv_autocorr_cands(kde_lscv_cands cands, int64_t n, const void* 
  * kde_lscv_autocorr_cands gives for dataset s alone.  Two launches per 1024
  * candidates and 256 datasets (nsets <= 65535).  workspace: at least
  * kde_lscv_autocorr_cands_batch_workspace_bytes(cands, nsets), 256-byte
- * aligned; n is copied from pageable memory, so the call is not for
- * CUDA-graph capture. */
+ * aligned.  Captured into a graph, the call's n stay in the graph. */
 kde_status kde_lscv_autocorr_cands_batch(kde_lscv_cands cands, int nsets, const int64_t* n,
                                          const void* R, double* pair_sums, double* lscv,
                                          void* workspace, size_t workspace_bytes,
@@ -405,8 +403,8 @@ kde_status kde_lscv_autocorr_cands_batch_workspace_bytes(kde_lscv_cands cands, i
  * LSCV, the reference candidate's LSCV, that candidate's theta (3 values; 0
  * if none fits)}.  KDE_F32 2-D plans.  workspace: at
  * least kde_lscv_theta_select_workspace_bytes(plan, nsets, J), 256-byte
- * aligned; the host inputs are copied from pageable memory, so the call is
- * not for CUDA-graph capture.  (Not in the paper.) */
+ * aligned.  Captured into a graph, the call's host inputs stay in the graph.
+ * (Not in the paper.) */
 kde_status kde_lscv_theta_select(kde_plan plan, int nsets, const int64_t* n, const float* theta,
                                  const double* box, int J, const double* offsets,
                                  const double* ref, const void* R, double* lscv, double* out,
@@ -605,8 +603,8 @@ kde_status kde_features2(const int64_t* counts, int M, int64_t n, const double* 
  * kde_autocorrelation).  workspace: at least
  * kde_prepare2_batch_workspace_bytes(plan, nsets, offsets[nsets]), 256-byte
  * aligned (it holds the standardised samples and the transforms'
- * intermediates).  offsets are copied from pageable memory, so the call is
- * not for CUDA-graph capture. */
+ * intermediates).  Captured into a graph, the call's offsets stay in the
+ * graph. */
 kde_status kde_prepare2_batch(kde_plan plan, int nsets, const float* X, const int64_t* offsets,
                               int64_t* counts, double* moments, float* feat, void* R,
                               void* workspace, size_t workspace_bytes, kde_stream_t stream);

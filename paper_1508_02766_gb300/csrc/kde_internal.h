@@ -41,9 +41,9 @@ kde_status fail(kde_status s, const std::string& msg);
 kde_status matrix_support(const kde_plan_s* plan, const double* A, double* Ainv, double* detA,
                           int64_t* L);
 kde_status cuda_fail(cudaError_t e, const char* what);
-// Asynchronous upload of a small host array (copied into a page-locked
-// staging slot first, so the caller's array may be reused at once).  Not for
-// stream capture: a captured copy would replay the slot's later contents.
+// Asynchronous upload of a small host array, copied before the call returns
+// (into a page-locked staging slot; into the graph on a captured stream), so
+// the caller's array may be reused at once.
 kde_status upload_async(void* dst, const void* src, size_t bytes, cudaStream_t st);
 // K_A(delta o l) = C exp(sum_k D_k (l_k + sum_{j<k} B_kj l_j)^2) from the
 // Cholesky factor of A (no cancellation when A is nearly singular);

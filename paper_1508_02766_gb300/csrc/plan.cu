@@ -41,6 +41,11 @@ kde_status cuda_fail(cudaError_t e, const char* what) {
 // which would stop the host from enqueueing the next batch while the GPU
 // works on this one.  Each thread keeps, per device, a ring of slots; a slot
 // is refilled only after the event recorded behind its last copy completed.
+//
+// On a stream that is being captured the ring is left alone: a captured copy
+// would read whatever its slot holds, or has been freed, by the time the graph
+// is replayed, and the event of a capture cannot be waited for afterwards.
+// There the bytes travel as kernel arguments, which the graph keeps by value.
 // ---------------------------------------------------------------------------
 namespace {
 struct UploadSlot {
@@ -56,13 +61,37 @@ struct UploadRing {
   int next = 0;
 };
 thread_local UploadRing g_upload[kUploadDevices];
+
+struct UploadChunk {
+  unsigned char b[32000];   // kernel arguments take up to 32764 bytes
+};
+__global__ void __launch_bounds__(256)
+kde_upload_kernel(unsigned char* dst, int n, const __grid_constant__ UploadChunk c) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = c.b[i];
+}
+
+kde_status upload_captured(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+  UploadChunk c;
+  for (size_t at = 0; at < bytes; at += sizeof(c.b)) {
+    const size_t n = std::min(sizeof(c.b), bytes - at);
+    std::memcpy(c.b, (const char*)src + at, n);
+    LaunchScope ls("kde_upload_kernel", st);
+    kde_upload_kernel<<<1, 256, 0, st>>>((unsigned char*)dst + at, (int)n, c);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(e, "kde_upload_kernel");
+  }
+  return KDE_OK;
+}
 }  // namespace
 
 kde_status upload_async(void* dst, const void* src, size_t bytes, cudaStream_t st) {
   if (bytes == 0) return KDE_OK;
+  cudaStreamCaptureStatus cap_st = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(st, &cap_st);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaStreamIsCapturing(upload)");
+  if (cap_st != cudaStreamCaptureStatusNone) return upload_captured(dst, src, bytes, st);
   int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
   if (dev < 0 || dev >= kUploadDevices) {   // no ring: a plain (possibly waiting) copy
     e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
     return e == cudaSuccess ? KDE_OK : cuda_fail(e, "cudaMemcpyAsync(upload)");
@@ -77,17 +106,12 @@ kde_status upload_async(void* dst, const void* src, size_t bytes, cudaStream_t s
   if (!sl.ev && (e = cudaEventCreateWithFlags(&sl.ev, cudaEventDisableTiming)) != cudaSuccess)
     return cuda_fail(e, "cudaEventCreate(upload)");
   if (sl.cap < bytes) {
-    const size_t cap = std::max<size_t>(bytes, 64 << 10);
-    // a call of many bandwidths takes one slot, so a captured one can be the
-    // first to reach its slot: the allocation is allowed while capturing
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
     if (sl.host) cudaFreeHost(sl.host);
     sl.host = nullptr;
     sl.cap = 0;
-    e = cudaHostAlloc(&sl.host, cap, cudaHostAllocPortable);
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaHostAlloc(upload)");
+    const size_t cap = std::max<size_t>(bytes, 64 << 10);
+    if ((e = cudaHostAlloc(&sl.host, cap, cudaHostAllocPortable)) != cudaSuccess)
+      return cuda_fail(e, "cudaHostAlloc(upload)");
     sl.cap = cap;
   }
   std::memcpy(sl.host, src, bytes);
