@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "kde_internal.h"
+#include "smem_limit.cuh"
 #include "tc_wait.cuh"
 
 namespace kde {
@@ -251,13 +252,8 @@ __global__ void __launch_bounds__(128) kde_rows_r2c_tc_kernel(TcArgs a) {
 template <int BN>
 cudaError_t launch_tc(const TcArgs& a, int N, cudaStream_t st) {
   const int smem = 2 * (2 * 16384 + 2 * BN * 128);
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(kde_rows_r2c_tc_kernel<BN>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  const cudaError_t e = allow_smem(kde_rows_r2c_tc_kernel<BN>);
+  if (e != cudaSuccess) return e;
   LaunchScope ls("kde_rows_r2c_tc_kernel", st);
   kde_rows_r2c_tc_kernel<BN><<<dim3((unsigned)((a.rows + 127) / 128), N / BN), 128, smem, st>>>(a);
   return cudaGetLastError();

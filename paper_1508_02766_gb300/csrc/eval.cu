@@ -24,7 +24,6 @@
 #include <cstdint>
 #include <cstring>
 #include <mutex>
-#include <set>
 #include <string>
 #include <type_traits>
 #include <vector>
@@ -36,6 +35,7 @@
 #include "kde_debug.cuh"
 #include "kgen.cuh"
 #include "pdl.cuh"
+#include "smem_limit.cuh"
 
 namespace kde {
 namespace {
@@ -1470,24 +1470,6 @@ __global__ void __launch_bounds__(kColsMaxThreads) kde_cols_inv_kernel(ColsParam
 // ---------------------------------------------------------------------------
 // Host side.
 // ---------------------------------------------------------------------------
-constexpr size_t kSmemMax = 227 * 1024;
-
-template <typename F>
-cudaError_t allow_smem(F* fn) {
-  static std::mutex mu;
-  static std::set<const void*> done;
-  std::lock_guard<std::mutex> lk(mu);
-  if (done.count((const void*)fn)) return cudaSuccess;
-  // the opt-in limit covers static and dynamic shared memory together
-  cudaFuncAttributes attr{};
-  cudaError_t e = cudaFuncGetAttributes(&attr, fn);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(kSmemMax - attr.sharedSizeBytes));
-  if (e == cudaSuccess) done.insert((const void*)fn);
-  return e;
-}
-
 LinePlan line_plan(const kde_plan_info& info, int k) {
   LinePlan lp{};
   lp.N = (int)info.P[k];

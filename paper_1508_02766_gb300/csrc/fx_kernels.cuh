@@ -29,8 +29,6 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
-#include <mutex>
-#include <set>
 #include <type_traits>
 
 #include "fx_dft.cuh"
@@ -39,6 +37,7 @@
 #include "kde_internal.h"
 #include "kgen.cuh"
 #include "pdl.cuh"
+#include "smem_limit.cuh"
 
 namespace kde {
 namespace fx {
@@ -792,23 +791,6 @@ kde_fx_cols_kmid_kernel(KmidArgs a) {
 // Launchers, one translation unit each (fx_launch_*.cu, compiled in
 // parallel): kernel of size class cls (0: factors <= 20) on the stream.
 // ---------------------------------------------------------------------------
-constexpr size_t kSmemMax = 227 * 1024;
-
-template <typename F>
-cudaError_t allow_smem(F* fn) {
-  static std::mutex mu;
-  static std::set<const void*> done;
-  std::lock_guard<std::mutex> lk(mu);
-  if (done.count((const void*)fn)) return cudaSuccess;
-  cudaFuncAttributes attr{};
-  cudaError_t e = cudaFuncGetAttributes(&attr, fn);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)(kSmemMax - attr.sharedSizeBytes));
-  if (e == cudaSuccess) done.insert((const void*)fn);
-  return e;
-}
-
 // Every pass kernel starts with pdl_trigger(); pdl_wait(); so it may be
 // launched as a programmatic dependent of the kernel before it.
 template <typename Kern, typename... Args>

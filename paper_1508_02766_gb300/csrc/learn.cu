@@ -21,6 +21,7 @@
 
 #include "kde_internal.h"
 #include "pdl.cuh"
+#include "smem_limit.cuh"
 #include "tc_wait.cuh"
 
 namespace kde {
@@ -277,15 +278,10 @@ cudaError_t launch_gemm_st(const GemmPair& p, dim3 grid, cudaStream_t st) {
   // for as much as the wide ones, so that at most four CTAs share an SM and
   // their tensor memory (64 columns each) stays within its 512 columns.
   const int smem = kStages * (16384 + 64 * 128);
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(kde_gemm_tc_kernel<BN, kStages>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  cudaError_t e = allow_smem(kde_gemm_tc_kernel<BN, kStages>);
+  if (e != cudaSuccess) return e;
   LaunchScope ls("kde_gemm_tc_kernel", st);
-  const cudaError_t e = launch_pdl(kde_gemm_tc_kernel<BN, kStages>, grid, dim3(128), (size_t)smem, st, p);
+  e = launch_pdl(kde_gemm_tc_kernel<BN, kStages>, grid, dim3(128), (size_t)smem, st, p);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
