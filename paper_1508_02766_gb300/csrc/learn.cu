@@ -337,14 +337,16 @@ kde_status launch_gemm2(GemmArgs a, int epi_a, GemmArgs b, int epi_b, cudaStream
 // ---------------------------------------------------------------------------
 // X (B x in, FP32) -> Xb (Bp x in, BF16) and its transpose Xt (in x Bp);
 // rows B .. Bp-1 are zero.  Tiles of 32 x 64 go through shared memory, so that
-// both copies are written in rows.  Grid (in / 64, Bp / 32).
+// both copies are written in rows.  One block a tile, (in / 64) (Bp / 32) along
+// x: a batch may have more rows than the other grid dimensions take tiles.
 __global__ void __launch_bounds__(256) kde_mlp_cast_kernel(const float* __restrict__ X, int B,
                                                            int Bp, int in, bf16* __restrict__ Xb,
                                                            bf16* __restrict__ Xt) {
   __shared__ bf16 tile[32][66];
   pdl_trigger();
   pdl_wait();   // X, and the last reader of Xb and Xt
-  const int k0 = blockIdx.x * 64, b0 = blockIdx.y * 32, t = threadIdx.x;
+  const int cols = in / 64, k0 = (int)(blockIdx.x % cols) * 64, b0 = (int)(blockIdx.x / cols) * 32,
+            t = threadIdx.x;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const int b = (t >> 6) + 4 * i, k = t & 63;
@@ -747,9 +749,9 @@ GemmArgs gemm_args(const bf16* A, int lda, const bf16* B, int ldb, int M, int N,
 kde_status mlp_forward(kde_mlp_s* m, const float* X, int B, int Bp, bool keep_t, cudaStream_t st) {
   {
     LaunchScope ls("kde_mlp_cast_kernel", st);
-    const cudaError_t e = launch_pdl(kde_mlp_cast_kernel, dim3((unsigned)(m->in / 64), (unsigned)(Bp / 32)),
-                                     dim3(256), 0, st, X, B, Bp, m->in, m->Xb,
-                                     keep_t ? m->Xt : (bf16*)nullptr);
+    const dim3 grid((unsigned)(m->in / 64) * (unsigned)(Bp / 32));
+    const cudaError_t e = launch_pdl(kde_mlp_cast_kernel, grid, dim3(256), 0, st, X, B, Bp, m->in,
+                                     m->Xb, keep_t ? m->Xt : (bf16*)nullptr);
     if (e != cudaSuccess) return cuda_fail(e, "kde_mlp_cast_kernel");
   }
   GemmArgs g1 = gemm_args(m->Xb, m->in, m->W1b, m->in, Bp, m->hid, m->in, m->Z1, m->hid, m->status);
