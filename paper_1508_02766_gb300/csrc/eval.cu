@@ -983,38 +983,33 @@ __device__ __forceinline__ float2 ac_term2(float2 l, float2 D1, float2 t_hi, flo
 
 // The sum over the work unit of matrix g that starts at lag row row0, by one
 // warp (lane = class); valid in lane 0.  at(r, l1): R at lag (row0 + r, l1).
-template <typename T, typename F>
-__device__ __forceinline__ double ac_unit_sum(const AcGen<T>& g, int row0, int lane, F&& at) {
+template <typename F>
+__device__ __forceinline__ double ac_unit_sum(const AcGen<float>& g, int row0, int lane, F&& at) {
   const int r1 = min(g.L0, row0 + kAcRows - 1), first = lane - g.L1;
-  T acc = 0;
+  float acc = 0.f;
   int l0 = row0;
   if (l0 == 0) {
-    const AcRow<T> r = ac_row(g, 0);
+    const AcRow<float> r = ac_row(g, 0);
     for (int l1 = first; l1 <= g.L1; l1 += 32)
-      if (l1 >= 0) acc = fma(ac_term0(g, r, (T)l1), at(0, l1), acc);
+      if (l1 >= 0) acc = fma(ac_term0(g, r, (float)l1), at(0, l1), acc);
     ++l0;
   }
   for (; l0 <= r1; ++l0) {
-    const AcRow<T> r = ac_row(g, l0);
-    T f = (T)first;
-    if constexpr (sizeof(T) == 4) {
-      const float2 D1 = make_float2(g.D1, g.D1), th = make_float2(r.t_hi, r.t_hi),
-                   tl = make_float2(r.t_lo, r.t_lo), e0 = make_float2(r.e0, r.e0);
-      for (int l1 = first; l1 <= g.L1; l1 += 64, f += 64.f) {
-        float2 l = make_float2(f, f + 32.f);
-        if (g.wand) l = make_float2(fabsf(l.x), fabsf(l.y));
-        const float2 k = ac_term2(l, D1, th, tl, e0);
-        acc = fmaf(k.x, at(l0 - row0, l1), acc);
-        if (l1 + 32 <= g.L1) acc = fmaf(k.y, at(l0 - row0, l1 + 32), acc);
-      }
-    } else {
-      for (int l1 = first; l1 <= g.L1; l1 += 32, f += T(32))
-        acc = fma(ac_term(g, r, f), at(l0 - row0, l1), acc);
+    const AcRow<float> r = ac_row(g, l0);
+    float f = (float)first;
+    const float2 D1 = make_float2(g.D1, g.D1), th = make_float2(r.t_hi, r.t_hi),
+                 tl = make_float2(r.t_lo, r.t_lo), e0 = make_float2(r.e0, r.e0);
+    for (int l1 = first; l1 <= g.L1; l1 += 64, f += 64.f) {
+      float2 l = make_float2(f, f + 32.f);
+      if (g.wand) l = make_float2(fabsf(l.x), fabsf(l.y));
+      const float2 k = ac_term2(l, D1, th, tl, e0);
+      acc = fmaf(k.x, at(l0 - row0, l1), acc);
+      if (l1 + 32 <= g.L1) acc = fmaf(k.y, at(l0 - row0, l1 + 32), acc);
     }
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-  return (double)(T(2) * g.C * acc);
+  return (double)(2.f * g.C * acc);
 }
 
 // Lag rows row0 .. row0 + nrow - 1 of R, lags -L1 .. L1, into tile (rows of
@@ -1030,6 +1025,35 @@ __device__ __forceinline__ void ac_stage(float* tile, const float* __restrict__ 
   }
 }
 
+// FP64: a block a work unit, a warp a lag row.  The terms are bound by the
+// FP64 pipe (about twenty instructions of it each), so what counts is that
+// every SM has rows: with a warp a whole unit and its sixteen to a block, as
+// the FP32 kernel has them, 16 candidates of 460-lag supports took 723 us
+// against 398.
+__global__ void __launch_bounds__(256) kde_lscv_ac64_kernel(const AcGen<double>* __restrict__ gens,
+                                                            const int2* __restrict__ units,
+                                                            const double* __restrict__ Rall, int P1,
+                                                            int64_t set_stride,
+                                                            double* __restrict__ partial) {
+  const int2 u = units[blockIdx.x];
+  const AcGen<double> g = gens[u.x];
+  const int lane = threadIdx.x & 31, l0 = u.y + (threadIdx.x >> 5);
+  double acc = 0.0;
+  if (l0 <= g.L0) {
+    const double* R = Rall + (int64_t)(g.set + blockIdx.y) * set_stride + (int64_t)l0 * P1;
+    const AcRow<double> r = ac_row(g, l0);
+#pragma unroll 4
+    for (int l1 = (l0 == 0 ? 0 : -g.L1) + lane; l1 <= g.L1; l1 += 32) {
+      const double v = ((double)(g.wand ? abs(l1) : l1) + r.t_hi) + r.t_lo;
+      acc = fma(exp2(fma(g.D1 * v, v, r.e0)), __ldg(R + (l1 < 0 ? l1 + P1 : l1)), acc);
+    }
+    // every lag of the half plane counts twice, the lag 0 (K = C) once
+    if (l0 == 0 && lane == 0) acc -= 0.5 * __ldg(R);
+  }
+  block_sum_to(2.0 * g.C * acc,
+               partial + (int64_t)(g.u0 + u.y / kAcRows) * gridDim.y + blockIdx.y);
+}
+
 // A block takes up to kAcBlock work units (matrix, first row) of one dataset
 // and first row, blocks[..] = (first unit, count), two to a warp:
 // partial[u nsets + y] with u the unit's place among its matrix's units, for
@@ -1037,37 +1061,27 @@ __device__ __forceinline__ void ac_stage(float* tile, const float* __restrict__ 
 // (the first unit's L_1 is the largest); read from the L2 as they are used,
 // one load's latency for 32 terms was most of the kernel.
 constexpr int kAcBlock = 16;
-template <typename T>
-__global__ void __launch_bounds__(256) kde_lscv_ac_kernel(const AcGen<T>* __restrict__ gens,
+__global__ void __launch_bounds__(256) kde_lscv_ac_kernel(const AcGen<float>* __restrict__ gens,
                                                           const int2* __restrict__ units,
                                                           const int2* __restrict__ blocks,
-                                                          const T* __restrict__ Rall, int P1,
+                                                          const float* __restrict__ Rall, int P1,
                                                           int64_t set_stride,
                                                           double* __restrict__ partial) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* tile = reinterpret_cast<T*>(smem_raw);
+  extern __shared__ __align__(16) float tile[];
   const int2 blk = blocks[blockIdx.x];
   units += blk.x;
   const int2 lead = units[0];
-  const AcGen<T>& gl = gens[lead.x];
-  const T* __restrict__ R = Rall + (int64_t)(gl.set + blockIdx.y) * set_stride;
+  const AcGen<float>& gl = gens[lead.x];
+  const float* __restrict__ R = Rall + (int64_t)(gl.set + blockIdx.y) * set_stride;
   const int lane = threadIdx.x & 31, L1 = gl.L1, W = 2 * L1 + 1, row0 = lead.y;
-  if constexpr (sizeof(T) == 4) {
-    // rows below the support of the block's longest matrix (never past R)
-    int L0 = 0;
-    for (int i = 0; i < blk.y; ++i) L0 = max(L0, gens[units[i].x].L0);
-    ac_stage(tile, R, P1, row0, min(kAcRows, L0 + 1 - row0), L1);
-    __syncthreads();
-  }
+  // rows below the support of the block's longest matrix (never past R)
+  int L0 = 0;
+  for (int i = 0; i < blk.y; ++i) L0 = max(L0, gens[units[i].x].L0);
+  ac_stage(tile, R, P1, row0, min(kAcRows, L0 + 1 - row0), L1);
+  __syncthreads();
   for (int i = threadIdx.x >> 5; i < blk.y; i += 8) {
-    const AcGen<T> g = gens[units[i].x];
-    double v;
-    if constexpr (sizeof(T) == 4)
-      v = ac_unit_sum(g, row0, lane, [&](int r, int l1) { return tile[r * W + L1 + l1]; });
-    else
-      v = ac_unit_sum(g, row0, lane, [&](int r, int l1) {
-        return __ldg(R + (size_t)(row0 + r) * P1 + (l1 < 0 ? l1 + P1 : l1));
-      });
+    const AcGen<float> g = gens[units[i].x];
+    const double v = ac_unit_sum(g, row0, lane, [&](int r, int l1) { return tile[r * W + L1 + l1]; });
     if (lane == 0) partial[(int64_t)(g.u0 + row0 / kAcRows) * gridDim.y + blockIdx.y] = v;
   }
 }
@@ -2268,7 +2282,11 @@ kde_status ac_build_chunk(kde_plan_s* plan, int64_t c0, int nh, int nH, const do
   // matrices by dataset and falling L_1, then each dataset's rows in turn
   const std::vector<int> order = ac_order(gens);
   units.reserve(nunits);
-  for (size_t i = 0, j = 0; i < order.size(); i = j) {
+  if (sizeof(T) == 8) {   // a block a unit: the longest rows first
+    for (int m : order)
+      for (int r = 0; r <= gens[m].L0; r += kAcRows) units.push_back(make_int2(m, r));
+  }
+  for (size_t i = 0, j = 0; sizeof(T) == 4 && i < order.size(); i = j) {
     int L0 = 0;
     for (j = i; j < order.size() && gens[order[j]].set == gens[order[i]].set; ++j)
       L0 = std::max(L0, gens[order[j]].L0);
@@ -2335,16 +2353,20 @@ kde_status ac_launch_chunk(const kde_plan_info& I, const void* img, int nh, cons
                            int64_t nH_all, double* S_out, double* lscv_out, cudaStream_t st) {
   const AcImage<T> im(img, nh, sh.nunits);
   cudaError_t e;
-  {
-    // FP32: kAcRows staged rows of at most 2 (KDE_MAX_P / 2) - 1 lags
-    const size_t smem = sizeof(T) == 4 ? (size_t)kAcRows * (2 * sh.L1 + 1) * sizeof(T) : 0;
-    if ((e = allow_smem(kde_lscv_ac_kernel<T>)) != cudaSuccess)
-      return cuda_fail(e, "cudaFuncSetAttribute");
+  const int64_t per = I.P[0] * I.P[1];
+  if constexpr (std::is_same<T, double>::value) {
+    LaunchScope ls("kde_lscv_ac64_kernel", st);
+    kde_lscv_ac64_kernel<<<dim3((unsigned)sh.nunits, (unsigned)ns), 256, 0, st>>>(
+        im.gens, im.units, R, (int)I.P[1], per, partial);
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_ac64_kernel");
+  } else {
+    // kAcRows staged rows of at most 2 (KDE_MAX_P / 2) - 1 lags
+    const size_t smem = (size_t)kAcRows * (2 * sh.L1 + 1) * sizeof(float);
+    if ((e = allow_smem(kde_lscv_ac_kernel)) != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
     LaunchScope ls("kde_lscv_ac_kernel", st);
-    kde_lscv_ac_kernel<T><<<dim3((unsigned)sh.nblocks, (unsigned)ns), 256, smem, st>>>(
-        im.gens, im.units, im.blocks, R, (int)I.P[1], (int64_t)I.P[0] * I.P[1], partial);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "kde_lscv_ac_kernel");
+    kde_lscv_ac_kernel<<<dim3((unsigned)sh.nblocks, (unsigned)ns), 256, smem, st>>>(
+        im.gens, im.units, im.blocks, R, (int)I.P[1], per, partial);
+    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_ac_kernel");
   }
   return ac_reduce<T>(im, nh, ns, partial, nk_set, nk_all, nH_all, S_out, lscv_out, st);
 }
