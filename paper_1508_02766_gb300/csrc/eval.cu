@@ -927,16 +927,73 @@ struct AcGen {
 // parameters and work units are uploaded to the workspace.  A work unit is
 // kAcRows lag rows of one matrix (the last of a matrix fewer).
 //
-// The order of the additions is the same in every form below, so that a
-// candidate's score does not depend on how many datasets are scored with it:
-// lag l_1 belongs to class (l_1 + L_1) mod 32; a unit's class sums run over
-// its rows and, within a row, over l_1 ascending (FP32); the 32 class sums are added
-// as a warp's shuffle tree adds its lanes (FP32); a matrix's units are added
-// in order in FP64.  The FP64 part is one addition per unit: FP64 runs at 2
-// lanes a clock and SM, and a tree over 256 FP64 values for every 4096 terms
-// took longer than the terms.
+// FP32 sums.  The terms are FP32; how they are added is fixed here, for every
+// kernel below, so that a candidate's score does not depend on how many
+// datasets are scored with it or on how the work is spread:
+//   chain   the lags l_1 = c (mod 8) of one row inside one window [S w, S (w +
+//           1)), ascending, in FP32: S = ac_window(first row, L_1) / 8 terms;
+//   group   the 4 x 8 chains of four rows (first row a multiple of four), in
+//           order of 8 (row mod 4) + c, as a pair of FP32 (AcPair: the sum and
+//           the sum of its rounding errors);
+//   unit    the groups of its two sets of four rows, windows ascending;
+//   matrix  its units, in order.
+// From the chains on nothing is lost to FP32: LSCV subtracts two such sums,
+// and rows of small far terms vanish in one long chain.  FP64 additions would
+// do, but run at 2 lanes a clock and SM; a pair costs four to eight FP32 ones.  Error
+// of the additions alone, rms over random bandwidths (x 1e-9), with chains
+// through eight rows and a FP32 tree / with a warp's row sums added in FP32 and
+// the lanes in FP64 (what the widths below are held against) / now: supports
+// of 39 x 39 lags 27 / 4.9 / 2.3, 120 x 120 21 / 2.8 / 2.8, 7 x 2000 1100 / 41
+// / 3, 27 x 70 - / 4.5 / 2.1, 7 x 32 - / 4.6 / 4.7, 10 x 10 52 / 8.2 / 5.4.
 constexpr int kAcChunk = 1024;
 constexpr int kAcRows = 8;
+constexpr int kAcGroup = 4;       // rows of a group
+constexpr int kAcWindow = 128;    // widest window
+// Width of the windows: short chains in the first unit, which holds the
+// largest terms and with a support of few rows is all there is (every unit at
+// 64 lags: 1.5 times the error at 5 x 48 lags); about sixteen a side at least.
+__host__ __device__ constexpr int ac_window(int row0, int L1) {
+  int S = row0 ? kAcWindow : 16;
+  while (S < kAcWindow && 16 * S < L1) S *= 2;
+  return S;
+}
+// Windows that hold lags -L1 .. L1: ac_first .. L1 / S.
+__host__ __device__ constexpr int ac_first(int L1, int S) { return -((L1 + S - 1) / S); }
+__host__ __device__ constexpr int ac_windows(int L1, int S) { return L1 / S - ac_first(L1, S) + 1; }
+constexpr int kAcMaxWindows = 33;
+
+// A sum as value + error, |error| about half an ulp of the value.
+struct AcPair {
+  float s, e;
+};
+// The exact error of s = a + b rounded (Knuth's two-sum).
+__device__ __forceinline__ float sum_error(float a, float b, float s) {
+  const float bb = __fsub_rn(s, a);
+  return __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+__device__ __forceinline__ AcPair ac_add(AcPair a, AcPair b) {
+  AcPair r;
+  r.s = __fadd_rn(a.s, b.s);
+  r.e = __fadd_rn(__fadd_rn(a.e, b.e), sum_error(a.s, b.s, r.s));
+  return r;
+}
+// The same two at a time (component by component).
+struct AcPair2 {
+  float2 s, e;
+};
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
+}
+__device__ __forceinline__ float2 sum_error2(float2 a, float2 b, float2 s) {
+  const float2 bb = sub2(s, a);
+  return __fadd2_rn(sub2(a, sub2(s, bb)), sub2(b, bb));
+}
+__device__ __forceinline__ AcPair2 ac_add2(AcPair2 a, AcPair2 b) {
+  AcPair2 r;
+  r.s = __fadd2_rn(a.s, b.s);
+  r.e = __fadd2_rn(__fadd2_rn(a.e, b.e), sum_error2(a.s, b.s, r.s));
+  return r;
+}
 
 // K_A at lag (l0, l1) over 2 C: every lag of the half plane counts twice,
 // the lag 0 once; zero outside the support and on the other half of row 0.
@@ -960,69 +1017,159 @@ __device__ __forceinline__ float ac_ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ double ac_ex2(double x) { return exp2(x); }
-// l1: the lag as T (an integer conversion would take the exponential's unit).
-template <typename T>
-__device__ __forceinline__ T ac_term(const AcGen<T>& g, const AcRow<T>& r, T l1) {
-  const T v = ((g.wand ? fabs(l1) : l1) + r.t_hi) + r.t_lo;
-  return ac_ex2(fma(g.D1 * v, v, r.e0));
-}
-// Row 0: the lag 0 counts half, the lags below it not at all.
-template <typename T>
-__device__ __forceinline__ T ac_term0(const AcGen<T>& g, const AcRow<T>& r, T l1) {
-  const T k = ac_term(g, r, l1);
-  return l1 > T(0) ? k : l1 == T(0) ? T(0.5) * k : T(0);
-}
-// Two terms in packed arithmetic, each component rounded as ac_term's:
-// lags l.x, l.y with the parameters D1, t_hi, t_lo, e0 of each.
+// Two terms in packed arithmetic: lags l.x, l.y (as floats: an integer
+// conversion would take the exponential's unit) with the parameters D1, t_hi,
+// t_lo, e0 of each.
 __device__ __forceinline__ float2 ac_term2(float2 l, float2 D1, float2 t_hi, float2 t_lo, float2 e0) {
   const float2 v = __fadd2_rn(__fadd2_rn(l, t_hi), t_lo);
   const float2 e = __ffma2_rn(__fmul2_rn(D1, v), v, e0);
   return make_float2(ac_ex2(e.x), ac_ex2(e.y));
 }
 
-// The sum over the work unit of matrix g that starts at lag row row0, by one
-// warp (lane = class); valid in lane 0.  at(r, l1): R at lag (row0 + r, l1).
-template <typename F>
-__device__ __forceinline__ double ac_unit_sum(const AcGen<float>& g, int row0, int lane, F&& at) {
-  const int r1 = min(g.L0, row0 + kAcRows - 1), first = lane - g.L1;
+// A lane's row of a group: its parameters and its lags [lo, lo + span].
+struct AcLane {
+  float2 D1, th, tl, e0;
+  const float* x;   // lag 0 of the row in shared memory
+  int lo;
+  unsigned span;
+};
+__device__ __forceinline__ AcLane ac_lane(const AcGen<float>& g, int l0, const float* x) {
+  AcLane a;
+  const AcRow<float> r = ac_row(g, l0);
+  a.D1 = make_float2(g.D1, g.D1);
+  a.th = make_float2(r.t_hi, r.t_hi);
+  a.tl = make_float2(r.t_lo, r.t_lo);
+  a.e0 = make_float2(r.e0, r.e0);
+  a.x = x;
+  // none in a row beyond the support, half of them in row 0
+  a.lo = l0 > g.L0 ? KDE_MAX_P : l0 == 0 ? 0 : -g.L1;
+  a.span = l0 > g.L0 ? 0u : (unsigned)(g.L1 - a.lo);
+  return a;
+}
+// This lane's chain of the window of S lags from w0 on, for the group of rows
+// r0 .. r0 + 3 of matrix g.
+__device__ __forceinline__ float ac_chain(const AcGen<float>& g, const AcLane& a, int r0, int w0,
+                                          int S, int c) {
+  const unsigned sign = g.wand ? 0x7FFFFFFFu : 0xFFFFFFFFu;
   float acc = 0.f;
-  int l0 = row0;
-  if (l0 == 0) {
-    const AcRow<float> r = ac_row(g, 0);
-    for (int l1 = first; l1 <= g.L1; l1 += 32)
-      if (l1 >= 0) acc = fma(ac_term0(g, r, (float)l1), at(0, l1), acc);
-    ++l0;
-  }
-  for (; l0 <= r1; ++l0) {
-    const AcRow<float> r = ac_row(g, l0);
-    float f = (float)first;
-    const float2 D1 = make_float2(g.D1, g.D1), th = make_float2(r.t_hi, r.t_hi),
-                 tl = make_float2(r.t_lo, r.t_lo), e0 = make_float2(r.e0, r.e0);
-    for (int l1 = first; l1 <= g.L1; l1 += 64, f += 64.f) {
-      float2 l = make_float2(f, f + 32.f);
-      if (g.wand) l = make_float2(fabsf(l.x), fabsf(l.y));
-      const float2 k = ac_term2(l, D1, th, tl, e0);
-      acc = fmaf(k.x, at(l0 - row0, l1), acc);
-      if (l1 + 32 <= g.L1) acc = fmaf(k.y, at(l0 - row0, l1 + 32), acc);
+  auto terms = [&](float2 f) {
+    const float2 l = make_float2(__uint_as_float(__float_as_uint(f.x) & sign),
+                                 __uint_as_float(__float_as_uint(f.y) & sign));
+    return ac_term2(l, a.D1, a.th, a.tl, a.e0);
+  };
+  const float2 step = make_float2(16.f, 16.f);
+  if (w0 >= -g.L1 && w0 + S <= g.L1 && r0 > 0 && r0 + kAcGroup - 1 <= g.L0) {   // all of it
+    const float* x = a.x + w0 + c;
+    float2 f = make_float2((float)(w0 + c), (float)(w0 + c + 8));
+#pragma unroll 4
+    for (int i = 0; i < S / 16; ++i, x += 16) {
+      const float2 k = terms(f);
+      acc = fmaf(k.x, x[0], acc);
+      acc = fmaf(k.y, x[8], acc);
+      f = __fadd2_rn(f, step);
     }
+    return acc;
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-  return (double)(2.f * g.C * acc);
+  const int i0 = max(0, (-g.L1 - w0) >> 3), i1 = min(S - 1, g.L1 - w0) >> 3;
+  int l = w0 + 8 * i0 + c;
+  float2 f = make_float2((float)l, (float)(l + 8));
+  for (int i = i0; i <= i1; i += 2, l += 16) {
+    float2 k = terms(f);
+    if (r0 == 0 && (threadIdx.x & 24) == 0) {   // row 0: its lag 0 counts once, the others twice
+      if (l == 0) k.x *= 0.5f;
+      if (l + 8 == 0) k.y *= 0.5f;
+    }
+    if ((unsigned)(l - a.lo) <= a.span) acc = fmaf(k.x, a.x[l], acc);
+    if (i < i1 && (unsigned)(l + 8 - a.lo) <= a.span) acc = fmaf(k.y, a.x[l + 8], acc);
+    f = __fadd2_rn(f, step);
+  }
+  return acc;
 }
 
-// Lag rows row0 .. row0 + nrow - 1 of R, lags -L1 .. L1, into tile (rows of
-// 2 L1 + 1) by the whole block.
+// A group's sum from its chains v[0] .. v[31].  The error is taken as for |sum|
+// >= |chain|; where the first few chains grow it falls short by what one FP32
+// addition of them rounds (no larger errors in the sums measured above).
+__device__ __forceinline__ AcPair ac_group_sum(const float* v) {
+  AcPair p{v[0], 0.f};
+#pragma unroll
+  for (int r = 1; r < 32; ++r) {
+    const float b = v[r], s = __fadd_rn(p.s, b);
+    p.e = __fadd_rn(p.e, __fadd_rn(__fsub_rn(p.s, s), b));
+    p.s = s;
+  }
+  return p;
+}
+
+// A block's groups: those of unit row0 of nm <= 32 matrices (gs) dealt out to
+// its warps in runs, their sums into sums in order (matrix, set of four rows,
+// window), matrix m's at off[m].  A warp leaves the chains of up to 32 groups
+// in its turn of shared memory and a lane then adds each group's: shuffles for
+// each took a third of the kernel.  tile: lag (row0, 0).
+constexpr int kAcTurn1 = 33;   // pitch of the chains
+// off, by one warp; complete after the block's next barrier.
+__device__ __forceinline__ void ac_offsets(const AcGen<float>* gs, int nm, int row0, int* off) {
+  const int lane = threadIdx.x & 31;
+  int v = 0;
+  if (lane < nm && row0 <= gs[lane].L0)
+    v = (kAcRows / kAcGroup) * ac_windows(gs[lane].L1, ac_window(row0, gs[lane].L1));
+#pragma unroll
+  for (int d = 1; d < 32; d *= 2) {
+    const int u = __shfl_up_sync(0xffffffffu, v, d);
+    if (lane >= d) v += u;
+  }
+  if (lane < nm) off[lane + 1] = v;
+  if (lane == 0) off[0] = 0;
+}
+__device__ __forceinline__ void ac_groups(const AcGen<float>* gs, const int* off, int nm, int row0,
+                                          const float* tile, int pitch, float* turn, AcPair* sums) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const int end = off[nm] * (warp + 1) / warps, rs = lane >> 3, c = lane & 7;
+  int t = off[nm] * warp / warps, m = 0, w = 0, S = 0, last = -1, r0 = 0;
+  turn += warp * 32 * kAcTurn1;
+  AcLane a{};
+  while (t < end) {
+    const int n = min(32, end - t);
+    for (int k = 0; k < n; ++k, ++w) {
+      if (w > last) {   // the next set of four rows, or where the run begins
+        while (off[m + 1] <= t + k) ++m;
+        S = ac_window(row0, gs[m].L1);
+        const int nw = ac_windows(gs[m].L1, S), j = t + k - off[m];
+        const int h = j >= nw;
+        w = ac_first(gs[m].L1, S) + j - h * nw;
+        last = gs[m].L1 / S;
+        r0 = row0 + kAcGroup * h;
+        a = ac_lane(gs[m], r0 + rs, tile + (kAcGroup * h + rs) * pitch);
+      }
+      turn[k * kAcTurn1 + lane] = r0 <= gs[m].L0 ? ac_chain(gs[m], a, r0, w * S, S, c) : 0.f;
+    }
+    __syncwarp();
+    if (lane < n) sums[t + lane] = ac_group_sum(turn + lane * kAcTurn1);
+    __syncwarp();
+    t += n;
+  }
+}
+
+// Lag rows row0 .. row0 + nrow - 1 of R, lags -L1 .. L1, into tile by the
+// whole block; complete for the block after ac_staged.  Row r starts at r
+// pitch; the pitch of 8 (mod 32) words keeps a group's four rows on different
+// banks.
+__host__ __device__ constexpr int ac_pitch(int L1) { return (2 * L1 + 1 + 23) / 32 * 32 + 8; }
 __device__ __forceinline__ void ac_stage(float* tile, const float* __restrict__ R, int P1, int row0,
                                          int nrow, int L1) {
-  const int W = 2 * L1 + 1;
+  const int W = 2 * L1 + 1, pitch = ac_pitch(L1);
   for (int r = threadIdx.x >> 5; r < nrow; r += blockDim.x >> 5) {
     const float* Rrow = R + (size_t)(row0 + r) * P1;
-#pragma unroll 4
-    for (int i = threadIdx.x & 31; i < W; i += 32)
-      tile[r * W + i] = __ldg(Rrow + (i < L1 ? i - L1 + P1 : i - L1));
+    uint32_t dst = (uint32_t)__cvta_generic_to_shared(tile + r * pitch + (threadIdx.x & 31));
+    for (int i = threadIdx.x & 31; i < W; i += 32, dst += 128)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst),
+                   "l"(__cvta_generic_to_global(Rrow + (i < L1 ? i - L1 + P1 : i - L1)))
+                   : "memory");
   }
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+}
+__device__ __forceinline__ void ac_staged() {
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  __syncthreads();
 }
 
 // FP64: a block a work unit, a warp a lag row.  The terms are bound by the
@@ -1050,62 +1197,83 @@ __global__ void __launch_bounds__(256) kde_lscv_ac64_kernel(const AcGen<double>*
     // every lag of the half plane counts twice, the lag 0 (K = C) once
     if (l0 == 0 && lane == 0) acc -= 0.5 * __ldg(R);
   }
-  block_sum_to(2.0 * g.C * acc,
-               partial + (int64_t)(g.u0 + u.y / kAcRows) * gridDim.y + blockIdx.y);
+  block_sum_to(acc, partial + (int64_t)(g.u0 + u.y / kAcRows) * gridDim.y + blockIdx.y);
 }
 
 // A block takes up to kAcBlock work units (matrix, first row) of one dataset
-// and first row, blocks[..] = (first unit, count), two to a warp:
-// partial[u nsets + y] with u the unit's place among its matrix's units, for
-// the autocorrelation g.set + y, y = blockIdx.y.  FP32: the units' lag rows are staged in shared memory once
+// and first row, blocks[..] = (first unit, count): partial[u nsets + y] with u
+// the unit's place among its matrix's units, for the autocorrelation g.set +
+// y, y = blockIdx.y.  The units' lag rows are staged in shared memory once
 // (the first unit's L_1 is the largest); read from the L2 as they are used,
-// one load's latency for 32 terms was most of the kernel.
+// one load's latency for 32 terms was most of the kernel.  The block's groups
+// are dealt out to its warps, their sums left in shared memory and added
+// there in order, so that a few wide supports keep every warp at work too.
 constexpr int kAcBlock = 16;
-__global__ void __launch_bounds__(256) kde_lscv_ac_kernel(const AcGen<float>* __restrict__ gens,
-                                                          const int2* __restrict__ units,
-                                                          const int2* __restrict__ blocks,
-                                                          const float* __restrict__ Rall, int P1,
-                                                          int64_t set_stride,
-                                                          double* __restrict__ partial) {
+constexpr int kAcThreads = 256;
+__host__ __device__ constexpr size_t ac_block_smem(int L1, int matrices, int threads) {
+  return (size_t)kAcRows * ac_pitch(L1) * sizeof(float) + (size_t)threads * kAcTurn1 * sizeof(float) +
+         (size_t)matrices * (kAcRows / kAcGroup) * kAcMaxWindows * sizeof(AcPair);
+}
+static_assert(ac_windows(KDE_MAX_P / 2 - 1, kAcWindow) <= kAcMaxWindows &&
+                  ac_windows(KDE_MAX_P / 2 - 1, ac_window(0, KDE_MAX_P / 2 - 1)) <= kAcMaxWindows &&
+                  ac_windows(256, ac_window(0, 256)) <= kAcMaxWindows,
+              "windows of a row");
+static_assert(ac_block_smem(KDE_MAX_P / 2 - 1, kAcBlock, kAcThreads) + 4096 <= kSmemMax,
+              "the widest support's rows and groups fit in shared memory");
+
+__global__ void __launch_bounds__(kAcThreads) kde_lscv_ac_kernel(
+    const AcGen<float>* __restrict__ gens, const int2* __restrict__ units,
+    const int2* __restrict__ blocks, const float* __restrict__ Rall, int P1, int64_t set_stride,
+    AcPair* __restrict__ partial) {
   extern __shared__ __align__(16) float tile[];
+  __shared__ AcGen<float> gs[kAcBlock];
+  __shared__ int off[kAcBlock + 1];
   const int2 blk = blocks[blockIdx.x];
   units += blk.x;
-  const int2 lead = units[0];
-  const AcGen<float>& gl = gens[lead.x];
-  const float* __restrict__ R = Rall + (int64_t)(gl.set + blockIdx.y) * set_stride;
-  const int lane = threadIdx.x & 31, L1 = gl.L1, W = 2 * L1 + 1, row0 = lead.y;
+  const int row0 = units[0].y, tid = threadIdx.x;
+  if (tid < blk.y) gs[tid] = gens[units[tid].x];
+  __syncthreads();
+  const float* __restrict__ R = Rall + (int64_t)(gs[0].set + blockIdx.y) * set_stride;
+  const int L1 = gs[0].L1, pitch = ac_pitch(L1);
   // rows below the support of the block's longest matrix (never past R)
   int L0 = 0;
-  for (int i = 0; i < blk.y; ++i) L0 = max(L0, gens[units[i].x].L0);
+  for (int i = 0; i < blk.y; ++i) L0 = max(L0, gs[i].L0);
   ac_stage(tile, R, P1, row0, min(kAcRows, L0 + 1 - row0), L1);
+  float* turn = tile + kAcRows * pitch;
+  AcPair* sums = reinterpret_cast<AcPair*>(turn + kAcThreads * kAcTurn1);
+  if (tid < 32) ac_offsets(gs, blk.y, row0, off);
+  ac_staged();
+  ac_groups(gs, off, blk.y, row0, tile + L1, pitch, turn, sums);
   __syncthreads();
-  for (int i = threadIdx.x >> 5; i < blk.y; i += 8) {
-    const AcGen<float> g = gens[units[i].x];
-    const double v = ac_unit_sum(g, row0, lane, [&](int r, int l1) { return tile[r * W + L1 + l1]; });
-    if (lane == 0) partial[(int64_t)(g.u0 + row0 / kAcRows) * gridDim.y + blockIdx.y] = v;
+  if (tid < blk.y) {
+    AcPair v{0.f, 0.f};
+#pragma unroll 4
+    for (int j = off[tid]; j < off[tid + 1]; ++j) v = ac_add(v, sums[j]);
+    partial[(int64_t)(gs[tid].u0 + row0 / kAcRows) * gridDim.y + blockIdx.y] = v;
   }
 }
 
 // Many datasets scored against one candidate set.  A kernel value serves
 // every dataset, so the sums are a matrix product (matrices x lags) (lags x
 // datasets).  A warp takes the work units of kAcQuad matrices with the same
-// L_1 on one first row, lane = class as above: per lag it forms the four
+// L_1 on one first row, a lane one chain of a group: per lag it forms the four
 // kernel values once and sums them against kAcSets datasets, whose lags a
-// block stages in shared memory (datasets innermost, so that a lane's
-// kAcSets values are four 16-byte loads; the pitch of 20 words keeps them
-// free of bank conflicts) for its 16 warps, the next rows' copies in flight.
-// That is about 1.2 instructions a term, where one dataset at a time takes the exponential
-// again for each: 256 datasets x 2016 matrices on 256^2 grids 3181 -> 255 us
-// (event times; 1.8 G terms, 44 us at the FP32 pipes' rate; what is left is
-// the staging's copies, one block of 16 warps an SM for its registers, and
-// lanes past the supports).  Tried: the datasets innermost in memory, a
-// thread a dataset, classes one after another (897 us with four matrices a
-// thread, 323 with eight: the L2's latency at 8 to 12 warps an SM).
+// block stages in shared memory kAcWindow lags of four rows at a time
+// (datasets innermost, so that a lane's kAcSets values are four 16-byte loads;
+// the pitch of 20 words keeps them free of bank conflicts) for its 16 warps,
+// the next window's copies in flight.  After a window each warp turns its 64 x
+// 32 chains through shared memory, so that a lane adds the 32 chains of two
+// sums.  A lane outside the support reads a slot of zeros, so that a value
+// that does not count is never touched.
 constexpr int kAcQuad = 4, kAcSets = 16, kAcPitch = 20;
-constexpr int kAcTileRows = 2;   // lag rows staged at a time, two tiles in turn
 constexpr int kAcWarps = 16;
+constexpr int kAcTurn = kAcQuad * kAcSets + 4;   // pitch of the turned chains
 constexpr int kAcSlab = 256;     // datasets per launch
 constexpr int kAcMinSets = 8;    // fewer are scored one by one
+constexpr int kAcTile = kAcGroup * kAcWindow * kAcPitch;
+constexpr size_t kAcSetsSmem =
+    sizeof(float) * (2 * kAcTile + 2 * kAcPitch + (size_t)kAcWarps * 32 * kAcTurn);
+static_assert(kAcSetsSmem <= kSmemMax, "tiles and turned chains fit in shared memory");
 
 // The matrices of one warp: the same L_1, falling L_0 (m[0]'s the largest).
 struct AcGroup {
@@ -1113,17 +1281,19 @@ struct AcGroup {
   int L0, L1;
 };
 
-// Lag rows t0 .. t0 + nrow - 1 of the datasets s0 .. s0 + nset - 1 into a tile
-// (one committed group of 4-byte asynchronous copies; no copy and no value
-// for datasets beyond).
+// Lags max(w0, -Lw) .. min(w0 + 63, Lw) of lag rows t0 .. t0 + nrow - 1 of
+// nset datasets into a tile (one committed group of 4-byte asynchronous
+// copies; no copy and no value for datasets beyond).
 __device__ __forceinline__ void ac_stage_sets(float* tile, const float* __restrict__ R, int P1,
-                                              int64_t set_stride, int t0, int nrow, int nset, int Lw) {
-  const int W = 2 * Lw + 1, lane = threadIdx.x & 31;
+                                              int64_t set_stride, int t0, int nrow, int nset,
+                                              int w0, int Lw) {
+  const int lane = threadIdx.x & 31, b = max(w0, -Lw), e = min(w0 + kAcWindow - 1, Lw);
   for (int q = threadIdx.x >> 5; q < nrow * nset; q += kAcWarps) {
     const int r = q / nset, d = q - r * nset;
     const float* Rrow = R + (int64_t)d * set_stride + (int64_t)(t0 + r) * P1;
-    uint32_t dst = (uint32_t)__cvta_generic_to_shared(tile + (r * W + lane) * kAcPitch + d);
-    for (int l1 = lane - Lw; l1 <= Lw; l1 += 32, dst += 32 * kAcPitch * 4)
+    uint32_t dst = (uint32_t)__cvta_generic_to_shared(
+        tile + (r * kAcWindow + b - w0 + lane) * kAcPitch + d);
+    for (int l1 = b + lane; l1 <= e; l1 += 32, dst += 32 * kAcPitch * 4)
       asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst),
                    "l"(__cvta_generic_to_global(Rrow + (l1 < 0 ? l1 + P1 : l1)))
                    : "memory");
@@ -1131,122 +1301,146 @@ __device__ __forceinline__ void ac_stage_sets(float* tile, const float* __restri
   asm volatile("cp.async.commit_group;\n" ::: "memory");
 }
 
+// ac_group_sum for two sums at a time (v: their columns, rows kAcTurn apart).
+__device__ __forceinline__ AcPair2 ac_group_sum2(const float* v) {
+  AcPair2 p{*reinterpret_cast<const float2*>(v), make_float2(0.f, 0.f)};
+#pragma unroll
+  for (int r = 1; r < 32; ++r) {
+    const float2 b = *reinterpret_cast<const float2*>(v + r * kAcTurn), s = __fadd2_rn(p.s, b);
+    p.e = __fadd2_rn(p.e, __fadd2_rn(sub2(p.s, s), b));
+    p.s = s;
+  }
+  return p;
+}
+
 __global__ void __launch_bounds__(32 * kAcWarps, 1) kde_lscv_ac_sets_kernel(
     const AcGen<float>* __restrict__ gens, const AcGroup* __restrict__ groups,
     const int3* __restrict__ items, const float* __restrict__ Rall, int P1, int64_t set_stride,
-    int ns, double* __restrict__ partial) {
-  extern __shared__ __align__(16) float tiles[];   // 2 x [row][l1 + Lw][kAcPitch]
+    int ns, AcPair* __restrict__ partial) {
+  extern __shared__ __align__(16) float tiles[];   // 2 x [row][lag][kAcPitch]
+  float* zero = tiles + 2 * kAcTile;               // a lag's datasets: zeros,
+  float* half = zero + kAcPitch;                   // and half of lag (0, 0)
   const int3 it = items[blockIdx.x];              // first group, groups, first row
   const int s0 = blockIdx.y * kAcSets, nset = min(kAcSets, ns - s0);
-  const int Lw = groups[it.x].L1, W = 2 * Lw + 1, row0 = it.z;   // L_1 falls along the groups
+  const int Lw = groups[it.x].L1, row0 = it.z;   // L_1 falls along the groups
   int Lmax = 0;
   for (int i = 0; i < it.y; ++i) Lmax = max(Lmax, groups[it.x + i].L0);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, rs = lane >> 3, c = lane & 7;
+  float* turn = half + kAcPitch + warp * 32 * kAcTurn;
   const bool act = warp < it.y && groups[it.x + (warp < it.y ? warp : 0)].L0 >= row0;
   const AcGroup gr = groups[it.x + (act ? warp : 0)];
-  AcGen<float> g[kAcQuad];
-#pragma unroll
-  for (int m = 0; m < kAcQuad; ++m) {
-    g[m] = gens[gr.m[m] >= 0 ? gr.m[m] : gr.m[0]];
-    if (gr.m[m] < 0) g[m].L0 = -1;
-  }
-  const int wand = g[0].wand;
   float2 acc[kAcQuad][kAcSets / 2];
 #pragma unroll
   for (int m = 0; m < kAcQuad; ++m)
 #pragma unroll
     for (int d = 0; d < kAcSets / 2; ++d) acc[m][d] = make_float2(0.f, 0.f);
   const float* R = Rall + (int64_t)s0 * set_stride;
-  const int end = min(Lmax + 1, row0 + kAcRows), tile_len = kAcTileRows * W * kAcPitch;
-  if (nset < kAcSets) {   // datasets beyond the last read as zeros
-    for (int i = threadIdx.x; i < 2 * tile_len; i += blockDim.x) tiles[i] = 0.f;
-    __syncthreads();
-  }
-  ac_stage_sets(tiles, R, P1, set_stride, row0, min(kAcTileRows, end - row0), nset, Lw);
-  int cur = 0;
-  for (int t0 = row0; t0 < end; t0 += kAcTileRows, cur ^= 1) {
-    const int nrow = min(kAcTileRows, end - t0);
-    const float* tile = tiles + cur * tile_len;
-    if (t0 + kAcTileRows < end)
-      ac_stage_sets(tiles + (cur ^ 1) * tile_len, R, P1, set_stride, t0 + kAcTileRows,
-                    min(kAcTileRows, end - t0 - kAcTileRows), nset, Lw);
-    else
+  // datasets beyond the last read as zeros
+  for (int i = threadIdx.x; i < 2 * kAcTile + 2 * kAcPitch; i += blockDim.x) tiles[i] = 0.f;
+  __syncthreads();
+  const int nw = ac_windows(Lw, kAcWindow), first = ac_first(Lw, kAcWindow);
+  const int ntile = nw * ((min(kAcRows, Lmax + 1 - row0) + kAcGroup - 1) / kAcGroup);
+  auto stage = [&](int t) {
+    if (t < ntile) {
+      const int h = t / nw, r0 = row0 + kAcGroup * h;
+      ac_stage_sets(tiles + (t & 1) * kAcTile, R, P1, set_stride, r0, min(kAcGroup, Lmax + 1 - r0),
+                    nset, (first + t - h * nw) * kAcWindow, Lw);
+    } else {
       asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+  };
+  stage(0);
+  AcPair2 sum{make_float2(0.f, 0.f), make_float2(0.f, 0.f)};   // sums 2 lane, 2 lane + 1
+  float2 D1[2], th[2], tl[2], e0[2];
+  int lo = 0;
+  unsigned span = 0, sign = 0;
+  const int S = ac_window(row0, gr.L1);
+  for (int t = 0; t < ntile; ++t) {
+    const int h = t / nw, w0 = (first + t - h * nw) * kAcWindow, r0 = row0 + kAcGroup * h;
+    const float* tile = tiles + (t & 1) * kAcTile;
+    stage(t + 1);
     asm volatile("cp.async.wait_group 1;\n" ::: "memory");
     __syncthreads();
-    if (act) {
-      const int r1 = min(nrow, gr.L0 + 1 - t0);
-      for (int r = 0; r < r1; ++r) {
-        const int l0 = t0 + r;
-        float2 D1[2], th[2], tl[2], e0[2];
-        float on[kAcQuad];   // 0 for a matrix whose support ends before this row
+    if (r0 == 0 && w0 == 0) {
+      if (threadIdx.x < kAcSets) half[threadIdx.x] = 0.5f * tile[threadIdx.x];
+      __syncthreads();
+    }
+    const int l0 = r0 + rs;
+    if (act && t == h * nw) {   // the lane's row of each matrix
+      lo = l0 > gr.L0 ? KDE_MAX_P : l0 == 0 ? 0 : -gr.L1;
+      span = l0 > gr.L0 ? 0u : (unsigned)(gr.L1 - lo);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const AcRow<float> a = ac_row(g[2 * h], l0), b = ac_row(g[2 * h + 1], l0);
-          D1[h] = make_float2(g[2 * h].D1, g[2 * h + 1].D1);
-          th[h] = make_float2(a.t_hi, b.t_hi);
-          tl[h] = make_float2(a.t_lo, b.t_lo);
-          e0[h] = make_float2(a.e0, b.e0);
+      for (int q = 0; q < 2; ++q) {
+        AcGen<float> g[2];
+        AcRow<float> a[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int m = gr.m[2 * q + j];
+          g[j] = gens[m >= 0 ? m : gr.m[0]];
+          a[j] = ac_row(g[j], l0);
+          if (m < 0 || l0 > g[j].L0) a[j].e0 = -INFINITY;   // no term
         }
-#pragma unroll
-        for (int m = 0; m < kAcQuad; ++m) on[m] = l0 <= g[m].L0 ? 1.f : 0.f;
-        float f = (float)(lane - gr.L1);
-        const float* x = tile + (r * W + lane - gr.L1 + Lw) * kAcPitch;
-        for (int l1 = lane - gr.L1; l1 - lane <= gr.L1; l1 += 32, f += 32.f, x += 32 * kAcPitch) {
-          // one factor for the lane's place: beyond the support, or row 0's
-          // other half, the terms are zero; the lag 0 counts half
-          const float w = l1 > gr.L1 ? 0.f : l0 > 0 || l1 > 0 ? 1.f : l1 == 0 ? 0.5f : 0.f;
-          const float lf = wand ? fabsf(f) : f;
+        D1[q] = make_float2(g[0].D1, g[1].D1);
+        th[q] = make_float2(a[0].t_hi, a[1].t_hi);
+        tl[q] = make_float2(a[0].t_lo, a[1].t_lo);
+        e0[q] = make_float2(a[0].e0, a[1].e0);
+        sign = g[0].wand ? 0x7FFFFFFFu : 0xFFFFFFFFu;
+      }
+    }
+    if (act && r0 <= gr.L0) {
+      // the tile's windows, the support's first to its last
+      const int v0 = max(w0, ac_first(gr.L1, S) * S), v1 = min(w0 + kAcWindow - 1, gr.L1);
+      for (int v = v0; v <= v1; v += S) {
+        const int i0 = max(0, (-gr.L1 - v) >> 3), i1 = min(S - 1, gr.L1 - v) >> 3;
+        int l = v + 8 * i0 + c;
+        float f = (float)l;
+        const float* x = tile + (rs * kAcWindow + l - w0) * kAcPitch;
+        for (int i = i0; i <= i1; ++i, l += 8, f += 8.f, x += 8 * kAcPitch) {
+          const float lf = __uint_as_float(__float_as_uint(f) & sign);
           float2 k[2];
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            k[h] = ac_term2(make_float2(lf, lf), D1[h], th[h], tl[h], e0[h]);
-            k[h] = __fmul2_rn(k[h], make_float2(w * on[2 * h], w * on[2 * h + 1]));
-          }
-          // lanes beyond the tile's last lag read its end (times zero)
-          const float4* xv = reinterpret_cast<const float4*>(l1 > gr.L1 ? tile : x);
+          for (int q = 0; q < 2; ++q) k[q] = ac_term2(make_float2(lf, lf), D1[q], th[q], tl[q], e0[q]);
+          const float* xs = (unsigned)(l - lo) <= span ? x : zero;
+          if (l == 0 && l0 == 0) xs = half;
+          const float4* xv = reinterpret_cast<const float4*>(xs);
           const float km[kAcQuad] = {k[0].x, k[0].y, k[1].x, k[1].y};
 #pragma unroll
           for (int q = 0; q < kAcSets / 4; ++q) {
-            const float4 v = xv[q];
+            const float4 y = xv[q];
 #pragma unroll
             for (int m = 0; m < kAcQuad; ++m) {
               const float2 kk = make_float2(km[m], km[m]);
-              acc[m][2 * q] = __ffma2_rn(kk, make_float2(v.x, v.y), acc[m][2 * q]);
-              acc[m][2 * q + 1] = __ffma2_rn(kk, make_float2(v.z, v.w), acc[m][2 * q + 1]);
+              acc[m][2 * q] = __ffma2_rn(kk, make_float2(y.x, y.y), acc[m][2 * q]);
+              acc[m][2 * q + 1] = __ffma2_rn(kk, make_float2(y.z, y.w), acc[m][2 * q + 1]);
             }
           }
         }
+        // turn: this lane's chains into a row, then two columns of 32 back
+        float4* row = reinterpret_cast<float4*>(turn + lane * kAcTurn);
+#pragma unroll
+        for (int m = 0; m < kAcQuad; ++m)
+#pragma unroll
+          for (int q = 0; q < kAcSets / 4; ++q) {
+            const float2 a = acc[m][2 * q], b = acc[m][2 * q + 1];
+            row[m * (kAcSets / 4) + q] = make_float4(a.x, a.y, b.x, b.y);
+            acc[m][2 * q] = acc[m][2 * q + 1] = make_float2(0.f, 0.f);
+          }
+        __syncwarp();
+        sum = ac_add2(sum, ac_group_sum2(turn + 2 * lane));
+        __syncwarp();
       }
     }
     __syncthreads();
   }
   if (!act) return;
-  // the 64 sums over the lanes, halving the values a lane carries at each
-  // step: value i adds the lanes in the order of a shuffle-down tree
-  float* a = &acc[0][0].x;
-  float c[kAcQuad * kAcSets];
-#pragma unroll
-  for (int i = 0; i < kAcQuad * kAcSets; ++i) c[i] = a[i];
-  int first = 0;
-#pragma unroll
-  for (int off = 16, n = kAcQuad * kAcSets / 2; off > 0; off >>= 1, n >>= 1) {
-    const bool up = lane & off;
-#pragma unroll
-    for (int i = 0; i < n; ++i) {
-      const float send = up ? c[i] : c[i + n], keep = up ? c[i + n] : c[i];
-      c[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-    }
-    first += up ? n : 0;
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int m = (first + i) / kAcSets, d = (first + i) % kAcSets;
-    if (d >= nset || gr.m[m] < 0) continue;
-    const AcGen<float>& gm = gens[gr.m[m]];
-    if (row0 <= gm.L0)
-      partial[(int64_t)(gm.u0 + row0 / kAcRows) * ns + s0 + d] = (double)(2.f * gm.C * c[i]);
-  }
+  const int m = groups[it.x + warp].m[(2 * lane) / kAcSets];
+  if (m < 0) return;
+  const AcGen<float>& g = gens[m];
+  if (row0 > g.L0) return;
+  AcPair* out = partial + (int64_t)(g.u0 + row0 / kAcRows) * ns + s0;
+  const int d = (2 * lane) % kAcSets;
+  if (d < nset) out[d] = AcPair{sum.s.x, sum.e.x};
+  if (d + 1 < nset) out[d + 1] = AcPair{sum.s.y, sum.e.y};
 }
 
 // {n, 1 / n^2, 2 / (n (n - 1))}: the LSCV's factors, formed once per dataset
@@ -1256,6 +1450,13 @@ struct NTerms {
   double v[3];
 };
 
+// A work unit's sum over 2 C as it is stored, and such sums added.
+template <typename T>
+using AcPart = std::conditional_t<std::is_same<T, float>::value, AcPair, double>;
+__device__ __forceinline__ double ac_add(double a, double b) { return a + b; }
+__device__ __forceinline__ double ac_value(double v) { return v; }
+__device__ __forceinline__ double ac_value(AcPair v) { return (double)v.s + (double)v.e; }
+
 // One thread per (candidate, dataset): S(H), S(2H) as the sums of their
 // units' partials in order, and the LSCV.  The n terms are the dataset's
 // (nk_set), or nk_all, or with nk_all.v[0] = 0 the candidate's (kn: {K_H(0),
@@ -1263,7 +1464,7 @@ struct NTerms {
 template <typename T>
 __global__ void __launch_bounds__(256) kde_lscv_ac_reduce_kernel(
     const AcGen<T>* __restrict__ gens, const double* __restrict__ kn,
-    const NTerms* __restrict__ nk_set, NTerms nk_all, const double* __restrict__ partial, int nh,
+    const NTerms* __restrict__ nk_set, NTerms nk_all, const AcPart<T>* __restrict__ partial, int nh,
     int ns, int64_t nH_all, double* __restrict__ S_out, double* __restrict__ lscv_out) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (int64_t)nh * ns) return;
@@ -1272,10 +1473,10 @@ __global__ void __launch_bounds__(256) kde_lscv_ac_reduce_kernel(
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int u0 = gens[2 * i + h].u0, nu = gens[2 * i + h].nu;
-    double v = 0.0;
+    AcPart<T> v{};
 #pragma unroll 8
-    for (int j = 0; j < nu; ++j) v += __ldg(partial + (int64_t)(u0 + j) * ns + y);
-    s[h] = v;
+    for (int j = 0; j < nu; ++j) v = ac_add(v, partial[(int64_t)(u0 + j) * ns + y]);
+    s[h] = 2.0 * (double)gens[2 * i + h].C * ac_value(v);
   }
   double nk[3];
 #pragma unroll
@@ -1365,57 +1566,54 @@ __global__ void __launch_bounds__(32) kde_theta_gen_kernel(ThetaArgs t) {
 }
 
 // A block takes up to kThetaCands candidates of one dataset (two matrices
-// each, two to a warp): S(A) = sum over the support of K_A(delta o l) R(l),
-// kAcRows lag rows staged in shared memory at a time, the units of
-// kde_lscv_ac_kernel added in order; NaN for a matrix that does not fit the
-// plan.  256 datasets of 28 candidates with supports near the box's widest:
-// 201 -> 152 us; bound by the exponentials (336 M terms, 67 us at 16 a clock
-// and SM) and their arithmetic.
+// each): S(A) = sum over the support of K_A(delta o l) R(l), kAcRows lag rows
+// staged in shared memory at a time, their groups dealt out to the warps and
+// added as kde_lscv_ac_kernel's are; NaN for a matrix that does not fit the
+// plan.  Bound by the exponentials and their arithmetic (256 datasets of 28
+// candidates with supports near the box's widest: 336 M terms, 67 us at 16
+// exponentials a clock and SM).
 constexpr int kThetaCands = 7;
 constexpr int kThetaThreads = 32 * kThetaCands;
+// L1max: an upper bound of the supports along axis 1.
 __global__ void __launch_bounds__(kThetaThreads) kde_lscv_theta_sums_kernel(
     const AcGen<float>* __restrict__ gens, int per, const float* __restrict__ Rall, int P1,
-    int64_t set_stride, double* __restrict__ S) {
+    int64_t set_stride, int L1max, double* __restrict__ S) {
   extern __shared__ __align__(16) float tile[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __shared__ AcGen<float> gs[2 * kThetaCands];
+  __shared__ int off[2 * kThetaCands + 1];
+  float* turn = tile + kAcRows * ac_pitch(L1max);
+  AcPair* sums = reinterpret_cast<AcPair*>(turn + kThetaThreads * kAcTurn1);
+  const int tid = threadIdx.x;
   const int ngroups = (per + 2 * kThetaCands - 1) / (2 * kThetaCands), set = blockIdx.x / ngroups;
   const int first = 2 * kThetaCands * (blockIdx.x - set * ngroups);
   const int nm = min(2 * kThetaCands, per - first);
   gens += (int64_t)set * per + first;
   S += (int64_t)set * per + first;
   const float* __restrict__ R = Rall + (int64_t)set * set_stride;
+  if (tid < nm) gs[tid] = gens[tid];
+  __syncthreads();
   int L0 = -1, L1 = 0;
   for (int m = 0; m < nm; ++m)
-    if (gens[m].L0 >= 0) {
-      L0 = max(L0, gens[m].L0);
-      L1 = max(L1, gens[m].L1);
+    if (gs[m].L0 >= 0) {
+      L0 = max(L0, gs[m].L0);
+      L1 = max(L1, gs[m].L1);
     }
-  const int W = 2 * L1 + 1;
-  AcGen<float> g[2];
-  double sum[2] = {0.0, 0.0};
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int m = warp + kThetaCands * h;
-    if (m < nm) g[h] = gens[m];
-    else g[h].L0 = -1;
-  }
+  AcPair sum{0.f, 0.f};
   for (int row0 = 0; row0 <= L0; row0 += kAcRows) {
     ac_stage(tile, R, P1, row0, min(kAcRows, L0 + 1 - row0), L1);
+    if (tid < 32) ac_offsets(gs, nm, row0, off);
+    ac_staged();
+    ac_groups(gs, off, nm, row0, tile + L1, ac_pitch(L1), turn, sums);
     __syncthreads();
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-      const AcGen<float> gh = h ? g[1] : g[0];
-      if (row0 > gh.L0) continue;
-      const double v =
-          ac_unit_sum(gh, row0, lane, [&](int r, int l1) { return tile[r * W + L1 + l1]; });
-      if (h) sum[1] += v;
-      else sum[0] += v;
+    if (tid < nm) {
+      AcPair v{0.f, 0.f};
+  #pragma unroll 4
+    for (int j = off[tid]; j < off[tid + 1]; ++j) v = ac_add(v, sums[j]);
+      sum = ac_add(sum, v);
     }
-    __syncthreads();
+    __syncthreads();   // off is written again
   }
-  if (lane == 0)
-    for (int h = 0; h < 2; ++h)
-      if (warp + kThetaCands * h < nm) S[warp + kThetaCands * h] = g[h].L0 < 0 ? nan("") : sum[h];
+  if (tid < nm) S[tid] = gs[tid].L0 < 0 ? nan("") : 2.0 * (double)gs[tid].C * ac_value(sum);
 }
 
 // One warp per dataset: LSCV of its J + 1 candidates (optionally stored),
@@ -2332,7 +2530,7 @@ struct AcImage {
 };
 
 template <typename T>
-kde_status ac_reduce(const AcImage<T>& im, int nh, int ns, const double* partial,
+kde_status ac_reduce(const AcImage<T>& im, int nh, int ns, const AcPart<T>* partial,
                      const NTerms* nk_set, const NTerms& nk_all, int64_t nH_all, double* S_out,
                      double* lscv_out, cudaStream_t st) {
   LaunchScope ls("kde_lscv_ac_reduce_kernel", st);
@@ -2346,12 +2544,14 @@ kde_status ac_reduce(const AcImage<T>& im, int nh, int ns, const double* partial
 
 // One chunk whose image (ac_build_chunk) is at `img` against ns
 // autocorrelations from R on, one by one (n terms as the reduction takes
-// them).  partial: nunits ns values.
+// them).  sums: nunits ns of AcPart.
 template <typename T>
 kde_status ac_launch_chunk(const kde_plan_info& I, const void* img, int nh, const AcShape& sh, const T* R,
-                           int ns, double* partial, const NTerms* nk_set, const NTerms& nk_all,
+                           int ns, void* sums, const NTerms* nk_set, const NTerms& nk_all,
                            int64_t nH_all, double* S_out, double* lscv_out, cudaStream_t st) {
   const AcImage<T> im(img, nh, sh.nunits);
+  AcPart<T>* partial = (AcPart<T>*)sums;
+  static_assert(sizeof(AcPart<T>) == sizeof(double), "the workspaces count 8 bytes a unit");
   cudaError_t e;
   const int64_t per = I.P[0] * I.P[1];
   if constexpr (std::is_same<T, double>::value) {
@@ -2360,11 +2560,10 @@ kde_status ac_launch_chunk(const kde_plan_info& I, const void* img, int nh, cons
         im.gens, im.units, R, (int)I.P[1], per, partial);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_ac64_kernel");
   } else {
-    // kAcRows staged rows of at most 2 (KDE_MAX_P / 2) - 1 lags
-    const size_t smem = (size_t)kAcRows * (2 * sh.L1 + 1) * sizeof(float);
+    const size_t smem = ac_block_smem(sh.L1, kAcBlock, kAcThreads);
     if ((e = allow_smem(kde_lscv_ac_kernel)) != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
     LaunchScope ls("kde_lscv_ac_kernel", st);
-    kde_lscv_ac_kernel<<<dim3((unsigned)sh.nblocks, (unsigned)ns), 256, smem, st>>>(
+    kde_lscv_ac_kernel<<<dim3((unsigned)sh.nblocks, (unsigned)ns), kAcThreads, smem, st>>>(
         im.gens, im.units, im.blocks, R, (int)I.P[1], per, partial);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_ac_kernel");
   }
@@ -2815,7 +3014,7 @@ struct kde_lscv_cands_s {
     int64_t c0;
     int nh;
     AcShape sh;
-    AcGroup* groups;   // null: scored one by one (FP64, or a support too wide)
+    AcGroup* groups;   // null: scored one by one (FP64)
     int3* items;
     int nitems;
   };
@@ -2826,13 +3025,6 @@ static void cands_free(kde_lscv_cands_s* c) {
   for (auto& ch : c->chunks) cudaFree(ch.dev);
   delete c;
 }
-
-// Supports along axis 1 up to this fit the batched sums' shared memory.
-constexpr int kAcMaxL1 = 319;
-constexpr size_t ac_tile_bytes(int L1) {
-  return (size_t)2 * kAcTileRows * (2 * L1 + 1) * kAcPitch * sizeof(float);
-}
-static_assert(ac_tile_bytes(kAcMaxL1) <= 220 * 1024, "a block's lag rows fit in shared memory");
 
 // Groups of up to kAcQuad matrices, and items of up to kAcWarps groups and a
 // first row (the widest first).
@@ -2873,7 +3065,7 @@ static kde_status cands_build(kde_lscv_cands_s* c, const double* H) {
     std::vector<int3> items;
     const size_t at = (up.size() + 255) & ~(size_t)255;
     size_t at_items = at;
-    if (sizeof(T) == 4 && ch.sh.L1 <= kAcMaxL1) {
+    if (sizeof(T) == 4) {
       cands_group(gens, groups, items);
       at_items = at + groups.size() * sizeof(AcGroup);
       up.resize(at_items + items.size() * sizeof(int3));
@@ -2977,7 +3169,7 @@ extern "C" kde_status kde_lscv_autocorr_cands_batch_workspace_bytes(kde_lscv_can
 
 // The batched sums of one chunk against ns autocorrelations from R on.
 static kde_status ac_product_chunk(const kde_plan_info& I, const kde_lscv_cands_s::Chunk& ch,
-                                   const float* R, int ns, double* partial, const NTerms* nk_set,
+                                   const float* R, int ns, AcPair* partial, const NTerms* nk_set,
                                    int64_t nH_all, double* S, double* lscv, cudaStream_t st) {
   const AcImage<float> im(ch.dev, ch.nh, ch.sh.nunits);
   cudaError_t e;
@@ -2986,8 +3178,7 @@ static kde_status ac_product_chunk(const kde_plan_info& I, const kde_lscv_cands_
       return cuda_fail(e, "cudaFuncSetAttribute");
     LaunchScope ls("kde_lscv_ac_sets_kernel", st);
     kde_lscv_ac_sets_kernel<<<dim3((unsigned)ch.nitems, (unsigned)((ns + kAcSets - 1) / kAcSets)),
-                              32 * kAcWarps,
-                              ac_tile_bytes(ch.sh.L1), st>>>(
+                              32 * kAcWarps, kAcSetsSmem, st>>>(
         im.gens, ch.groups, ch.items, R, (int)I.P[1], (int64_t)I.P[0] * I.P[1], ns, partial);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_ac_sets_kernel");
   }
@@ -3018,7 +3209,7 @@ extern "C" kde_status kde_lscv_autocorr_cands_batch(kde_lscv_cands cands, int ns
   const kde_plan_info& I = plan->info;
   cudaStream_t st = (cudaStream_t)stream;
   NTerms* nset = (NTerms*)workspace;
-  double* partial = (double*)((char*)workspace + lay.off_part);
+  void* partial = (char*)workspace + lay.off_part;
   if ((s = upload_async(nset, nd.data(), nd.size() * sizeof(NTerms), st)) != KDE_OK) return s;
   const int64_t per = I.P[0] * I.P[1], nH = cands->nH;
   for (int y = 0; y < nsets; y += lay.slab) {
@@ -3027,7 +3218,7 @@ extern "C" kde_status kde_lscv_autocorr_cands_batch(kde_lscv_cands cands, int ns
       double* S = pair_sums ? pair_sums + 2 * (y * nH + ch.c0) : nullptr;
       double* out = lscv + y * nH + ch.c0;
       if (lay.product)
-        s = ac_product_chunk(I, ch, (const float*)R + y * per, ns, partial, nset + y, nH, S, out, st);
+        s = ac_product_chunk(I, ch, (const float*)R + y * per, ns, (AcPair*)partial, nset + y, nH, S, out, st);
       else if (I.precision == KDE_F32)
         s = ac_launch_chunk<float>(I, ch.dev, ch.nh, ch.sh, (const float*)R + y * per, ns, partial,
                                    nset + y, NTerms{}, nH, S, out, st);
@@ -3138,14 +3329,14 @@ extern "C" kde_status kde_lscv_theta_select(kde_plan plan, int nsets, const int6
   {
     // a candidate's support that fits has L_1 <= P_1 - M_1, and never more than
     // M_1 - 1 (the padding alone can be far wider than any support)
-    const int64_t L1 = std::min(I.P[1] - I.M[1], I.M[1] - 1);
-    const size_t smem = (size_t)kAcRows * (2 * L1 + 1) * sizeof(float);
+    const int L1 = (int)std::min(I.P[1] - I.M[1], I.M[1] - 1);
+    const size_t smem = ac_block_smem(L1, 2 * kThetaCands, kThetaThreads);
     if ((e = allow_smem(kde_lscv_theta_sums_kernel)) != cudaSuccess)
       return cuda_fail(e, "cudaFuncSetAttribute");
     LaunchScope ls("kde_lscv_theta_sums_kernel", st);
     kde_lscv_theta_sums_kernel<<<(unsigned)((int64_t)nsets * ((J + kThetaCands) / kThetaCands)),
                                  kThetaThreads, smem, st>>>(t.gens, 2 * (J + 1), (const float*)R,
-                                                            (int)I.P[1], (int64_t)I.P[0] * I.P[1], S);
+                                                            (int)I.P[1], (int64_t)I.P[0] * I.P[1], L1, S);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_theta_sums_kernel");
   }
   {
