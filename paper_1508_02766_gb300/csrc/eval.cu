@@ -936,7 +936,8 @@ struct AcGen {
 //           order of 8 (row mod 4) + c, as a pair of FP32 (AcPair: the sum and
 //           the sum of its rounding errors);
 //   unit    the groups of its two sets of four rows, windows ascending;
-//   matrix  its units, in order.
+//   matrix  its units, every eighth in order, the eight sums as a tree
+//           (kde_lscv_ac_reduce_kernel).
 // From the chains on nothing is lost to FP32: LSCV subtracts two such sums,
 // and rows of small far terms vanish in one long chain.  FP64 additions would
 // do, but run at 2 lanes a clock and SM; a pair costs four to eight FP32 ones.  Error
@@ -960,7 +961,6 @@ __host__ __device__ constexpr int ac_window(int row0, int L1) {
 // Windows that hold lags -L1 .. L1: ac_first .. L1 / S.
 __host__ __device__ constexpr int ac_first(int L1, int S) { return -((L1 + S - 1) / S); }
 __host__ __device__ constexpr int ac_windows(int L1, int S) { return L1 / S - ac_first(L1, S) + 1; }
-constexpr int kAcMaxWindows = 33;
 
 // A sum as value + error, |error| about half an ulp of the value.
 struct AcPair {
@@ -1102,7 +1102,7 @@ __device__ __forceinline__ AcPair ac_group_sum(const float* v) {
 
 // A block's groups: those of unit row0 of nm <= 32 matrices (gs) dealt out to
 // its warps in runs, their sums into sums in order (matrix, set of four rows,
-// window), matrix m's at off[m].  A warp leaves the chains of up to 32 groups
+// window), matrix m's at off[m].  A warp leaves the chains of `held` <= 32 groups
 // in its turn of shared memory and a lane then adds each group's: shuffles for
 // each took a third of the kernel.  tile: lag (row0, 0).
 constexpr int kAcTurn1 = 33;   // pitch of the chains
@@ -1121,14 +1121,15 @@ __device__ __forceinline__ void ac_offsets(const AcGen<float>* gs, int nm, int r
   if (lane == 0) off[0] = 0;
 }
 __device__ __forceinline__ void ac_groups(const AcGen<float>* gs, const int* off, int nm, int row0,
-                                          const float* tile, int pitch, float* turn, AcPair* sums) {
+                                          const float* tile, int pitch, float* turn, int held,
+                                          AcPair* sums) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   const int end = off[nm] * (warp + 1) / warps, rs = lane >> 3, c = lane & 7;
   int t = off[nm] * warp / warps, m = 0, w = 0, S = 0, last = -1, r0 = 0;
-  turn += warp * 32 * kAcTurn1;
+  turn += warp * held * kAcTurn1;
   AcLane a{};
   while (t < end) {
-    const int n = min(32, end - t);
+    const int n = min(held, end - t);
     for (int k = 0; k < n; ++k, ++w) {
       if (w > last) {   // the next set of four rows, or where the run begins
         while (off[m + 1] <= t + k) ++m;
@@ -1147,6 +1148,11 @@ __device__ __forceinline__ void ac_groups(const AcGen<float>* gs, const int* off
     __syncwarp();
     t += n;
   }
+}
+
+// The groups' sums, behind the turns of the block's warps.
+__device__ __forceinline__ AcPair* ac_sums(float* turn, int held) {
+  return reinterpret_cast<AcPair*>(turn + (((int)(blockDim.x >> 5) * held * kAcTurn1 + 1) & ~1));
 }
 
 // Lag rows row0 .. row0 + nrow - 1 of R, lags -L1 .. L1, into tile by the
@@ -1200,8 +1206,8 @@ __global__ void __launch_bounds__(256) kde_lscv_ac64_kernel(const AcGen<double>*
   block_sum_to(acc, partial + (int64_t)(g.u0 + u.y / kAcRows) * gridDim.y + blockIdx.y);
 }
 
-// A block takes up to kAcBlock work units (matrix, first row) of one dataset
-// and first row, blocks[..] = (first unit, count): partial[u nsets + y] with u
+// A block takes up to `sub` work units (matrix, first row) of one dataset and
+// first row, a part of blocks[..] = (first unit, count <= kAcBlock): partial[u nsets + y] with u
 // the unit's place among its matrix's units, for the autocorrelation g.set +
 // y, y = blockIdx.y.  The units' lag rows are staged in shared memory once
 // (the first unit's L_1 is the largest); read from the L2 as they are used,
@@ -1209,14 +1215,30 @@ __global__ void __launch_bounds__(256) kde_lscv_ac64_kernel(const AcGen<double>*
 // are dealt out to its warps, their sums left in shared memory and added
 // there in order, so that a few wide supports keep every warp at work too.
 constexpr int kAcBlock = 16;
-constexpr int kAcThreads = 256;
-__host__ __device__ constexpr size_t ac_block_smem(int L1, int matrices, int threads) {
-  return (size_t)kAcRows * ac_pitch(L1) * sizeof(float) + (size_t)threads * kAcTurn1 * sizeof(float) +
-         (size_t)matrices * (kAcRows / kAcGroup) * kAcMaxWindows * sizeof(AcPair);
+// Warps of a block: twice as many where the staged rows leave room for one
+// block an SM.
+constexpr int kAcThreads = 512;
+__host__ __device__ constexpr int ac_threads(int L1) {
+  return 2 * kAcRows * ac_pitch(L1) * (int)sizeof(float) > 110 * 1024 ? kAcThreads : kAcThreads / 2;
 }
-static_assert(ac_windows(KDE_MAX_P / 2 - 1, kAcWindow) <= kAcMaxWindows &&
-                  ac_windows(KDE_MAX_P / 2 - 1, ac_window(0, KDE_MAX_P / 2 - 1)) <= kAcMaxWindows &&
-                  ac_windows(256, ac_window(0, 256)) <= kAcMaxWindows,
+// Groups of a unit at most, over supports up to L1.
+__host__ __device__ constexpr int ac_unit_groups(int L1) {
+  return (kAcRows / kAcGroup) * (L1 <= 256 ? ac_windows(L1, 16) : 33);
+}
+// Groups whose chains a warp holds at a time, with `matrices` units a block.
+__host__ __device__ constexpr int ac_turn(int L1, int matrices, int threads) {
+  const int n = (matrices * ac_unit_groups(L1) * 32 + threads - 1) / threads;
+  return n < 32 ? n : 32;
+}
+__host__ __device__ constexpr size_t ac_block_smem(int L1, int matrices, int threads) {
+  return (size_t)kAcRows * ac_pitch(L1) * sizeof(float) +
+         (size_t)(threads / 32) * ac_turn(L1, matrices, threads) * kAcTurn1 * sizeof(float) +
+         (size_t)matrices * ac_unit_groups(L1) * sizeof(AcPair) + sizeof(AcPair);
+}
+static_assert(ac_windows(KDE_MAX_P / 2 - 1, kAcWindow) <= 33 &&
+                  ac_windows(KDE_MAX_P / 2 - 1, ac_window(0, KDE_MAX_P / 2 - 1)) <= 33 &&
+                  ac_windows(257, ac_window(0, 257)) <= 33 && ac_windows(512, ac_window(0, 512)) <= 33 &&
+                  ac_windows(1024, ac_window(0, 1024)) <= 33,
               "windows of a row");
 static_assert(ac_block_smem(KDE_MAX_P / 2 - 1, kAcBlock, kAcThreads) + 4096 <= kSmemMax,
               "the widest support's rows and groups fit in shared memory");
@@ -1224,12 +1246,15 @@ static_assert(ac_block_smem(KDE_MAX_P / 2 - 1, kAcBlock, kAcThreads) + 4096 <= k
 __global__ void __launch_bounds__(kAcThreads) kde_lscv_ac_kernel(
     const AcGen<float>* __restrict__ gens, const int2* __restrict__ units,
     const int2* __restrict__ blocks, const float* __restrict__ Rall, int P1, int64_t set_stride,
-    AcPair* __restrict__ partial) {
+    int sub, int held, AcPair* __restrict__ partial) {
   extern __shared__ __align__(16) float tile[];
   __shared__ AcGen<float> gs[kAcBlock];
   __shared__ int off[kAcBlock + 1];
-  const int2 blk = blocks[blockIdx.x];
-  units += blk.x;
+  const int parts = (kAcBlock + sub - 1) / sub, part = blockIdx.x % parts;
+  int2 blk = blocks[blockIdx.x / parts];
+  blk.y = min(sub, blk.y - part * sub);
+  if (blk.y <= 0) return;
+  units += blk.x + part * sub;
   const int row0 = units[0].y, tid = threadIdx.x;
   if (tid < blk.y) gs[tid] = gens[units[tid].x];
   __syncthreads();
@@ -1240,10 +1265,10 @@ __global__ void __launch_bounds__(kAcThreads) kde_lscv_ac_kernel(
   for (int i = 0; i < blk.y; ++i) L0 = max(L0, gs[i].L0);
   ac_stage(tile, R, P1, row0, min(kAcRows, L0 + 1 - row0), L1);
   float* turn = tile + kAcRows * pitch;
-  AcPair* sums = reinterpret_cast<AcPair*>(turn + kAcThreads * kAcTurn1);
+  AcPair* sums = ac_sums(turn, held);
   if (tid < 32) ac_offsets(gs, blk.y, row0, off);
   ac_staged();
-  ac_groups(gs, off, blk.y, row0, tile + L1, pitch, turn, sums);
+  ac_groups(gs, off, blk.y, row0, tile + L1, pitch, turn, held, sums);
   __syncthreads();
   if (tid < blk.y) {
     AcPair v{0.f, 0.f};
@@ -1457,37 +1482,86 @@ __device__ __forceinline__ double ac_add(double a, double b) { return a + b; }
 __device__ __forceinline__ double ac_value(double v) { return v; }
 __device__ __forceinline__ double ac_value(AcPair v) { return (double)v.s + (double)v.e; }
 
-// One thread per (candidate, dataset): S(H), S(2H) as the sums of their
-// units' partials in order, and the LSCV.  The n terms are the dataset's
-// (nk_set), or nk_all, or with nk_all.v[0] = 0 the candidate's (kn: {K_H(0),
-// n terms}).  Outputs at y nH_all + i.
-template <typename T>
+// S(H), S(2H) per (candidate, dataset) as the sums of their units' partials,
+// and the LSCV.  Class c of a matrix's units takes every eighth from c on, in
+// order; the classes' sums are added as a tree.  With many scores a thread
+// takes a score; with few a warp takes a class of 32 scores, as one thread
+// waited for one load after another (64 candidates of 1800 lags 85 us, now
+// 15).  The n terms are the dataset's (nk_set), or nk_all, or with nk_all.v[0]
+// = 0 the candidate's (kn: {K_H(0), n terms}).  Outputs at y nH_all + i.
+constexpr int kAcClasses = 8;
+template <typename T, bool MANY>
 __global__ void __launch_bounds__(256) kde_lscv_ac_reduce_kernel(
     const AcGen<T>* __restrict__ gens, const double* __restrict__ kn,
     const NTerms* __restrict__ nk_set, NTerms nk_all, const AcPart<T>* __restrict__ partial, int nh,
     int ns, int64_t nH_all, double* __restrict__ S_out, double* __restrict__ lscv_out) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)nh * ns) return;
-  const int i = (int)(t / ns), y = (int)(t - (int64_t)i * ns);
-  double s[2];
+  constexpr int kScores = MANY ? 256 : 32;
+  const int lane = threadIdx.x % kScores, p = threadIdx.x / kScores;
+  const int64_t t = (int64_t)blockIdx.x * kScores + lane;
+  const bool in = t < (int64_t)nh * ns;
+  const int i = in ? (int)(t / ns) : 0, y = (int)(t - (int64_t)i * ns);
+  const AcGen<T>*g0 = gens + 2 * i, *g1 = g0 + 1;
+  const int nu0 = in ? g0->nu : 0, nu1 = in ? g1->nu : 0;
+  const AcPart<T>*p0 = partial + (int64_t)g0->u0 * ns + y, *p1 = partial + (int64_t)g1->u0 * ns + y;
+  AcPart<T> v[2] = {};
+  if constexpr (MANY) {
+    AcPart<T> c[2][kAcClasses] = {};
+    for (int j = 0; j < max(nu0, nu1); j += kAcClasses)
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int u0 = gens[2 * i + h].u0, nu = gens[2 * i + h].nu;
-    AcPart<T> v{};
-#pragma unroll 8
-    for (int j = 0; j < nu; ++j) v = ac_add(v, partial[(int64_t)(u0 + j) * ns + y]);
-    s[h] = 2.0 * (double)gens[2 * i + h].C * ac_value(v);
+      for (int k = 0; k < kAcClasses; ++k) {
+        c[0][k] = ac_add(c[0][k], j + k < nu0 ? p0[(int64_t)(j + k) * ns] : AcPart<T>{});
+        c[1][k] = ac_add(c[1][k], j + k < nu1 ? p1[(int64_t)(j + k) * ns] : AcPart<T>{});
+      }
+#pragma unroll
+    for (int off = kAcClasses / 2; off > 0; off >>= 1)
+#pragma unroll
+      for (int k = 0; k < off; ++k)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) c[h][k] = ac_add(c[h][k], c[h][k + off]);
+    v[0] = c[0][0];
+    v[1] = c[1][0];
+  } else {
+    __shared__ AcPart<T> part[2][kAcClasses][kScores];
+    for (int j = p; j < max(nu0, nu1); j += 8 * kAcClasses) {
+      AcPart<T> a[8], b[8];   // loads in flight
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int u = j + k * kAcClasses;
+        a[k] = u < nu0 ? p0[(int64_t)u * ns] : AcPart<T>{};
+        b[k] = u < nu1 ? p1[(int64_t)u * ns] : AcPart<T>{};
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        v[0] = ac_add(v[0], a[k]);
+        v[1] = ac_add(v[1], b[k]);
+      }
+    }
+    part[0][p][lane] = v[0];
+    part[1][p][lane] = v[1];
+#pragma unroll
+    for (int off = kAcClasses / 2; off > 0; off >>= 1) {
+      __syncthreads();
+      if (p < off)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          v[h] = ac_add(v[h], part[h][p + off][lane]);
+          part[h][p][lane] = v[h];
+        }
+    }
+    if (p) return;
   }
+  if (!in) return;
+  const double s0 = 2.0 * (double)g0->C * ac_value(v[0]), s1 = 2.0 * (double)g1->C * ac_value(v[1]);
   double nk[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k)
     nk[k] = nk_set ? nk_set[y].v[k] : nk_all.v[0] > 0.0 ? nk_all.v[k] : kn[4 * (int64_t)i + 1 + k];
   const int64_t o = y * nH_all + i;
   if (S_out) {
-    S_out[2 * o] = s[0];
-    S_out[2 * o + 1] = s[1];
+    S_out[2 * o] = s0;
+    S_out[2 * o + 1] = s1;
   }
-  lscv_out[o] = s[1] * nk[1] - nk[2] * (s[0] - nk[0] * kn[4 * (int64_t)i]);
+  lscv_out[o] = s1 * nk[1] - nk[2] * (s0 - nk[0] * kn[4 * (int64_t)i]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1577,12 +1651,12 @@ constexpr int kThetaThreads = 32 * kThetaCands;
 // L1max: an upper bound of the supports along axis 1.
 __global__ void __launch_bounds__(kThetaThreads) kde_lscv_theta_sums_kernel(
     const AcGen<float>* __restrict__ gens, int per, const float* __restrict__ Rall, int P1,
-    int64_t set_stride, int L1max, double* __restrict__ S) {
+    int64_t set_stride, int L1max, int held, double* __restrict__ S) {
   extern __shared__ __align__(16) float tile[];
   __shared__ AcGen<float> gs[2 * kThetaCands];
   __shared__ int off[2 * kThetaCands + 1];
   float* turn = tile + kAcRows * ac_pitch(L1max);
-  AcPair* sums = reinterpret_cast<AcPair*>(turn + kThetaThreads * kAcTurn1);
+  AcPair* sums = ac_sums(turn, held);
   const int tid = threadIdx.x;
   const int ngroups = (per + 2 * kThetaCands - 1) / (2 * kThetaCands), set = blockIdx.x / ngroups;
   const int first = 2 * kThetaCands * (blockIdx.x - set * ngroups);
@@ -1603,7 +1677,7 @@ __global__ void __launch_bounds__(kThetaThreads) kde_lscv_theta_sums_kernel(
     ac_stage(tile, R, P1, row0, min(kAcRows, L0 + 1 - row0), L1);
     if (tid < 32) ac_offsets(gs, nm, row0, off);
     ac_staged();
-    ac_groups(gs, off, nm, row0, tile + L1, ac_pitch(L1), turn, sums);
+    ac_groups(gs, off, nm, row0, tile + L1, ac_pitch(L1), turn, held, sums);
     __syncthreads();
     if (tid < nm) {
       AcPair v{0.f, 0.f};
@@ -2492,6 +2566,11 @@ kde_status ac_build_chunk(kde_plan_s* plan, int64_t c0, int nh, int nH, const do
       for (size_t k = i; k < j; ++k)
         if (r <= gens[order[k]].L0) units.push_back(make_int2(order[k], r));
   }
+  *shape = AcShape{(int)units.size(), 0, 0, 0};
+  for (const auto& g : gens) {
+    shape->L0 = std::max(shape->L0, g.L0);
+    shape->L1 = std::max(shape->L1, g.L1);
+  }
   std::vector<int2> blocks;
   for (int u = 0; u < (int)units.size(); ++u) {
     const bool same = !blocks.empty() && blocks.back().y < kAcBlock &&
@@ -2500,11 +2579,7 @@ kde_status ac_build_chunk(kde_plan_s* plan, int64_t c0, int nh, int nH, const do
     if (same) ++blocks.back().y;
     else blocks.push_back(make_int2(u, 1));
   }
-  *shape = AcShape{(int)units.size(), (int)blocks.size(), 0, 0};
-  for (const auto& g : gens) {
-    shape->L0 = std::max(shape->L0, g.L0);
-    shape->L1 = std::max(shape->L1, g.L1);
-  }
+  shape->nblocks = (int)blocks.size();
   const size_t gb = gens.size() * sizeof(AcGen<T>), kb = kn.size() * sizeof(double),
                ub = units.size() * sizeof(int2), bb = blocks.size() * sizeof(int2);
   up.resize(gb + kb + ub + bb);
@@ -2534,12 +2609,28 @@ kde_status ac_reduce(const AcImage<T>& im, int nh, int ns, const AcPart<T>* part
                      const NTerms* nk_set, const NTerms& nk_all, int64_t nH_all, double* S_out,
                      double* lscv_out, cudaStream_t st) {
   LaunchScope ls("kde_lscv_ac_reduce_kernel", st);
-  const int64_t threads = (int64_t)nh * ns;
-  const int block = threads < 64 * 256 ? 64 : 256;
-  kde_lscv_ac_reduce_kernel<T><<<(unsigned)((threads + block - 1) / block), block, 0, st>>>(
-      im.gens, im.kn, nk_set, nk_all, partial, nh, ns, nH_all, S_out, lscv_out);
+  const int64_t scores = (int64_t)nh * ns;
+  auto launch = [&](auto fn, int per) {
+    fn<<<(unsigned)((scores + per - 1) / per), 256, 0, st>>>(im.gens, im.kn, nk_set, nk_all, partial,
+                                                             nh, ns, nH_all, S_out, lscv_out);
+  };
+  if (scores >= 256 * (int64_t)num_sms()) launch(kde_lscv_ac_reduce_kernel<T, true>, 256);
+  else launch(kde_lscv_ac_reduce_kernel<T, false>, 32);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? KDE_OK : cuda_fail(e, "kde_lscv_ac_reduce_kernel");
+}
+
+// Units of a block: fewer where there are few in all, so that every SM has the
+// blocks that it can hold, up to four (16 candidates of 230 lags 18.1 us with
+// sixteen a block, 12.8 with a lag row a warp, 13.1 now; 512 x 512, 460 lags
+// 29.1, 19.4, 18.3), but 24 groups at least.
+int ac_block_units(int64_t nunits, int L1) {
+  const int64_t fit = 220 * 1024 / ac_block_smem(L1, kAcBlock, ac_threads(L1));
+  const int64_t blocks = std::min<int64_t>(4, std::max<int64_t>(1, fit)) * num_sms();
+  const int64_t least = (23 + ac_unit_groups(L1)) / ac_unit_groups(L1);
+  int sub = 1;   // parts of a block are alike
+  while (sub < kAcBlock && (sub < least || 2 * sub <= nunits / blocks)) sub *= 2;
+  return sub;
 }
 
 // One chunk whose image (ac_build_chunk) is at `img` against ns
@@ -2560,11 +2651,14 @@ kde_status ac_launch_chunk(const kde_plan_info& I, const void* img, int nh, cons
         im.gens, im.units, R, (int)I.P[1], per, partial);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_ac64_kernel");
   } else {
-    const size_t smem = ac_block_smem(sh.L1, kAcBlock, kAcThreads);
+    const int threads = ac_threads(sh.L1), sub = ac_block_units((int64_t)sh.nunits * ns, sh.L1);
+    const size_t smem = ac_block_smem(sh.L1, sub, threads);
+    const unsigned grid = (unsigned)sh.nblocks * (unsigned)((kAcBlock + sub - 1) / sub);
     if ((e = allow_smem(kde_lscv_ac_kernel)) != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
     LaunchScope ls("kde_lscv_ac_kernel", st);
-    kde_lscv_ac_kernel<<<dim3((unsigned)sh.nblocks, (unsigned)ns), kAcThreads, smem, st>>>(
-        im.gens, im.units, im.blocks, R, (int)I.P[1], per, partial);
+    kde_lscv_ac_kernel<<<dim3(grid, (unsigned)ns), threads, smem, st>>>(
+        im.gens, im.units, im.blocks, R, (int)I.P[1], per, sub,
+        ac_turn(sh.L1, sub, threads), partial);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_ac_kernel");
   }
   return ac_reduce<T>(im, nh, ns, partial, nk_set, nk_all, nH_all, S_out, lscv_out, st);
@@ -3336,7 +3430,8 @@ extern "C" kde_status kde_lscv_theta_select(kde_plan plan, int nsets, const int6
     LaunchScope ls("kde_lscv_theta_sums_kernel", st);
     kde_lscv_theta_sums_kernel<<<(unsigned)((int64_t)nsets * ((J + kThetaCands) / kThetaCands)),
                                  kThetaThreads, smem, st>>>(t.gens, 2 * (J + 1), (const float*)R,
-                                                            (int)I.P[1], (int64_t)I.P[0] * I.P[1], L1, S);
+                                                            (int)I.P[1], (int64_t)I.P[0] * I.P[1], L1,
+                                                            ac_turn(L1, 2 * kThetaCands, kThetaThreads), S);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_theta_sums_kernel");
   }
   {
