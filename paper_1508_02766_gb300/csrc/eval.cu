@@ -931,7 +931,7 @@ struct AcGen {
 // kernel below, so that a candidate's score does not depend on how many
 // datasets are scored with it or on how the work is spread:
 //   chain   the lags l_1 = c (mod 8) of one row inside one window [S w, S (w +
-//           1)), ascending, in FP32: S = ac_window(first row, L_1) / 8 terms;
+//           1)), ascending, in FP32: S = 2^ac_shift(first row, L_1), S / 8 terms;
 //   group   the 4 x 8 chains of four rows (first row a multiple of four), in
 //           order of 8 (row mod 4) + c, as a pair of FP32 (AcPair: the sum and
 //           the sum of its rounding errors);
@@ -953,14 +953,16 @@ constexpr int kAcWindow = 128;    // widest window
 // Width of the windows: short chains in the first unit, which holds the
 // largest terms and with a support of few rows is all there is (every unit at
 // 64 lags: 1.5 times the error at 5 x 48 lags); about sixteen a side at least.
-__host__ __device__ constexpr int ac_window(int row0, int L1) {
-  int S = row0 ? kAcWindow : 16;
-  while (S < kAcWindow && 16 * S < L1) S *= 2;
-  return S;
+// (The windows' log2, so that nothing is divided.)
+__host__ __device__ constexpr int ac_shift(int row0, int L1) {
+  int b = row0 ? 7 : 4;
+  while (b < 7 && (16 << b) < L1) ++b;
+  return b;
 }
-// Windows that hold lags -L1 .. L1: ac_first .. L1 / S.
-__host__ __device__ constexpr int ac_first(int L1, int S) { return -((L1 + S - 1) / S); }
-__host__ __device__ constexpr int ac_windows(int L1, int S) { return L1 / S - ac_first(L1, S) + 1; }
+static_assert(kAcWindow == 1 << 7, "");
+// Windows that hold lags -L1 .. L1: ac_first .. L1 >> b.
+__host__ __device__ constexpr int ac_first(int L1, int b) { return -((L1 + (1 << b) - 1) >> b); }
+__host__ __device__ constexpr int ac_windows(int L1, int b) { return (L1 >> b) - ac_first(L1, b) + 1; }
 
 // A sum as value + error, |error| about half an ulp of the value.
 struct AcPair {
@@ -1058,19 +1060,28 @@ __device__ __forceinline__ float ac_chain(const AcGen<float>& g, const AcLane& a
     return ac_term2(l, a.D1, a.th, a.tl, a.e0);
   };
   const float2 step = make_float2(16.f, 16.f);
-  if (w0 >= -g.L1 && w0 + S <= g.L1 && r0 > 0 && r0 + kAcGroup - 1 <= g.L0) {   // all of it
-    const float* x = a.x + w0 + c;
-    float2 f = make_float2((float)(w0 + c), (float)(w0 + c + 8));
+  const int i0 = max(0, (-g.L1 - w0) >> 3), i1 = min(S - 1, g.L1 - w0) >> 3;
+  if (r0 > 0 && r0 + kAcGroup - 1 <= g.L0) {   // whole rows: only the ends can lie outside
+    auto end = [&](int i) {
+      const int l = w0 + 8 * i + c;
+      const float2 k = terms(make_float2((float)l, 0.f));
+      if ((unsigned)(l - a.lo) <= a.span) acc = fmaf(k.x, a.x[l], acc);
+    };
+    int i = i0;
+    const int last = w0 + 8 * i1 + 7 > g.L1 ? i1 - 1 : i1;
+    if (w0 + 8 * i0 < -g.L1) end(i++);
+    const float* x = a.x + w0 + 8 * i + c;
+    float2 f = make_float2((float)(w0 + 8 * i + c), (float)(w0 + 8 * i + c + 8));
 #pragma unroll 4
-    for (int i = 0; i < S / 16; ++i, x += 16) {
+    for (; i < last; i += 2, x += 16) {
       const float2 k = terms(f);
       acc = fmaf(k.x, x[0], acc);
       acc = fmaf(k.y, x[8], acc);
       f = __fadd2_rn(f, step);
     }
+    for (; i <= i1; ++i) end(i);
     return acc;
   }
-  const int i0 = max(0, (-g.L1 - w0) >> 3), i1 = min(S - 1, g.L1 - w0) >> 3;
   int l = w0 + 8 * i0 + c;
   float2 f = make_float2((float)l, (float)(l + 8));
   for (int i = i0; i <= i1; i += 2, l += 16) {
@@ -1111,7 +1122,7 @@ __device__ __forceinline__ void ac_offsets(const AcGen<float>* gs, int nm, int r
   const int lane = threadIdx.x & 31;
   int v = 0;
   if (lane < nm && row0 <= gs[lane].L0)
-    v = (kAcRows / kAcGroup) * ac_windows(gs[lane].L1, ac_window(row0, gs[lane].L1));
+    v = (kAcRows / kAcGroup) * ac_windows(gs[lane].L1, ac_shift(row0, gs[lane].L1));
 #pragma unroll
   for (int d = 1; d < 32; d *= 2) {
     const int u = __shfl_up_sync(0xffffffffu, v, d);
@@ -1125,23 +1136,25 @@ __device__ __forceinline__ void ac_groups(const AcGen<float>* gs, const int* off
                                           AcPair* sums) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   const int end = off[nm] * (warp + 1) / warps, rs = lane >> 3, c = lane & 7;
-  int t = off[nm] * warp / warps, m = 0, w = 0, S = 0, last = -1, r0 = 0;
+  int t = off[nm] * warp / warps, m = 0, w = 0, b = 0, last = -1, r0 = 0;
   turn += warp * held * kAcTurn1;
   AcLane a{};
+  AcGen<float> g{};
   while (t < end) {
     const int n = min(held, end - t);
     for (int k = 0; k < n; ++k, ++w) {
       if (w > last) {   // the next set of four rows, or where the run begins
         while (off[m + 1] <= t + k) ++m;
-        S = ac_window(row0, gs[m].L1);
-        const int nw = ac_windows(gs[m].L1, S), j = t + k - off[m];
-        const int h = j >= nw;
-        w = ac_first(gs[m].L1, S) + j - h * nw;
-        last = gs[m].L1 / S;
+        g = gs[m];
+        b = ac_shift(row0, g.L1);
+        const int first = ac_first(g.L1, b), j = t + k - off[m];
+        last = g.L1 >> b;
+        const int nw = last - first + 1, h = j >= nw;
+        w = first + j - h * nw;
         r0 = row0 + kAcGroup * h;
-        a = ac_lane(gs[m], r0 + rs, tile + (kAcGroup * h + rs) * pitch);
+        a = ac_lane(g, r0 + rs, tile + (kAcGroup * h + rs) * pitch);
       }
-      turn[k * kAcTurn1 + lane] = r0 <= gs[m].L0 ? ac_chain(gs[m], a, r0, w * S, S, c) : 0.f;
+      turn[k * kAcTurn1 + lane] = r0 <= g.L0 ? ac_chain(g, a, r0, w << b, 1 << b, c) : 0.f;
     }
     __syncwarp();
     if (lane < n) sums[t + lane] = ac_group_sum(turn + lane * kAcTurn1);
@@ -1223,7 +1236,7 @@ __host__ __device__ constexpr int ac_threads(int L1) {
 }
 // Groups of a unit at most, over supports up to L1.
 __host__ __device__ constexpr int ac_unit_groups(int L1) {
-  return (kAcRows / kAcGroup) * (L1 <= 256 ? ac_windows(L1, 16) : 33);
+  return (kAcRows / kAcGroup) * (L1 <= 256 ? ac_windows(L1, 4) : 33);
 }
 // Groups whose chains a warp holds at a time, with `matrices` units a block.
 __host__ __device__ constexpr int ac_turn(int L1, int matrices, int threads) {
@@ -1235,10 +1248,9 @@ __host__ __device__ constexpr size_t ac_block_smem(int L1, int matrices, int thr
          (size_t)(threads / 32) * ac_turn(L1, matrices, threads) * kAcTurn1 * sizeof(float) +
          (size_t)matrices * ac_unit_groups(L1) * sizeof(AcPair) + sizeof(AcPair);
 }
-static_assert(ac_windows(KDE_MAX_P / 2 - 1, kAcWindow) <= 33 &&
-                  ac_windows(KDE_MAX_P / 2 - 1, ac_window(0, KDE_MAX_P / 2 - 1)) <= 33 &&
-                  ac_windows(257, ac_window(0, 257)) <= 33 && ac_windows(512, ac_window(0, 512)) <= 33 &&
-                  ac_windows(1024, ac_window(0, 1024)) <= 33,
+static_assert(ac_windows(KDE_MAX_P / 2 - 1, 7) <= 33 && ac_windows(256, ac_shift(0, 256)) <= 33 &&
+                  ac_windows(512, ac_shift(0, 512)) <= 33 && ac_windows(1024, ac_shift(0, 1024)) <= 33 &&
+                  ac_shift(0, 1025) == 7,
               "windows of a row");
 static_assert(ac_block_smem(KDE_MAX_P / 2 - 1, kAcBlock, kAcThreads) + 4096 <= kSmemMax,
               "the widest support's rows and groups fit in shared memory");
@@ -1363,7 +1375,7 @@ __global__ void __launch_bounds__(32 * kAcWarps, 1) kde_lscv_ac_sets_kernel(
   // datasets beyond the last read as zeros
   for (int i = threadIdx.x; i < 2 * kAcTile + 2 * kAcPitch; i += blockDim.x) tiles[i] = 0.f;
   __syncthreads();
-  const int nw = ac_windows(Lw, kAcWindow), first = ac_first(Lw, kAcWindow);
+  const int nw = ac_windows(Lw, 7), first = ac_first(Lw, 7);
   const int ntile = nw * ((min(kAcRows, Lmax + 1 - row0) + kAcGroup - 1) / kAcGroup);
   auto stage = [&](int t) {
     if (t < ntile) {
@@ -1379,7 +1391,7 @@ __global__ void __launch_bounds__(32 * kAcWarps, 1) kde_lscv_ac_sets_kernel(
   float2 D1[2], th[2], tl[2], e0[2];
   int lo = 0;
   unsigned span = 0, sign = 0;
-  const int S = ac_window(row0, gr.L1);
+  const int shift = ac_shift(row0, gr.L1), S = 1 << shift;
   for (int t = 0; t < ntile; ++t) {
     const int h = t / nw, w0 = (first + t - h * nw) * kAcWindow, r0 = row0 + kAcGroup * h;
     const float* tile = tiles + (t & 1) * kAcTile;
@@ -1414,7 +1426,7 @@ __global__ void __launch_bounds__(32 * kAcWarps, 1) kde_lscv_ac_sets_kernel(
     }
     if (act && r0 <= gr.L0) {
       // the tile's windows, the support's first to its last
-      const int v0 = max(w0, ac_first(gr.L1, S) * S), v1 = min(w0 + kAcWindow - 1, gr.L1);
+      const int v0 = max(w0, ac_first(gr.L1, shift) * S), v1 = min(w0 + kAcWindow - 1, gr.L1);
       for (int v = v0; v <= v1; v += S) {
         const int i0 = max(0, (-gr.L1 - v) >> 3), i1 = min(S - 1, gr.L1 - v) >> 3;
         int l = v + 8 * i0 + c;
@@ -1564,6 +1576,18 @@ __global__ void __launch_bounds__(256) kde_lscv_ac_reduce_kernel(
   lscv_out[o] = s1 * nk[1] - nk[2] * (s0 - nk[0] * kn[4 * (int64_t)i]);
 }
 
+// S(A) from a matrix's class sums, stride apart.
+__device__ __forceinline__ double ac_class_sum(const AcGen<float>& g, const AcPair* c, int64_t stride) {
+  AcPair v[kAcClasses];
+#pragma unroll
+  for (int k = 0; k < kAcClasses; ++k) v[k] = c[k * stride];
+#pragma unroll
+  for (int off = kAcClasses / 2; off > 0; off >>= 1)
+#pragma unroll
+    for (int k = 0; k < off; ++k) v[k] = ac_add(v[k], v[k + off]);
+  return g.L0 < 0 ? nan("") : 2.0 * (double)g.C * ac_value(v[0]);
+}
+
 // ---------------------------------------------------------------------------
 // Candidates of the learned proposal built and scored on the device: for
 // dataset s, candidate j < J is the network's theta_s clipped to a box plus
@@ -1639,32 +1663,54 @@ __global__ void __launch_bounds__(32) kde_theta_gen_kernel(ThetaArgs t) {
   if (h == 0) t.K0[m >> 1] = C;
 }
 
-// A block takes up to kThetaCands candidates of one dataset (two matrices
-// each): S(A) = sum over the support of K_A(delta o l) R(l), kAcRows lag rows
-// staged in shared memory at a time, their groups dealt out to the warps and
-// added as kde_lscv_ac_kernel's are; NaN for a matrix that does not fit the
-// plan.  Bound by the exponentials and their arithmetic (256 datasets of 28
-// candidates with supports near the box's widest: 336 M terms, 67 us at 16
-// exponentials a clock and SM).
+// A block takes up to nc <= kThetaCands candidates of one dataset (two matrices
+// each) and every nr-th unit of eight lag rows (nr divides kAcClasses): S(A) =
+// sum over the support of K_A(delta o l) R(l), the rows staged in shared memory
+// a unit at a time, their groups dealt out to the warps and added as
+// kde_lscv_ac_kernel's are, the units in the classes of
+// kde_lscv_ac_reduce_kernel (classes: [class][matrix] over 2 C; with nr = 1 the
+// block adds them, S).  NaN for a matrix that does not fit the plan.  Few
+// datasets take fewer candidates and rows a block, so that every SM has work:
+// one dataset of 28 candidates 78 us with seven and all rows a block, 6 now.
+// 256 datasets of 28 candidates of 12 to 130 lags (116 M terms) take 165 us: a
+// group has six terms a lane on average, and its setup and sum cost about as
+// much as they do.
 constexpr int kThetaCands = 7;
-constexpr int kThetaThreads = 32 * kThetaCands;
+constexpr int kThetaThreads = 256;
+// Blocks of nsets x cands candidates: nc to a block (as many as leave ten
+// blocks an SM with the rows split eight ways), nr blocks to their rows.
+struct ThetaSplit {
+  int nc, nr;
+};
+ThetaSplit theta_split(int64_t nsets, int64_t cands, int sms) {
+  const int64_t want = 10 * (int64_t)sms;
+  ThetaSplit p{1, 1};
+  while (p.nc < kThetaCands && nsets * cands * kAcClasses >= (p.nc + 1) * want) ++p.nc;
+  const int64_t blocks = nsets * ((cands + p.nc - 1) / p.nc);
+  while (p.nr < kAcClasses && blocks * p.nr < want) p.nr *= 2;
+  return p;
+}
 // L1max: an upper bound of the supports along axis 1.
 __global__ void __launch_bounds__(kThetaThreads) kde_lscv_theta_sums_kernel(
-    const AcGen<float>* __restrict__ gens, int per, const float* __restrict__ Rall, int P1,
-    int64_t set_stride, int L1max, int held, double* __restrict__ S) {
+    const AcGen<float>* __restrict__ gens, int per, int nc, const float* __restrict__ Rall, int P1,
+    int64_t set_stride, int L1max, int held, int64_t nmat, AcPair* __restrict__ classes,
+    double* __restrict__ S) {
   extern __shared__ __align__(16) float tile[];
   __shared__ AcGen<float> gs[2 * kThetaCands];
   __shared__ int off[2 * kThetaCands + 1];
+  __shared__ AcPair cls[2 * kThetaCands][kAcClasses];
   float* turn = tile + kAcRows * ac_pitch(L1max);
   AcPair* sums = ac_sums(turn, held);
   const int tid = threadIdx.x;
-  const int ngroups = (per + 2 * kThetaCands - 1) / (2 * kThetaCands), set = blockIdx.x / ngroups;
-  const int first = 2 * kThetaCands * (blockIdx.x - set * ngroups);
-  const int nm = min(2 * kThetaCands, per - first);
-  gens += (int64_t)set * per + first;
-  S += (int64_t)set * per + first;
+  const int ngroups = (per + 2 * nc - 1) / (2 * nc), set = blockIdx.x / ngroups;
+  const int first = 2 * nc * (blockIdx.x - set * ngroups);
+  const int nm = min(2 * nc, per - first);
+  const int64_t mat = (int64_t)set * per + first;
   const float* __restrict__ R = Rall + (int64_t)set * set_stride;
-  if (tid < nm) gs[tid] = gens[tid];
+  if (tid < nm) {
+    gs[tid] = gens[mat + tid];
+    for (int k = 0; k < kAcClasses; ++k) cls[tid][k] = AcPair{0.f, 0.f};
+  }
   __syncthreads();
   int L0 = -1, L1 = 0;
   for (int m = 0; m < nm; ++m)
@@ -1672,8 +1718,7 @@ __global__ void __launch_bounds__(kThetaThreads) kde_lscv_theta_sums_kernel(
       L0 = max(L0, gs[m].L0);
       L1 = max(L1, gs[m].L1);
     }
-  AcPair sum{0.f, 0.f};
-  for (int row0 = 0; row0 <= L0; row0 += kAcRows) {
+  for (int row0 = kAcRows * blockIdx.y; row0 <= L0; row0 += kAcRows * gridDim.y) {
     ac_stage(tile, R, P1, row0, min(kAcRows, L0 + 1 - row0), L1);
     if (tid < 32) ac_offsets(gs, nm, row0, off);
     ac_staged();
@@ -1681,21 +1726,30 @@ __global__ void __launch_bounds__(kThetaThreads) kde_lscv_theta_sums_kernel(
     __syncthreads();
     if (tid < nm) {
       AcPair v{0.f, 0.f};
-  #pragma unroll 4
-    for (int j = off[tid]; j < off[tid + 1]; ++j) v = ac_add(v, sums[j]);
-      sum = ac_add(sum, v);
+#pragma unroll 4
+      for (int j = off[tid]; j < off[tid + 1]; ++j) v = ac_add(v, sums[j]);
+      AcPair& c = cls[tid][row0 / kAcRows % kAcClasses];
+      c = ac_add(c, v);
     }
     __syncthreads();   // off is written again
   }
-  if (tid < nm) S[tid] = gs[tid].L0 < 0 ? nan("") : 2.0 * (double)gs[tid].C * ac_value(sum);
+  if (tid >= nm) return;
+  if (gridDim.y == 1) {
+    S[mat + tid] = ac_class_sum(gs[tid], cls[tid], 1);
+  } else {
+    for (int k = blockIdx.y; k < kAcClasses; k += gridDim.y) classes[k * nmat + mat + tid] = cls[tid][k];
+  }
 }
 
-// One warp per dataset: LSCV of its J + 1 candidates (optionally stored),
+// One warp per dataset: LSCV of its J + 1 candidates (optionally stored; S, or
+// with classes not null the sums' classes),
 // the first index of the smallest among the first J (a candidate that does
 // not fit counts as +inf) and out[s] = {that index, its LSCV, the reference
 // candidate's LSCV, that candidate's theta}.
 __global__ void __launch_bounds__(32) kde_lscv_theta_pick_kernel(ThetaArgs t,
                                                                  const double* __restrict__ S,
+                                                                 const AcPair* __restrict__ classes,
+                                                                 int64_t nmat,
                                                                  double* __restrict__ lscv,
                                                                  double* __restrict__ out) {
   const int J = t.J;
@@ -1708,7 +1762,8 @@ __global__ void __launch_bounds__(32) kde_lscv_theta_pick_kernel(ThetaArgs t,
   double ref = HUGE_VAL;
   for (int j = threadIdx.x; j <= J; j += 32) {
     const int64_t c = (int64_t)s * (J + 1) + j;
-    const double s1 = S[2 * c], s2 = S[2 * c + 1];
+    const double s1 = classes ? ac_class_sum(t.gens[2 * c], classes + 2 * c, nmat) : S[2 * c];
+    const double s2 = classes ? ac_class_sum(t.gens[2 * c + 1], classes + 2 * c + 1, nmat) : S[2 * c + 1];
     double v = s2 / (n * n) - 2.0 * (s1 - n * K0[c]) / (n * (n - 1.0));
     if (isnan(v)) v = HUGE_VAL;
     if (lscv) lscv[c] = v;
@@ -3328,7 +3383,8 @@ extern "C" kde_status kde_lscv_autocorr_cands_batch(kde_lscv_cands cands, int ns
 // Workspace of kde_lscv_theta_select: the uploaded n, reference thetas and
 // offsets; the candidates' parameters, K_H(0) and pair sums.
 struct ThetaLayout {
-  size_t off_up, off_gens, off_K0, off_S, total;
+  size_t off_up, off_gens, off_K0, off_S, off_cls, total;
+  ThetaSplit split;
 };
 
 static ThetaLayout theta_layout(int64_t nsets, int64_t J) {
@@ -3339,7 +3395,9 @@ static ThetaLayout theta_layout(int64_t nsets, int64_t J) {
   L.off_gens = up((size_t)(nsets + 3 * nsets + 3 * J) * sizeof(double));
   L.off_K0 = L.off_gens + up((size_t)2 * cands * sizeof(AcGen<float>));
   L.off_S = L.off_K0 + up((size_t)cands * sizeof(double));
-  L.total = L.off_S + up((size_t)2 * cands * sizeof(double));
+  L.off_cls = L.off_S + up((size_t)2 * cands * sizeof(double));
+  L.split = theta_split(nsets, J + 1, num_sms());
+  L.total = L.off_cls + (L.split.nr > 1 ? up((size_t)2 * cands * kAcClasses * sizeof(AcPair)) : 0);
   return L;
 }
 
@@ -3414,6 +3472,7 @@ extern "C" kde_status kde_lscv_theta_select(kde_plan plan, int nsets, const int6
   t.gens = (AcGen<float>*)(ws + L.off_gens);
   t.K0 = (double*)(ws + L.off_K0);
   double* S = (double*)(ws + L.off_S);
+  AcPair* cls = L.split.nr > 1 ? (AcPair*)(ws + L.off_cls) : nullptr;
   const int64_t nmat = (int64_t)nsets * 2 * (J + 1);
   {
     LaunchScope ls("kde_theta_gen_kernel", st);
@@ -3424,19 +3483,20 @@ extern "C" kde_status kde_lscv_theta_select(kde_plan plan, int nsets, const int6
     // a candidate's support that fits has L_1 <= P_1 - M_1, and never more than
     // M_1 - 1 (the padding alone can be far wider than any support)
     const int L1 = (int)std::min(I.P[1] - I.M[1], I.M[1] - 1);
-    const size_t smem = ac_block_smem(L1, 2 * kThetaCands, kThetaThreads);
+    const ThetaSplit sp = L.split;
+    const size_t smem = ac_block_smem(L1, 2 * sp.nc, kThetaThreads);
     if ((e = allow_smem(kde_lscv_theta_sums_kernel)) != cudaSuccess)
       return cuda_fail(e, "cudaFuncSetAttribute");
     LaunchScope ls("kde_lscv_theta_sums_kernel", st);
-    kde_lscv_theta_sums_kernel<<<(unsigned)((int64_t)nsets * ((J + kThetaCands) / kThetaCands)),
-                                 kThetaThreads, smem, st>>>(t.gens, 2 * (J + 1), (const float*)R,
-                                                            (int)I.P[1], (int64_t)I.P[0] * I.P[1], L1,
-                                                            ac_turn(L1, 2 * kThetaCands, kThetaThreads), S);
+    kde_lscv_theta_sums_kernel<<<dim3((unsigned)((int64_t)nsets * ((J + sp.nc) / sp.nc)), (unsigned)sp.nr),
+                                 kThetaThreads, smem, st>>>(
+        t.gens, 2 * (J + 1), sp.nc, (const float*)R, (int)I.P[1], (int64_t)I.P[0] * I.P[1], L1,
+        ac_turn(L1, 2 * sp.nc, kThetaThreads), nmat, cls, S);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_theta_sums_kernel");
   }
   {
     LaunchScope ls("kde_lscv_theta_pick_kernel", st);
-    kde_lscv_theta_pick_kernel<<<nsets, 32, 0, st>>>(t, S, lscv, out);
+    kde_lscv_theta_pick_kernel<<<nsets, 32, 0, st>>>(t, S, cls, nmat, lscv, out);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_lscv_theta_pick_kernel");
   }
   return KDE_OK;
