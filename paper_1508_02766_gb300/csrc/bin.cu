@@ -412,7 +412,6 @@ __device__ __forceinline__ bool axis_node(T x, const BinAxis<T>& a, int& i, unsi
 // 64-bit shared atomic is six times slower here), exact for the at most
 // kPrivSamples = 2^15 samples between two flushes.  The blocks start their
 // flush at different cells, so that they do not queue on the same ones.
-constexpr int kPrivThreads = 512;
 constexpr int kPrivSamples = 1 << 15;
 constexpr int kPrivCells = 24576;      // 192 KB of sums
 static_assert(2ll * kPrivCells * 4 <= 227 * 1024 - 1024, "private counts fit in shared memory");
@@ -420,7 +419,7 @@ static_assert(2ll * kPrivCells * 4 <= 227 * 1024 - 1024, "private counts fit in 
 // Words of one of the two sums (a multiple of 4: cleared as uint4).
 __host__ __device__ constexpr int priv_words(int64_t cells) { return (int)((cells + 3) & ~(int64_t)3); }
 
-template <typename T, int D>
+template <typename T, int D, int kPrivThreads>
 __global__ void __launch_bounds__(kPrivThreads)
 kde_bin_private_kernel(const T* __restrict__ X, int64_t n, int64_t chunk, BinParams<T> p,
                        unsigned long long* __restrict__ counts,
@@ -933,38 +932,56 @@ cudaError_t allow_smem(F* fn, size_t bytes) {
   return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// Grids whose sums leave room for one block an SM: twice the warps (28^3 cells,
+// FP32: 11.5 -> 9.4 us), and for FP32 samples a line of their own below.
+bool private_wide(int64_t cells) { return 2 * (size_t)priv_words(cells) * sizeof(unsigned) > 100 * 1024; }
+
 // Private counts where the grid fits and the samples are many for its cells.
-// The line per dimension is where the two kernels met for normal samples
-// (direct / private, us with the zeroing, FP32, graph of ten, GB300):
-//   d = 1: 2001 cells, 16e3 samples 3.9 / 3.3, 1e6 115 / 6.7, 5e6 567 / 12;
-//          20000 cells, 256e3 5.7 / 6.4, 1e6 16 / 8.6;
-//   d = 2: 64^2, 16e3 4.3 / 4.1, 1e6 109 / 8.9; 128^2, 64e3 4.7 / 6.8,
-//          256e3 10.8 / 6.8, 5e6 155 / 41;
-//   d = 3: 16^3, 16e3 9.2 / 5.3, 1e6 381 / 16; 28^3, 32e3 8.0 / 11,
-//          256e3 46 / 11, 5e6 861 / 69.
 // A block copies and flushes the whole grid whatever its samples, which is
-// what the line grows with; more corners per sample bring it down.
+// what the line grows with; more corners per sample bring it down.  Where it
+// lies is a matter of the samples: the direct kernel is slow where they crowd
+// (standard normal on [-6, 6]) and at its best where they spread (uniform).
+// The line is where a wrong choice costs the same factor either way, direct /
+// private in us with the zeroing (graph of five, GB300), normal then uniform:
+//   d = 1: 2001 cells, 32e3 FP32 5.8 / 3.3, 3.3 / 3.7; FP64 6.6 / 4.1, 4.1 / 4.1;
+//          20000 cells, 284e3 FP32 6.6 / 6.4, 5.3 / 6.6, 426e3 9.9 / 7.0, 7.4 / 7.4;
+//          FP64 284e3 12.3 / 7.8, 12.3 / 7.8;
+//   d = 2: 100^2, 84e3 FP32 11.5 / 5.7, 4.9 / 6.2; FP64 16 / 7.0, 9.4 / 7.4;
+//          150 x 160, 196e3 FP32 11.1 / 7.6, 6.6 / 8.2, 490e3 24 / 8.5, 12.2 / 10.3;
+//          FP64 17 / 10.5, 17 / 10.7;
+//   d = 3: 16^3, 16e3 FP32 9.0 / 5.4, 4.1 / 5.3; FP64 10.3 / 6.6, 5.7 / 6.6;
+//          28^3, 70e3 FP32 15 / 9.0, 5.8 / 10.2, 105e3 21 / 9.1, 6.2 / 10.2, 175e3
+//          33 / 9.4, 10.3 / 10.3; FP64 70e3 18 / 12.3, 11.5 / 13.5.
+template <typename T>
 bool use_private(int64_t n, int64_t cells, int d) {
-  const int64_t per_cell = d == 1 ? 14 : d == 2 ? 8 : 3;
+  const bool wide = sizeof(T) == 4 && private_wide(cells);
+  const int64_t per_cell = d == 1 ? (wide ? 20 : 14) : d == 2 ? 8 : wide ? 4 : 3;
   return cells <= kPrivCells && n >= 4096 + per_cell * cells;
 }
 
-template <typename T, int D>
-kde_status launch_private(const T* X, int64_t n, const BinParams<T>& p, unsigned long long* counts,
+template <typename T, int D, int kPrivThreads>
+kde_status launch_private_at(const T* X, int64_t n, const BinParams<T>& p, unsigned long long* counts,
                           unsigned long long* n_out, cudaStream_t stream) {
-  auto* fn = kde_bin_private_kernel<T, D>;
+  auto* fn = kde_bin_private_kernel<T, D, kPrivThreads>;
   const size_t smem = 2 * (size_t)priv_words(p.cells) * sizeof(unsigned);
   // the largest grid's, so that calls from several threads set the same limit
   cudaError_t e = allow_smem(fn, 2 * (size_t)priv_words(kPrivCells) * sizeof(unsigned));
   if (e != cudaSuccess) return kde::cuda_fail(e, "smem attr");
   const int64_t per = std::max<int64_t>(1024, p.cells / 8);
-  const int64_t cap = (int64_t)num_sms() * (smem <= 100 * 1024 ? 2 : 1);
+  const int64_t cap = (int64_t)num_sms() * (private_wide(p.cells) ? 1 : 2);
   const int64_t blocks = std::min(cap, (n + per - 1) / per);
   kde::LaunchScope ls("kde_bin_private_kernel", stream);
   e = kde::launch_pdl(fn, dim3((unsigned)blocks), dim3(kPrivThreads), smem, stream, X, n,
                       (n + blocks - 1) / blocks, p, counts, n_out);
   if (e == cudaSuccess) e = cudaGetLastError();
   return e == cudaSuccess ? KDE_OK : kde::cuda_fail(e, "kde_bin_private_kernel launch");
+}
+
+template <typename T, int D>
+kde_status launch_private(const T* X, int64_t n, const BinParams<T>& p, unsigned long long* counts,
+                          unsigned long long* n_out, cudaStream_t stream) {
+  return private_wide(p.cells) ? launch_private_at<T, D, 1024>(X, n, p, counts, n_out, stream)
+                               : launch_private_at<T, D, 512>(X, n, p, counts, n_out, stream);
 }
 
 template <typename T>
@@ -981,7 +998,7 @@ kde_status launch_direct(const T* X, int64_t n, int d, const double* lo, const d
   }
   if (n == 0) return KDE_OK;
   BinParams<T> p = make_params<T>(d, lo, hi, M, nullptr);
-  if (use_private(n, cells, d)) {
+  if (use_private<T>(n, cells, d)) {
     switch (d) {
       case 1: return launch_private<T, 1>(X, n, p, counts, n_out, stream);
       case 2: return launch_private<T, 2>(X, n, p, counts, n_out, stream);

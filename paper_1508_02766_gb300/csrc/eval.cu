@@ -3687,9 +3687,8 @@ __global__ void __launch_bounds__(256) kde_batch_bin_kernel(BatchArgs<T> a) {
 // grids: the binning 325 us by direct adds alone, 156 + 61 with these (event
 // times); side by side on the plan's two streams the batch takes 661 us, one
 // after the other 699, by direct adds alone 829.
-constexpr int kBatchPrivThreads = 512;
 constexpr int kBatchPrivCells[2] = {6144, 24576};   // 48 and 192 KB of sums
-template <typename T>
+template <typename T, int kBatchPrivThreads>
 __global__ void __launch_bounds__(kBatchPrivThreads)
 kde_batch_bin_private_kernel(BatchArgs<T> a, int pass) {
   extern __shared__ __align__(16) unsigned priv_sm[];
@@ -4247,11 +4246,12 @@ kde_status batch_eval_impl(kde_batch_plan_s* bp, const void* X, void* density, v
   for (int cls = 0; cls < 2; ++cls) {
     const int total = bp->wstart[(size_t)(BP_PBIN + cls) * (c + 1) + c];
     if (total == 0) continue;
-    auto* fn = kde_batch_bin_private_kernel<T>;
-    if ((e = allow_smem(fn)) != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
     const size_t smem = 2 * (size_t)((bp->priv_cells[cls] + 3) & ~3) * sizeof(unsigned);
+    const bool wide = smem > 100 * 1024;   // one block an SM: twice the warps
+    auto* fn = wide ? kde_batch_bin_private_kernel<T, 1024> : kde_batch_bin_private_kernel<T, 512>;
+    if ((e = allow_smem(fn)) != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
     LaunchScope ls("kde_batch_bin_private_kernel", bp->side);
-    fn<<<total, kBatchPrivThreads, smem, bp->side>>>(a, BP_PBIN + cls);
+    fn<<<total, wide ? 1024 : 512, smem, bp->side>>>(a, BP_PBIN + cls);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "kde_batch_bin_private_kernel");
   }
   e = cudaEventRecord(bp->join, bp->side);
