@@ -125,6 +125,13 @@ const float2* twiddles(const kde_plan_s* plan, int k) {
   return reinterpret_cast<const float2*>((const char*)plan->tw_dev + plan->tw_offset[k]);
 }
 
+// Planes with a line above kMaxNamedP take the wide constants on every axis.
+bool wide_constants(const kde_plan_info& I) {
+  for (int k = 0; k < I.d; ++k)
+    if (I.P[k] > fxp::kMaxNamedP) return true;
+  return false;
+}
+
 // Row pass: SRC_COUNTS (counts rows -> half spectra), SRC_KGEN (kernel-grid
 // rows -> half spectra) or the inverse (half spectra -> rows, cropped).
 // Batched bandwidths of one launch (grid.y = bandwidth): per-bandwidth
@@ -167,7 +174,7 @@ kde_status rows_pass(const kde_plan_s* plan, int kind, int64_t nrows, const long
                       sizeof(float2);
   if (smem > kSmemMax) return fail(KDE_ERR_UNSUPPORTED, "two-phase row block too large");
   const Launch l{a.ln.N1, a.ln.N2, a.ln.N3, dim3((unsigned)((pairs + a.B - 1) / a.B), (unsigned)bt.nh),
-                 threads, smem, st};
+                 threads, smem, st, wide_constants(I)};
   if (kind == 2) {
     LaunchScope ls("kde_fx_rows_c2r_kernel", st);
     return done(half ? launch_rows_c2r_even(l, RowsEvenArgs{a, half, (int)I.P[0]}) : launch_rows_c2r(l, a),
@@ -232,7 +239,8 @@ kde_status cols_pass(const kde_plan_s* plan, int k, const char* name, const floa
   const size_t smem = ((size_t)a.ln.N1 * a.SK + (MODE == COL_KMID && !a.ln.N3 ? (size_t)B * a.ln.P : 0)) *
                       sizeof(float2);
   if (smem > kSmemMax) return fail(KDE_ERR_UNSUPPORTED, "two-phase column block too large");
-  const Launch l{a.ln.N1, a.ln.N2, a.ln.N3, dim3((unsigned)((lines + B - 1) / B), (unsigned)O), threads, smem, st};
+  const Launch l{a.ln.N1, a.ln.N2, a.ln.N3, dim3((unsigned)((lines + B - 1) / B), (unsigned)O),
+                 threads, smem, st, wide_constants(I)};
   LaunchScope ls(name, st);
   cudaError_t e;
   switch (MODE) {
@@ -271,7 +279,7 @@ kde_status slab_pass(const kde_plan_s* plan, bool fwd, const long long* counts, 
   a.ex_elems = g.ex_elems;
   a.status = plan->status_dev;
   const Launch l{a.lr.N1, a.lr.N2, 0, dim3((unsigned)(I.M[0] * kSlabC)), g.threads,
-                 (size_t)(fwd ? g.smem_fwd : g.smem_inv), st};
+                 (size_t)(fwd ? g.smem_fwd : g.smem_inv), st, false};
   if (fwd) {
     LaunchScope ls("kde_fx_slab_fwd_kernel", st);
     return done(launch_slab_fwd(l, a), "kde_fx_slab_fwd_kernel");

@@ -35,45 +35,45 @@ constexpr int threads_per_line3() {
 // ---- shared phase bodies on one line's exchange buffer --------------------
 
 // Phase A forward: x (N1 values of thread n23) -> slots (k1, n23).
-template <int N1, int N2, int N3>
+template <int N1, int N2, int N3, bool WIDE>
 __device__ __forceinline__ void p3_a_fwd(float2 (&x)[N1], int n23, const float2* __restrict__ tw,
                                          float2* line, int SK, int SJ) {
-  dft<N1>(x);
+  dft<N1, WIDE>(x);
   line[n23 * SJ] = x[0];
 #pragma unroll
   for (int k1 = 1; k1 < N1; ++k1) line[k1 * SK + n23 * SJ] = cmul(x[k1], __ldg(tw + n23 * k1));
 }
 
 // Phase B forward on thread (k1, n3): slots (k1, n3 + N3 n2) in place.
-template <int N1, int N2, int N3>
+template <int N1, int N2, int N3, bool WIDE>
 __device__ __forceinline__ void p3_b_fwd(int k1, int n3, const float2* __restrict__ tw, float2* line,
                                          int SK, int SJ) {
   float2* base = line + k1 * SK + n3 * SJ;
   float2 y[N2];
 #pragma unroll
   for (int n2 = 0; n2 < N2; ++n2) y[n2] = base[N3 * n2 * SJ];
-  dft<N2>(y);
+  dft<N2, WIDE>(y);
   base[0] = y[0];
 #pragma unroll
   for (int k2 = 1; k2 < N2; ++k2) base[N3 * k2 * SJ] = cmul(y[k2], __ldg(tw + N1 * n3 * k2));
 }
 
 // Phase C forward on thread (k1, k2): z[k3] = X[k1 + N1 (k2 + N2 k3)].
-template <int N1, int N2, int N3>
+template <int N1, int N2, int N3, bool WIDE>
 __device__ __forceinline__ void p3_c_fwd(float2 (&z)[N3], int k1, int k2, const float2* line, int SK,
                                          int SJ) {
   const float2* base = line + k1 * SK + N3 * k2 * SJ;
 #pragma unroll
   for (int n3 = 0; n3 < N3; ++n3) z[n3] = base[n3 * SJ];
-  dft<N3>(z);
+  dft<N3, WIDE>(z);
 }
 
 // Phase C inverse on thread (k1, k2): z[k3] = X[k1 + N1 (k2 + N2 k3)] ->
 // slots (k1, n3 + N3 k2).
-template <int N1, int N2, int N3>
+template <int N1, int N2, int N3, bool WIDE>
 __device__ __forceinline__ void p3_c_inv(float2 (&z)[N3], int k1, int k2,
                                          const float2* __restrict__ tw, float2* line, int SK, int SJ) {
-  idft<N3>(z);
+  idft<N3, WIDE>(z);
   float2* base = line + k1 * SK + N3 * k2 * SJ;
   base[0] = z[0];
 #pragma unroll
@@ -82,14 +82,14 @@ __device__ __forceinline__ void p3_c_inv(float2 (&z)[N3], int k1, int k2,
 
 // Phase B inverse on thread (k1, n3): slots (k1, n3 + N3 k2) in place, the
 // value for n2 times e^{+2 pi i (n3 + N3 n2) k1 / P}.
-template <int N1, int N2, int N3>
+template <int N1, int N2, int N3, bool WIDE>
 __device__ __forceinline__ void p3_b_inv(int k1, int n3, const float2* __restrict__ tw, float2* line,
                                          int SK, int SJ) {
   float2* base = line + k1 * SK + n3 * SJ;
   float2 y[N2];
 #pragma unroll
   for (int k2 = 0; k2 < N2; ++k2) y[k2] = base[N3 * k2 * SJ];
-  idft<N2>(y);
+  idft<N2, WIDE>(y);
 #pragma unroll
   for (int n2 = 0; n2 < N2; ++n2) {
     const int n23 = n3 + N3 * n2;
@@ -98,12 +98,12 @@ __device__ __forceinline__ void p3_b_inv(int k1, int n3, const float2* __restric
 }
 
 // Phase A inverse on thread n23: x[n1] = value at position n23 + N23 n1.
-template <int N1, int N2, int N3>
+template <int N1, int N2, int N3, bool WIDE>
 __device__ __forceinline__ void p3_a_inv(float2 (&x)[N1], int n23, const float2* line, int SK,
                                          int SJ) {
 #pragma unroll
   for (int k1 = 0; k1 < N1; ++k1) x[k1] = line[k1 * SK + n23 * SJ];
-  idft<N1>(x);
+  idft<N1, WIDE>(x);
 }
 
 // Slot of X[k] after phase C (rows): k1 = k mod N1, k2, k3 from k / N1.
@@ -114,7 +114,7 @@ __device__ __forceinline__ int p3_slot(int k, int SK) {
 }
 
 // ---- rows ------------------------------------------------------------------
-template <int N1, int N2, int N3, int SRC>
+template <int N1, int N2, int N3, int SRC, bool WIDE>
 __global__ void __launch_bounds__(kThreads3)
 kde_fx3_rows_fwd_kernel(RowsArgs a, const long long* __restrict__ counts, KGen<float> g) {
   pdl_trigger();
@@ -152,20 +152,20 @@ kde_fx3_rows_fwd_kernel(RowsArgs a, const long long* __restrict__ counts, KGen<f
 #pragma unroll
         for (int n1 = 0; n1 < N1; ++n1) x[n1] = stage[n23 + N23 * n1];
       }
-      p3_a_fwd<N1, N2, N3>(x, n23, a.tw, fx_sm + b * LS, SK, 1);
+      p3_a_fwd<N1, N2, N3, WIDE>(x, n23, a.tw, fx_sm + b * LS, SK, 1);
     }
   }
   __syncthreads();
   if (t < a.B * N1 * N3) {  // phase B
     const int b = t / (N1 * N3), r = t - b * (N1 * N3);
-    p3_b_fwd<N1, N2, N3>(r / N3, r % N3, a.tw, fx_sm + b * LS, SK, 1);
+    p3_b_fwd<N1, N2, N3, WIDE>(r / N3, r % N3, a.tw, fx_sm + b * LS, SK, 1);
   }
   __syncthreads();
   if (t < a.B * N1 * N2) {  // phase C, results back to the slots
     const int b = t / (N1 * N2), r = t - b * (N1 * N2);
     const int k1 = r % N1, k2 = r / N1;
     float2 z[N3];
-    p3_c_fwd<N1, N2, N3>(z, k1, k2, fx_sm + b * LS, SK, 1);
+    p3_c_fwd<N1, N2, N3, WIDE>(z, k1, k2, fx_sm + b * LS, SK, 1);
     float2* base = fx_sm + b * LS + k1 * SK + N3 * k2;
 #pragma unroll
     for (int k3 = 0; k3 < N3; ++k3) base[k3] = z[k3];
@@ -189,7 +189,7 @@ kde_fx3_rows_fwd_kernel(RowsArgs a, const long long* __restrict__ counts, KGen<f
   }
 }
 
-template <int N1, int N2, int N3, bool EVEN>
+template <int N1, int N2, int N3, bool EVEN, bool WIDE>
 __global__ void __launch_bounds__(kThreads3) kde_fx3_rows_c2r_kernel(C2rArgs<EVEN> a) {
   pdl_trigger();
   pdl_wait();
@@ -217,13 +217,13 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_rows_c2r_kernel(C2rArgs<EVE
         const float2 Y = two ? __ldg(x1 + kk) : make_float2(0.f, 0.f);
         z[k3] = lo ? make_float2(X.x - Y.y, X.y + Y.x) : make_float2(X.x + Y.y, Y.x - X.y);
       }
-      p3_c_inv<N1, N2, N3>(z, k1, k2, a.tw, fx_sm + b * LS, SK, 1);
+      p3_c_inv<N1, N2, N3, WIDE>(z, k1, k2, a.tw, fx_sm + b * LS, SK, 1);
     }
   }
   __syncthreads();
   if (t < a.B * N1 * N3) {
     const int b = t / (N1 * N3), r = t - b * (N1 * N3);
-    p3_b_inv<N1, N2, N3>(r / N3, r % N3, a.tw, fx_sm + b * LS, SK, 1);
+    p3_b_inv<N1, N2, N3, WIDE>(r / N3, r % N3, a.tw, fx_sm + b * LS, SK, 1);
   }
   __syncthreads();
   if (t < a.B * N23) {
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_rows_c2r_kernel(C2rArgs<EVE
     if (r0 < a.nrows) {
       const bool two = r0 + 1 < a.nrows;
       float2 x[N1];
-      p3_a_inv<N1, N2, N3>(x, n23, fx_sm + b * LS, SK, 1);
+      p3_a_inv<N1, N2, N3, WIDE>(x, n23, fx_sm + b * LS, SK, 1);
       float *m0, *m1 = nullptr, *o0 = c2r_row<EVEN>(a, r0, &m0),
                  *o1 = two ? c2r_row<EVEN>(a, r0 + 1, &m1) : nullptr;
 #pragma unroll
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_rows_c2r_kernel(C2rArgs<EVE
 
 // ---- columns: W = 2^lgB adjacent columns, column index fastest; entry
 // (column c, k1, j) at c + j W + k1 SK ------------------------------------------
-template <int N1, int N2, int N3, int MODE>
+template <int N1, int N2, int N3, int MODE, bool WIDE>
 __global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kernel(ColsArgs a) {
   pdl_trigger();
   pdl_wait();
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kernel(ColsArgs a) {
         z[k3] = v ? __ldg(in) : make_float2(0.f, 0.f);
         in += step;
       }
-      p3_c_inv<N1, N2, N3>(z, k1, k2, a.tw, line, SK, W);
+      p3_c_inv<N1, N2, N3, WIDE>(z, k1, k2, a.tw, line, SK, W);
     }
   } else {
     if (r < N23) {  // phase A
@@ -320,15 +320,15 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kernel(ColsArgs a) {
           }
         }
       }
-      p3_a_fwd<N1, N2, N3>(x, n23, a.tw, line, SK, W);
+      p3_a_fwd<N1, N2, N3, WIDE>(x, n23, a.tw, line, SK, W);
     }
     __syncthreads();
-    if (r < N1 * N3) p3_b_fwd<N1, N2, N3>(r / N3, r % N3, a.tw, line, SK, W);
+    if (r < N1 * N3) p3_b_fwd<N1, N2, N3, WIDE>(r / N3, r % N3, a.tw, line, SK, W);
     __syncthreads();
     if (r < N1 * N2) {  // phase C
       const int k1 = r % N1, k2 = r / N1;
       float2 z[N3];
-      p3_c_fwd<N1, N2, N3>(z, k1, k2, line, SK, W);
+      p3_c_fwd<N1, N2, N3, WIDE>(z, k1, k2, line, SK, W);
       if constexpr (MODE == COL_FWD) {
         const int64_t s = first + c;
         if (s < a.S) {
@@ -366,19 +366,19 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kernel(ColsArgs a) {
             z[k3].y *= kpre[k3];
           }
         }
-        p3_c_inv<N1, N2, N3>(z, k1, k2, a.tw, line, SK, W);
+        p3_c_inv<N1, N2, N3, WIDE>(z, k1, k2, a.tw, line, SK, W);
       }
     }
   }
   if constexpr (MODE == COL_MID || MODE == COL_AUTO || MODE == COL_INV) {
     __syncthreads();
-    if (r < N1 * N3) p3_b_inv<N1, N2, N3>(r / N3, r % N3, a.tw, line, SK, W);
+    if (r < N1 * N3) p3_b_inv<N1, N2, N3, WIDE>(r / N3, r % N3, a.tw, line, SK, W);
     __syncthreads();
     if (r < N23) {
       const int64_t s = first + c;
       if (s < a.S) {
         float2 x[N1];
-        p3_a_inv<N1, N2, N3>(x, r, line, SK, W);
+        p3_a_inv<N1, N2, N3, WIDE>(x, r, line, SK, W);
         float2* out = a.out + s + (int64_t)r * a.S;
         const int64_t step = (int64_t)N23 * a.S;
 #pragma unroll
@@ -419,12 +419,12 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kmid_kernel(KmidArgs a
     float2 x[N1];
 #pragma unroll
     for (int n1 = 0; n1 < N1; ++n1) x[n1] = col_pair(a, r + N23 * n1, P, s, v0, v1);
-    p3_a_fwd<N1, N2, N3>(x, r, a.tw, line, SK, W);
+    p3_a_fwd<N1, N2, N3, false>(x, r, a.tw, line, SK, W);
   }
   __syncthreads();
-  if (r < N1 * N3) p3_b_fwd<N1, N2, N3>(r / N3, r % N3, a.tw, line, SK, W);
+  if (r < N1 * N3) p3_b_fwd<N1, N2, N3, false>(r / N3, r % N3, a.tw, line, SK, W);
   __syncthreads();
-  if (vc) p3_c_fwd<N1, N2, N3>(z, k1, k2, line, SK, W);
+  if (vc) p3_c_fwd<N1, N2, N3, false>(z, k1, k2, line, SK, W);
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     if (vc) {
@@ -434,18 +434,18 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_cols_kmid_kernel(KmidArgs a
         cv[k3].x *= k;
         cv[k3].y *= k;
       }
-      p3_c_inv<N1, N2, N3>(cv, k1, k2, a.tw, line, SK, W);
+      p3_c_inv<N1, N2, N3, false>(cv, k1, k2, a.tw, line, SK, W);
       if (h == 0) {
 #pragma unroll
         for (int k3 = 0; k3 < N3; ++k3) cv[k3] = v1 ? __ldg(pc + half + k3 * step) : make_float2(0.f, 0.f);
       }
     }
     __syncthreads();
-    if (r < N1 * N3) p3_b_inv<N1, N2, N3>(r / N3, r % N3, a.tw, line, SK, W);
+    if (r < N1 * N3) p3_b_inv<N1, N2, N3, false>(r / N3, r % N3, a.tw, line, SK, W);
     __syncthreads();
     if (r < N23 && (h ? v1 : v0)) {
       float2 x[N1];
-      p3_a_inv<N1, N2, N3>(x, r, line, SK, W);
+      p3_a_inv<N1, N2, N3, false>(x, r, line, SK, W);
       float2* out = a.out + s + (h ? half : 0) + (int64_t)r * a.S;
       const int64_t ostep = (int64_t)N23 * a.S;
 #pragma unroll

@@ -14,6 +14,15 @@
 // (+-1, -+1) (a product with +-1 is exact, so each component is still one
 // rounded addition).  Every component is rounded as the scalar FP32
 // operation of the same form would be.
+//
+// WIDE: every constant as the sum of two floats.  An FP32 cosine or sine is
+// off by up to half an ulp, and those of the powers of two and three all round
+// down (1/sqrt 2 by 1.7e-8 of it, sqrt 3 / 2 by 1.8e-8, cos pi/8 by 3e-8), so
+// that each such factor shrinks the transform a little and lengths made of
+// them alone give densities 1e-7 too small, where fives and sevens even out.
+// Planes with a line above 2048 points, which only splits of that kind serve,
+// take it: 2017 x 3001 2.1e-7 -> 1.6e-7 rms against 64 bits (7-smooth lengths
+// 1.7e-7), 1 to 3% of their time.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -39,6 +48,19 @@ __device__ __forceinline__ float2 p_scale(float2 a, float c) { return __fmul2_rn
 __device__ __forceinline__ float2 p_fma(float2 a, float c, float2 acc) {
   return __ffma2_rn(a, make_float2(c, c), acc);
 }
+// a c and acc + a c for a constant c given in double
+template <bool WIDE>
+__device__ __forceinline__ float2 p_scale_c(float2 a, double c) {
+  const float hi = (float)c, lo = (float)(c - (double)hi);
+  if constexpr (WIDE) return p_fma(a, hi, p_scale(a, lo));
+  return p_scale(a, hi);
+}
+template <bool WIDE>
+__device__ __forceinline__ float2 p_fma_c(float2 a, double c, float2 acc) {
+  const float hi = (float)c, lo = (float)(c - (double)hi);
+  if constexpr (WIDE) return p_fma(a, hi, p_fma(a, lo, acc));
+  return p_fma(a, hi, acc);
+}
 // rot(b) = -i b (forward) or +i b (inverse); a + rot(b) and a - rot(b)
 template <bool INV>
 __device__ __forceinline__ float2 p_add_rot(float2 a, float2 b) {
@@ -51,7 +73,7 @@ __device__ __forceinline__ float2 p_sub_rot(float2 a, float2 b) {
 
 // x e^{-+2 pi i E / N} with the exponent known at compile time; quarter
 // turns are exact component moves and sign changes.
-template <int N, int E, bool INV>
+template <int N, int E, bool INV, bool WIDE>
 __device__ __forceinline__ float2 twiddle_mul(float2 x) {
   constexpr int e = E % N;
   if constexpr (e == 0) {
@@ -65,17 +87,25 @@ __device__ __forceinline__ float2 twiddle_mul(float2 x) {
     constexpr fxm::CS cs = fxm::cossin_2pi(e, N);
     constexpr float c = (float)cs.c, s = (float)cs.s;
     // forward x (c - i s) = (x.x c + x.y s, x.y c - x.x s); inverse with -s
-    const float2 t = __fmul2_rn(x, make_float2(c, c));
+    float2 t;
+    if constexpr (WIDE) {
+      constexpr float cl = (float)(cs.c - (double)c), sl = (float)(cs.s - (double)s);
+      t = __fmul2_rn(x, make_float2(cl, cl));
+      t = __ffma2_rn(make_float2(x.y, x.x), INV ? make_float2(-sl, sl) : make_float2(sl, -sl), t);
+      t = __ffma2_rn(x, make_float2(c, c), t);
+    } else {
+      t = __fmul2_rn(x, make_float2(c, c));
+    }
     return __ffma2_rn(make_float2(x.y, x.x), INV ? make_float2(-s, s) : make_float2(s, -s), t);
   }
 }
 
 // Length-R DFTs of the base radices.
-template <int R, bool INV>
+template <int R, bool INV, bool WIDE = false>
 struct BaseDFT;
 
-template <bool INV>
-struct BaseDFT<2, INV> {
+template <bool INV, bool WIDE>
+struct BaseDFT<2, INV, WIDE> {
   __device__ __forceinline__ static void run(float2* x) {
     const float2 a = x[0], b = x[1];
     x[0] = p_add(a, b);
@@ -83,8 +113,8 @@ struct BaseDFT<2, INV> {
   }
 };
 
-template <bool INV>
-struct BaseDFT<4, INV> {
+template <bool INV, bool WIDE>
+struct BaseDFT<4, INV, WIDE> {
   __device__ __forceinline__ static void run(float2* x) {
     const float2 t0 = p_add(x[0], x[2]), t1 = p_sub(x[0], x[2]);
     const float2 t2 = p_add(x[1], x[3]), d = p_sub(x[1], x[3]);
@@ -95,18 +125,18 @@ struct BaseDFT<4, INV> {
   }
 };
 
-template <bool INV>
-struct BaseDFT<8, INV> {
+template <bool INV, bool WIDE>
+struct BaseDFT<8, INV, WIDE> {
   __device__ __forceinline__ static void run(float2* x) {
-    constexpr float h = 0.70710678118654752440f;
+    constexpr double h = 0.70710678118654752440;
     float2 e[4] = {x[0], x[2], x[4], x[6]};
     float2 o[4] = {x[1], x[3], x[5], x[7]};
-    BaseDFT<4, INV>::run(e);
-    BaseDFT<4, INV>::run(o);
+    BaseDFT<4, INV, WIDE>::run(e);
+    BaseDFT<4, INV, WIDE>::run(o);
     // o_k times w_8^k, w_8 = e^{-+ i pi / 4}: (o_1 + rot o_1) / sqrt 2,
     // rot o_2, (rot o_3 - o_3) / sqrt 2
-    const float2 w1 = p_scale(p_add_rot<INV>(o[1], o[1]), h);
-    const float2 w3 = p_scale(p_sub_rot<INV>(o[3], o[3]), -h);
+    const float2 w1 = p_scale_c<WIDE>(p_add_rot<INV>(o[1], o[1]), h);
+    const float2 w3 = p_scale_c<WIDE>(p_sub_rot<INV>(o[3], o[3]), -h);
     x[0] = p_add(e[0], o[0]);
     x[4] = p_sub(e[0], o[0]);
     x[1] = p_add(e[1], w1);
@@ -121,7 +151,7 @@ struct BaseDFT<8, INV> {
 // Odd R: pair legs n and R - n; A_k = x_0 + sum_n (x_n + x_{R-n}) cos(2 pi n k / R),
 // B_k = sum_n (x_n - x_{R-n}) sin(2 pi n k / R); X_k = A_k + rot B_k,
 // X_{R-k} = A_k - rot B_k.
-template <int R, bool INV>
+template <int R, bool INV, bool WIDE>
 struct BaseDFT {
   static constexpr int H = (R - 1) / 2;
   __device__ __forceinline__ static void run(float2* x) {
@@ -156,29 +186,28 @@ struct BaseDFT {
                                                  float2& B) {
     if constexpr (N <= H) {
       constexpr fxm::CS cs = fxm::cossin_2pi((long long)N * K, R);
-      constexpr float c = (float)cs.c, s = (float)cs.s;
-      A = p_fma(sp[N - 1], c, A);
-      B = N == 1 ? p_scale(sm[0], s) : p_fma(sm[N - 1], s, B);
+      A = p_fma_c<WIDE>(sp[N - 1], cs.c, A);
+      B = N == 1 ? p_scale_c<WIDE>(sm[0], cs.s) : p_fma_c<WIDE>(sm[N - 1], cs.s, B);
       odd_sum<K, N + 1>(sp, sm, A, B);
     }
   }
 };
 
-template <int N, bool INV, int R = base_radix(N), bool BASE = is_base(N)>
+template <int N, bool INV, bool WIDE, int R = base_radix(N), bool BASE = is_base(N)>
 struct DFT;
 
-template <int N, bool INV, int R>
-struct DFT<N, INV, R, true> {
-  __device__ __forceinline__ static void run(float2* x) { BaseDFT<N, INV>::run(x); }
+template <int N, bool INV, bool WIDE, int R>
+struct DFT<N, INV, WIDE, R, true> {
+  __device__ __forceinline__ static void run(float2* x) { BaseDFT<N, INV, WIDE>::run(x); }
 };
 
-template <bool INV, int R>
-struct DFT<1, INV, R, false> {
+template <bool INV, bool WIDE, int R>
+struct DFT<1, INV, WIDE, R, false> {
   __device__ __forceinline__ static void run(float2*) {}
 };
 
-template <int N, bool INV, int R>
-struct DFT<N, INV, R, false> {
+template <int N, bool INV, bool WIDE, int R>
+struct DFT<N, INV, WIDE, R, false> {
   static constexpr int M = N / R;
   template <int r>
   __device__ __forceinline__ static void twiddle_row(float2 (&y)[R][M]) {
@@ -190,7 +219,7 @@ struct DFT<N, INV, R, false> {
   template <int r, int k>
   __device__ __forceinline__ static void twiddle_cols(float2 (&y)[R][M]) {
     if constexpr (k < M) {
-      y[r][k] = twiddle_mul<N, r * k, INV>(y[r][k]);
+      y[r][k] = twiddle_mul<N, r * k, INV, WIDE>(y[r][k]);
       twiddle_cols<r, k + 1>(y);
     }
   }
@@ -201,29 +230,29 @@ struct DFT<N, INV, R, false> {
 #pragma unroll
       for (int m = 0; m < M; ++m) y[r][m] = x[R * m + r];
 #pragma unroll
-    for (int r = 0; r < R; ++r) DFT<M, INV>::run(y[r]);
+    for (int r = 0; r < R; ++r) DFT<M, INV, WIDE>::run(y[r]);
     twiddle_row<1>(y);
 #pragma unroll
     for (int k = 0; k < M; ++k) {
       float2 t[R];
 #pragma unroll
       for (int r = 0; r < R; ++r) t[r] = y[r][k];
-      BaseDFT<R, INV>::run(t);
+      BaseDFT<R, INV, WIDE>::run(t);
 #pragma unroll
       for (int q = 0; q < R; ++q) x[k + M * q] = t[q];
     }
   }
 };
 
-template <int N>
+template <int N, bool WIDE = false>
 __device__ __forceinline__ void dft(float2* x) {
-  DFT<N, false>::run(x);
+  DFT<N, false, WIDE>::run(x);
 }
 
 // Unnormalised inverse: X_k = sum_n x_n e^{+2 pi i n k / N}.
-template <int N>
+template <int N, bool WIDE = false>
 __device__ __forceinline__ void idft(float2* x) {
-  DFT<N, true>::run(x);
+  DFT<N, true, WIDE>::run(x);
 }
 
 }  // namespace fx

@@ -772,10 +772,17 @@ kde_fx_cols_kmid_kernel(KmidArgs a) {
 // Launch of the kernel for the split (N1, N2): the one compiled for it if it
 // is in the list, else the generic kernel for factors up to 20.
 #define KDE_FX_DISPATCH(KERNEL_T, ...)                                                   \
+  if (l.n3 && l.wide) {                                                                \
+    switch (l.n1 * 4096 + l.n2 * 64 + l.n3) {                                          \
+      KDE_FX_TRIPLES(KDE_FX_CASE_WIDE)                                                 \
+      KDE_FX_LONG_TRIPLES(KDE_FX_CASE_WIDE)                                            \
+      default:                                                                         \
+        return cudaErrorInvalidConfiguration;                                          \
+    }                                                                                  \
+  }                                                                                    \
   if (l.n3) {                                                                          \
     switch (l.n1 * 4096 + l.n2 * 64 + l.n3) {                                          \
       KDE_FX_TRIPLES(KDE_FX_CASE_TRIPLE)                                               \
-      KDE_FX_LONG_TRIPLES(KDE_FX_CASE_TRIPLE)                                          \
       default:                                                                         \
         return cudaErrorInvalidConfiguration;                                          \
     }                                                                                  \
@@ -808,6 +815,7 @@ struct Launch {
   int threads;
   size_t smem;
   cudaStream_t st;
+  bool wide;       // wide transform constants (fx_dft.cuh)
 };
 
 cudaError_t launch_rows_counts(const Launch& l, const RowsArgs& a, const long long* counts);

@@ -13,7 +13,11 @@ cudaError_t launch_cols_kmid(const Launch& l, const KmidArgs& a) {
 #define KDE_FX_CASE_TRIPLE(n1, n2, n3)  \
   case n1 * 4096 + n2 * 64 + n3:       \
     return launch_kernel(kde_fx3_cols_kmid_kernel<n1, n2, n3>, l.grid, l.threads, l.smem, l.st, a);
+#define KDE_FX_CASE_WIDE(n1, n2, n3)  \
+  case n1 * 4096 + n2 * 64 + n3:       \
+    return cudaErrorInvalidConfiguration;
   KDE_FX_DISPATCH(KDE_FX_KERNEL, a)
+#undef KDE_FX_CASE_WIDE
 #undef KDE_FX_CASE_TRIPLE
 #undef KDE_FX_CASE_PAIR
 #undef KDE_FX_KERNEL

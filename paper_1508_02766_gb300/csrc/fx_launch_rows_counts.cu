@@ -12,8 +12,12 @@ cudaError_t launch_rows_counts(const Launch& l, const RowsArgs& a, const long lo
     return launch_kernel(KDE_FX_KERNEL(n1, n2), l.grid, l.threads, l.smem, l.st, a, counts, KGen<float>{});
 #define KDE_FX_CASE_TRIPLE(n1, n2, n3)  \
   case n1 * 4096 + n2 * 64 + n3:       \
-    return launch_kernel(kde_fx3_rows_fwd_kernel<n1, n2, n3, SRC_COUNTS>, l.grid, l.threads, l.smem, l.st, a, counts, KGen<float>{});
+    return launch_kernel(kde_fx3_rows_fwd_kernel<n1, n2, n3, SRC_COUNTS, false>, l.grid, l.threads, l.smem, l.st, a, counts, KGen<float>{});
+#define KDE_FX_CASE_WIDE(n1, n2, n3)  \
+  case n1 * 4096 + n2 * 64 + n3:       \
+    return launch_kernel(kde_fx3_rows_fwd_kernel<n1, n2, n3, SRC_COUNTS, true>, l.grid, l.threads, l.smem, l.st, a, counts, KGen<float>{});
   KDE_FX_DISPATCH(KDE_FX_KERNEL, a, counts, KGen<float>{})
+#undef KDE_FX_CASE_WIDE
 #undef KDE_FX_CASE_TRIPLE
 #undef KDE_FX_CASE_PAIR
 #undef KDE_FX_KERNEL

@@ -12,8 +12,12 @@ cudaError_t launch_rows_kgen(const Launch& l, const RowsArgs& a, const KGen<floa
     return launch_kernel(KDE_FX_KERNEL(n1, n2), l.grid, l.threads, l.smem, l.st, a, (const long long*)nullptr, g);
 #define KDE_FX_CASE_TRIPLE(n1, n2, n3)  \
   case n1 * 4096 + n2 * 64 + n3:       \
-    return launch_kernel(kde_fx3_rows_fwd_kernel<n1, n2, n3, SRC_KGEN>, l.grid, l.threads, l.smem, l.st, a, (const long long*)nullptr, g);
+    return launch_kernel(kde_fx3_rows_fwd_kernel<n1, n2, n3, SRC_KGEN, false>, l.grid, l.threads, l.smem, l.st, a, (const long long*)nullptr, g);
+#define KDE_FX_CASE_WIDE(n1, n2, n3)  \
+  case n1 * 4096 + n2 * 64 + n3:       \
+    return launch_kernel(kde_fx3_rows_fwd_kernel<n1, n2, n3, SRC_KGEN, true>, l.grid, l.threads, l.smem, l.st, a, (const long long*)nullptr, g);
   KDE_FX_DISPATCH(KDE_FX_KERNEL, a, (const long long*)nullptr, g)
+#undef KDE_FX_CASE_WIDE
 #undef KDE_FX_CASE_TRIPLE
 #undef KDE_FX_CASE_PAIR
 #undef KDE_FX_KERNEL
