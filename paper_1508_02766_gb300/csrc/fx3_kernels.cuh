@@ -230,18 +230,13 @@ __global__ void __launch_bounds__(kThreads3) kde_fx3_rows_c2r_kernel(C2rArgs<EVE
     const int b = t / N23, n23 = t - b * N23;
     const int64_t r0 = 2 * ((int64_t)blockIdx.x * a.B + b);
     if (r0 < a.nrows) {
-      const bool two = r0 + 1 < a.nrows;
       float2 x[N1];
       p3_a_inv<N1, N2, N3, WIDE>(x, n23, fx_sm + b * LS, SK, 1);
-      float *m0, *m1 = nullptr, *o0 = c2r_row<EVEN>(a, r0, &m0),
-                 *o1 = two ? c2r_row<EVEN>(a, r0 + 1, &m1) : nullptr;
+      const C2rOut<EVEN> out(a, r0, r0 + 1 < a.nrows);
 #pragma unroll
       for (int n1 = 0; n1 < N1; ++n1) {
         const int pos = n23 + N23 * n1;
-        if (pos < a.Mout) {
-          c2r_store<EVEN>(o0, m0, pos, a.Mout, x[n1].x);
-          if (two) c2r_store<EVEN>(o1, m1, pos, a.Mout, x[n1].y);
-        }
+        if (pos < a.Mout) out.store(pos, x[n1]);
       }
     }
   }

@@ -171,29 +171,44 @@ struct RowsEvenArgs : RowsArgs {
 template <bool EVEN>
 using C2rArgs = std::conditional_t<EVEN, RowsEvenArgs, RowsArgs>;
 
-// Where c2r row r goes: its output row (null: the mirror of an earlier row),
-// and (mirror) the row that takes it reversed, or null.  EVEN: its own
-// kernels, as the branches cost the others' stores 10%.
+// Stores of the c2r row pair r, r + 1 (two: the second exists), value by value.
+// EVEN: r is even inside its grid, so the pair is rows p, p + 1 of one grid and
+// its mirrors P0 - p, P0 - p - 1; the rest of the last pair is the mirror of an
+// earlier row.  The plain form keeps one pointer: with one a row the generic
+// kernel took 82 registers instead of 64 and 13.6 us instead of 9.7 at 128^3.
 template <bool EVEN>
-__device__ __forceinline__ float* c2r_row(const C2rArgs<EVEN>& a, int64_t r, float** mirror) {
-  *mirror = nullptr;
-  if constexpr (!EVEN) {
-    return a.out_real + r * a.Mout;
-  } else {
-    const int64_t grid = r / a.half;
-    const int p = (int)(r - grid * a.half);
-    if (2 * p > a.P0) return nullptr;
-    float* base = a.out_real + grid * (int64_t)a.P0 * a.Mout;
-    if (p > 0 && 2 * p < a.P0) *mirror = base + (int64_t)(a.P0 - p) * a.Mout;
-    return base + (int64_t)p * a.Mout;
+struct C2rOut {
+  float *row, *mirror;
+  int M;
+  bool w[2], q[2];
+  __device__ __forceinline__ C2rOut(const C2rArgs<EVEN>& a, int64_t r, bool two) {
+    M = a.Mout;
+    if constexpr (!EVEN) {
+      row = a.out_real + r * M;
+      w[0] = true;
+      w[1] = two;
+    } else {
+      const int64_t grid = r / a.half;
+      const int p = (int)(r - grid * a.half);
+      float* base = a.out_real + grid * (int64_t)a.P0 * M;
+      row = base + (int64_t)p * M;
+      mirror = base + (int64_t)(a.P0 - p) * M;
+      w[0] = 2 * p <= a.P0;
+      w[1] = two && 2 * (p + 1) <= a.P0;
+      q[0] = p > 0 && 2 * p < a.P0;
+      q[1] = two && 2 * (p + 1) < a.P0;
+    }
   }
-}
-// Value v at position pos of a row and, reversed, of its mirror.
-template <bool EVEN>
-__device__ __forceinline__ void c2r_store(float* row, float* mirror, int pos, int M, float v) {
-  if (!EVEN || row) row[pos] = v;
-  if (EVEN && mirror) mirror[pos ? M - pos : 0] = v;
-}
+  __device__ __forceinline__ void store(int pos, float2 v) const {
+    if (!EVEN || w[0]) row[pos] = v.x;
+    if (w[1]) row[M + pos] = v.y;
+    if constexpr (EVEN) {
+      const int back = pos ? M - pos : 0;
+      if (q[0]) mirror[back] = v.x;
+      if (q[1]) mirror[back - M] = v.y;
+    }
+  }
+};
 
 // Per-bandwidth view of the arguments (h = blockIdx.y).
 __device__ __forceinline__ void rows_slab(RowsArgs& a, KGen<float>& g) {
@@ -389,21 +404,16 @@ __device__ __forceinline__ void rows_a_inv(const C2rArgs<EVEN>& a, const float2*
   const int b = t / N2, n2 = t - b * N2;
   const int64_t r0 = 2 * ((int64_t)blockIdx.x * a.B + b);
   if (r0 >= a.nrows) return;
-  const bool two = r0 + 1 < a.nrows;
   const float2* src = sm + b * (N1 * a.SK) + n2;
   float2 x[N1];
 #pragma unroll
   for (int k1 = 0; k1 < N1; ++k1) x[k1] = src[k1 * a.SK];
   idft<N1>(x);
-  float *m0, *m1 = nullptr, *o0 = c2r_row<EVEN>(a, r0, &m0),
-             *o1 = two ? c2r_row<EVEN>(a, r0 + 1, &m1) : nullptr;
+  const C2rOut<EVEN> out(a, r0, r0 + 1 < a.nrows);
 #pragma unroll
   for (int n1 = 0; n1 < N1; ++n1) {
     const int pos = n2 + N2 * n1;
-    if (pos < a.Mout && KDE_DCHECK(r0 < a.nrows, KDE_DBG_ROWS_STORE)) {
-      c2r_store<EVEN>(o0, m0, pos, a.Mout, x[n1].x);
-      if (two) c2r_store<EVEN>(o1, m1, pos, a.Mout, x[n1].y);
-    }
+    if (pos < a.Mout && KDE_DCHECK(r0 < a.nrows, KDE_DBG_ROWS_STORE)) out.store(pos, x[n1]);
   }
 }
 
