@@ -1306,7 +1306,20 @@ constexpr int kAcQuad = 4, kAcSets = 16, kAcPitch = 20;
 constexpr int kAcWarps = 16;
 constexpr int kAcTurn = kAcQuad * kAcSets + 4;   // pitch of the turned chains
 constexpr int kAcSlab = 256;     // datasets per launch
-constexpr int kAcMinSets = 8;    // fewer are scored one by one
+// Fewer datasets are scored one by one, and so are few work units: an item of
+// the product takes as long for one dataset as for sixteen (18 us + 0.4 a lag of
+// its widest support), and few items leave SMs idle, where a (unit, dataset)
+// pair one by one takes 2.1 ns + 0.004 a lag.  One by one / product, us with
+// the reduction: 343 candidates up to 30 lags (2e3 units) 32 / 36 with 7 / 8
+// datasets, 32 up to 60 lags (340 units) 32 / 47 with 24, 46 / 47 with 64, 32 up
+// to 190 lags (1100 units) 52 / 94 with 12, 78 / 95 with 24, 4 of them 45 / 69
+// with 64.
+constexpr int kAcMinSets = 8;
+bool ac_product(int ns, int nunits, int nitems, int L1, int sms) {
+  const int64_t blocks = (int64_t)nitems * ((ns + kAcSets - 1) / kAcSets);
+  return ns >= kAcMinSets && (int64_t)nunits * ns * (2.1 + 0.004 * L1) >
+                                 (double)((blocks + sms - 1) / sms) * (18000.0 + 400.0 * L1);
+}
 constexpr int kAcTile = kAcGroup * kAcWindow * kAcPitch;
 constexpr size_t kAcSetsSmem =
     sizeof(float) * (2 * kAcTile + 2 * kAcPitch + (size_t)kAcWarps * 32 * kAcTurn);
@@ -3289,7 +3302,6 @@ extern "C" kde_status kde_lscv_autocorr_cands(kde_lscv_cands cands, int64_t n, c
 // a slab of datasets one FP64 partial per work unit of the largest chunk.
 struct CandsBatch {
   int slab;            // datasets per launch
-  bool product;        // batched sums (else the datasets one by one)
   size_t off_part, total;
 };
 
@@ -3297,11 +3309,7 @@ static CandsBatch cands_batch_layout(const kde_lscv_cands_s* c, int nsets) {
   auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
   int units = 0;
   CandsBatch b{};
-  b.product = nsets >= kAcMinSets;
-  for (const auto& ch : c->chunks) {
-    units = std::max(units, ch.sh.nunits);
-    b.product = b.product && ch.groups;
-  }
+  for (const auto& ch : c->chunks) units = std::max(units, ch.sh.nunits);
   b.slab = std::min(nsets, kAcSlab);
   b.off_part = up((size_t)nsets * sizeof(NTerms));
   b.total = b.off_part + up((size_t)b.slab * units * sizeof(double));
@@ -3366,7 +3374,7 @@ extern "C" kde_status kde_lscv_autocorr_cands_batch(kde_lscv_cands cands, int ns
     for (const auto& ch : cands->chunks) {
       double* S = pair_sums ? pair_sums + 2 * (y * nH + ch.c0) : nullptr;
       double* out = lscv + y * nH + ch.c0;
-      if (lay.product)
+      if (ch.groups && ac_product(ns, ch.sh.nunits, ch.nitems, ch.sh.L1, num_sms()))
         s = ac_product_chunk(I, ch, (const float*)R + y * per, ns, (AcPair*)partial, nset + y, nH, S, out, st);
       else if (I.precision == KDE_F32)
         s = ac_launch_chunk<float>(I, ch.dev, ch.nh, ch.sh, (const float*)R + y * per, ns, partial,
