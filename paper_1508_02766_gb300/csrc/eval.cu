@@ -931,7 +931,7 @@ struct AcGen {
 // kernel below, so that a candidate's score does not depend on how many
 // datasets are scored with it or on how the work is spread:
 //   chain   the lags l_1 = c (mod 8) of one row inside one window [S w, S (w +
-//           1)), ascending, in FP32: S = 2^ac_shift(first row, L_1), S / 8 terms;
+//           1)), ascending, in FP32: S = 2^ac_shift(first row, L_0, L_1), S / 8 terms;
 //   group   the 4 x 8 chains of four rows (first row a multiple of four), in
 //           order of 8 (row mod 4) + c, as a pair of FP32 (AcPair: the sum and
 //           the sum of its rounding errors);
@@ -944,18 +944,20 @@ struct AcGen {
 // of the additions alone, rms over random bandwidths (x 1e-9), with chains
 // through eight rows and a FP32 tree / with a warp's row sums added in FP32 and
 // the lanes in FP64 (what the widths below are held against) / now: supports
-// of 39 x 39 lags 27 / 4.9 / 2.3, 120 x 120 21 / 2.8 / 2.8, 7 x 2000 1100 / 41
-// / 3, 27 x 70 - / 4.5 / 2.1, 7 x 32 - / 4.6 / 4.7, 10 x 10 52 / 8.2 / 5.4.
+// of 39 x 39 lags 31 / 4.9 / 3.2, 120 x 120 22 / 2.4 / 1.8, 7 x 2000 1000 / 39
+// / 5, 27 x 70 36 / 4.4 / 4.1, 7 x 32 43 / 5.3 / 5.1, 10 x 10 45 / 8.3 / 5.6; over
+// 60 random shapes 0.39 of the second on average.
 constexpr int kAcChunk = 1024;
 constexpr int kAcRows = 8;
 constexpr int kAcGroup = 4;       // rows of a group
 constexpr int kAcWindow = 128;    // widest window
-// Width of the windows: short chains in the first unit, which holds the
-// largest terms and with a support of few rows is all there is (every unit at
-// 64 lags: 1.5 times the error at 5 x 48 lags); about sixteen a side at least.
-// (The windows' log2, so that nothing is divided.)
-__host__ __device__ constexpr int ac_shift(int row0, int L1) {
-  int b = row0 ? 7 : 4;
+// Width of the windows, as its log2 (nothing is divided): 64 lags, chains of
+// eight terms, but short chains in the first unit, which holds the largest
+// terms, of a support of few rows, where it is nearly all there is (64 lags
+// there too: 1.5 times the error at 5 x 48 lags); and sixteen windows a side
+// at most, up to 128 lags wide.
+__host__ __device__ constexpr int ac_shift(int row0, int L0, int L1) {
+  int b = row0 == 0 && L0 < 24 ? 4 : 6;
   while (b < 7 && (16 << b) < L1) ++b;
   return b;
 }
@@ -1122,7 +1124,7 @@ __device__ __forceinline__ void ac_offsets(const AcGen<float>* gs, int nm, int r
   const int lane = threadIdx.x & 31;
   int v = 0;
   if (lane < nm && row0 <= gs[lane].L0)
-    v = (kAcRows / kAcGroup) * ac_windows(gs[lane].L1, ac_shift(row0, gs[lane].L1));
+    v = (kAcRows / kAcGroup) * ac_windows(gs[lane].L1, ac_shift(row0, gs[lane].L0, gs[lane].L1));
 #pragma unroll
   for (int d = 1; d < 32; d *= 2) {
     const int u = __shfl_up_sync(0xffffffffu, v, d);
@@ -1146,7 +1148,7 @@ __device__ __forceinline__ void ac_groups(const AcGen<float>* gs, const int* off
       if (w > last) {   // the next set of four rows, or where the run begins
         while (off[m + 1] <= t + k) ++m;
         g = gs[m];
-        b = ac_shift(row0, g.L1);
+        b = ac_shift(row0, g.L0, g.L1);
         const int first = ac_first(g.L1, b), j = t + k - off[m];
         last = g.L1 >> b;
         const int nw = last - first + 1, h = j >= nw;
@@ -1248,9 +1250,9 @@ __host__ __device__ constexpr size_t ac_block_smem(int L1, int matrices, int thr
          (size_t)(threads / 32) * ac_turn(L1, matrices, threads) * kAcTurn1 * sizeof(float) +
          (size_t)matrices * ac_unit_groups(L1) * sizeof(AcPair) + sizeof(AcPair);
 }
-static_assert(ac_windows(KDE_MAX_P / 2 - 1, 7) <= 33 && ac_windows(256, ac_shift(0, 256)) <= 33 &&
-                  ac_windows(512, ac_shift(0, 512)) <= 33 && ac_windows(1024, ac_shift(0, 1024)) <= 33 &&
-                  ac_shift(0, 1025) == 7,
+static_assert(ac_windows(KDE_MAX_P / 2 - 1, 7) <= 33 && ac_windows(256, ac_shift(0, 0, 256)) <= 33 &&
+                  ac_windows(512, ac_shift(0, 0, 512)) <= 33 && ac_windows(1024, ac_shift(8, 8, 1024)) <= 33 &&
+                  ac_shift(8, 8, 1025) == 7,
               "windows of a row");
 static_assert(ac_block_smem(KDE_MAX_P / 2 - 1, kAcBlock, kAcThreads) + 4096 <= kSmemMax,
               "the widest support's rows and groups fit in shared memory");
@@ -1298,10 +1300,16 @@ __global__ void __launch_bounds__(kAcThreads) kde_lscv_ac_kernel(
 // block stages in shared memory kAcWindow lags of four rows at a time
 // (datasets innermost, so that a lane's kAcSets values are four 16-byte loads;
 // the pitch of 20 words keeps them free of bank conflicts) for its 16 warps,
-// the next window's copies in flight.  After a window each warp turns its 64 x
+// the next tile's copies in flight.  After a window each warp turns its 64 x
 // 32 chains through shared memory, so that a lane adds the 32 chains of two
 // sums.  A lane outside the support reads a slot of zeros, so that a value
-// that does not count is never touched.
+// that does not count is never touched.  256 datasets x 2016 matrices of 5 to
+// 108 lags (1.8 G terms, 49 us at the FP32 rate): 392 us, 3172 one by one.  Its
+// shared memory moves as much for the chains' ends as for the terms, half of
+// its rate with the four warps a scheduler that 64 sums a lane leave.  Tried: a
+// thread 4 x 4 or 8 x 4 sums with the kernel values formed in shared memory,
+// chains ending in registers (446 us: a third of its instructions are the ends
+// of short chains, and an item of 190 lags alone takes 310).
 constexpr int kAcQuad = 4, kAcSets = 16, kAcPitch = 20;
 constexpr int kAcWarps = 16;
 constexpr int kAcTurn = kAcQuad * kAcSets + 4;   // pitch of the turned chains
@@ -1325,7 +1333,8 @@ constexpr size_t kAcSetsSmem =
     sizeof(float) * (2 * kAcTile + 2 * kAcPitch + (size_t)kAcWarps * 32 * kAcTurn);
 static_assert(kAcSetsSmem <= kSmemMax, "tiles and turned chains fit in shared memory");
 
-// The matrices of one warp: the same L_1, falling L_0 (m[0]'s the largest).
+// The matrices of one warp: the same L_1 and windows, falling L_0 (m[0]'s the
+// largest).
 struct AcGroup {
   int m[kAcQuad];   // matrix or -1
   int L0, L1;
@@ -1404,7 +1413,7 @@ __global__ void __launch_bounds__(32 * kAcWarps, 1) kde_lscv_ac_sets_kernel(
   float2 D1[2], th[2], tl[2], e0[2];
   int lo = 0;
   unsigned span = 0, sign = 0;
-  const int shift = ac_shift(row0, gr.L1), S = 1 << shift;
+  const int shift = ac_shift(row0, gr.L0, gr.L1), S = 1 << shift;
   for (int t = 0; t < ntile; ++t) {
     const int h = t / nw, w0 = (first + t - h * nw) * kAcWindow, r0 = row0 + kAcGroup * h;
     const float* tile = tiles + (t & 1) * kAcTile;
@@ -3199,7 +3208,8 @@ static void cands_group(const std::vector<AcGen<T>>& gens, std::vector<AcGroup>&
     g.L0 = gens[order[i]].L0;
     g.L1 = gens[order[i]].L1;
     for (int k = 0; k < kAcQuad; ++k) {
-      const bool same = i < order.size() && gens[order[i]].L1 == g.L1;
+      const bool same = i < order.size() && gens[order[i]].L1 == g.L1 &&
+                        ac_shift(0, gens[order[i]].L0, g.L1) == ac_shift(0, g.L0, g.L1);
       g.m[k] = same ? order[i++] : -1;
     }
     groups.push_back(g);
