@@ -952,12 +952,13 @@ constexpr int kAcRows = 8;
 constexpr int kAcGroup = 4;       // rows of a group
 constexpr int kAcWindow = 128;    // widest window
 // Width of the windows, as its log2 (nothing is divided): 64 lags, chains of
-// eight terms, but short chains in the first unit, which holds the largest
-// terms, of a support of few rows, where it is nearly all there is (64 lags
-// there too: 1.5 times the error at 5 x 48 lags); and sixteen windows a side
-// at most, up to 128 lags wide.
+// eight terms; 128 lags for supports above 256, where a row had as many terms
+// to a lane before (60 x 165 lags 3.1 / 2.2 with 64, 3.7 with 128; 60 x 400 6.1 /
+// 1.6, 3.1); and short ones, but at most sixteen a side, in the first unit, which
+// holds the largest terms, of a support of few rows, where it is nearly all
+// there is (5 x 48 lags 5.2 / 8.1 with 64, 4.3 with 16).
 __host__ __device__ constexpr int ac_shift(int row0, int L0, int L1) {
-  int b = row0 == 0 && L0 < 24 ? 4 : 6;
+  int b = row0 == 0 && L0 < 24 ? 4 : L1 > 256 ? 7 : 6;
   while (b < 7 && (16 << b) < L1) ++b;
   return b;
 }
@@ -1064,24 +1065,24 @@ __device__ __forceinline__ float ac_chain(const AcGen<float>& g, const AcLane& a
   const float2 step = make_float2(16.f, 16.f);
   const int i0 = max(0, (-g.L1 - w0) >> 3), i1 = min(S - 1, g.L1 - w0) >> 3;
   if (r0 > 0 && r0 + kAcGroup - 1 <= g.L0) {   // whole rows: only the ends can lie outside
-    auto end = [&](int i) {
-      const int l = w0 + 8 * i + c;
-      const float2 k = terms(make_float2((float)l, 0.f));
-      if ((unsigned)(l - a.lo) <= a.span) acc = fmaf(k.x, a.x[l], acc);
-    };
+    int l = w0 + 8 * i0 + c;
+    const float* x = a.x + l;
+    float2 f = make_float2((float)l, (float)(l + 8));
     int i = i0;
-    const int last = w0 + 8 * i1 + 7 > g.L1 ? i1 - 1 : i1;
-    if (w0 + 8 * i0 < -g.L1) end(i++);
-    const float* x = a.x + w0 + 8 * i + c;
-    float2 f = make_float2((float)(w0 + 8 * i + c), (float)(w0 + 8 * i + c + 8));
-#pragma unroll 4
-    for (; i < last; i += 2, x += 16) {
+    auto pair = [&](bool whole) {
       const float2 k = terms(f);
-      acc = fmaf(k.x, x[0], acc);
-      acc = fmaf(k.y, x[8], acc);
+      if (whole || (l >= -g.L1 && l <= g.L1)) acc = fmaf(k.x, x[0], acc);
+      if (whole || (i < i1 && l + 8 <= g.L1)) acc = fmaf(k.y, x[8], acc);
       f = __fadd2_rn(f, step);
-    }
-    for (; i <= i1; ++i) end(i);
+      l += 16;
+      x += 16;
+      i += 2;
+    };
+    const int last = w0 + 8 * i1 + 7 > g.L1 ? i1 - 1 : i1;
+    if (w0 + 8 * i0 < -g.L1) pair(false);
+#pragma unroll 4
+    while (i < last) pair(true);
+    while (i <= i1) pair(false);
     return acc;
   }
   int l = w0 + 8 * i0 + c;
@@ -1251,8 +1252,7 @@ __host__ __device__ constexpr size_t ac_block_smem(int L1, int matrices, int thr
          (size_t)matrices * ac_unit_groups(L1) * sizeof(AcPair) + sizeof(AcPair);
 }
 static_assert(ac_windows(KDE_MAX_P / 2 - 1, 7) <= 33 && ac_windows(256, ac_shift(0, 0, 256)) <= 33 &&
-                  ac_windows(512, ac_shift(0, 0, 512)) <= 33 && ac_windows(1024, ac_shift(8, 8, 1024)) <= 33 &&
-                  ac_shift(8, 8, 1025) == 7,
+                  ac_windows(512, ac_shift(0, 0, 512)) <= 33 && ac_windows(1024, ac_shift(0, 0, 1024)) <= 33,
               "windows of a row");
 static_assert(ac_block_smem(KDE_MAX_P / 2 - 1, kAcBlock, kAcThreads) + 4096 <= kSmemMax,
               "the widest support's rows and groups fit in shared memory");
@@ -1539,21 +1539,24 @@ __global__ void __launch_bounds__(256) kde_lscv_ac_reduce_kernel(
   const AcPart<T>*p0 = partial + (int64_t)g0->u0 * ns + y, *p1 = partial + (int64_t)g1->u0 * ns + y;
   AcPart<T> v[2] = {};
   if constexpr (MANY) {
-    AcPart<T> c[2][kAcClasses] = {};
-    for (int j = 0; j < max(nu0, nu1); j += kAcClasses)
 #pragma unroll
-      for (int k = 0; k < kAcClasses; ++k) {
-        c[0][k] = ac_add(c[0][k], j + k < nu0 ? p0[(int64_t)(j + k) * ns] : AcPart<T>{});
-        c[1][k] = ac_add(c[1][k], j + k < nu1 ? p1[(int64_t)(j + k) * ns] : AcPart<T>{});
+    for (int h = 0; h < 2; ++h) {
+      const AcPart<T>* ph = h ? p1 : p0;
+      const int nu = h ? nu1 : nu0;
+      AcPart<T> c[kAcClasses] = {};
+      for (int j = 0; j < nu; j += kAcClasses) {
+        AcPart<T> a[kAcClasses];   // loads in flight
+#pragma unroll
+        for (int k = 0; k < kAcClasses; ++k) a[k] = j + k < nu ? ph[(int64_t)(j + k) * ns] : AcPart<T>{};
+#pragma unroll
+        for (int k = 0; k < kAcClasses; ++k) c[k] = ac_add(c[k], a[k]);
       }
 #pragma unroll
-    for (int off = kAcClasses / 2; off > 0; off >>= 1)
+      for (int off = kAcClasses / 2; off > 0; off >>= 1)
 #pragma unroll
-      for (int k = 0; k < off; ++k)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) c[h][k] = ac_add(c[h][k], c[h][k + off]);
-    v[0] = c[0][0];
-    v[1] = c[1][0];
+        for (int k = 0; k < off; ++k) c[k] = ac_add(c[k], c[k + off]);
+      v[h] = c[0];
+    }
   } else {
     __shared__ AcPart<T> part[2][kAcClasses][kScores];
     for (int j = p; j < max(nu0, nu1); j += 8 * kAcClasses) {
@@ -1698,7 +1701,7 @@ __global__ void __launch_bounds__(32) kde_theta_gen_kernel(ThetaArgs t) {
 // group has six terms a lane on average, and its setup and sum cost about as
 // much as they do.
 constexpr int kThetaCands = 7;
-constexpr int kThetaThreads = 256;
+constexpr int kThetaThreads = 128;
 // Blocks of nsets x cands candidates: nc to a block (as many as leave ten
 // blocks an SM with the rows split eight ways), nr blocks to their rows.
 struct ThetaSplit {
