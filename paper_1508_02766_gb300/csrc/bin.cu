@@ -137,12 +137,13 @@ __device__ __forceinline__ void corner_weights(const unsigned* q, unsigned long 
 // ---------------------------------------------------------------------------
 // Direct path.
 // ---------------------------------------------------------------------------
-// A pair of adjacent lanes takes one sample: lane parity p adds the 2^(D-1)
-// corners at offset p along the last axis.  Corners (.., j) and (.., j + 1)
+// A pair of adjacent lanes adds one sample's corners: lane parity p the
+// 2^(D-1) at offset p along the last axis.  Corners (.., j) and (.., j + 1)
 // are adjacent 8-byte words, in one 32-byte sector unless j = 3 mod 4, so
 // each warp instruction's lane pairs coalesce into one sector request where
 // one lane per sample would issue two: the scattered-sector rate of the L2
-// is what bounds this kernel.
+// is what bounds these adds.
+
 // The corners of lane parity par of a sample at (i, q) into counts.
 template <typename T, int D>
 __device__ __forceinline__ void add_corners(const int* i, const unsigned* q, int par,

@@ -141,7 +141,7 @@ struct Batch {
   int nh = 1;
   const KGen<float>* gens = nullptr;
   const int* L0 = nullptr;
-  int64_t slab_in = 0, slab_out = 0, slab_real = 0, slab_K = 0;
+  int64_t slab_in = 0, slab_out = 0, slab_real = 0;
 };
 
 kde_status rows_pass(const kde_plan_s* plan, int kind, int64_t nrows, const long long* counts,
@@ -207,7 +207,6 @@ kde_status cols_pass(const kde_plan_s* plan, int k, const char* name, const floa
     a.slab_in = bt->slab_in;
     a.slab_out = bt->slab_out;
     a.slab_real = bt->slab_real;
-    a.slab_K = bt->slab_K;
   } else {   // outer slabs of a 3-D pass: [O][Nin][S] in, [O][Nout or P][S] out
     a.slab_in = (int64_t)Nin * S;
     a.slab_out = (int64_t)(MODE == COL_FWD ? (int)I.P[k] : Nout) * S;
@@ -224,7 +223,9 @@ kde_status cols_pass(const kde_plan_s* plan, int k, const char* name, const floa
   a.tw = twiddles(plan, k);
   const int64_t lines = (MODE == COL_FWD_REAL || MODE == COL_KMID ? (S + 1) / 2 : S);
   // lines per block over all slabs: at least 4 adjacent columns (a 32-byte
-  // sector per row; fewer make every load a partial sector), at most 16
+  // sector per row; fewer make every load a partial sector) where the block's
+  // threads allow, which lines of more than 128 threads (most three-factor
+  // splits above 1100 points) do not: two columns there; at most 16
   int B = std::max(4, pick_lines(lines * O, a.ln, true));
   while (B * threads_per_line(a.ln) > max_threads(a.ln)) B /= 2;
   while (B > 1 && B > lines) B /= 2;
@@ -426,7 +427,7 @@ kde_status fx_autocorr(kde_plan_s* plan, const long long* counts, float* R, floa
   if (s != KDE_OK) return s;
   // R is even: the inverse keeps rows 0 .. P_0 / 2, and the output rows store
   // each row's reverse too (256 grids of 256^2 padded to 448^2, event times:
-  // axis 0 133 -> 104 us, rows 91 -> 61 us)
+  // axis 0 133 -> 111 us, rows 91 -> 55 us)
   const int half = (int)std::min<int64_t>(I.P[0], (I.P[0] / 2 + 2) & ~(int64_t)1);
   s = cols_pass<COL_AUTO>(plan, 0, "kde_fx_cols_auto_kernel", A, B, nullptr, nullptr, I.Q, nsets,
                          (int)I.M[0], half, -1, st, nullptr, 2.3283064365386963e-10f,

@@ -462,6 +462,8 @@ struct ColsArgs {
   // 3-D pass, or batched bandwidths (in 0 when they share the input); with
   // h_L0 (batched kernel spectra) the input of slab h holds L0 + 1 rows (lags
   // 0 .. L0) with L0 = h_L0[h].
+  // slab_K: always 0 (every slab reads the same K); without the member and its
+  // use the 256^3 evaluation takes 180.3 us instead of 178.5.
   int64_t slab_in, slab_out, slab_real, slab_K;
   const int* h_L0;
   float s_pre, s_post;  // COL_AUTO scales
@@ -808,8 +810,12 @@ kde_fx_cols_kmid_kernel(KmidArgs a) {
 // Launchers, one translation unit each (fx_launch_*.cu, compiled in
 // parallel): kernel of size class cls (0: factors <= 20) on the stream.
 // ---------------------------------------------------------------------------
-// Every pass kernel starts with pdl_trigger(); pdl_wait(); so it may be
-// launched as a programmatic dependent of the kernel before it.
+// Every pass kernel may be launched as a programmatic dependent of the kernel
+// before it: it starts with pdl_trigger() and waits (pdl_wait) before it reads
+// anything that an earlier kernel wrote and before its own stores.  All wait at
+// once but the kernel-grid rows whose parameters are kernel arguments; those
+// read only the plan's twiddles, complete since the plan was made, and wait
+// before their store.
 template <typename Kern, typename... Args>
 cudaError_t launch_kernel(Kern* fn, dim3 grid, int threads, size_t smem, cudaStream_t st,
                           Args... args) {

@@ -300,10 +300,13 @@ const typename Cplx<T>::type* table(const kde_plan_s* plan) {
 // and the two transposes are about 5 us of it).
 template <typename T>
 constexpr int min_line() { return sizeof(T) == 8 ? 512 : 1536; }
-// Widest support of the cosine sums (their terms grow with L, the
-// transform's do not).  Transform against sums: FP64 L = 20 34 / 1.4 us (P =
-// 2025), L = 600 52 / 3.5 (P = 2625), L = 525 65 / 4.1 (P = 4032); FP32 6.2 /
-// 1.0, 7.0 / 1.2, 8.6 / 1.4.
+// Widest support of the cosine sums.  Their terms grow with L, the transform's
+// do not, but the two do not meet: transform against sums (us) FP64 L = 20 34 /
+// 1.4 (P = 2025), L = 600 52 / 3.5 (P = 2625), L = 1025 47 / 7.4 (P = 2560), L =
+// 2039 70 / 18 (P = 4096); FP32 6.2 / 1.0, 7.0 / 1.2, 7.4 / 2.5, 11.1 / 4.9.  The
+// line is where the FP32 sums' error has been held against the transform's
+// (level, over drawn cases); above it single supports went either way (4.1e-8 /
+// 7.0e-8 at L = 1700, 5.9e-8 / 2.5e-8 at 2039).
 constexpr int kMaxLags = 1024;
 
 }  // namespace
@@ -343,7 +346,7 @@ kde_status line1d_eval(const kde_plan_s* plan, const long long* counts, const T*
 }
 
 // The cosine-sum spectrum of a d = 1 plan; *taken = false for supports above
-// kMaxLags, where the one-block transform is the shorter.
+// kMaxLags.
 template <typename T>
 kde_status line1d_kernel_grid(const kde_plan_s* plan, const KGen<T>& gen, T* Kspec,
                               cudaStream_t st, bool* taken) {
