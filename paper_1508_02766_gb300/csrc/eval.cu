@@ -1340,7 +1340,7 @@ struct AcGroup {
   int L0, L1;
 };
 
-// Lags max(w0, -Lw) .. min(w0 + 63, Lw) of lag rows t0 .. t0 + nrow - 1 of
+// Lags max(w0, -Lw) .. min(w0 + kAcWindow - 1, Lw) of lag rows t0 .. t0 + nrow - 1 of
 // nset datasets into a tile (one committed group of 4-byte asynchronous
 // copies; no copy and no value for datasets beyond).
 __device__ __forceinline__ void ac_stage_sets(float* tile, const float* __restrict__ R, int P1,
