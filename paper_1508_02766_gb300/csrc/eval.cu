@@ -1230,6 +1230,10 @@ __global__ void __launch_bounds__(256) kde_lscv_ac64_kernel(const AcGen<double>*
 // one load's latency for 32 terms was most of the kernel.  The block's groups
 // are dealt out to its warps, their sums left in shared memory and added
 // there in order, so that a few wide supports keep every warp at work too.
+// The 2048 matrices of 1024 candidates at 512^2 take 31 us (24 with chains
+// through eight rows and a tree of shuffles, whose additions err ten times as
+// far): 72% of the issue slots, integer and comparison work 59% of its pipe,
+// exponentials 10%, shared memory 19%.
 constexpr int kAcBlock = 16;
 // Warps of a block: twice as many where the staged rows leave room for one
 // block an SM.
@@ -3705,9 +3709,10 @@ __global__ void __launch_bounds__(256) kde_batch_bin_kernel(BatchArgs<T> a) {
 // memory and added into the problem's counts once, as kde_bin_private_kernel
 // does (the same split sums, exact for the at most 2^15 samples of a chunk).
 // One block an item; 64 datasets of 10^3 to 10^6 samples on 64^2 to 1024^2
-// grids: the binning 325 us by direct adds alone, 156 + 61 with these (event
-// times); side by side on the plan's two streams the batch takes 661 us, one
-// after the other 699, by direct adds alone 829.
+// grids: the binning 325 us by direct adds alone, 145 + 66 with these (event
+// times); side by side on the plan's two streams the batch takes 656 us, one
+// after the other 699 and by direct adds alone 829 (with 512 threads a block,
+// 661 side by side).
 constexpr int kBatchPrivCells[2] = {6144, 24576};   // 48 and 192 KB of sums
 template <typename T, int kBatchPrivThreads>
 __global__ void __launch_bounds__(kBatchPrivThreads)
